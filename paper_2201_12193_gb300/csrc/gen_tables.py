@@ -469,13 +469,146 @@ def flop_count(dim):
     return n
 
 
+FX_VF = 60      # value coefficients of the fixed-point form: g 2^FX_VF, rounded
+
+
+def _fx_halves(x):
+    """round(x 2^FX_VF) as signed halves h 2^32 + l, |l| <= 2^31."""
+    v = int((x * (1 << FX_VF)).to_integral_value())
+    l = (v + (1 << 31)) % (1 << 32) - (1 << 31)
+    h = (v - l) >> 32
+    assert -(1 << 31) <= h < (1 << 31) and h * (1 << 32) + l == v
+    return h, l
+
+
+def fx_columns(dim, P):
+    """Per class, the s indices of the fixed-point form in its order: without the
+    target average's column (it works on the deviations from it: every row and
+    every q_l - u_5 vanishes on constants).  2D: class (0,1) in the order in
+    which it is the x <-> y image of class (1,0)."""
+    d4, basis, sl, bases, VP, RCP = P
+    cen = d4.index((0, 0, 0))
+    cols = {c: [sl[c][j] for j, r in enumerate(basis[c]) if not r[cen]] for c in parity_classes(dim)}
+    if dim == 2:
+        swap = [d4.index(({0: 0, 1: 2, 2: 1}[k], oy, ox)) for (k, ox, oy) in d4]
+        order = []
+        for r in basis[(1, 0)]:
+            img = [0] * len(d4)
+            for q, a in enumerate(r):
+                img[swap[q]] = a
+            order.append(sl[(0, 1)][basis[(0, 1)].index(img)])
+        cols[(0, 1)] = order
+    return cols
+
+
+def emit_fx(w, dim, P):
+    """The same reconstruction in block fixed point (hweno_fx.cuh)."""
+    d4, basis, sl, bases, VP, RCP = P
+    classes = parity_classes(dim)
+    n = len(d4)
+    cols = fx_columns(dim, P)
+    row_of = {sl[c][j]: r for c in classes for j, r in enumerate(basis[c])}
+    cname = {(0, 0): "a", (1, 0): "b", (0, 1): "c", (1, 1): "e"}
+    args = ", ".join(f"hwfx::Half2 (&{cname[c]})[{len(cols[c])}]" for c in classes)
+    cargs = ", ".join(f"const hwfx::Half2 (&{cname[c]})[{len(cols[c])}]" for c in classes)
+    w("\n// Fixed-point form, on the deviations from the target average (d of it is not read): the classes'\n")
+    w("// parity combinations" + ("; c is the x <-> y image of b" if dim == 2 else "") + ".\n")
+    w(f"__device__ __forceinline__ void fx_split{dim}d(const long long (&d)[{n}], {args}) {{\n")
+    for c in classes:
+        for k, j in enumerate(cols[c]):
+            r = row_of[j]
+            assert all(abs(a) <= 1 for a in r) and sum(abs(a) for a in r) <= 4
+            expr = " ".join(("+" if a > 0 else "-") + f" d[{q}]" for q, a in enumerate(r) if a)
+            expr = expr[2:] if expr.startswith("+ ") else "-" + expr[2:]
+            w(f"  {cname[c]}[{k}] = hwfx::halves({expr});\n")
+    w("}\n\n")
+    # rows of beta_l, per class: over the class's columns, levels in turn
+    def coef(lvl, c, b):
+        return {sl[c][j]: g.to_decimal() for j, g in enumerate(VP[(lvl, b, c)]) if g.a != 0 or g.b != 0}
+    if dim == 1:
+        npt = 4
+        w("// x[p] = (c2 q2 + c3 q3 + c4 q4)(point p) - (c2 + c3 + c4) u_5 in fixed point; ca = c2 + c3 weights the\n"
+          "// parts q2 and q3 share.\n")
+        w(f"__device__ __forceinline__ void fx_values1d({cargs}, hwfx::Half2 c2, hwfx::Half2 c3, hwfx::Half2 c4, "
+          f"hwfx::Half2 ca, long long (&x)[{npt}]) {{\n")
+        seen = {}
+        for bi, b in enumerate(bases):
+            for ci, cl in enumerate(classes):
+                names = {}
+                for lvl in (2, 3, 4):
+                    co = coef(lvl, cl, b)
+                    terms = [(k, co[j]) for k, j in enumerate(cols[cl]) if j in co]
+                    key = (cl,) + tuple((j, str(v)) for j, v in terms)
+                    if key not in seen:
+                        nm = seen[key] = f"q{lvl}_{ci}_{bi}"
+                        w(f"  hwfx::Half2 {nm};\n  {{")
+                        for t, (k, v) in enumerate(terms):
+                            h, l = _fx_halves(v)
+                            w(f" hwfx::Acc t = hwfx::prod({cname[cl]}[{k}], {h}, {l});" if t == 0 else
+                              f" hwfx::mac(t, {cname[cl]}[{k}], {h}, {l});")
+                        w(f" {nm} = hwfx::halves(hwfx::scaled<{FX_VF}>(t)); }}\n")
+                    names[lvl] = seen[key]
+                parts = [("ca", names[2]), ("c4", names[4])] if names[2] == names[3] else \
+                    [("c2", names[2]), ("c3", names[3]), ("c4", names[4])]
+                w(f"  long long E{ci}_{bi};\n  {{")
+                for t, (c, q) in enumerate(parts):
+                    w(f" hwfx::Acc t = hwfx::prod({q}, {c}.h, {c}.l);" if t == 0 else f" hwfx::mac(t, {q}, {c}.h, {c}.l);")
+                w(f" E{ci}_{bi} = hwfx::scaled<hwfx::CF>(t); }}\n")
+            k = b[0]
+            w(f"  x[{k}] = E0_{bi} + E1_{bi};\n  x[{3 - k}] = E0_{bi} - E1_{bi};\n")
+        w("}\n\n")
+    else:
+        # value coefficients per base point (|xi|, |eta|) = (.2236, .2236), (.2236, .5), (.5, .2236), (.5, .5)
+        def row(lvl, c, b, use):
+            co = coef(lvl, c, b)
+            assert set(co) - {sl[(0, 0)][[r[d4.index((0, 0, 0))] != 0 for r in basis[(0, 0)]].index(True)]} <= set(cols[c][k] for k in use)
+            return [co.get(cols[c][k], decimal.Decimal(0)) for k in use]
+        na, nb, ne = len(cols[(0, 0)]), len(cols[(1, 0)]), len(cols[(1, 1)])
+        use = {"A2": (2, (0, 0), (0, 1, 2)), "A4": (4, (0, 0), range(na)), "B2": (2, (1, 0), (0, 1)),
+               "B3": (3, (1, 0), (0, 1, 4)), "B4": (4, (1, 0), range(nb)), "E2": (2, (1, 1), (0,)),
+               "E4": (4, (1, 1), range(ne))}
+        w("// Coefficients of q_l - u_5 at the points (|xi|, |eta|), by 2 i + j with i, j = 0: sqrt(5)/10, 1: 1/2, as\n"
+          f"// (h 2^32 + l) 2^-{FX_VF}.  q_2 and q_3 agree on the classes (even, even) and (odd, odd); class c takes those\n"
+          "// of class b at (|eta|, |xi|).\n")
+        for nm, (lvl, c, us) in use.items():
+            rows = []
+            for b in bases:
+                r = row(lvl, c, b, us)
+                if nm[0] in "AE" and lvl == 2:
+                    assert r == row(3, c, b, us) and coef(3, c, b) == coef(2, c, b)
+                if c == (1, 0):
+                    bt = (b[1], b[0])
+                    assert r == row(lvl, (0, 1), bt, us)
+                rows.append("{" + ", ".join("{%d, %d}" % _fx_halves(v) for v in r) + "}")
+            w(f"static __constant__ int2 D2_V{nm}[4][{len(us)}] = {{\n  " + ",\n  ".join(rows) + "};\n".replace("-2147483648", "(-2147483647 - 1)"))
+        w("\n")
+
+
+def fx_rows(dim, P):
+    """Rows of beta_2..beta_4 over the fixed-point columns: (class, level) -> list of
+    (q_l part, q_{l-1} part) rows.  2D: class (0,1) uses the rows of class (1,0)
+    on its x <-> y image (the same quadratic form)."""
+    d4, basis, sl, bases, VP, RCP = P
+    cols = fx_columns(dim, P)
+    out = {}
+    for c in parity_classes(dim):
+        if c == (0, 1):
+            continue
+        pos = [sl[c].index(j) for j in cols[c]]
+        for lvl in (2, 3, 4):
+            A, Bm = RCP.get((lvl, lvl, c)), RCP.get((lvl, lvl - 1, c))
+            out[(c, lvl)] = [([A[r][j] for j in pos], [Bm[r][j] if Bm is not None else decimal.Decimal(0) for j in pos])
+                             for r in range(len(A))]
+    return out
+
+
 def emit_parity(out):
     w = out.write
     w("// Generated by gen_tables.py (mirror-parity form); do not edit.\n")
     w("// Reconstruction of one variable in the parity basis s of the stencil data:\n")
     w("// split (d -> s), smoothness indicators beta_2..beta_4 from run-time rows, and the\n")
     w("// Gauss-Lobatto values u = c1 q1 + c2 q2 + c3 q3 + c4 q4 at all points.\n")
-    w("#pragma once\n\nnamespace hwp {\n\n")
+    w('#pragma once\n\n#include "hweno_fx.cuh"\n\nnamespace hwp {\n\n')
     host = []
     for dim in (1, 2):
         P = build_parity(dim)
@@ -556,6 +689,20 @@ def emit_parity(out):
                 w(f"    out[{pp}] = P + Q;\n    out[{mp}] = P - Q;\n    out[{pm}] = R + S;\n    out[{mm}] = R - S;\n")
             w("  }\n")
         w("}\n\n")
+        emit_fx(w, dim, P)
+        fr = fx_rows(dim, P)
+        for c, nm in (((0, 0), "A"), ((1, 0), "B"), ((1, 1), "E")):
+            if (c, 2) not in fr:
+                continue
+            rows = [(lvl, a, b) for lvl in (2, 3, 4) for a, b in fr[(c, lvl)]]
+            cnt = [len(fr[(c, lvl)]) for lvl in (2, 3, 4)]
+            w(f"// beta rows of class {c}: first of levels 2, 3, 4 (k = 0, 1, 2), end (k = 3)\n")
+            w(f"__host__ __device__ constexpr int {tag}_R{nm}(int k) {{ return k == 0 ? 0 : k == 1 ? {cnt[0]} : "
+              f"k == 2 ? {cnt[0] + cnt[1]} : {sum(cnt)}; }}\n")
+            w(f"constexpr int {tag}_NR{nm} = {len(rows)}, {tag}_NC{nm} = {len(rows[0][1])};\n")
+            for part, src in ((1, "L"), (2, "M")):
+                host.append(f"static const double {tag}P_{nm}{src}[{len(rows)}][{len(rows[0][1])}] = {{" +
+                            ", ".join("{" + ", ".join(_lit(v) for v in r[part]) + "}" for r in rows) + "};\n")
         for lvl in (2, 3, 4):
             flat = [e for ent in lay[lvl] for e in ent]
             host.append(f"static const double {tag}P_RC{lvl}_{lvl}[{len(flat)}] = {{" +
@@ -565,6 +712,7 @@ def emit_parity(out):
     w("}  // namespace hwp\n\n")
     w("#ifdef HWP_HOST_TABLES\n// Host: coefficient rows in the flat order the beta functions read them;\n")
     w("// B_l = (S_l/g_l) RC_l_l - (S_{l-1}/g_l) RC_l_(l-1)  (eq. (p)), or RC_l_l alone for beta of q_l.\n")
+    w("// P_<class>L, P_<class>M: the same two parts over the columns of the fixed-point form, levels in turn.\n")
     w("namespace hwp {\n")
     for h in host:
         w(h)

@@ -410,11 +410,11 @@ void run_stage_1d(const Prob& P, const HostTabs& T, int prec, const Bufs& B, con
   if (P.nvar == 3) {
     if (prec == PREC_FP32) stage_t<float, 3>(P, T.wf, T.b1f, B, S, st);
     else if (prec == PREC_DF64) stage_t<df64, 3>(P, T.wx, T.b1x, B, S, st);
-    else stage_t<double, 3>(P, T.wd, T.b1d, B, S, st);
+    else stage_t<fx64, 3>(P, T.wd, T.b1d, B, S, st);
   } else {
     if (prec == PREC_FP32) stage_t<float, 1>(P, T.wf, T.b1f, B, S, st);
     else if (prec == PREC_DF64) stage_t<df64, 1>(P, T.wx, T.b1x, B, S, st);
-    else stage_t<double, 1>(P, T.wd, T.b1d, B, S, st);
+    else stage_t<fx64, 1>(P, T.wd, T.b1d, B, S, st);
   }
 }
 

@@ -17,7 +17,8 @@
 // the point values in HBM rather than recomputing a halo.
 //
 // This unit holds the FP64 instantiations and the precision dispatch; FP32,
-// double-float and the batched kernels compile in their own units.
+// double-float, FP64 with the learned indicator and the batched kernels compile
+// in their own units.
 #include "hweno_2d_kernels.cuh"
 
 namespace hw {
@@ -25,8 +26,10 @@ namespace hw {
 void run_stage_2d(const Prob& P, const HostTabs& T, int prec, const Bufs& B, const StageCall& S, cudaStream_t st) {
   if (prec == PREC_FP32) return run_stage_2d_fp32(P, T, B, S, st);
   if (prec == PREC_DF64) return run_stage_2d_df64(P, T, B, S, st);
-  if (P.nvar == 4) stage_t<double, 4>(P, T, T.wd, T.b2d, B, S, st);
-  else stage_t<double, 1>(P, T, T.wd, T.b2d, B, S, st);
+  // above a confidence of 1 the network decides nothing: the plain scheme, bit for bit
+  if (P.indicator == IND_MLP && B.mlp_conf <= 1.0f) return run_stage_2d_learned(P, T, B, S, st);
+  if (P.nvar == 4) stage_t<fx64, 4>(P, T, T.wd, T.b2d, B, S, st);
+  else stage_t<fx64, 1>(P, T, T.wd, T.b2d, B, S, st);
 }
 
 }  // namespace hw

@@ -12,9 +12,9 @@ cudaError_t run_batch_stage(const HostTabs& T, int fp32, int tile_variant, const
     if (tile_variant == 2) return launch_batch<float, 64, 2>(T.wf, T.b2f, S, nsm, st);
     return launch_batch<float, 32, 4>(T.wf, T.b2f, S, nsm, st);
   }
-  if (tile_variant == 1) return launch_batch<double, 16, 8>(T.wd, T.b2d, S, nsm, st);
-  if (tile_variant == 2) return launch_batch<double, 64, 2>(T.wd, T.b2d, S, nsm, st);
-  return launch_batch<double, 32, 4>(T.wd, T.b2d, S, nsm, st);
+  if (tile_variant == 1) return launch_batch<fx64, 16, 8>(T.wd, T.b2d, S, nsm, st);
+  if (tile_variant == 2) return launch_batch<fx64, 64, 2>(T.wd, T.b2d, S, nsm, st);
+  return launch_batch<fx64, 32, 4>(T.wd, T.b2d, S, nsm, st);
 }
 
 }  // namespace hw

@@ -144,12 +144,18 @@ __device__ __forceinline__ void rec2d_cell(const Prob& P, const Weights<T>& W, c
   const bool usemod = MODE == REC_FLAGGED || (MODE == REC_MIXED && mask[(long long)j * P.nx + i] == 1);
   const Nbr nb = neighbours<FIX>(P, i, j);
   const long long o = goff(P, i, j);
-  // float copy, plain pass, all 3 x 3 cells inside the grid: no image to apply,
+  // FP32 from the float copy and fx64, plain pass, all 3 x 3 cells inside the grid: no image to apply,
   // the moments are read at fixed offsets from the cell's own
-  const bool inner = S32 && MODE == REC_PLAIN && i > 0 && i < P.nx - 1 && j > 0 && j < P.ny - 1;
-  const float* __restrict__ Uc = S32 ? U32 + ((long long)j * P.pitch + i) : nullptr;
+  constexpr bool DIRECT = (S32 || (std::is_same<T, fx64>::value && !FIX)) && MODE == REC_PLAIN;
+  const bool inner = DIRECT && i > 0 && i < P.nx - 1 && j > 0 && j < P.ny - 1;
+  using Src = std::conditional_t<S32, float, double>;
+  const Src* __restrict__ Uc;
+  if constexpr (S32) Uc = U32 + ((long long)j * P.pitch + i);
+  else Uc = U + ((long long)j * P.pitch + i);
+  constexpr bool D64 = std::is_same<T, fx64>::value;
   T rinv[16];
   T pxl = T(0), pxr = T(0), pyb = T(0), pyt = T(0), nrm = T(0);
+  [[maybe_unused]] long long nrmb = 0;   // FP64: the norm's bits (non-negative doubles order like them)
 #pragma unroll 1
   for (int v = 0; v < NV; ++v) {
     T d[23];
@@ -158,7 +164,7 @@ __device__ __forceinline__ void rec2d_cell(const Prob& P, const Weights<T>& W, c
       for (int c = 0; c < 23; ++c) {
         int kind, ox, oy;
         d4_slot(c, kind, ox, oy);
-        d[c] = T(Uc[(long long)(v * 3 + kind) * P.plane + (long long)oy * P.pitch + ox]);
+        if constexpr (DIRECT) d[c] = T(Uc[(long long)(v * 3 + kind) * P.plane + (long long)oy * P.pitch + ox]);
       }
     } else {
 #pragma unroll
@@ -172,10 +178,20 @@ __device__ __forceinline__ void rec2d_cell(const Prob& P, const Weights<T>& W, c
       }
     }
     T out[16];
-    recon2d<T>(W, B, d, out);
+    if constexpr (D64) {
+      // the point values go out as they are formed (four base points in turn);
+      // the partials read them back below
+      T* __restrict__ Gv = G + (long long)(v * 16) * P.gplane + o;
+      recon2d<T>(W, B, d, [&](int p, T x) {
+        Gv[p * P.gplane] = x;
+        if (!FLAGGED && v == 0) nrmb = max(nrmb, __double_as_longlong(x.v) & 0x7FFFFFFFFFFFFFFFLL);
+      });
+    } else {
+      recon2d<T>(W, B, d, [&](int p, T x) { out[p] = x; });
 #pragma unroll
-    for (int p = 0; p < 16; ++p) G[(long long)(v * 16 + p) * P.gplane + o] = out[p];
-    if (!FLAGGED) {
+      for (int p = 0; p < 16; ++p) G[(long long)(v * 16 + p) * P.gplane + o] = out[p];
+    }
+    if (!FLAGGED && !D64) {
       if (v == 0) {
 #pragma unroll
         for (int p = 0; p < 16; ++p) nrm = tmax(nrm, tabs(out[p]));
@@ -220,6 +236,27 @@ __device__ __forceinline__ void rec2d_cell(const Prob& P, const Weights<T>& W, c
       }
     }
   }
+  if constexpr (D64 && !FLAGGED) {
+    nrm = __longlong_as_double(nrmb);
+    if (P.eq == EQ_ADV) {
+      pxl = pxr = P.adv_a;
+      pyb = pyt = P.adv_b;
+    } else {
+      // faces x-lo, x-hi, y-lo, y-hi: point indices p0 + q dp, velocity (rho mu)/rho, (rho nu)/rho or u
+      const T* Gr = G + o;
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        const int p0 = f == 0 ? 0 : f == 1 ? 12 : f == 2 ? 0 : 3, dp = f < 2 ? 1 : 4, v = NV == 4 ? (f < 2 ? 1 : 2) : 0;
+        T s = T(0);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const T m = Gr[(long long)(v * 16 + p0 + q * dp) * P.gplane];
+          s += gl_w<T>(q) * (NV == 4 ? m * rcp(Gr[(long long)(p0 + q * dp) * P.gplane]) : m);
+        }
+        (f == 0 ? pxl : f == 1 ? pxr : f == 2 ? pyb : pyt) = s;
+      }
+    }
+  }
   if (!FLAGGED) {
     aux[0 * P.gplane + o] = pxl;
     aux[1 * P.gplane + o] = pxr;
@@ -234,10 +271,13 @@ __device__ __forceinline__ void rec2d_cell(const Prob& P, const Weights<T>& W, c
 // Double-float: 4 resident blocks per SM (at most 128 registers, a few spills)
 // beat 3 (168 registers, none): 7.0 vs 8.3 ms per launch at 2048^2.  FP32 with
 // the float copy: 8 blocks (64 registers, 164 B of spills) measured 0.545 ms per
-// 2048^2 launch against 0.685 at 4 blocks (119 registers).  FP64 is pipe-bound:
-// 2, 3 or 4 blocks run alike.
+// 2048^2 launch against 0.685 at 4 blocks (119 registers).  FP64: 5 blocks (96
+// registers, 20 spilled) 5.52 ms per 2048^2 launch, 4 blocks 5.71, 2 blocks 6.34;
+// the linear part in integers took it there from 18.1 ms (all in FP64): 696 FP64
+// operations per cell instead of 2330, the FP64 pipe 80 % busy beside 20 k
+// integer instructions per cell.
 template <typename T, int NV, int MODE, bool FIX = false, bool S32 = false>
-__global__ void __launch_bounds__(RB, (is_df64<T>::value ? 4 : (std::is_same<T, float>::value ? 8 : 1))) rec2d_kernel(Prob P, Weights<T> W, Beta2<T> B, const double* __restrict__ U,
+__global__ void __launch_bounds__(RB, (is_df64<T>::value ? 4 : std::is_same<T, float>::value ? 8 : std::is_same<T, fx64>::value ? 5 : 1)) rec2d_kernel(const __grid_constant__ Prob P, const __grid_constant__ Weights<T> W, const __grid_constant__ Beta2<T> B, const double* __restrict__ U,
                                                   const uint8_t* __restrict__ mask, const double* __restrict__ Mod,
                                                   const int* __restrict__ list, const int* __restrict__ count,
                                                   T* __restrict__ G, T* __restrict__ aux,
@@ -754,7 +794,7 @@ void launch_rec2d(int blocks, cudaStream_t st, const Prob& P, const Weights<T>& 
       return;
     }
   }
-  if constexpr (NV == 4 && std::is_same<T, double>::value) {
+  if constexpr (NV == 4 && std::is_same<T, fx64>::value) {
     if (P.fixtab || P.sol_j > 0) {
       rec2d_kernel<T, NV, MODE, true><<<blocks, RB, 0, st>>>(P, W, Bt, U, mask, Mod, list, count, G, aux, rerec);
       return;
@@ -766,7 +806,7 @@ void launch_rec2d(int blocks, cudaStream_t st, const Prob& P, const Weights<T>& 
 template <typename T, int NV>
 void stage_t(const Prob& P, const HostTabs& HT, const Weights<T>& W, const Beta2<T>& Bt, const Bufs& B,
              const StageCall& S, cudaStream_t st) {
-  if constexpr (NV == 4) {
+  if constexpr (NV == 4 && !std::is_same<T, double>::value) {
     if (fused_applies(P, NV)) {   // the whole stage in one launch
       Rk r{S.Uin, S.Un, S.Uout, S.mask, S.Mod, S.maskN, S.ModN, S.dt, S.cA, S.cB, S.Lout, S.Umod, B.status, S.dtp};
       FzOut o{S.mask, S.Mod, S.aleph, B.rerec};
@@ -782,25 +822,30 @@ void stage_t(const Prob& P, const HostTabs& HT, const Weights<T>& W, const Beta2
   const int rblocks = (int)((ncell + RB - 1) / RB);
   const int fblocks = (int)std::min<long long>(rblocks, (long long)P.nsm * 8);
   const dim3 blk(TX, TY), grd((P.nx + TX - 1) / TX, (P.ny + TY - 1) / TY);
-  if (NV == 4 && P.indicator == IND_MLP) {
-    // Learned indicator first (moments only): confident cells are decided and
-    // modified before Step 1, which then reconstructs them from the modified
-    // moments; KXRCF decides the rest from the Step-1 point values, and only
-    // the cells it flags are reconstructed again.
-    int* ucnt = B.und_count + S.stage;
-    cudaMemsetAsync(ucnt, 0, sizeof(int), st);
-    if (B.prof) B.prof->begin(4, st);
-    run_mlpre2d(P, B.mlp, B.mlp_conf, S.Uin, S.mask, S.Mod, B.und, ucnt, B.mlp_stats, B.mlp_prob, st);
-    if (B.prof) B.prof->end(st);
-    if (B.prof) B.prof->begin(0, st);
-    rec2d_kernel<T, NV, REC_MIXED><<<rblocks, RB, 0, st>>>(P, W, Bt, S.Uin, S.mask, S.Mod, nullptr, nullptr,
-                                                           (T*)B.G, (T*)B.aux, nullptr);
-    if (B.prof) B.prof->end(st);
-    if (B.prof) B.prof->begin(1, st);
-    fallback2d_kernel<T, NV><<<fblocks, RB, 0, st>>>(P, W, S.Uin, (const T*)B.G, (const T*)B.aux, B.und, ucnt,
-                                                     S.mask, S.Mod, B.list, cnt, S.aleph);
-    if (B.prof) B.prof->end(st);
-  } else {
+  bool learned = false;
+  if constexpr (NV == 4) {
+    learned = P.indicator == IND_MLP;
+    if (learned) {
+      // Learned indicator first (moments only): confident cells are decided and
+      // modified before Step 1, which then reconstructs them from the modified
+      // moments; KXRCF decides the rest from the Step-1 point values, and only
+      // the cells it flags are reconstructed again.
+      int* ucnt = B.und_count + S.stage;
+      cudaMemsetAsync(ucnt, 0, sizeof(int), st);
+      if (B.prof) B.prof->begin(4, st);
+      run_mlpre2d(P, B.mlp, B.mlp_conf, S.Uin, S.mask, S.Mod, B.und, ucnt, B.mlp_stats, B.mlp_prob, st);
+      if (B.prof) B.prof->end(st);
+      if (B.prof) B.prof->begin(0, st);
+      rec2d_kernel<T, NV, REC_MIXED><<<rblocks, RB, 0, st>>>(P, W, Bt, S.Uin, S.mask, S.Mod, nullptr, nullptr,
+                                                             (T*)B.G, (T*)B.aux, nullptr);
+      if (B.prof) B.prof->end(st);
+      if (B.prof) B.prof->begin(1, st);
+      fallback2d_kernel<T, NV><<<fblocks, RB, 0, st>>>(P, W, S.Uin, (const T*)B.G, (const T*)B.aux, B.und, ucnt,
+                                                       S.mask, S.Mod, B.list, cnt, S.aleph);
+      if (B.prof) B.prof->end(st);
+    }
+  }
+  if (!learned) {
     if (B.prof) B.prof->begin(0, st);
     launch_rec2d<T, NV, REC_PLAIN>(rblocks, st, P, W, Bt, S.Uin, nullptr, nullptr, nullptr, nullptr, (T*)B.G,
                                    (T*)B.aux, nullptr, S.U32in);
@@ -819,7 +864,7 @@ void stage_t(const Prob& P, const HostTabs& HT, const Weights<T>& W, const Beta2
   Rk r{S.Uin, S.Un, S.Uout, S.mask, S.Mod, S.maskN, S.ModN, S.dt, S.cA, S.cB, S.Lout, S.Umod, B.status, S.dtp,
        std::is_same<T, float>::value ? S.U32out : nullptr};
   if (B.prof) B.prof->begin(3, st);
-  if constexpr (NV == 4 && std::is_same<T, double>::value) {
+  if constexpr (NV == 4 && std::is_same<T, fx64>::value) {
     if (P.sol_j > 0) update2d_kernel<T, NV, true><<<grd, blk, 0, st>>>(P, (const T*)B.G, r);
     else update2d_kernel<T, NV><<<grd, blk, 0, st>>>(P, (const T*)B.G, r);
   } else if constexpr (NV == 4 && std::is_same<T, float>::value) {
@@ -883,7 +928,8 @@ __device__ __forceinline__ int owner(const BProb* __restrict__ probs, int n, int
 }
 
 template <typename T, int TXV, int TYV>
-__global__ void __launch_bounds__(TXV * TYV) batch_stage_kernel(BatchStage A, Weights<T> W, Beta2<T> B) {
+__global__ void __launch_bounds__(TXV * TYV) batch_stage_kernel(const __grid_constant__ BatchStage A, const __grid_constant__ Weights<T> W,
+                                                                const __grid_constant__ Beta2<T> B) {
   static_assert(TXV * TYV == RB, "tiles and rows use the same block");
   __shared__ T xf[TYV][TXV + 1][4][4];
   __shared__ T yf[TYV + 1][TXV][4][4];

@@ -126,7 +126,7 @@ void build_tables(hweno_s* h) {
   const double* g = h->g.gamma_bar;
   long double S[5] = {0, 0, 0, 0, 0};
   for (int l = 1; l <= 4; ++l) S[l] = S[l - 1] + g[l - 1];
-  auto& wd = h->T.wd;
+  auto& wd = h->T.wl;
   auto& wf = h->T.wf;
   for (int l = 1; l <= 4; ++l) {
     wd.gam[l - 1] = (double)(g[l - 1] / S[4]);
@@ -135,6 +135,13 @@ void build_tables(hweno_s* h) {
     wf.gam[l - 1] = (float)wd.gam[l - 1];
     wf.sg[l - 1] = (float)wd.sg[l - 1];
     wf.s1g[l - 1] = (float)wd.s1g[l - 1];
+    wd.ss[l - 1] = (double)(S[l] / S[4]);
+    wf.ss[l - 1] = (float)wd.ss[l - 1];
+    h->T.wx.ss[l - 1] = dfx(S[l] / S[4]);
+    h->T.wd.gam[l - 1] = wd.gam[l - 1];
+    h->T.wd.sg[l - 1] = wd.sg[l - 1];
+    h->T.wd.s1g[l - 1] = wd.s1g[l - 1];
+    h->T.wd.ss[l - 1] = wd.ss[l - 1];
     h->T.wx.gam[l - 1] = dfx(g[l - 1] / S[4]);
     h->T.wx.sg[l - 1] = dfx(S[l] / g[l - 1]);
     h->T.wx.s1g[l - 1] = dfx(S[l - 1] / g[l - 1]);
@@ -142,6 +149,7 @@ void build_tables(hweno_s* h) {
   wd.eps = 1e-10;
   wf.eps = 1e-10f;
   h->T.wx.eps = dfx(1e-10L);
+  h->T.wd.eps = 1e-10;
   auto coef = [&](int l, long double& a, long double& b) {
     if (h->g.beta_of_q) { a = 1.0L; b = 0.0L; return; }
     a = S[l] / g[l - 1];
@@ -149,23 +157,50 @@ void build_tables(hweno_s* h) {
   };
   long double a, b;
   // flat rows: B_l[k] = a_l RC_l_l[k] + b_l RC_l_(l-1)[k]; q_1 is constant, so level 2 has no b part
-  auto fill = [&](int l, const double* rl, const double* rm, int n, double* outd, float* outf, hw::df64* outx) {
+  auto fill = [&](int l, const double* rl, const double* rm, int n, float* outf, hw::df64* outx, double* outl) {
     coef(l, a, b);
     for (int k = 0; k < n; ++k) {
       const long double v = a * rl[k] + (rm ? b * rm[k] : 0.0L);
-      outd[k] = (double)v;
       outf[k] = (float)v;
       outx[k] = dfx(v);
+      if (outl) outl[k] = (double)v;
+    }
+  };
+  // FP64: the rows of a parity class in fixed point, the sum of each one's |coefficients|
+  // between 2^61.9 and 2^62.9 units; first[]: its rows of levels 2, 3, 4
+  auto fill_fx = [&](int (*first)(int), int nc, const double* rl, const double* rm, int2* out, int* f) {
+    for (int r = 0; r < first(3); ++r) {
+      coef(r < first(1) ? 2 : r < first(2) ? 3 : 4, a, b);
+      std::vector<long double> v(nc);
+      long double sum = 0.0L;
+      for (int k = 0; k < nc; ++k) {
+        v[k] = a * rl[r * nc + k] + b * rm[r * nc + k];
+        sum += fabsl(v[k]);
+      }
+      const int F = sum > 0.0L ? (int)floorl(62.9L - log2l(sum)) : 60;
+      f[r] = 60 - F;
+      for (int k = 0; k < nc; ++k) {
+        const long long c = llrintl(ldexpl(v[k], F));
+        const int lo = (int)(unsigned)(unsigned long long)c;
+        out[r * nc + k] = make_int2((int)((c - lo) >> 32), lo);
+      }
     }
   };
   if (h->g.dim == 1) {
-    fill(2, hwp::D1P_RC2_2, nullptr, hwp::D1_NB2, h->T.b1d.B2, h->T.b1f.B2, h->T.b1x.B2);
-    fill(3, hwp::D1P_RC3_3, hwp::D1P_RC3_2, hwp::D1_NB3, h->T.b1d.B3, h->T.b1f.B3, h->T.b1x.B3);
-    fill(4, hwp::D1P_RC4_4, hwp::D1P_RC4_3, hwp::D1_NB4, h->T.b1d.B4, h->T.b1f.B4, h->T.b1x.B4);
+    fill(2, hwp::D1P_RC2_2, nullptr, hwp::D1_NB2, h->T.b1f.B2, h->T.b1x.B2, nullptr);
+    fill(3, hwp::D1P_RC3_3, hwp::D1P_RC3_2, hwp::D1_NB3, h->T.b1f.B3, h->T.b1x.B3, nullptr);
+    fill(4, hwp::D1P_RC4_4, hwp::D1P_RC4_3, hwp::D1_NB4, h->T.b1f.B4, h->T.b1x.B4, nullptr);
+    auto& B = h->T.b1d;
+    fill_fx(hwp::D1_RA, hwp::D1_NCA, &hwp::D1P_AL[0][0], &hwp::D1P_AM[0][0], &B.a[0][0], B.fa);
+    fill_fx(hwp::D1_RB, hwp::D1_NCB, &hwp::D1P_BL[0][0], &hwp::D1P_BM[0][0], &B.b[0][0], B.fb);
   } else {
-    fill(2, hwp::D2P_RC2_2, nullptr, hwp::D2_NB2, h->T.b2d.B2, h->T.b2f.B2, h->T.b2x.B2);
-    fill(3, hwp::D2P_RC3_3, hwp::D2P_RC3_2, hwp::D2_NB3, h->T.b2d.B3, h->T.b2f.B3, h->T.b2x.B3);
-    fill(4, hwp::D2P_RC4_4, hwp::D2P_RC4_3, hwp::D2_NB4, h->T.b2d.B4, h->T.b2f.B4, h->T.b2x.B4);
+    fill(2, hwp::D2P_RC2_2, nullptr, hwp::D2_NB2, h->T.b2f.B2, h->T.b2x.B2, h->T.b2l.B2);
+    fill(3, hwp::D2P_RC3_3, hwp::D2P_RC3_2, hwp::D2_NB3, h->T.b2f.B3, h->T.b2x.B3, h->T.b2l.B3);
+    fill(4, hwp::D2P_RC4_4, hwp::D2P_RC4_3, hwp::D2_NB4, h->T.b2f.B4, h->T.b2x.B4, h->T.b2l.B4);
+    auto& B = h->T.b2d;
+    fill_fx(hwp::D2_RA, hwp::D2_NCA, &hwp::D2P_AL[0][0], &hwp::D2P_AM[0][0], &B.a[0][0], B.fa);
+    fill_fx(hwp::D2_RB, hwp::D2_NCB, &hwp::D2P_BL[0][0], &hwp::D2P_BM[0][0], &B.b[0][0], B.fb);
+    fill_fx(hwp::D2_RE, hwp::D2_NCE, &hwp::D2P_EL[0][0], &hwp::D2P_EM[0][0], &B.e[0][0], B.fe);
   }
 }
 

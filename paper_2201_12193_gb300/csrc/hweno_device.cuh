@@ -3,8 +3,8 @@
 // Scheme: moment-based multi-resolution HWENO, Li, Shu & Qiu (arXiv 2201.12193).
 // Section and equation names below are the paper's.
 //
-// Precision: T = double (FP64 path), float (FP32-bulk path) or df64 (double-float
-// path, df64.cuh).  The state, the Runge-Kutta combination and the conservation
+// Precision: T = fx64 (FP64 path, fx64.cuh), double (FP64 path of the learned
+// indicator), float (FP32-bulk path) or df64 (double-float path, df64.cuh).  The state, the Runge-Kutta combination and the conservation
 // sums stay FP64 in all three.
 #pragma once
 
@@ -15,6 +15,7 @@
 
 #include "hweno_parity.h"
 #include "df64.cuh"
+#include "fx64.cuh"
 
 namespace hw {
 
@@ -40,6 +41,7 @@ template <typename T> __device__ __forceinline__ T pc(const PConst& c);
 template <> __device__ __forceinline__ double pc<double>(const PConst& c) { return c.d; }
 template <> __device__ __forceinline__ float pc<float>(const PConst& c) { return c.f; }
 template <> __device__ __forceinline__ df64 pc<df64>(const PConst& c) { return c.x; }
+template <> __device__ __forceinline__ fx64 pc<fx64>(const PConst& c) { return c.d; }
 
 // Problem description passed by value to every kernel.
 struct Prob {
@@ -93,6 +95,7 @@ struct Weights {
   T gam[4];      // gamma_{l,4}
   T sg[4];       // S_l / g_l
   T s1g[4];      // S_{l-1} / g_l  (0 for l = 1)
+  T ss[4];       // S_l / S_4
   T eps;         // 1e-10 of eqs. (w1_-LR), (non-linear-weight)
 };
 
@@ -101,6 +104,17 @@ struct Weights {
 // with row = (S_l/g_l) R C_l - (S_{l-1}/g_l) R C_{l-1}  (eq. (beta), (2D-beta), (p)).
 template <typename T> struct Beta1 { T B2[hwp::D1_NB2]; T B3[hwp::D1_NB3]; T B4[hwp::D1_NB4]; };
 template <typename T> struct Beta2 { T B2[hwp::D2_NB2]; T B3[hwp::D2_NB3]; T B4[hwp::D2_NB4]; };
+// fx64: the rows in fixed point (hweno_fx.cuh), per parity class and over the class's
+// columns; a coefficient is (x = h, y = l): (h 2^32 + l) 2^-F with F the row's own (the
+// sum of its |coefficients| below 2^63 units), f = 60 - F.
+template <int RA, int CA, int RB, int CB, int RE, int CE>
+struct FxRows {
+  int2 a[RA][CA], b[RB][CB], e[RE][CE];
+  int fa[RA], fb[RB], fe[RE];
+};
+template <> struct Beta1<fx64> : FxRows<hwp::D1_NRA, hwp::D1_NCA, hwp::D1_NRB, hwp::D1_NCB, 1, 1> {};
+template <> struct Beta2<fx64>
+    : FxRows<hwp::D2_NRA, hwp::D2_NCA, hwp::D2_NRB, hwp::D2_NCB, hwp::D2_NRE, hwp::D2_NCE> {};
 
 // Gauss-Lobatto nodes and weights of eq. (F)
 template <typename T> __device__ __forceinline__ T gl_w(int k) { return (k == 0 || k == 3) ? T(1.0 / 12.0) : T(5.0 / 12.0); }
@@ -224,11 +238,24 @@ __device__ __forceinline__ double avg_img(const Prob& P, const double* __restric
 // ---------------------------------------------------------------- physics
 // Physical flux of eq. (1D-Euler) / (2D-Euler) or of the scalar laws in
 // direction dir (0 = x, 1 = y); NV = 1 (scalar), 3 (1D Euler), 4 (2D Euler).
-// 1/x correctly rounded (the same value as the IEEE division 1/x) by the
-// reciprocal intrinsics of the two hardware precisions; double-float divides.
+// 1/x.  FP32, double: correctly rounded.  fx64: the hardware's approximation y (2^-20) and
+// one third-order step of Householder's iteration, y (1 + e + e^2) with e = 1 - x y:
+// the truncation is e^3 (2^-60), the result within 0.5 + 2^-7 units in the last
+// place, and three FP64 operations where the IEEE reciprocal takes 5.4 (measured
+// rates; FP64 issues at 2 per clock and SM).  0 and infinity give NaN.
 template <typename T> __device__ __forceinline__ T rcp(T x) { return T(1) / x; }
 template <> __device__ __forceinline__ float rcp<float>(float x) { return __frcp_rn(x); }
 template <> __device__ __forceinline__ double rcp<double>(double x) { return __drcp_rn(x); }
+template <> __device__ __forceinline__ fx64 rcp<fx64>(fx64 a) {
+  const double x = a.v;
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  double e = fma(-x, y, 1.0);
+  e = fma(e, e, e);
+  return fma(y, e, y);
+}
+
+__device__ __forceinline__ double rcp64(double x) { return rcp<fx64>(x).v; }
 
 template <typename T, int NV>
 __device__ __forceinline__ void phys_flux(const Prob& P, const T* u, int dir, T* f) {
@@ -355,7 +382,7 @@ __device__ __forceinline__ void hllc(const Prob& P, const T* uL, const T* uR, in
   // the branches below then fall through to f_R.
   const T k = pc<T>(P.chk);
   T sL, sR;
-  if constexpr (std::is_same<T, double>::value) {
+  if constexpr (one_division<T>::value) {
     const T coefL = ps <= pL ? T(1) : sqrt(T(1) + k * (ps / pL - T(1)));
     const T coefR = ps <= pR ? T(1) : sqrt(T(1) + k * (ps / pR - T(1)));
     sL = mL - cL * coefL;
@@ -448,11 +475,98 @@ __device__ __forceinline__ void combine_weights(const Weights<T>& W, const T bet
   c[3] = om[3] * W.sg[3];
 }
 
+// fx64: the same weights with one division.  With x_l = beta_l + eps,
+// wbar_l = gamma_l (x_l + tau) / x_l; scaling every wbar_l by prod_m x_m gives
+// omega_l = gamma_l n_l / sum_m gamma_m n_m with n_l = (x_l + tau) prod_{m != l} x_m,
+// and, gamma_l S_l/g_l being S_l/S_4, c_k = (S_k/S_4) (n_k - n_{k+1}) / sum_m gamma_m n_m.
+// c_1 = 1 - c_2 - c_3 - c_4 is not formed: q_1 is the target average u_5 and
+// u = u_5 + sum_{k>1} c_k (q_k - u_5).  c[3] is c_2 + c_3.
+__device__ __forceinline__ void combine_weights_fp64(const Weights<fx64>& W, const double beta[4], double c[4]) {
+  const double tau4s = fabs(beta[3] - beta[0]) + fabs(beta[3] - beta[1]) + fabs(beta[3] - beta[2]);
+  const double tau4 = (tau4s * (1.0 / 3.0)) * (tau4s * (1.0 / 3.0));
+  const double eps = W.eps.v;
+  const double x0 = beta[0] + eps, x1 = beta[1] + eps, x2 = beta[2] + eps, x3 = beta[3] + eps;
+  const double p01 = x0 * x1, p23 = x2 * x3;
+  const double n0 = (x0 + tau4) * (x1 * p23), n1 = (x1 + tau4) * (x0 * p23);
+  const double n2 = (x2 + tau4) * (p01 * x3), n3 = (x3 + tau4) * (p01 * x2);
+  const double inv = rcp64(fma(W.gam[3].v, n3, fma(W.gam[2].v, n2, fma(W.gam[1].v, n1, W.gam[0].v * n0))));
+  c[0] = (W.ss[1].v * (n1 - n2)) * inv;
+  c[1] = (W.ss[2].v * (n2 - n3)) * inv;
+  c[2] = n3 * inv;
+  c[3] = c[0] + c[1];
+}
+
+// sum_k c[k] s[k] of a beta row as a double: the row's units are 2^(e0 + f).
+template <int N>
+__device__ __forceinline__ double fx_row(const hwfx::Half2 (&s)[N], const int2 (&c)[N], int ef) {
+  hwfx::Acc t = hwfx::prod(s[0], c[0].x, c[0].y);
+#pragma unroll
+  for (int k = 1; k < N; ++k) hwfx::mac(t, s[k], c[k].x, c[k].y);
+  return hwfx::from_fx(hwfx::scaled<60>(t), ef);
+}
+
+// The FP64 weights as fixed-point integers of one exponent; returns it (2047 if one is not finite).
+__device__ __forceinline__ int fx_weights(const double (&c)[4], hwfx::Half2 (&h)[4]) {
+  const int e = max(max(max(hwfx::bexp(c[0]), hwfx::bexp(c[1])), max(hwfx::bexp(c[2]), hwfx::bexp(c[3]))), hwfx::CEMIN);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) h[k] = hwfx::halves(hwfx::to_fx<hwfx::CBITS>(c[k], e));
+  return e;
+}
+
 // ---------------------------------------------------------------- 1D reconstruction
 // d = (u_{i-1}, u_i, u_{i+1}, v_{i-1}, v_i, v_{i+1}) of one variable; out = the
 // four Gauss-Lobatto values of eq. (re-u).  Steps 1.1-1.3 of the 1D algorithm.
+// fx64: the linear part in block fixed point (hweno_fx.cuh).
+__device__ __forceinline__ void recon1d_fp64(const Weights<fx64>& W, const Beta1<fx64>& B, const fx64 (&d)[6],
+                                             fx64 (&out)[4]) {
+  const double dl = d[1].v - d[0].v, dr = d[2].v - d[1].v;
+  const double dv[6] = {-dl, 0.0, dr, d[3].v, d[4].v, d[5].v};
+  int e = hwfx::EMIN;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) if (k != 1) e = max(e, hwfx::bexp(dv[k]));
+  long long q[6];
+#pragma unroll
+  for (int k = 0; k < 6; ++k) q[k] = k == 1 ? 0 : hwfx::to_fx<hwfx::BITS>(dv[k], e);
+  hwfx::Half2 sa[2], sb[3];
+  hwp::fx_split1d(q, sa, sb);
+  double beta[4];
+  const int e0 = e - (1022 + hwfx::BITS);
+#pragma unroll
+  for (int l = 0; l < 3; ++l) {
+    double bl = 0.0;
+#pragma unroll
+    for (int r = hwp::D1_RA(l); r < hwp::D1_RA(l + 1); ++r) { const double x = fx_row(sa, B.a[r], e0 + B.fa[r]); bl = fma(x, x, bl); }
+#pragma unroll
+    for (int r = hwp::D1_RB(l); r < hwp::D1_RB(l + 1); ++r) { const double x = fx_row(sb, B.b[r], e0 + B.fb[r]); bl = fma(x, x, bl); }
+    beta[l + 1] = bl;
+  }
+  // beta_1: eqs. (beta1-LR), (tau1), (w1_-LR), (w1-LR), (beta1) over a common denominator
+  {
+    const double bl = dl * dl, br = dr * dr;
+    const double t1 = (br - bl) * (br - bl);
+    const double xl = bl + W.eps.v, xr = br + W.eps.v;
+    const double nl = (xl + t1) * xr, nr = (xr + t1) * xl;
+    const double gg = (nl * dl + nr * dr) * rcp64(nl + nr);
+    beta[0] = gg * gg;
+  }
+  double c[4];
+  combine_weights_fp64(W, beta, c);
+  hwfx::Half2 h[4];
+  const int ec = fx_weights(c, h);
+  long long x[4];
+  hwp::fx_values1d(sa, sb, h[0], h[1], h[2], h[3], x);
+  const double u = e > hwfx::EMAX || ec == 0x7FF ? __longlong_as_double(0x7FF8000000000000LL) : d[1].v;
+  const int eb = ec + e + (hwfx::CF - (1022 + hwfx::CBITS) - (1022 + hwfx::BITS));
+#pragma unroll
+  for (int p = 0; p < 4; ++p) out[p] = u + hwfx::from_fx(x[p], eb);
+}
+
 template <typename T>
 __device__ __forceinline__ void recon1d(const Weights<T>& W, const Beta1<T>& B, const T (&d)[6], T (&out)[4]) {
+  if constexpr (std::is_same<T, fx64>::value) {
+    recon1d_fp64(W, B, d, out);
+    return;
+  } else {
   T s[6];
   hwp::split1d<T>(d, s);
   T beta[4];
@@ -478,15 +592,145 @@ __device__ __forceinline__ void recon1d(const Weights<T>& W, const Beta1<T>& B, 
   T c[4];
   combine_weights(W, beta, c);
   hwp::values1d<T>(s, d[1], c, out);
+  }
 }
 
 // ---------------------------------------------------------------- 2D reconstruction
 // d = the 23 data of q_4 (u at labels 1..9, v at 1,3,4,5,6,7,9, w at
-// 1,2,3,5,7,8,9; labels of the paper's 3x3 stencil table), out[k*4+l] =
-// u_{i,j}(xi_k, eta_l) of eq. (2D-re-u).  Steps 1.1-1.3 of the 2D algorithm.
+// 1,2,3,5,7,8,9; labels of the paper's 3x3 stencil table); put(k*4+l, value)
+// receives u_{i,j}(xi_k, eta_l) of eq. (2D-re-u).  Steps 1.1-1.3 of the 2D algorithm.
 // Square cells: beta_1 of eq. (2D-beta1) is (sum w_1k Dx_k)^2 + (sum w_1k Dy_k)^2.
-template <typename T>
-__device__ __forceinline__ void recon2d(const Weights<T>& W, const Beta2<T>& B, const T (&d)[23], T (&out)[16]) {
+// fx64: the linear part in block fixed point (hweno_fx.cuh).  The beta rows and
+// the four base points (+-|xi|, +-|eta|) run as loops over coefficient tables:
+// unrolled, a variable's code is 100 KB and the warps wait for instructions.
+template <typename Put>
+__device__ __forceinline__ void recon2d_fp64(const Weights<fx64>& W, const Beta2<fx64>& B, const fx64 (&d)[23],
+                                             Put put) {
+  using hwfx::Half2;
+  const double u5 = d[4].v;
+  double dv[23];
+#pragma unroll
+  for (int k = 0; k < 23; ++k) dv[k] = k < 9 ? d[k].v - u5 : d[k].v;
+  int e = hwfx::EMIN;
+#pragma unroll
+  for (int k = 0; k < 23; ++k) if (k != 4) e = max(e, hwfx::bexp(dv[k]));
+  Half2 sa[7], sb[6], sc[6], se[3];   // parity classes (even, even), (odd, even), (even, odd), (odd, odd)
+  {
+    long long q[23];
+#pragma unroll
+    for (int k = 0; k < 23; ++k) q[k] = k == 4 ? 0 : hwfx::to_fx<hwfx::BITS>(dv[k], e);
+    hwp::fx_split2d(q, sa, sb, sc, se);
+  }
+  double beta[4];
+  {
+    const int e0 = e - (1022 + hwfx::BITS);
+    int ra = 0, rb = 0, re = 0;
+#pragma unroll 1
+    for (int l = 0; l < 3; ++l) {
+      const int na = l == 0 ? hwp::D2_RA(1) : l == 1 ? hwp::D2_RA(2) : hwp::D2_RA(3);
+      const int nb = l == 0 ? hwp::D2_RB(1) : l == 1 ? hwp::D2_RB(2) : hwp::D2_RB(3);
+      const int ne = l == 0 ? hwp::D2_RE(1) : l == 1 ? hwp::D2_RE(2) : hwp::D2_RE(3);
+      double bl = 0.0;
+#pragma unroll 1
+      for (; ra < na; ++ra) { const double x = fx_row(sa, B.a[ra], e0 + B.fa[ra]); bl = fma(x, x, bl); }
+#pragma unroll 1
+      for (; rb < nb; ++rb) {   // the same rows for both odd classes (x <-> y images)
+        const double x = fx_row(sb, B.b[rb], e0 + B.fb[rb]), y = fx_row(sc, B.b[rb], e0 + B.fb[rb]);
+        bl = fma(x, x, fma(y, y, bl));
+      }
+#pragma unroll 1
+      for (; re < ne; ++re) { const double x = fx_row(se, B.e[re], e0 + B.fe[re]); bl = fma(x, x, bl); }
+      if (l == 0) beta[1] = bl; else if (l == 1) beta[2] = bl; else beta[3] = bl;
+    }
+  }
+  // beta_1: eqs. (2D-q1-1234) .. (2D-beta1).  With x differences a (west), b (east)
+  // and y differences g (south), h (north), the four one-sided |grad|^2 are a^2 + h^2,
+  // b^2 + h^2, b^2 + g^2, a^2 + g^2; their six unordered differences are +-A twice,
+  // +-B twice, +-(A + B) and +-(A - B), A = a^2 - b^2, B = h^2 - g^2, so that
+  // tau_1 = ((|A| + |B| + max(|A|, |B|)) / 3)^2.
+  {
+    const double a = -dv[3], b = dv[5], g = -dv[1], h = dv[7];
+    const double a2 = a * a, b2 = b * b, g2 = g * g, h2 = h * h;
+    const double A = fabs(a2 - b2), Bq = fabs(h2 - g2);
+    const double ts = (A + Bq + (A > Bq ? A : Bq)) * (1.0 / 3.0);
+    const double t1 = ts * ts;
+    const double he = h2 + W.eps.v, ge = g2 + W.eps.v;
+    const double y0 = a2 + he, y1 = b2 + he, y2 = b2 + ge, y3 = a2 + ge;
+    const double p01 = y0 * y1, p23 = y2 * y3;
+    const double n0 = (y0 + t1) * (y1 * p23), n1 = (y1 + t1) * (y0 * p23);
+    const double n2 = (y2 + t1) * (p01 * y3), n3 = (y3 + t1) * (p01 * y2);
+    const double n03 = n0 + n3, n12 = n1 + n2, n01 = n0 + n1, n23 = n2 + n3;
+    const double inv = rcp64(n01 + n23);
+    const double gx = fma(n03, a, n12 * b) * inv, gy = fma(n01, h, n23 * g) * inv;
+    beta[0] = fma(gx, gx, gy * gy);
+  }
+  double c[4];
+  combine_weights_fp64(W, beta, c);
+  Half2 hc[4];
+  const int ec = fx_weights(c, hc);
+  const double u = e > hwfx::EMAX || ec == 0x7FF ? __longlong_as_double(0x7FF8000000000000LL) : u5;
+  const int eb = ec + e + (hwfx::CF - (1022 + hwfx::CBITS) - (1022 + hwfx::BITS));
+  using namespace hwp;
+#pragma unroll 1
+  for (int b = 0; b < 4; ++b) {
+    const int bt = ((b & 1) << 1) | (b >> 1);     // the point with |xi| and |eta| exchanged
+    auto dot = [](const int2& c0, const Half2& s0) { return hwfx::prod(s0, c0.x, c0.y); };
+    auto add = [](hwfx::Acc& t, const int2& ck, const Half2& sk) { hwfx::mac(t, sk, ck.x, ck.y); };
+    auto fin = [](const hwfx::Acc& t) { return hwfx::halves(hwfx::scaled<60>(t)); };
+    long long E[4];
+    // c_2 q_2 + c_3 q_3 + c_4 q_4 of one class
+    auto comb = [&](const Half2& q2, const Half2& q3, const Half2& q4) {
+      hwfx::Acc t = hwfx::prod(q2, hc[0].h, hc[0].l);
+      hwfx::mac(t, q3, hc[1].h, hc[1].l);
+      hwfx::mac(t, q4, hc[2].h, hc[2].l);
+      return hwfx::scaled<hwfx::CF>(t);
+    };
+    auto comb_a = [&](const Half2& q23, const Half2& q4) {   // q_2 = q_3
+      hwfx::Acc t = hwfx::prod(q23, hc[3].h, hc[3].l);
+      hwfx::mac(t, q4, hc[2].h, hc[2].l);
+      return hwfx::scaled<hwfx::CF>(t);
+    };
+    {
+      hwfx::Acc t = dot(D2_VA2[b][0], sa[0]);
+      add(t, D2_VA2[b][1], sa[1]); add(t, D2_VA2[b][2], sa[2]);
+      hwfx::Acc r = dot(D2_VA4[b][0], sa[0]);
+#pragma unroll
+      for (int k = 1; k < 7; ++k) add(r, D2_VA4[b][k], sa[k]);
+      E[0] = comb_a(fin(t), fin(r));
+    }
+    auto odd = [&](int p, const Half2 (&x)[6]) {
+      hwfx::Acc t = dot(D2_VB2[p][0], x[0]);
+      add(t, D2_VB2[p][1], x[1]);
+      hwfx::Acc r = dot(D2_VB3[p][0], x[0]);
+      add(r, D2_VB3[p][1], x[1]); add(r, D2_VB3[p][2], x[4]);
+      hwfx::Acc z = dot(D2_VB4[p][0], x[0]);
+#pragma unroll
+      for (int k = 1; k < 6; ++k) add(z, D2_VB4[p][k], x[k]);
+      return comb(fin(t), fin(r), fin(z));
+    };
+    E[1] = odd(b, sb);
+    E[2] = odd(bt, sc);
+    {
+      hwfx::Acc t = dot(D2_VE2[b][0], se[0]);
+      hwfx::Acc r = dot(D2_VE4[b][0], se[0]);
+      add(r, D2_VE4[b][1], se[1]); add(r, D2_VE4[b][2], se[2]);
+      E[3] = comb_a(fin(t), fin(r));
+    }
+    const int k = 2 + (b >> 1), l = 2 + (b & 1);
+    const long long p = E[0] + E[2], q = E[1] + E[3], r = E[0] - E[2], t = E[1] - E[3];
+    put(k * 4 + l, fx64(u + hwfx::from_fx(p + q, eb)));
+    put((3 - k) * 4 + l, fx64(u + hwfx::from_fx(p - q, eb)));
+    put(k * 4 + 3 - l, fx64(u + hwfx::from_fx(r + t, eb)));
+    put((3 - k) * 4 + 3 - l, fx64(u + hwfx::from_fx(r - t, eb)));
+  }
+}
+
+template <typename T, typename Put>
+__device__ __forceinline__ void recon2d(const Weights<T>& W, const Beta2<T>& B, const T (&d)[23], Put put) {
+  if constexpr (std::is_same<T, fx64>::value) {
+    recon2d_fp64(W, B, d, put);
+    return;
+  } else {
   T s[23];
   hwp::split2d<T>(d, s);
   T beta[4];
@@ -527,7 +771,11 @@ __device__ __forceinline__ void recon2d(const Weights<T>& W, const Beta2<T>& B, 
   }
   T c[4];
   combine_weights(W, beta, c);
+  T out[16];
   hwp::values2d<T>(s, d[4], c, out);
+#pragma unroll
+  for (int p = 0; p < 16; ++p) put(p, out[p]);
+  }
 }
 
 // Positions (ox, oy, kind) of the 23 data of q_4 in gather order.

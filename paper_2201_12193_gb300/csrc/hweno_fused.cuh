@@ -49,6 +49,7 @@ __device__ __forceinline__ int ring5(int r) { return (r + 20) % 5; }   // rows >
 __device__ __forceinline__ int ring4(int r) { return (r + 20) & 3; }
 // Butterfly shuffle of a value of the compute precision (all 32 lanes take part).
 template <typename T> __device__ __forceinline__ T shfl_xor_t(T x, int o) { return __shfl_xor_sync(0xffffffffu, x, o); }
+template <> __device__ __forceinline__ fx64 shfl_xor_t<fx64>(fx64 x, int o) { return __shfl_xor_sync(0xffffffffu, x.v, o); }
 template <> __device__ __forceinline__ df64 shfl_xor_t<df64>(df64 x, int o) {
   return df64(__shfl_xor_sync(0xffffffffu, x.hi, o), __shfl_xor_sync(0xffffffffu, x.lo, o));
 }
@@ -123,7 +124,7 @@ struct FzOut {
 
 template <typename T>
 __global__ void __launch_bounds__(FZ_NT, sizeof(T) == 4 ? 4 : 2)
-    fused2d_kernel(Prob P, Weights<T> W, Beta2<T> B, Rk S, FzOut O) {
+    fused2d_kernel(Prob P, const __grid_constant__ Weights<T> W, const __grid_constant__ Beta2<T> B, Rk S, FzOut O) {
   static_assert(FZ_WC == 32, "one warp spans the window's columns");
   extern __shared__ __align__(16) unsigned char fz_raw[];
   FusedSmem<T>& sm = *reinterpret_cast<FusedSmem<T>*>(fz_raw);
@@ -236,11 +237,8 @@ __global__ void __launch_bounds__(FZ_NT, sizeof(T) == 4 ? 4 : 2)
         d4_slot(e, kind, ox, oy);
         d[e] = sm.M[ring5(jg + oy)][v * 3 + kind][c + 1 + ox];
       }
-      T out[16];
-      recon2d<T>(W, B, d, out);
       const int s4 = ring4(jg);
-#pragma unroll
-      for (int p = 0; p < 16; ++p) sm.G[s4][v][p][c] = out[p];
+      recon2d<T>(W, B, d, [&](int p, T x) { sm.G[s4][v][p][c] = x; });
     }
     __syncthreads();
     // KXRCF partials of row jg: GL-weighted face velocities and the density norm
@@ -345,11 +343,8 @@ __global__ void __launch_bounds__(FZ_NT, sizeof(T) == 4 ? 4 : 2)
           else
             d[e] = sm.M[ring5(jr + oy)][v * 3 + kind][c + 1 + ox];
         }
-        T out[16];
-        recon2d<T>(W, B, d, out);
         const int s4 = ring4(jr);
-#pragma unroll
-        for (int p = 0; p < 16; ++p) sm.G[s4][v][p][c] = out[p];
+        recon2d<T>(W, B, d, [&](int p, T x) { sm.G[s4][v][p][c] = x; });
       }
     }
     __syncthreads();

@@ -62,7 +62,8 @@ __device__ __forceinline__ double f1_flip(double x, bool neg) {
 }
 
 template <typename T, int NV, int S, int NT>
-__global__ void __launch_bounds__(NT) fused1d_kernel(Prob P, Weights<T> W, Beta1<T> B, Rk1 R,
+__global__ void __launch_bounds__(NT) fused1d_kernel(const __grid_constant__ Prob P, const __grid_constant__ Weights<T> W,
+                                                     const __grid_constant__ Beta1<T> B, Rk1 R,
                                                      uint8_t* __restrict__ mask, double* __restrict__ ModOut,
                                                      double* __restrict__ aleph,
                                                      unsigned long long* __restrict__ rerec) {

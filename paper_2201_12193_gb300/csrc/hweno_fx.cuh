@@ -1,0 +1,80 @@
+// 64-bit block fixed point for the linear part of the FP64 reconstruction.
+//
+// GB300 issues 2 FP64 operations per clock and SM against 64 32-bit integer
+// multiply-adds with a 64-bit sum (measured: DFMA 2.0, IMAD.WIDE 52-64 per
+// clock and SM, each at its full rate beside the other).  The dot products of
+// the reconstruction (smoothness-indicator rows, polynomial values) therefore
+// run in integers: the stencil data of one variable share an exponent and are
+// held as 57-bit integers, a coefficient is a 64-bit integer, and one
+// multiply-add is three 32 x 32 -> 64 products (the low x low one, below the
+// last place kept, is left out): 0.05 clocks per SM against 0.5.  The data are deviations from the target
+// cell's average, so their common exponent is that of the variation: the
+// rounding is 2^-55 to 2^-57 of the largest deviation (FP64's is 2^-53 of the
+// largest datum).  Nonlinear parts stay FP64.
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace hwfx {
+
+// x = h 2^32 + l with both halves signed (|l| <= 2^31)
+struct Half2 { int h, l; };
+
+// The halves pass through an empty asm: seen as parts of a 64-bit value, the
+// compiler multiplies them as 64 x 64 bits (measured: three times the instructions).
+__device__ __forceinline__ Half2 halves(long long x) {
+  int h = (int)((x + 0x80000000LL) >> 32), l = (int)x;
+  asm("" : "+r"(h), "+r"(l));
+  return Half2{h, l};
+}
+
+// Sum of products a b: the h h products and the mixed ones (2^-32 of them).
+struct Acc { long long hh, m; };
+
+__device__ __forceinline__ Acc prod(Half2 a, int bh, int bl) {
+  return Acc{(long long)a.h * bh, (long long)a.h * bl + (long long)a.l * bh};
+}
+__device__ __forceinline__ void mac(Acc& s, Half2 a, int bh, int bl) {
+  s.hh += (long long)a.h * bh;
+  s.m += (long long)a.h * bl;
+  s.m += (long long)a.l * bh;
+}
+// the sum times 2^-F (33 <= F <= 64)
+template <int F>
+__device__ __forceinline__ long long scaled(const Acc& s) {
+  return (s.hh << (64 - F)) + (s.m >> (F - 32));
+}
+
+constexpr int BITS = 57;        // data: |d| < 2^BITS units
+constexpr int EMIN = 500;       // smallest block exponent (biased): variations below 2^-580 vanish
+constexpr int EMAX = 1900;      // largest one: above it the FP64 weights overflow (they are not finite)
+constexpr int CBITS = 61;       // weights c_k: |c| < 2^CBITS units
+constexpr int CEMIN = 700;
+constexpr int CF = 61;          // the weighted sums keep the product times 2^-CF
+
+__device__ __forceinline__ int bexp(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
+
+// x in units of 2^(e - 1022 - B), truncated; e at least x's biased exponent and
+// at least 64 (a zero then shifts out).
+template <int B>
+__device__ __forceinline__ long long to_fx(double x, int e) {
+  const int hi = __double2hiint(x);
+  const int k = min(e - ((hi >> 20) & 0x7FF), 63);
+  unsigned long long m =
+      ((unsigned long long)(unsigned)((hi & 0xFFFFF) | 0x100000) << 32) | (unsigned)__double2loint(x);
+  m = (m << (B - 53)) >> k;
+  const long long s = (long long)(hi >> 31);
+  return ((long long)m ^ s) - s;
+}
+
+// x 2^eb as a double (integer work; truncated to 53 bits).  The caller keeps the exponent in range.
+__device__ __forceinline__ double from_fx(long long x, int eb) {
+  const long long s = x >> 63;
+  const unsigned long long a = (unsigned long long)((x ^ s) - s);
+  const int n = __clzll((long long)a);
+  const unsigned long long m = (a << (n & 63)) >> 11;
+  const unsigned long long r = m + ((unsigned long long)(unsigned)(1085 - n + eb) << 52);
+  return __longlong_as_double(a ? (long long)(r | ((unsigned long long)s << 63)) : 0LL);
+}
+
+}  // namespace hwfx

@@ -13,15 +13,17 @@ namespace hw {
 
 // Per-handle tables in both precisions (filled once at creation).
 struct HostTabs {
-  Weights<double> wd;
+  Weights<fx64> wd;
   Weights<float> wf;
   Weights<df64> wx;      // double-float (precision 2)
-  Beta1<double> b1d;
+  Weights<double> wl;    // FP64 with the learned indicator
+  Beta1<fx64> b1d;
   Beta1<float> b1f;
   Beta1<df64> b1x;
-  Beta2<double> b2d;
+  Beta2<fx64> b2d;
   Beta2<float> b2f;
   Beta2<df64> b2x;
+  Beta2<double> b2l;
 };
 
 // Compute precision of a handle: 0 FP64, 1 FP32 bulk, 2 double-float (FP32 pairs).
@@ -170,6 +172,7 @@ cudaError_t run_mlpre2d(const Prob& P, const float* th, float conf, const double
                         int* und, int* und_count, int* stats, float* prob, cudaStream_t st);
 void run_stage_2d(const Prob& P, const HostTabs& T, int prec, const Bufs& B, const StageCall& S, cudaStream_t st);
 void run_stage_2d_fp32(const Prob& P, const HostTabs& T, const Bufs& B, const StageCall& S, cudaStream_t st);
+void run_stage_2d_learned(const Prob& P, const HostTabs& T, const Bufs& B, const StageCall& S, cudaStream_t st);
 void run_stage_2d_df64(const Prob& P, const HostTabs& T, const Bufs& B, const StageCall& S, cudaStream_t st);
 cudaError_t run_batch_stage_df64(const HostTabs& T, int tile_variant, const BatchStage& S, int nsm, cudaStream_t st);
 
