@@ -421,7 +421,8 @@ __device__ __forceinline__ void face_flux(const Prob& P, T (&uL)[NV], T (&uR)[NV
       uR[1] = uR[2]; uR[2] = b;
     }
     T F[4];
-    hllc<T, 4>(P, uL, uR, 0, F, wall);
+    if constexpr (lean<T>::value) hllc_lean<T, 4>(P, uL, uR, 0, F, wall);
+    else hllc<T, 4>(P, uL, uR, 0, F, wall);
     out[0] = F[0];
     out[1] = xd ? F[1] : F[2];
     out[2] = xd ? F[2] : F[1];
@@ -482,13 +483,104 @@ struct StagedSrc {
   }
 };
 
+// Quadrature, L(U) and the Runge-Kutta combination of one cell (2D Euler, the
+// lean precisions), from the integrals of its faces (slot 0 the mean, 1 the first
+// moment; xm left, xp right, ym below, yp above).  The 16 points fall into three
+// groups of one weight (corners 1, edges 5, centre 25, over 144), summed without
+// weights.  With the kinetic terms A = sum w m^2/rho and S = sum w (m^2 + n^2)/rho
+// the momentum fluxes need no pressure per point: sum w p = (gamma - 1)(E - S/2),
+// and the sums of m, n and E are the cell's averages (every q_l has them, and the
+// quadrature is exact for degree 5).
+template <typename T, typename Src>
+__device__ __forceinline__ void update_cell_lean(const Prob& P, const Src& src, const Rk& S, int i, int j,
+                                                 const T (&xm)[4][4], const T (&xp)[4][4], const T (&ym)[4][4],
+                                                 const T (&yp)[4][4]) {
+  const long long so = (long long)j * P.pitch + i;
+  const long long cell = (long long)j * P.nx + i;
+  const T g = pc<T>(P.cgamma), gm1 = pc<T>(P.cgm1), kap = pc<T>(P.chg);
+  T A, C, K, X, Y;
+  A = C = K = X = Y = T(0);
+#pragma unroll
+  for (int grp = 2; grp >= 0; --grp) {               // 25 centre + 5 edges + corners (Horner in 5)
+    if (grp < 2) { A *= T(5); C *= T(5); K *= T(5); X *= T(5); Y *= T(5); }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+      for (int l = 0; l < 4; ++l) {
+        const bool ki = k == 1 || k == 2, li = l == 1 || l == 2;
+        if ((int)ki + (int)li != grp) continue;
+        const int p = k * 4 + l;
+        const T m = src.g(P, 1, p, i, j), n = src.g(P, 2, p, i, j), E = src.g(P, 3, p, i, j);
+        const T inv = rcp(src.g(P, 0, p, i, j));
+        const T mu = m * inv, nu = n * inv;
+        const T s = fma(m, mu, n * nu);
+        A = fma(m, mu, A);
+        C = fma(m, nu, C);
+        K = K + s;
+        const T H = fma(-kap, s, E);                 // (E + p) / gamma
+        X = fma(mu, H, X);
+        Y = fma(nu, H, Y);
+      }
+  }
+  const T w = T(1.0 / 144.0);
+  A *= w; C *= w; K *= w; X *= w * g; Y *= w * g;
+  const T mbar = from_double<T>(src.uin(P, S, 3, i, j)), nbar = from_double<T>(src.uin(P, S, 6, i, j)),
+          Ebar = from_double<T>(src.uin(P, S, 9, i, j));
+  const T pbar = gm1 * fma(T(-0.5), K, Ebar);
+  const T Fc[4] = {mbar, A + pbar, C, X}, Gc[4] = {nbar, C, (K - A) + pbar, Y};
+  // eq. (2D-equ-int-approximation); the average equation in FP64 (its flux differences telescope)
+  const double idx = P.crdx.d, idy = P.crdy.d;
+  const T tidx = pc<T>(P.crdx), tidy = pc<T>(P.crdy);
+  const bool fk = S.mask[cell] != 0 && (P.persist || S.Lout);
+  const bool fn = P.persist && S.maskN && S.maskN[cell] != 0;
+  const bool first = S.cA == 0.0;                    // U^(1) = U' + dt L: no U^n term
+  const bool owned = j >= P.jlo && j < P.jhi;
+  double newavg[4];
+  bool finite = true;
+#pragma unroll
+  for (int v = 0; v < 4; ++v) {
+    double L[3];
+    const T Fp = xp[0][v], Fm = xm[0][v], Gp = yp[0][v], Gm = ym[0][v];
+    L[0] = -(to_f64(Fp) - to_f64(Fm)) * idx - (to_f64(Gp) - to_f64(Gm)) * idy;
+    L[1] = to_f64(fma(T(-0.5), Fp + Fm, Fc[v]) * tidx - (yp[1][v] - ym[1][v]) * tidy);
+    L[2] = to_f64(fma(T(-0.5), Gp + Gm, Gc[v]) * tidy - (xp[1][v] - xm[1][v]) * tidx);
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+      const long long si = (long long)(v * 3 + m) * P.plane + so;
+      const double uin = (m > 0 && fk) ? S.Mod[(long long)(v * 2 + m - 1) * P.plane + so] : src.uin(P, S, v * 3 + m, i, j);
+      if (S.Lout) {
+        S.Lout[si] = L[m];
+        if (S.Umod) S.Umod[si] = uin;
+        continue;
+      }
+      double r;
+      if (first) {
+        r = fma(S.dt, L[m], uin);
+      } else {
+        const double un = (m > 0 && fn) ? S.ModN[(long long)(v * 2 + m - 1) * P.plane + so] : src.un(P, S, v * 3 + m, i, j);
+        r = fma(S.cA, un, S.cB * fma(S.dt, L[m], uin));
+      }
+      S.Uout[si] = r;
+      if (m == 0) newavg[v] = r;
+      finite = finite && ((__double_as_longlong(r) >> 52) & 0x7FF) != 0x7FF;
+    }
+  }
+  if (S.Lout || !owned) return;
+  if (!finite) atomicOr(S.status, ST_NONFINITE);
+  // rho > 0 and p = (gamma - 1)(E - |m|^2 / (2 rho)) > 0, the latter as 2 E rho > |m|^2 (no division)
+  const double m2 = newavg[1] * newavg[1] + newavg[2] * newavg[2];
+  if (!(newavg[0] > 0.0) || !(2.0 * newavg[3] * newavg[0] > m2)) atomicOr(S.status, ST_NONPOSITIVE);
+}
+
 // Step 3 for the TXV x TYV tile at (i0, j0): face fluxes into shared memory, then
 // quadrature, L(U) and the Runge-Kutta combination per cell.  tid = ty*TXV + tx.
+// above: the block has just done the tile below (its top faces are reused).
 // SOLID: the handle may have a solid block (FP64 2D Euler only); without it the
 // wall-face code is not compiled in (the batched kernel runs at the register limit).
 template <typename T, int NV, int TXV, int TYV, bool SOLID = false, typename Src = GlobalSrc<T>>
 __device__ __forceinline__ void update2d_tile(const Prob& P, const Src& src, const Rk& S, int i0, int j0,
-                                              int tid, T (&xf)[TYV][TXV + 1][4][NV], T (&yf)[TYV + 1][TXV][4][NV]) {
+                                              int tid, T (&xf)[TYV][TXV + 1][4][NV], T (&yf)[TYV + 1][TXV][4][NV],
+                                              bool above = false) {
   const int tx = tid % TXV, ty = tid / TXV;
   const int i = i0 + tx, j = j0 + ty;
   const bool live = i < P.nx && j < P.ny;
@@ -501,7 +593,12 @@ __device__ __forceinline__ void update2d_tile(const Prob& P, const Src& src, con
   // the point values at fixed offsets
   const bool tin = Src::staged || ((!SOLID || P.sol_j == 0) && i0 >= 1 && i0 + TXV < P.nx && j0 >= 1 && j0 + TYV < P.ny);
   __syncthreads();   // the shared arrays may still be read for a previous tile
-  for (int f = tid; f < NXP + NYP; f += TXV * TYV) {
+  if (above) {       // the tile below was this block's last: its top faces are this one's bottom faces
+    for (int q = tid; q < TXV * 4 * NV; q += TXV * TYV) (&yf[0][0][0][0])[q] = (&yf[TYV][0][0][0])[q];
+    __syncthreads();
+  }
+  for (int t = tid; t < NXP + NYP - (above ? TXV * 4 : 0); t += TXV * TYV) {
+    const int f = above && t >= NXP ? t + TXV * 4 : t;
     // the face's GL point q, its slot (c, r) in the tile, its two cells a
     // (left / below) and b (right / above) and their point indices
     const bool xd = f < NXP;
@@ -543,6 +640,20 @@ __device__ __forceinline__ void update2d_tile(const Prob& P, const Src& src, con
     face_flux<T, NV>(P, uL, uR, xd, wall, xd ? xf[r][c][q] : yf[r][c][q]);
   }
   __syncthreads();
+  if constexpr (NV == 4 && lean<T>::value) {
+    // face integrals (eq. (integral2), (integral3)), once per face: point slots 0
+    // and 1 become the mean and the first moment along the face
+    constexpr int NXF = (TXV + 1) * TYV * 4;
+    for (int t = tid; t < NXF + TXV * (TYV + 1) * 4 - (above ? TXV * 4 : 0); t += TXV * TYV) {
+      const int f = above && t >= NXF ? t + TXV * 4 : t;
+      const int g = (f < NXF ? f : f - NXF) >> 2, v = f & 3;
+      T* q = f < NXF ? &xf[0][0][0][0] + g * 16 + v : &yf[0][0][0][0] + g * 16 + v;
+      const T f0 = q[0], f1 = q[4], f2 = q[8], f3 = q[12];
+      q[0] = fma(T(5.0 / 12.0), f1 + f2, T(1.0 / 12.0) * (f0 + f3));
+      q[4] = fma(T(5.0 / 12.0 * 0.22360679774997896964), f2 - f1, T(1.0 / 24.0) * (f3 - f0));
+    }
+    __syncthreads();
+  }
   if (!live) return;
   if (SOLID && P.sol_j > 0 && is_solid(P, i, j)) {   // solid cells are not updated: the state passes through
     if (!S.Lout) {
@@ -562,6 +673,9 @@ __device__ __forceinline__ void update2d_tile(const Prob& P, const Src& src, con
     }
     return;
   }
+  if constexpr (NV == 4 && lean<T>::value) {
+    update_cell_lean<T>(P, src, S, i, j, xf[ty][tx], xf[ty][tx + 1], yf[ty][tx], yf[ty + 1][tx]);
+  } else {
   // face integrals (eq. (integral2), (integral3)) and the cell quadrature (eq. (integral1))
   T Fp[NV], Fm[NV], Fpe[NV], Fme[NV], Gp[NV], Gm[NV], Gpx[NV], Gmx[NV], Fc[NV], Gc[NV];
 #pragma unroll
@@ -666,27 +780,53 @@ __device__ __forceinline__ void update2d_tile(const Prob& P, const Src& src, con
     const double m2 = newavg[1] * newavg[1] + newavg[2] * newavg[2];
     if (!(rho > 0.0) || !(2.0 * newavg[NV - 1] * rho > m2)) atomicOr(S.status, ST_NONPOSITIVE);
   }
+  }
 }
 
+// fx64 and double-float: a block does `sweep` tiles, one above the other, and the
+// faces between them once (8.1 instead of 9.1 fluxes per cell at 16 tiles; float,
+// which waits for loads rather than for its arithmetic, measured 9 % slower so).
+// fx64 at 2048^2: 15.2 ms per launch with hllc and the quadrature per point, 9.6
+// with hllc_lean and update_cell_lean, 8.07 with the integer compares, the 5-operation
+// root and the sweep; bound by the FP64 pipe (87 % busy, 1053 operations per cell,
+// 1915 before).  Double-float 5.2 -> 3.0 ms.
 template <typename T, int NV, bool SOLID = false>
-__global__ void __launch_bounds__(TX * TY, (std::is_same<T, float>::value ? 8 : 3)) update2d_kernel(Prob P, const T* __restrict__ G, Rk S) {
+__global__ void __launch_bounds__(TX * TY, (std::is_same<T, float>::value ? 8 : lean<T>::value ? 4 : 3))
+    update2d_kernel(const __grid_constant__ Prob P, const T* __restrict__ G, Rk S, int sweep) {
   __shared__ T xf[TY][TX + 1][4][NV];
   __shared__ T yf[TY + 1][TX][4][NV];
+  const int i0 = blockIdx.x * TX, ja = blockIdx.y * sweep * TY, jb = min(ja + sweep * TY, P.ny);
   if (S.dtp) {
     S.dt = *S.dtp;
     if (S.dt < 0.0) {   // a skipped step (block-uniform): the state passes through unchanged
-      const int i = blockIdx.x * TX + threadIdx.x, j = blockIdx.y * TY + threadIdx.y;
-      if (i < P.nx && j < P.ny && !S.Lout)
-        for (int q = 0; q < NV * 3; ++q) {
-          const long long si = (long long)q * P.plane + (long long)j * P.pitch + i;
-          S.Uout[si] = S.Uin[si];
-          if (S.U32out) S.U32out[si] = f32_rn(S.Uin[si]);
-        }
+      const int i = i0 + threadIdx.x;
+      for (int j = ja + threadIdx.y; j < jb; j += TY)
+        if (i < P.nx && !S.Lout)
+          for (int q = 0; q < NV * 3; ++q) {
+            const long long si = (long long)q * P.plane + (long long)j * P.pitch + i;
+            S.Uout[si] = S.Uin[si];
+            if (S.U32out) S.U32out[si] = f32_rn(S.Uin[si]);
+          }
       return;
     }
   }
-  update2d_tile<T, NV, TX, TY, SOLID>(P, GlobalSrc<T>{G}, S, blockIdx.x * TX, blockIdx.y * TY,
-                                      threadIdx.y * TX + threadIdx.x, xf, yf);
+  const int tid = threadIdx.y * TX + threadIdx.x;
+  if constexpr (lean<T>::value) {
+#pragma unroll 1
+    for (int j0 = ja; j0 < jb; j0 += TY)
+      update2d_tile<T, NV, TX, TY, SOLID>(P, GlobalSrc<T>{G}, S, i0, j0, tid, xf, yf, j0 > ja);
+  } else {
+    update2d_tile<T, NV, TX, TY, SOLID>(P, GlobalSrc<T>{G}, S, i0, ja, tid, xf, yf);
+  }
+}
+
+// Tiles per block: as many as leave six waves of resident blocks (4 per SM), at
+// most 16; small grids keep one, their blocks must reach every SM first.
+template <typename T>
+inline int update_sweep(const Prob& P) {
+  if (!lean<T>::value) return 1;
+  const long long tiles = (long long)((P.nx + TX - 1) / TX) * ((P.ny + TY - 1) / TY);
+  return (int)std::max<long long>(1, std::min<long long>(16, tiles / (6LL * P.nsm * 4)));
 }
 
 // ---------------------------------------------------------------- TMA-staged update (FP32 form)
@@ -864,16 +1004,18 @@ void stage_t(const Prob& P, const HostTabs& HT, const Weights<T>& W, const Beta2
   Rk r{S.Uin, S.Un, S.Uout, S.mask, S.Mod, S.maskN, S.ModN, S.dt, S.cA, S.cB, S.Lout, S.Umod, B.status, S.dtp,
        std::is_same<T, float>::value ? S.U32out : nullptr};
   if (B.prof) B.prof->begin(3, st);
+  const int sweep = update_sweep<T>(P);
+  const dim3 sgrd(grd.x, (grd.y + sweep - 1) / sweep);
   if constexpr (NV == 4 && std::is_same<T, fx64>::value) {
-    if (P.sol_j > 0) update2d_kernel<T, NV, true><<<grd, blk, 0, st>>>(P, (const T*)B.G, r);
-    else update2d_kernel<T, NV><<<grd, blk, 0, st>>>(P, (const T*)B.G, r);
+    if (P.sol_j > 0) update2d_kernel<T, NV, true><<<sgrd, blk, 0, st>>>(P, (const T*)B.G, r, sweep);
+    else update2d_kernel<T, NV><<<sgrd, blk, 0, st>>>(P, (const T*)B.G, r, sweep);
   } else if constexpr (NV == 4 && std::is_same<T, float>::value) {
     if (B.tmG && !S.Lout)
       update2d_tma_kernel<<<grd, blk, TMA_SMEM, st>>>(P, (const float*)B.G, r, *B.tmG);
     else
-      update2d_kernel<T, NV><<<grd, blk, 0, st>>>(P, (const T*)B.G, r);
+      update2d_kernel<T, NV><<<sgrd, blk, 0, st>>>(P, (const T*)B.G, r, sweep);
   } else {
-    update2d_kernel<T, NV><<<grd, blk, 0, st>>>(P, (const T*)B.G, r);
+    update2d_kernel<T, NV><<<sgrd, blk, 0, st>>>(P, (const T*)B.G, r, sweep);
   }
   if (B.prof) B.prof->end(st);
 }

@@ -106,6 +106,7 @@ void fill_consts(Prob& P) {
   P.cgamma = pconst(P.gamma);
   P.cgm1 = pconst(P.gamma - 1.0);
   P.chk = pconst((P.gamma + 1.0) / (2.0 * P.gamma));
+  P.chg = pconst((P.gamma - 1.0) / (2.0 * P.gamma));
   P.cdx = pconst(P.dx);
   P.cdy = pconst(P.dy);
   P.crdx = pconst(1.0 / P.dx);

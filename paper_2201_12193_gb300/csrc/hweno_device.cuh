@@ -71,6 +71,7 @@ struct Prob {
   int fused;              // one fused kernel per stage (1D default; 2D Euler option) instead of the pipeline
   PConst cgamma, cdx, cdy, crdx, crdy, cdx2;   // gamma, dx, dy, 1/dx, 1/dy, dx^2
   PConst cgm1, chk;   // gamma - 1 and (gamma + 1) / (2 gamma) of eq. (COEF)
+  PConst chg;         // (gamma - 1) / (2 gamma)
   int sol_i, sol_j;       // solid block (2D Euler, the forward step): cells i >= sol_i, j < sol_j;
                           //    sol_j = 0: none
   int jlo, jhi;           // owned rows [jlo, jhi): the rows a row-slab of a decomposed grid owns (the
@@ -424,6 +425,76 @@ __device__ __forceinline__ void hllc(const Prob& P, const T* uL, const T* uR, in
   for (int v = 0; v < NV; ++v) F[v] = fK[v] + sK * (us[v] - uK[v]);
 }
 
+// fx64 and double-float take the lean form below (fx64: 68 FP64 operations against
+// 150 of hllc); float and plain double keep hllc.
+template <typename T> struct lean { static constexpr bool value = is_df64<T>::value || std::is_same<T, fx64>::value; };
+template <typename T> __device__ __forceinline__ bool nonneg(T a) { return T(0) <= a; }
+template <typename T> __device__ __forceinline__ bool nonpos(T a) { return a <= T(0); }
+template <typename T> __device__ __forceinline__ bool below(T a, T b) { return a < b; }
+template <typename T> __device__ __forceinline__ T half(T a) { return T(0.5) * a; }
+
+// The same flux with fewer operations.  Only the chosen side's wave speed is
+// formed: s* < 0 with m_L < c_L implies s_L < 0 (its coefficient is at least 1),
+// so s_L matters for s* < 0 only in the remaining case.  The star flux is
+// written through the Rankine-Hugoniot relations of its wave: with
+// w = rho_K (s_K - m_K), p* = p_K + w (s* - m_K) and rho* = w / (s_K - s*) it is
+// (rho* s*, rho* s*^2 + p*, rho* s* t_K, s* (E* + p*)),
+// E* = (E_K (s_K - m_K) - p_K m_K + p* s*) / (s_K - s*).
+template <typename T, int NV>
+__device__ __forceinline__ void hllc_lean(const Prob& P, const T* uL, const T* uR, int dir, T* F, bool wall = false) {
+  constexpr bool two = NV == 4;
+  constexpr int iE = NV - 1;
+  const int in = 1 + dir, it = 2 - dir;
+  const T g = pc<T>(P.cgamma), gm1 = pc<T>(P.cgm1), k = pc<T>(P.chk);
+  const T rL = uL[0], rR = uR[0], EL = uL[iE], ER = uR[iE];
+  T iL, iR;
+  if constexpr (is_df64<T>::value) {   // one division for both
+    const T q = rcp(rL * rR);
+    iL = rR * q;
+    iR = rL * q;
+  } else {
+    iL = rcp(rL);
+    iR = rcp(rR);
+  }
+  const T mL = uL[in] * iL, mR = uR[in] * iR;
+  const T tL = two ? uL[it] * iL : T(0), tR = two ? uR[it] * iR : T(0);
+  T kL = uL[in] * mL, kR = uR[in] * mR;
+  if constexpr (two) { kL = fma(uL[it], tL, kL); kR = fma(uR[it], tR, kR); }
+  const T pL = gm1 * fma(T(-0.5), kL, EL), pR = gm1 * fma(T(-0.5), kR, ER);
+  const T gL = g * iL, gR = g * iR;
+  const T cL = sqrt(gL * pL), cR = sqrt(gR * pR);
+  const T x = (rL + rR) * (cL + cR);                 // four times the mean density times the mean sound speed
+  const T ps = fma((mL - mR) * x, T(0.125), half(pL + pR));
+  const T ss = fma((pL - pR) * rcp(x), T(2), half(mL + mR));
+  auto speed = [&](T gk, T pk, T ck) {               // c_K coef_K of eq. (COEF)
+    const T d = ps - pk;
+    return nonpos(d) ? ck : sqrt(gk * fma(k, d, pk));
+  };
+  bool left = nonneg(ss);
+  if (!left && !wall && !below(mL, cL)) left = nonneg(mL - speed(gL, pL, cL));
+  const T mK = left ? mL : mR, pK = left ? pL : pR, EK = left ? EL : ER, tK = left ? tL : tR;
+  const T sd = speed(left ? gL : gR, pK, left ? cL : cR);
+  const T sK = left ? mK - sd : mK + sd;
+  const bool ge = nonneg(sK);
+  if (!wall && (left ? ge : !ge)) {                  // supersonic: the physical flux of the side
+    const T q = left ? uL[in] : uR[in];
+    F[0] = q;
+    F[in] = fma(q, mK, pK);
+    if constexpr (two) F[it] = q * tK;
+    F[iE] = mK * (EK + pK);
+    return;
+  }
+  const T a = sK - mK, w = (left ? rL : rR) * a;
+  const T pst = fma(w, ss - mK, pK);
+  const T rb = rcp(sK - ss);
+  const T f0 = w * rb * ss;
+  F[0] = f0;
+  F[in] = fma(f0, ss, pst);
+  if constexpr (two) F[it] = f0 * tK;
+  const T e = fma(pst, ss, fma(EK, a, -(pK * mK)));
+  F[iE] = ss * fma(e, rb, pst);
+}
+
 // Scalar laws: local Lax-Friedrichs flux with alpha = max(|f'(uL)|, |f'(uR)|).
 template <typename T>
 __device__ __forceinline__ T llf(const Prob& P, T uL, T uR, int dir) {
@@ -437,6 +508,7 @@ __device__ __forceinline__ T llf(const Prob& P, T uL, T uR, int dir) {
 template <typename T, int NV>
 __device__ __forceinline__ void num_flux(const Prob& P, const T* uL, const T* uR, int dir, T* F) {
   if constexpr (NV == 1) F[0] = llf(P, uL[0], uR[0], dir);
+  else if constexpr (lean<T>::value) hllc_lean<T, NV>(P, uL, uR, dir, F);
   else hllc<T, NV>(P, uL, uR, dir, F);
 }
 

@@ -67,12 +67,12 @@ __device__ __forceinline__ long long to_fx(double x, int e) {
   return ((long long)m ^ s) - s;
 }
 
-// x 2^eb as a double (integer work; truncated to 53 bits).  The caller keeps the exponent in range.
+// x 2^eb as a double (integer work; rounded to 53 bits, halves up).  The caller keeps the exponent in range.
 __device__ __forceinline__ double from_fx(long long x, int eb) {
   const long long s = x >> 63;
   const unsigned long long a = (unsigned long long)((x ^ s) - s);
   const int n = __clzll((long long)a);
-  const unsigned long long m = (a << (n & 63)) >> 11;
+  const unsigned long long m = (((a << (n & 63)) >> 10) + 1) >> 1;   // a carry to 2^53 raises the exponent
   const unsigned long long r = m + ((unsigned long long)(unsigned)(1085 - n + eb) << 52);
   return __longlong_as_double(a ? (long long)(r | ((unsigned long long)s << 63)) : 0LL);
 }
