@@ -164,6 +164,7 @@ __device__ __forceinline__ double f64_of_f32(float x) {
 // A compute-type value as a double (float by the integer widening above).
 template <typename T> __device__ __forceinline__ double to_f64(T x) { return (double)x; }
 template <> __device__ __forceinline__ double to_f64<float>(float x) { return f64_of_f32(x); }
+template <> __device__ __forceinline__ double to_f64<df64>(df64 x) { return f64_of_f32(x.hi) + f64_of_f32(x.lo); }
 
 // A run-time double in the compute type (df64 by the integer split; float by
 // the FP64 conversion, which measured faster than f32_rn in the gathers of the

@@ -67,7 +67,7 @@ enum RecMode { REC_PLAIN = 0, REC_FLAGGED = 1, REC_MIXED = 2 };
 // Moment of kind 0 (average), 1 (x first moment) or 2 (y first moment) of
 // the stencil cell (ox, oy); when usemod, first moments of flagged stencil
 // cells come from the modified copy (eq. (vi) applied before Step 2.3).
-template <int MODE, bool SIGNBIT, bool FIX>
+template <int MODE, bool FIX>
 __device__ __forceinline__ double load_mom(const Prob& P, const double* __restrict__ U, const uint8_t* __restrict__ mask,
                                            const double* __restrict__ Mod, const Nbr& n, int var, int kind, int ox,
                                            int oy, bool usemod) {
@@ -78,37 +78,21 @@ __device__ __forceinline__ double load_mom(const Prob& P, const double* __restri
   const int ci = FIX ? n.ci[oy + 1][ox + 1] : n.xi[ox + 1], cj = FIX ? n.cj[oy + 1][ox + 1] : n.yj[oy + 1];
   const int sxm = FIX ? n.csx[oy + 1][ox + 1] : n.xs[ox + 1], sym = FIX ? n.csy[oy + 1][ox + 1] : n.ys[oy + 1];
   const long long so = (long long)cj * P.pitch + ci;
-  if constexpr (SIGNBIT) {
-    // FP64 / FP32 paths: the sign bit flipped by integer work (no FP64
-    // instruction; bitwise the same as negation), measured 6 % faster in FP64
-    unsigned long long flip = ((n.neg[oy + 1][ox + 1] >> var) & 1) ? 1ull : 0ull;
-    double v;
-    if (kind == 0) {
-      v = U[(long long)(var * 3) * P.plane + so];
-    } else {
-      if (MODE != REC_PLAIN && usemod && mask[(long long)cj * P.nx + ci] == 1)
-        v = Mod[(long long)(var * 2 + kind - 1) * P.plane + so];
-      else
-        v = U[(long long)(var * 3 + kind) * P.plane + so];
-      if (kind == 1 && sxm < 0) flip ^= 1ull;
-      if (kind == 2 && sym < 0) flip ^= 1ull;
-    }
-    return __longlong_as_double(__double_as_longlong(v) ^ (long long)(flip << 63));
+  // the sign bit flipped by integer work (no FP64 instruction; bitwise the same
+  // as negation), measured 6 % faster in FP64
+  unsigned long long flip = ((n.neg[oy + 1][ox + 1] >> var) & 1) ? 1ull : 0ull;
+  double v;
+  if (kind == 0) {
+    v = U[(long long)(var * 3) * P.plane + so];
   } else {
-    // double-float path: plain negation (fewer registers there, measured faster)
-    if (kind == 0) {
-      const double u = U[(long long)(var * 3) * P.plane + so];
-      return (n.neg[oy + 1][ox + 1] >> var) & 1 ? -u : u;
-    }
-    double v;
     if (MODE != REC_PLAIN && usemod && mask[(long long)cj * P.nx + ci] == 1)
       v = Mod[(long long)(var * 2 + kind - 1) * P.plane + so];
     else
       v = U[(long long)(var * 3 + kind) * P.plane + so];
-    if (kind == 1 && sxm < 0) v = -v;
-    if (kind == 2 && sym < 0) v = -v;
-    return (n.neg[oy + 1][ox + 1] >> var) & 1 ? -v : v;
+    if (kind == 1 && sxm < 0) flip ^= 1ull;
+    if (kind == 2 && sym < 0) flip ^= 1ull;
   }
+  return __longlong_as_double(__double_as_longlong(v) ^ (long long)(flip << 63));
 }
 
 // FP32 form: the moment from the float copy of the state the update kernel
@@ -136,8 +120,9 @@ __device__ __forceinline__ float load_mom32(const Prob& P, const float* __restri
 }
 
 template <typename T, int NV, int MODE, bool FIX = false, bool S32 = false>
-__device__ __forceinline__ void rec2d_cell(const Prob& P, const Weights<T>& W, const Beta2<T>& B,
-                                           const double* __restrict__ U, const uint8_t* __restrict__ mask,
+__device__ __forceinline__ void rec2d_cell(const Prob& P, const Weights<T>& W,
+                                           const typename rows2d<T>::type& B, const double* __restrict__ U,
+                                           const uint8_t* __restrict__ mask,
                                            const double* __restrict__ Mod, int i, int j, T* __restrict__ G,
                                            T* __restrict__ aux, const float* __restrict__ U32 = nullptr) {
   constexpr bool FLAGGED = MODE == REC_FLAGGED;
@@ -146,25 +131,26 @@ __device__ __forceinline__ void rec2d_cell(const Prob& P, const Weights<T>& W, c
   const long long o = goff(P, i, j);
   // FP32 from the float copy and fx64, plain pass, all 3 x 3 cells inside the grid: no image to apply,
   // the moments are read at fixed offsets from the cell's own
-  constexpr bool DIRECT = (S32 || (std::is_same<T, fx64>::value && !FIX)) && MODE == REC_PLAIN;
+  constexpr bool DIRECT = (S32 || (fixed2d<T>::value && !FIX)) && MODE == REC_PLAIN;
   const bool inner = DIRECT && i > 0 && i < P.nx - 1 && j > 0 && j < P.ny - 1;
   using Src = std::conditional_t<S32, float, double>;
   const Src* __restrict__ Uc;
   if constexpr (S32) Uc = U32 + ((long long)j * P.pitch + i);
   else Uc = U + ((long long)j * P.pitch + i);
-  constexpr bool D64 = std::is_same<T, fx64>::value;
+  constexpr bool FXD = fixed2d<T>::value;
+  using D = std::conditional_t<FXD, double, T>;   // the data's type
   T rinv[16];
   T pxl = T(0), pxr = T(0), pyb = T(0), pyt = T(0), nrm = T(0);
-  [[maybe_unused]] long long nrmb = 0;   // FP64: the norm's bits (non-negative doubles order like them)
+  [[maybe_unused]] long long nrmb = 0;   // fx64: the norm's bits (non-negative doubles order like them)
 #pragma unroll 1
   for (int v = 0; v < NV; ++v) {
-    T d[23];
+    D d[23];
     if (inner) {
 #pragma unroll
       for (int c = 0; c < 23; ++c) {
         int kind, ox, oy;
         d4_slot(c, kind, ox, oy);
-        if constexpr (DIRECT) d[c] = T(Uc[(long long)(v * 3 + kind) * P.plane + (long long)oy * P.pitch + ox]);
+        if constexpr (DIRECT) d[c] = D(Uc[(long long)(v * 3 + kind) * P.plane + (long long)oy * P.pitch + ox]);
       }
     } else {
 #pragma unroll
@@ -174,24 +160,27 @@ __device__ __forceinline__ void rec2d_cell(const Prob& P, const Weights<T>& W, c
         if constexpr (S32)
           d[c] = load_mom32<MODE>(P, U32, mask, Mod, nb, v, kind, ox, oy, usemod);
         else
-          d[c] = from_double<T>(load_mom<MODE, !is_df64<T>::value, FIX>(P, U, mask, Mod, nb, v, kind, ox, oy, usemod));
+          d[c] = from_double<D>(load_mom<MODE, FIX>(P, U, mask, Mod, nb, v, kind, ox, oy, usemod));
       }
     }
     T out[16];
-    if constexpr (D64) {
+    if constexpr (FXD) {
       // the point values go out as they are formed (four base points in turn);
       // the partials read them back below
       T* __restrict__ Gv = G + (long long)(v * 16) * P.gplane + o;
-      recon2d<T>(W, B, d, [&](int p, T x) {
+      recon2d_fx<T>(W, B, d, [&](int p, T x) {
         Gv[p * P.gplane] = x;
-        if (!FLAGGED && v == 0) nrmb = max(nrmb, __double_as_longlong(x.v) & 0x7FFFFFFFFFFFFFFFLL);
+        if (!FLAGGED && v == 0) {
+          if constexpr (is_df64<T>::value) nrm = tmax(nrm, tabs(x));
+          else nrmb = max(nrmb, __double_as_longlong(x.v) & 0x7FFFFFFFFFFFFFFFLL);
+        }
       });
     } else {
       recon2d<T>(W, B, d, [&](int p, T x) { out[p] = x; });
 #pragma unroll
       for (int p = 0; p < 16; ++p) G[(long long)(v * 16 + p) * P.gplane + o] = out[p];
     }
-    if (!FLAGGED && !D64) {
+    if (!FLAGGED && !FXD) {
       if (v == 0) {
 #pragma unroll
         for (int p = 0; p < 16; ++p) nrm = tmax(nrm, tabs(out[p]));
@@ -236,11 +225,11 @@ __device__ __forceinline__ void rec2d_cell(const Prob& P, const Weights<T>& W, c
       }
     }
   }
-  if constexpr (D64 && !FLAGGED) {
-    nrm = __longlong_as_double(nrmb);
+  if constexpr (FXD && !FLAGGED) {
+    if constexpr (!is_df64<T>::value) nrm = __longlong_as_double(nrmb);
     if (P.eq == EQ_ADV) {
-      pxl = pxr = P.adv_a;
-      pyb = pyt = P.adv_b;
+      pxl = pxr = T(P.adv_a);
+      pyb = pyt = T(P.adv_b);
     } else {
       // faces x-lo, x-hi, y-lo, y-hi: point indices p0 + q dp, velocity (rho mu)/rho, (rho nu)/rho or u
       const T* Gr = G + o;
@@ -268,8 +257,9 @@ __device__ __forceinline__ void rec2d_cell(const Prob& P, const Weights<T>& W, c
 
 // rerec (REC_FLAGGED only, may be null) accumulates the number of cells
 // reconstructed a second time.
-// Double-float: 4 resident blocks per SM (at most 128 registers, a few spills)
-// beat 3 (168 registers, none): 7.0 vs 8.3 ms per launch at 2048^2.  FP32 with
+// Double-float: 4 resident blocks per SM 5.41 ms per 2048^2 launch, 3 5.72, 5 5.79
+// (all in pairs: 7.6; 30 k instructions per cell, the ALU 45 % busy; its weights in
+// FP64 beside the integers measured alike, 5.6).  FP32 with
 // the float copy: 8 blocks (64 registers, 164 B of spills) measured 0.545 ms per
 // 2048^2 launch against 0.685 at 4 blocks (119 registers).  FP64: 5 blocks (96
 // registers, 20 spilled) 5.52 ms per 2048^2 launch, 4 blocks 5.71, 2 blocks 6.34;
@@ -277,7 +267,9 @@ __device__ __forceinline__ void rec2d_cell(const Prob& P, const Weights<T>& W, c
 // operations per cell instead of 2330, the FP64 pipe 80 % busy beside 20 k
 // integer instructions per cell.
 template <typename T, int NV, int MODE, bool FIX = false, bool S32 = false>
-__global__ void __launch_bounds__(RB, (is_df64<T>::value ? 4 : std::is_same<T, float>::value ? 8 : std::is_same<T, fx64>::value ? 5 : 1)) rec2d_kernel(const __grid_constant__ Prob P, const __grid_constant__ Weights<T> W, const __grid_constant__ Beta2<T> B, const double* __restrict__ U,
+__global__ void __launch_bounds__(RB, (is_df64<T>::value ? 4 : std::is_same<T, float>::value ? 8 : std::is_same<T, fx64>::value ? 5 : 1)) rec2d_kernel(
+    const __grid_constant__ Prob P, const __grid_constant__ Weights<T> W,
+    const __grid_constant__ typename rows2d<T>::type B, const double* __restrict__ U,
                                                   const uint8_t* __restrict__ mask, const double* __restrict__ Mod,
                                                   const int* __restrict__ list, const int* __restrict__ count,
                                                   T* __restrict__ G, T* __restrict__ aux,
@@ -296,7 +288,7 @@ __global__ void __launch_bounds__(RB, (is_df64<T>::value ? 4 : std::is_same<T, f
 
 // Step 2.1 for one cell: the troubled-cell decision of the configured indicator.
 template <typename T>
-__device__ __forceinline__ bool flag2d_cell(const Prob& P, const Weights<T>& W, const double* __restrict__ U,
+__device__ __forceinline__ bool flag2d_cell(const Prob& P, const double* __restrict__ U,
                                             const T* __restrict__ G, const T* __restrict__ aux, int i, int j,
                                             double* __restrict__ aleph) {
   if (P.sol_j > 0 && is_solid(P, i, j)) {
@@ -306,7 +298,7 @@ __device__ __forceinline__ bool flag2d_cell(const Prob& P, const Weights<T>& W, 
   if (P.indicator == IND_ALL) return true;
   if (P.indicator == IND_TVB) return tvb_cell(P, U, i, j);
   if (P.indicator != IND_KXRCF) return false;
-  const T a = kxrcf2d<T>(P, W, G, aux, i, j);
+  const T a = kxrcf2d<T>(P, G, aux, i, j);
   if (aleph) aleph[(long long)j * P.nx + i] = double(a);
   return a > T(1);
 }
@@ -349,14 +341,14 @@ __device__ __forceinline__ void warp_append(bool flag, E entry, E* __restrict__ 
 }
 
 template <typename T, int NV>
-__global__ void __launch_bounds__(TX * TY) flag2d_kernel(Prob P, Weights<T> W, const double* __restrict__ U,
+__global__ void __launch_bounds__(TX * TY) flag2d_kernel(const __grid_constant__ Prob P, const double* __restrict__ U,
                                                         const T* __restrict__ G, const T* __restrict__ aux,
                                                         uint8_t* __restrict__ mask, double* __restrict__ Mod,
                                                         int* __restrict__ list, int* __restrict__ count,
                                                         double* __restrict__ aleph) {
   const int i = blockIdx.x * TX + threadIdx.x, j = blockIdx.y * TY + threadIdx.y;
   const bool valid = i < P.nx && j < P.ny;
-  const bool flag = valid && flag2d_cell<T>(P, W, U, G, aux, i, j, aleph);
+  const bool flag = valid && flag2d_cell<T>(P, U, G, aux, i, j, aleph);
   warp_append<int>(flag, j * P.nx + i, list, count);   // a warp is one tile row
   if (!valid) return;
   mask[(long long)j * P.nx + i] = flag ? 1 : 0;
@@ -366,7 +358,7 @@ __global__ void __launch_bounds__(TX * TY) flag2d_kernel(Prob P, Weights<T> W, c
 // KXRCF for the cells the learned indicator left undecided (mask 2): the
 // decision, eq. (vi) for the troubled ones and their list for Step 2.3.
 template <typename T, int NV>
-__global__ void __launch_bounds__(RB) fallback2d_kernel(Prob P, Weights<T> W, const double* __restrict__ U,
+__global__ void __launch_bounds__(RB) fallback2d_kernel(const __grid_constant__ Prob P, const double* __restrict__ U,
                                                        const T* __restrict__ G, const T* __restrict__ aux,
                                                        const int* __restrict__ und, const int* __restrict__ und_count,
                                                        uint8_t* __restrict__ mask, double* __restrict__ Mod,
@@ -382,7 +374,7 @@ __global__ void __launch_bounds__(RB) fallback2d_kernel(Prob P, Weights<T> W, co
     if (t < n) {
       cell = und[t];
       const int i = cell % P.nx, j = cell / P.nx;
-      const T a = kxrcf2d<T>(P, W, G, aux, i, j);
+      const T a = kxrcf2d<T>(P, G, aux, i, j);
       if (aleph) aleph[cell] = double(a);
       flag = a > T(1);
       mask[cell] = flag ? 1 : 0;
@@ -522,12 +514,13 @@ __device__ __forceinline__ void update_cell_lean(const Prob& P, const Src& src, 
         Y = fma(nu, H, Y);
       }
   }
+  // (every product that meets a sum is a written fma: what the compiler would
+  // contract could differ between the kernels that share this, which agree bit for bit)
   const T w = T(1.0 / 144.0);
-  A *= w; C *= w; K *= w; X *= w * g; Y *= w * g;
   const T mbar = from_double<T>(src.uin(P, S, 3, i, j)), nbar = from_double<T>(src.uin(P, S, 6, i, j)),
           Ebar = from_double<T>(src.uin(P, S, 9, i, j));
-  const T pbar = gm1 * fma(T(-0.5), K, Ebar);
-  const T Fc[4] = {mbar, A + pbar, C, X}, Gc[4] = {nbar, C, (K - A) + pbar, Y};
+  const T pbar = gm1 * fma(T(-0.5) * w, K, Ebar);
+  const T Fc[4] = {mbar, fma(w, A, pbar), w * C, w * g * X}, Gc[4] = {nbar, w * C, fma(w, K - A, pbar), w * g * Y};
   // eq. (2D-equ-int-approximation); the average equation in FP64 (its flux differences telescope)
   const double idx = P.crdx.d, idy = P.crdy.d;
   const T tidx = pc<T>(P.crdx), tidy = pc<T>(P.crdy);
@@ -541,9 +534,9 @@ __device__ __forceinline__ void update_cell_lean(const Prob& P, const Src& src, 
   for (int v = 0; v < 4; ++v) {
     double L[3];
     const T Fp = xp[0][v], Fm = xm[0][v], Gp = yp[0][v], Gm = ym[0][v];
-    L[0] = -(to_f64(Fp) - to_f64(Fm)) * idx - (to_f64(Gp) - to_f64(Gm)) * idy;
-    L[1] = to_f64(fma(T(-0.5), Fp + Fm, Fc[v]) * tidx - (yp[1][v] - ym[1][v]) * tidy);
-    L[2] = to_f64(fma(T(-0.5), Gp + Gm, Gc[v]) * tidy - (xp[1][v] - xm[1][v]) * tidx);
+    L[0] = -fma(to_f64(Fp) - to_f64(Fm), idx, (to_f64(Gp) - to_f64(Gm)) * idy);
+    L[1] = to_f64(fma(fma(T(-0.5), Fp + Fm, Fc[v]), tidx, (ym[1][v] - yp[1][v]) * tidy));
+    L[2] = to_f64(fma(fma(T(-0.5), Gp + Gm, Gc[v]), tidy, (xm[1][v] - xp[1][v]) * tidx));
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
       const long long si = (long long)(v * 3 + m) * P.plane + so;
@@ -924,7 +917,7 @@ namespace {
 // Fixed-state ghosts are supported for 2D Euler in FP64 (the library rejects
 // other combinations), so only that instantiation carries the FIX variant.
 template <typename T, int NV, int MODE>
-void launch_rec2d(int blocks, cudaStream_t st, const Prob& P, const Weights<T>& W, const Beta2<T>& Bt,
+void launch_rec2d(int blocks, cudaStream_t st, const Prob& P, const Weights<T>& W, const typename rows2d<T>::type& Bt,
                   const double* U, const uint8_t* mask, const double* Mod, const int* list, const int* count, T* G,
                   T* aux, unsigned long long* rerec, const float* U32 = nullptr) {
   if constexpr (std::is_same<T, float>::value) {
@@ -944,14 +937,18 @@ void launch_rec2d(int blocks, cudaStream_t st, const Prob& P, const Weights<T>& 
 }
 
 template <typename T, int NV>
-void stage_t(const Prob& P, const HostTabs& HT, const Weights<T>& W, const Beta2<T>& Bt, const Bufs& B,
+void stage_t(const Prob& P, const HostTabs& HT, const Weights<T>& W, const Beta2<T>& Btf, const Bufs& B,
              const StageCall& S, cudaStream_t st) {
+  const typename rows2d<T>::type* rows;   // Btf serves the fused kernel, rows the pipeline's
+  if constexpr (is_df64<T>::value) rows = &HT.b2d;
+  else rows = &Btf;
+  const typename rows2d<T>::type& Bt = *rows;
   if constexpr (NV == 4 && !std::is_same<T, double>::value) {
     if (fused_applies(P, NV)) {   // the whole stage in one launch
       Rk r{S.Uin, S.Un, S.Uout, S.mask, S.Mod, S.maskN, S.ModN, S.dt, S.cA, S.cB, S.Lout, S.Umod, B.status, S.dtp};
       FzOut o{S.mask, S.Mod, S.aleph, B.rerec};
       if (B.prof) B.prof->begin(5, st);
-      launch_fused2d<T>(P, W, Bt, r, o, st);
+      launch_fused2d<T>(P, W, Btf, r, o, st);
       if (B.prof) B.prof->end(st);
       return;
     }
@@ -980,7 +977,7 @@ void stage_t(const Prob& P, const HostTabs& HT, const Weights<T>& W, const Beta2
                                                              (T*)B.G, (T*)B.aux, nullptr);
       if (B.prof) B.prof->end(st);
       if (B.prof) B.prof->begin(1, st);
-      fallback2d_kernel<T, NV><<<fblocks, RB, 0, st>>>(P, W, S.Uin, (const T*)B.G, (const T*)B.aux, B.und, ucnt,
+      fallback2d_kernel<T, NV><<<fblocks, RB, 0, st>>>(P, S.Uin, (const T*)B.G, (const T*)B.aux, B.und, ucnt,
                                                        S.mask, S.Mod, B.list, cnt, S.aleph);
       if (B.prof) B.prof->end(st);
     }
@@ -991,7 +988,7 @@ void stage_t(const Prob& P, const HostTabs& HT, const Weights<T>& W, const Beta2
                                    (T*)B.aux, nullptr, S.U32in);
     if (B.prof) B.prof->end(st);
     if (B.prof) B.prof->begin(1, st);
-    flag2d_kernel<T, NV><<<grd, blk, 0, st>>>(P, W, S.Uin, (const T*)B.G, (const T*)B.aux, S.mask, S.Mod, B.list,
+    flag2d_kernel<T, NV><<<grd, blk, 0, st>>>(P, S.Uin, (const T*)B.G, (const T*)B.aux, S.mask, S.Mod, B.list,
                                               cnt, S.aleph);
     if (B.prof) B.prof->end(st);
   }
@@ -1071,7 +1068,7 @@ __device__ __forceinline__ int owner(const BProb* __restrict__ probs, int n, int
 
 template <typename T, int TXV, int TYV>
 __global__ void __launch_bounds__(TXV * TYV) batch_stage_kernel(const __grid_constant__ BatchStage A, const __grid_constant__ Weights<T> W,
-                                                                const __grid_constant__ Beta2<T> B) {
+                                                                const __grid_constant__ typename rows2d<T>::type B) {
   static_assert(TXV * TYV == RB, "tiles and rows use the same block");
   __shared__ T xf[TYV][TXV + 1][4][4];
   __shared__ T yf[TYV + 1][TXV][4][4];
@@ -1123,7 +1120,7 @@ __global__ void __launch_bounds__(TXV * TYV) batch_stage_kernel(const __grid_con
     const int cell = (it - Q.rec_first) * RB + tid;
     const bool valid = cell < Q.P.nx * Q.P.ny;
     const int i = cell % Q.P.nx, j = cell / Q.P.nx;
-    const bool flag = valid && flag2d_cell<T>(Q.P, W, A.Uin + Q.uoff, G + Q.goff, aux + Q.aoff, i, j, nullptr);
+    const bool flag = valid && flag2d_cell<T>(Q.P, A.Uin + Q.uoff, G + Q.goff, aux + Q.aoff, i, j, nullptr);
     warp_append<unsigned long long>(flag, ((unsigned long long)p << 32) | (unsigned)cell, A.list, A.count);
     if (valid) {
       A.mask[Q.coff + cell] = flag ? 1 : 0;
@@ -1169,7 +1166,7 @@ __global__ void __launch_bounds__(TXV * TYV) batch_stage_kernel(const __grid_con
 }
 
 template <typename T, int TXV, int TYV>
-cudaError_t launch_batch(const Weights<T>& W, const Beta2<T>& Bt, const BatchStage& S, int nsm, cudaStream_t st) {
+cudaError_t launch_batch(const Weights<T>& W, const typename rows2d<T>::type& Bt, const BatchStage& S, int nsm, cudaStream_t st) {
   auto kern = batch_stage_kernel<T, TXV, TYV>;
   int per_sm = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, RB, 0);

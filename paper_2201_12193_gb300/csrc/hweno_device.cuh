@@ -125,6 +125,16 @@ template <typename T> __device__ __forceinline__ T gl_x(int k) {
 
 template <typename T> __device__ __forceinline__ T tabs(T x) { return x < T(0) ? -x : x; }
 template <typename T> __device__ __forceinline__ T tmax(T a, T b) { return a > b ? a : b; }
+template <> __device__ __forceinline__ fx64 tabs<fx64>(fx64 x) { return fabs(x.v); }
+// (of non-negative values everywhere: their bits order like them, and a NaN wins)
+template <> __device__ __forceinline__ fx64 tmax<fx64>(fx64 a, fx64 b) {
+  return __longlong_as_double(max(__double_as_longlong(a.v), __double_as_longlong(b.v)));
+}
+// The smoothness-indicator rows a pipeline kernel takes (double-float: those of
+// fx64), and the precisions it reconstructs in fixed point (recon2d_fx).
+template <typename T> struct rows2d { using type = Beta2<T>; };
+template <> struct rows2d<df64> { using type = Beta2<fx64>; };
+template <typename T> struct fixed2d { static constexpr bool value = is_df64<T>::value || std::is_same<T, fx64>::value; };
 
 // ---------------------------------------------------------------- boundary images
 // A ghost cell is the image of an interior cell: periodic wrap, or (transmissive)
@@ -552,36 +562,67 @@ __device__ __forceinline__ void combine_weights(const Weights<T>& W, const T bet
 // omega_l = gamma_l n_l / sum_m gamma_m n_m with n_l = (x_l + tau) prod_{m != l} x_m,
 // and, gamma_l S_l/g_l being S_l/S_4, c_k = (S_k/S_4) (n_k - n_{k+1}) / sum_m gamma_m n_m.
 // c_1 = 1 - c_2 - c_3 - c_4 is not formed: q_1 is the target average u_5 and
-// u = u_5 + sum_{k>1} c_k (q_k - u_5).  c[3] is c_2 + c_3.
-__device__ __forceinline__ void combine_weights_fp64(const Weights<fx64>& W, const double beta[4], double c[4]) {
+// u = u_5 + sum_{k>1} c_k (q_k - u_5).  c = (c_2, c_3, c_4, c_2 + c_3).
+__device__ __forceinline__ void weights_c(const Weights<fx64>& W, const fx64 (&bt)[4], fx64 (&c)[4]) {
+  const double beta[4] = {bt[0].v, bt[1].v, bt[2].v, bt[3].v};
   const double tau4s = fabs(beta[3] - beta[0]) + fabs(beta[3] - beta[1]) + fabs(beta[3] - beta[2]);
-  const double tau4 = (tau4s * (1.0 / 3.0)) * (tau4s * (1.0 / 3.0));
+  const double q = tau4s * (1.0 / 3.0);             // tau_4 = q^2
   const double eps = W.eps.v;
   const double x0 = beta[0] + eps, x1 = beta[1] + eps, x2 = beta[2] + eps, x3 = beta[3] + eps;
   const double p01 = x0 * x1, p23 = x2 * x3;
-  const double n0 = (x0 + tau4) * (x1 * p23), n1 = (x1 + tau4) * (x0 * p23);
-  const double n2 = (x2 + tau4) * (p01 * x3), n3 = (x3 + tau4) * (p01 * x2);
+  const double n0 = fma(q, q, x0) * (x1 * p23), n1 = fma(q, q, x1) * (x0 * p23);
+  const double n2 = fma(q, q, x2) * (p01 * x3), n3 = fma(q, q, x3) * (p01 * x2);
   const double inv = rcp64(fma(W.gam[3].v, n3, fma(W.gam[2].v, n2, fma(W.gam[1].v, n1, W.gam[0].v * n0))));
-  c[0] = (W.ss[1].v * (n1 - n2)) * inv;
-  c[1] = (W.ss[2].v * (n2 - n3)) * inv;
+  c[0] = (W.ss[1].v * __dsub_rn(n1, n2)) * inv;
+  c[1] = (W.ss[2].v * __dsub_rn(n2, n3)) * inv;
   c[2] = n3 * inv;
-  c[3] = c[0] + c[1];
+  c[3] = __dadd_rn(c[0].v, c[1].v);
 }
 
-// sum_k c[k] s[k] of a beta row as a double: the row's units are 2^(e0 + f).
-template <int N>
-__device__ __forceinline__ double fx_row(const hwfx::Half2 (&s)[N], const int2 (&c)[N], int ef) {
+__device__ __forceinline__ void weights_c(const Weights<df64>& W, const df64 (&beta)[4], df64 (&c)[4]) {
+  df64 k[4];
+  combine_weights<df64>(W, beta, k);
+  c[0] = k[1];
+  c[1] = k[2];
+  c[2] = k[3];
+  c[3] = k[1] + k[2];
+}
+
+// A fixed-point value x 2^eb in the compute precision.
+template <typename T> __device__ __forceinline__ T from_fixed(long long x, int eb);
+template <> __device__ __forceinline__ fx64 from_fixed<fx64>(long long x, int eb) { return hwfx::from_fx(x, eb); }
+template <> __device__ __forceinline__ df64 from_fixed<df64>(long long x, int eb) {
+  const float2 r = hwfx::from_fx_pair(x, eb);
+  return df64(r.x, r.y);
+}
+
+// sum_k c[k] s[k] of a beta row: the row's units are 2^ef.
+template <typename T, int N>
+__device__ __forceinline__ T fx_row(const hwfx::Half2 (&s)[N], const int2 (&c)[N], int ef) {
   hwfx::Acc t = hwfx::prod(s[0], c[0].x, c[0].y);
 #pragma unroll
   for (int k = 1; k < N; ++k) hwfx::mac(t, s[k], c[k].x, c[k].y);
-  return hwfx::from_fx(hwfx::scaled<60>(t), ef);
+  return from_fixed<T>(hwfx::scaled<60>(t), ef);
 }
 
-// The FP64 weights as fixed-point integers of one exponent; returns it (2047 if one is not finite).
-__device__ __forceinline__ int fx_weights(const double (&c)[4], hwfx::Half2 (&h)[4]) {
-  const int e = max(max(max(hwfx::bexp(c[0]), hwfx::bexp(c[1])), max(hwfx::bexp(c[2]), hwfx::bexp(c[3]))), hwfx::CEMIN);
+// The weights c_2, c_3, c_4, c_2 + c_3 as fixed-point integers of one exponent;
+// returns it (2047 if one is not finite).
+__device__ __forceinline__ int fx_weights(const fx64 (&c)[4], hwfx::Half2 (&h)[4]) {
+  const int e = max(max(max(hwfx::bexp(c[0].v), hwfx::bexp(c[1].v)), max(hwfx::bexp(c[2].v), hwfx::bexp(c[3].v))),
+                    hwfx::CEMIN);
 #pragma unroll
-  for (int k = 0; k < 4; ++k) h[k] = hwfx::halves(hwfx::to_fx<hwfx::CBITS>(c[k], e));
+  for (int k = 0; k < 4; ++k) h[k] = hwfx::halves(hwfx::to_fx<hwfx::CBITS>(c[k].v, e));
+  return e;
+}
+__device__ __forceinline__ int fx_weights(const df64 (&c)[4], hwfx::Half2 (&h)[4]) {
+  int f = 1;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) f = max(f, (int)((__float_as_uint(c[k].hi) >> 23) & 0xFF));
+  if (f == 0xFF) f = 0x7FF - 896;
+  const int e = f + 896;
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    h[k] = hwfx::halves(hwfx::to_fx<hwfx::CBITS>(c[k].hi, e) + hwfx::to_fx<hwfx::CBITS>(c[k].lo, e));
   return e;
 }
 
@@ -601,28 +642,27 @@ __device__ __forceinline__ void recon1d_fp64(const Weights<fx64>& W, const Beta1
   for (int k = 0; k < 6; ++k) q[k] = k == 1 ? 0 : hwfx::to_fx<hwfx::BITS>(dv[k], e);
   hwfx::Half2 sa[2], sb[3];
   hwp::fx_split1d(q, sa, sb);
-  double beta[4];
+  fx64 beta[4];
   const int e0 = e - (1022 + hwfx::BITS);
 #pragma unroll
   for (int l = 0; l < 3; ++l) {
-    double bl = 0.0;
+    fx64 bl = 0.0;
 #pragma unroll
-    for (int r = hwp::D1_RA(l); r < hwp::D1_RA(l + 1); ++r) { const double x = fx_row(sa, B.a[r], e0 + B.fa[r]); bl = fma(x, x, bl); }
+    for (int r = hwp::D1_RA(l); r < hwp::D1_RA(l + 1); ++r) { const fx64 x = fx_row<fx64>(sa, B.a[r], e0 + B.fa[r]); bl = fma(x, x, bl); }
 #pragma unroll
-    for (int r = hwp::D1_RB(l); r < hwp::D1_RB(l + 1); ++r) { const double x = fx_row(sb, B.b[r], e0 + B.fb[r]); bl = fma(x, x, bl); }
+    for (int r = hwp::D1_RB(l); r < hwp::D1_RB(l + 1); ++r) { const fx64 x = fx_row<fx64>(sb, B.b[r], e0 + B.fb[r]); bl = fma(x, x, bl); }
     beta[l + 1] = bl;
   }
   // beta_1: eqs. (beta1-LR), (tau1), (w1_-LR), (w1-LR), (beta1) over a common denominator
   {
-    const double bl = dl * dl, br = dr * dr;
-    const double t1 = (br - bl) * (br - bl);
-    const double xl = bl + W.eps.v, xr = br + W.eps.v;
-    const double nl = (xl + t1) * xr, nr = (xr + t1) * xl;
-    const double gg = (nl * dl + nr * dr) * rcp64(nl + nr);
+    const double td = fma(dr, dr, -(dl * dl));       // tau_1 = td^2
+    const double xl = fma(dl, dl, W.eps.v), xr = fma(dr, dr, W.eps.v);
+    const double nl = fma(td, td, xl) * xr, nr = fma(td, td, xr) * xl;
+    const double gg = fma(nl, dl, nr * dr) * rcp64(__dadd_rn(nl, nr));
     beta[0] = gg * gg;
   }
-  double c[4];
-  combine_weights_fp64(W, beta, c);
+  fx64 c[4];
+  weights_c(W, beta, c);
   hwfx::Half2 h[4];
   const int ec = fx_weights(c, h);
   long long x[4];
@@ -668,21 +708,53 @@ __device__ __forceinline__ void recon1d(const Weights<T>& W, const Beta1<T>& B, 
 }
 
 // ---------------------------------------------------------------- 2D reconstruction
+// beta_1: eqs. (2D-q1-1234) .. (2D-beta1).  With x differences a (west), b (east)
+// and y differences g (south), h (north), the four one-sided |grad|^2 are a^2 + h^2,
+// b^2 + h^2, b^2 + g^2, a^2 + g^2; their six unordered differences are +-A twice,
+// +-B twice, +-(A + B) and +-(A - B), A = a^2 - b^2, B = h^2 - g^2, so that
+// tau_1 = ((|A| + |B| + max(|A|, |B|)) / 3)^2.
+template <typename T> __device__ __forceinline__ T addrn(T a, T b) { return a + b; }
+template <> __device__ __forceinline__ fx64 addrn<fx64>(fx64 a, fx64 b) { return __dadd_rn(a.v, b.v); }
+template <typename T>
+__device__ __forceinline__ T beta1_2d(const Weights<T>& W, T a, T b, T g, T h) {
+  const T A = tabs(fma(a, a, -(b * b))), Bq = tabs(fma(h, h, -(g * g)));
+  const T ts = (A + Bq + tmax(A, Bq)) * T(1.0 / 3.0);
+  const T he = fma(h, h, W.eps), ge = fma(g, g, W.eps);
+  const T y0 = fma(a, a, he), y1 = fma(b, b, he), y2 = fma(b, b, ge), y3 = fma(a, a, ge);
+  T n0, n1, n2, n3;
+  if constexpr (one_division<T>::value) {   // over a common denominator
+    const T p01 = y0 * y1, p23 = y2 * y3;
+    n0 = fma(ts, ts, y0) * (y1 * p23);
+    n1 = fma(ts, ts, y1) * (y0 * p23);
+    n2 = fma(ts, ts, y2) * (p01 * y3);
+    n3 = fma(ts, ts, y3) * (p01 * y2);
+  } else {
+    n0 = T(1) + (ts * ts) / y0;
+    n1 = T(1) + (ts * ts) / y1;
+    n2 = T(1) + (ts * ts) / y2;
+    n3 = T(1) + (ts * ts) / y3;
+  }
+  // (n_k are products: sums of them stay sums, so that every kernel rounds alike)
+  const T n01 = addrn(n0, n1), n23 = addrn(n2, n3);
+  const T inv = rcp(n01 + n23);
+  const T gx = fma(addrn(n0, n3), a, addrn(n1, n2) * b) * inv, gy = fma(n01, h, n23 * g) * inv;
+  return fma(gx, gx, gy * gy);
+}
+
 // d = the 23 data of q_4 (u at labels 1..9, v at 1,3,4,5,6,7,9, w at
 // 1,2,3,5,7,8,9; labels of the paper's 3x3 stencil table); put(k*4+l, value)
 // receives u_{i,j}(xi_k, eta_l) of eq. (2D-re-u).  Steps 1.1-1.3 of the 2D algorithm.
 // Square cells: beta_1 of eq. (2D-beta1) is (sum w_1k Dx_k)^2 + (sum w_1k Dy_k)^2.
-// fx64: the linear part in block fixed point (hweno_fx.cuh).  The beta rows and
+// fx64 and double-float: the linear part in block fixed point (hweno_fx.cuh).  The beta rows and
 // the four base points (+-|xi|, +-|eta|) run as loops over coefficient tables:
 // unrolled, a variable's code is 100 KB and the warps wait for instructions.
-template <typename Put>
-__device__ __forceinline__ void recon2d_fp64(const Weights<fx64>& W, const Beta2<fx64>& B, const fx64 (&d)[23],
-                                             Put put) {
+template <typename T, typename Put>
+__device__ __forceinline__ void recon2d_fx(const Weights<T>& W, const Beta2<fx64>& B, const double (&d)[23], Put put) {
   using hwfx::Half2;
-  const double u5 = d[4].v;
+  const double u5 = d[4];
   double dv[23];
 #pragma unroll
-  for (int k = 0; k < 23; ++k) dv[k] = k < 9 ? d[k].v - u5 : d[k].v;
+  for (int k = 0; k < 23; ++k) dv[k] = k < 9 ? d[k] - u5 : d[k];
   int e = hwfx::EMIN;
 #pragma unroll
   for (int k = 0; k < 23; ++k) if (k != 4) e = max(e, hwfx::bexp(dv[k]));
@@ -693,7 +765,7 @@ __device__ __forceinline__ void recon2d_fp64(const Weights<fx64>& W, const Beta2
     for (int k = 0; k < 23; ++k) q[k] = k == 4 ? 0 : hwfx::to_fx<hwfx::BITS>(dv[k], e);
     hwp::fx_split2d(q, sa, sb, sc, se);
   }
-  double beta[4];
+  T beta[4];
   {
     const int e0 = e - (1022 + hwfx::BITS);
     int ra = 0, rb = 0, re = 0;
@@ -702,45 +774,25 @@ __device__ __forceinline__ void recon2d_fp64(const Weights<fx64>& W, const Beta2
       const int na = l == 0 ? hwp::D2_RA(1) : l == 1 ? hwp::D2_RA(2) : hwp::D2_RA(3);
       const int nb = l == 0 ? hwp::D2_RB(1) : l == 1 ? hwp::D2_RB(2) : hwp::D2_RB(3);
       const int ne = l == 0 ? hwp::D2_RE(1) : l == 1 ? hwp::D2_RE(2) : hwp::D2_RE(3);
-      double bl = 0.0;
+      T bl = T(0);
 #pragma unroll 1
-      for (; ra < na; ++ra) { const double x = fx_row(sa, B.a[ra], e0 + B.fa[ra]); bl = fma(x, x, bl); }
+      for (; ra < na; ++ra) { const T x = fx_row<T>(sa, B.a[ra], e0 + B.fa[ra]); bl = fma(x, x, bl); }
 #pragma unroll 1
       for (; rb < nb; ++rb) {   // the same rows for both odd classes (x <-> y images)
-        const double x = fx_row(sb, B.b[rb], e0 + B.fb[rb]), y = fx_row(sc, B.b[rb], e0 + B.fb[rb]);
+        const T x = fx_row<T>(sb, B.b[rb], e0 + B.fb[rb]), y = fx_row<T>(sc, B.b[rb], e0 + B.fb[rb]);
         bl = fma(x, x, fma(y, y, bl));
       }
 #pragma unroll 1
-      for (; re < ne; ++re) { const double x = fx_row(se, B.e[re], e0 + B.fe[re]); bl = fma(x, x, bl); }
+      for (; re < ne; ++re) { const T x = fx_row<T>(se, B.e[re], e0 + B.fe[re]); bl = fma(x, x, bl); }
       if (l == 0) beta[1] = bl; else if (l == 1) beta[2] = bl; else beta[3] = bl;
     }
   }
-  // beta_1: eqs. (2D-q1-1234) .. (2D-beta1).  With x differences a (west), b (east)
-  // and y differences g (south), h (north), the four one-sided |grad|^2 are a^2 + h^2,
-  // b^2 + h^2, b^2 + g^2, a^2 + g^2; their six unordered differences are +-A twice,
-  // +-B twice, +-(A + B) and +-(A - B), A = a^2 - b^2, B = h^2 - g^2, so that
-  // tau_1 = ((|A| + |B| + max(|A|, |B|)) / 3)^2.
-  {
-    const double a = -dv[3], b = dv[5], g = -dv[1], h = dv[7];
-    const double a2 = a * a, b2 = b * b, g2 = g * g, h2 = h * h;
-    const double A = fabs(a2 - b2), Bq = fabs(h2 - g2);
-    const double ts = (A + Bq + (A > Bq ? A : Bq)) * (1.0 / 3.0);
-    const double t1 = ts * ts;
-    const double he = h2 + W.eps.v, ge = g2 + W.eps.v;
-    const double y0 = a2 + he, y1 = b2 + he, y2 = b2 + ge, y3 = a2 + ge;
-    const double p01 = y0 * y1, p23 = y2 * y3;
-    const double n0 = (y0 + t1) * (y1 * p23), n1 = (y1 + t1) * (y0 * p23);
-    const double n2 = (y2 + t1) * (p01 * y3), n3 = (y3 + t1) * (p01 * y2);
-    const double n03 = n0 + n3, n12 = n1 + n2, n01 = n0 + n1, n23 = n2 + n3;
-    const double inv = rcp64(n01 + n23);
-    const double gx = fma(n03, a, n12 * b) * inv, gy = fma(n01, h, n23 * g) * inv;
-    beta[0] = fma(gx, gx, gy * gy);
-  }
-  double c[4];
-  combine_weights_fp64(W, beta, c);
+  beta[0] = beta1_2d<T>(W, from_double<T>(-dv[3]), from_double<T>(dv[5]), from_double<T>(-dv[1]), from_double<T>(dv[7]));
+  T c[4];
+  weights_c(W, beta, c);
   Half2 hc[4];
   const int ec = fx_weights(c, hc);
-  const double u = e > hwfx::EMAX || ec == 0x7FF ? __longlong_as_double(0x7FF8000000000000LL) : u5;
+  const T u = from_double<T>(e > hwfx::EMAX || ec == 0x7FF ? __longlong_as_double(0x7FF8000000000000LL) : u5);
   const int eb = ec + e + (hwfx::CF - (1022 + hwfx::CBITS) - (1022 + hwfx::BITS));
   using namespace hwp;
 #pragma unroll 1
@@ -790,17 +842,20 @@ __device__ __forceinline__ void recon2d_fp64(const Weights<fx64>& W, const Beta2
     }
     const int k = 2 + (b >> 1), l = 2 + (b & 1);
     const long long p = E[0] + E[2], q = E[1] + E[3], r = E[0] - E[2], t = E[1] - E[3];
-    put(k * 4 + l, fx64(u + hwfx::from_fx(p + q, eb)));
-    put((3 - k) * 4 + l, fx64(u + hwfx::from_fx(p - q, eb)));
-    put(k * 4 + 3 - l, fx64(u + hwfx::from_fx(r + t, eb)));
-    put((3 - k) * 4 + 3 - l, fx64(u + hwfx::from_fx(r - t, eb)));
+    put(k * 4 + l, u + from_fixed<T>(p + q, eb));
+    put((3 - k) * 4 + l, u + from_fixed<T>(p - q, eb));
+    put(k * 4 + 3 - l, u + from_fixed<T>(r + t, eb));
+    put((3 - k) * 4 + 3 - l, u + from_fixed<T>(r - t, eb));
   }
 }
 
 template <typename T, typename Put>
 __device__ __forceinline__ void recon2d(const Weights<T>& W, const Beta2<T>& B, const T (&d)[23], Put put) {
   if constexpr (std::is_same<T, fx64>::value) {
-    recon2d_fp64(W, B, d, put);
+    double x[23];
+#pragma unroll
+    for (int k = 0; k < 23; ++k) x[k] = d[k].v;
+    recon2d_fx<T>(W, B, x, put);
     return;
   } else {
   T s[23];
@@ -887,8 +942,7 @@ __device__ __forceinline__ long long goff(const Prob& P, int i, int j) { return 
 // the sign of the GL-weighted face velocity (average of both sides), jumps of
 // the indicator variable (variable 0) weighted by dy w_l or dx w_k.
 template <typename T>
-__device__ __forceinline__ T kxrcf2d(const Prob& P, const Weights<T>& W, const T* __restrict__ G,
-                                     const T* __restrict__ aux, int i, int j) {
+__device__ __forceinline__ T kxrcf2d(const Prob& P, const T* __restrict__ G, const T* __restrict__ aux, int i, int j) {
   const long long o = goff(P, i, j);
   const Img L = image(P, i - 1, j, i, j), R = image(P, i + 1, j, i, j), Bo = image(P, i, j - 1, i, j),
             Tp = image(P, i, j + 1, i, j);

@@ -77,4 +77,30 @@ __device__ __forceinline__ double from_fx(long long x, int eb) {
   return __longlong_as_double(a ? (long long)(r | ((unsigned long long)s << 63)) : 0LL);
 }
 
+// x 2^eb as a double-float pair hi + lo (truncated to 48 bits); magnitudes below 2^-126 become 0.
+__device__ __forceinline__ float2 from_fx_pair(long long x, int eb) {
+  const long long s = x >> 63;
+  const unsigned long long a = (unsigned long long)((x ^ s) - s);
+  const int n = __clzll((long long)a);
+  const unsigned long long m = a << (n & 63);
+  const int fe = 189 - n + eb;                       // hi's biased FP32 exponent less 1
+  if (a == 0 || fe < 0) return make_float2(0.0f, 0.0f);
+  const unsigned sg = (unsigned)s & 0x80000000u;
+  const float hi = __uint_as_float((((unsigned)fe << 23) + (unsigned)(m >> 40)) | sg);
+  // the next 32 bits, rounded to 24, times their unit 2^(8 - n + eb)
+  const float unit = __uint_as_float((unsigned)max(fe - 54, 0) << 23);
+  const float lo = __fmul_rn(__uint2float_rn((unsigned)(m >> 8)), unit);
+  return make_float2(hi, __uint_as_float(__float_as_uint(lo) ^ sg));
+}
+
+// A float in the units of to_fx<B> at biased (FP64) exponent e.
+template <int B>
+__device__ __forceinline__ long long to_fx(float x, int e) {
+  const int b = __float_as_int(x), f = (b >> 23) & 0xFF;
+  const int k = min(e - (f + 896), 63);
+  const long long m = (long long)((unsigned long long)(unsigned)(f ? (b & 0x7FFFFF) | 0x800000 : 0) << (B - 24)) >> k;
+  const long long s = (long long)(b >> 31);
+  return (m ^ s) - s;
+}
+
 }  // namespace hwfx
