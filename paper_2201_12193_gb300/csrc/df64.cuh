@@ -132,13 +132,14 @@ template <> struct is_df64<df64> { static constexpr bool value = true; };
 // bits and round on the 29 dropped bits (above half up; exactly half up when
 // the kept fraction is odd); a carry out of the fraction raises the exponent,
 // and out of the largest finite float gives infinity, as rounding must.
-// Results that are not normal floats (zero, subnormal, non-finite inputs)
-// take the FP64 conversion.
+// Other results that are not normal floats (subnormal, non-finite inputs) take
+// the FP64 conversion.
 __device__ __forceinline__ float f32_rn(double x) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const unsigned h = (unsigned)(b >> 32), l = (unsigned)b;
   const int e = (int)((h >> 20) & 0x7FFu);
-  if (e < 897 || e > 1150) return __double2float_rn(x);
+  if (e < 897 || e > 1150)    // zeros (first moments of flat data, momenta of gas at rest) stay integer work
+    return ((h << 1) | l) == 0u ? __uint_as_float(h) : __double2float_rn(x);
   const unsigned keep = ((h & 0xFFFFFu) << 3) | (l >> 29);
   const unsigned rest = l & 0x1FFFFFFFu;
   unsigned f = (h & 0x80000000u) | ((unsigned)(e - 896) << 23) | keep;

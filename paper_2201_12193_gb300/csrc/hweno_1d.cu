@@ -126,10 +126,14 @@ __global__ void __launch_bounds__(RB) rec1d_char_kernel(Prob P, Weights<T> W, Be
 // jl, jr of the density at the inflow faces (face velocities vl, vr), over
 // h^{(l+1)/3} (l = 5) times the cell's largest density point value nrm.  The
 // pipeline and the fused stage both call this, so their flags agree bit for bit.
+// The decision |s| / (h^2 nrm) > 1 is |s| > h^2 nrm without the division (the two
+// agree exactly under IEEE rounding); the value itself goes to aleph when asked for.
 template <typename T>
-__device__ __forceinline__ T kxrcf1(const Prob& P, T jl, T jr, T vl, T vr, T nrm) {
-  const T s = jl * (vl > T(KX_VDEAD) ? T(1) : T(0)) + jr * (-vr > T(KX_VDEAD) ? T(1) : T(0));
-  return nrm == T(0) ? T(0) : tabs(s) / (T(P.dx * P.dx) * nrm);
+__device__ __forceinline__ bool kxrcf1(const Prob& P, T jl, T jr, T vl, T vr, T nrm, double* aleph) {
+  const T s = tabs(jl * (vl > T(KX_VDEAD) ? T(1) : T(0)) + jr * (-vr > T(KX_VDEAD) ? T(1) : T(0)));
+  const T b = pc<T>(P.cdx2) * nrm;
+  if (aleph) *aleph = nrm == T(0) ? 0.0 : double(s / b);
+  return s > b && !(nrm == T(0));
 }
 
 // Modified first moment of a troubled cell, eq. (vi): from the neighbours'
@@ -138,11 +142,18 @@ __device__ __forceinline__ double mod1(double uL, double uR, double vL, double v
   return MOD_WU * (uR - uL) + MOD_WV * (vL + vR);
 }
 
+// Point velocity (rho u) / rho; fx64 by the three-operation reciprocal.
+template <typename T>
+__device__ __forceinline__ T vel1(T m, T rho) {
+  if constexpr (std::is_same<T, fx64>::value) return m * rcp(rho);
+  else return m / rho;
+}
+
 template <typename T, int NV>
 __device__ __forceinline__ T face_vel1(const Prob& P, const T* __restrict__ G, int c, int side) {
   const int p = side ? 3 : 0;
   if constexpr (NV == 1) return scalar_velocity(P, G[(long long)p * P.gplane + c], 0);
-  else return G[(long long)(4 + p) * P.gplane + c] / G[(long long)p * P.gplane + c];
+  else return vel1(G[(long long)(4 + p) * P.gplane + c], G[(long long)p * P.gplane + c]);
 }
 
 template <typename T, int NV>
@@ -172,9 +183,7 @@ __global__ void __launch_bounds__(RB) flag1d_kernel(Prob P, Weights<T> W, const 
       T nrm = T(0);
 #pragma unroll
       for (int p = 0; p < 4; ++p) nrm = tmax(nrm, tabs(G[(long long)p * P.gplane + i]));
-      const T a = kxrcf1<T>(P, jl, jr, vl, vr, nrm);
-      if (aleph) aleph[i] = double(a);
-      flag = a > T(1);
+      flag = kxrcf1<T>(P, jl, jr, vl, vr, nrm, aleph ? aleph + i : nullptr);
     }
   }
   const unsigned act = __ballot_sync(0xffffffffu, flag);
@@ -218,25 +227,29 @@ __device__ __forceinline__ void gl1(const Prob& P, const T* __restrict__ G, cons
 }
 
 // Quadrature of eq. (F): the weighted physical flux at the cell's 4
-// Gauss-Lobatto points u[k] (FP64 Euler: the four reciprocal densities with
-// one division).
+// Gauss-Lobatto points u[k].
+// fx64 Euler: the sums of the linear terms are the cell's averages ubar (the
+// quadrature is exact for degree 5), so with K = sum w m^2/rho the momentum flux
+// needs no pressure per point (K + (gamma - 1)(E - K/2)).
 template <typename T, int NV>
-__device__ __forceinline__ void quad1(const Prob& P, const T (&u)[4][NV], T (&F)[NV]) {
+__device__ __forceinline__ void quad1(const Prob& P, const T (&u)[4][NV], const double (&ubar)[NV], T (&F)[NV]) {
+  if constexpr (NV == 3 && std::is_same<T, fx64>::value) {
+    const T kap = pc<T>(P.chg), g = pc<T>(P.cgamma), gm1 = pc<T>(P.cgm1);
+    T k[4], x[4];
 #pragma unroll
-  for (int v = 0; v < NV; ++v) F[v] = T(0);
-  if constexpr (NV == 3 && one_division<T>::value) {
-    T rho[4], inv[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) rho[k] = u[k][0];
-    batch_inverse<4, T>(rho, inv);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      T f[NV];
-      euler_flux_inv<T, NV>(P, u[k], inv[k], 0, f);
-#pragma unroll
-      for (int v = 0; v < NV; ++v) F[v] += gl_w<T>(k) * f[v];
+    for (int q = 0; q < 4; ++q) {
+      const T mu = u[q][1] * rcp(u[q][0]);
+      k[q] = u[q][1] * mu;
+      x[q] = mu * fma(-kap, k[q], u[q][2]);        // u (E + p) / gamma
     }
+    const T K = fma(T(5.0 / 12.0), addrn(k[1], k[2]), T(1.0 / 12.0) * addrn(k[0], k[3]));
+    const T X = fma(T(5.0 / 12.0), addrn(x[1], x[2]), T(1.0 / 12.0) * addrn(x[0], x[3]));
+    F[0] = T(ubar[1]);
+    F[1] = fma(gm1, fma(T(-0.5), K, T(ubar[2])), K);
+    F[2] = g * X;
   } else {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) F[v] = T(0);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       T f[NV];
@@ -247,58 +260,55 @@ __device__ __forceinline__ void quad1(const Prob& P, const T (&u)[4][NV], T (&F)
   }
 }
 
-// L(U) of eq. (1D-equ-int-approximation) of cell i from its face fluxes fp
-// (right), fm (left) and quadrature F, and the SSP-RK3 combination of
+// L(U) of eq. (1D-equ-int-approximation) of variable v of cell i from its face
+// fluxes fp (right), fm (left) and quadrature F, and the SSP-RK3 combination of
 // eq. (Runge-Kutta) (or L and the stage input into Lout / Umod).  The average
 // equation is formed in FP64 from the widened face fluxes so that the flux
 // differences telescope in every precision; FP32 values are widened by integer
 // work and the first stage (cA = 0, cB = 1: U^(1) = U + dt L) is one FMA
-// without U^n, so the FP64 pipe carries only the sums.  uin: the cell's stage
-// input, its first moments replaced by those of eq. (vi) when it is flagged
-// and they persist (or Lout asks for them).  Both 1D stage forms call this.
-template <typename T, int NV>
-__device__ __forceinline__ void rk1_cell(const Prob& P, const Rk1& S, int i, const T* fp, const T* fm,
-                                         const T (&F)[NV], const double (&uinc)[2 * NV]) {
+// without U^n, so the FP64 pipe carries only the sums.  uin0, uin1: the cell's
+// stage input, its first moment replaced by that of eq. (vi) when it is flagged
+// and they persist (or Lout asks for them).  Returns the new average; finite is
+// cleared by a non-finite value.  Both 1D stage forms call this.
+template <typename T>
+__device__ __forceinline__ double rk1_var(const Prob& P, const Rk1& S, int i, int v, T fp, T fm, T F, double uin0,
+                                          double uin1, bool& finite) {
   const double idx = P.crdx.d;
   const T tidx = pc<T>(P.crdx);
-  const bool fn = P.persist && S.maskN && S.maskN[i] != 0;
-  const bool first = S.cA == 0.0;
-  double newavg[NV];
-  bool finite = true;
+  double L[2];
+  L[0] = -(to_f64(fp) - to_f64(fm)) * idx;
+  if constexpr (std::is_same<T, fx64>::value) L[1] = to_f64(fma(T(-0.5), fp + fm, F) * tidx);
+  else L[1] = to_f64(-(fp + fm) * T(0.5) * tidx + F * tidx);
+  double avg = 0.0;
 #pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    double L[2];
-    L[0] = -(to_f64(fp[v]) - to_f64(fm[v])) * idx;
-    L[1] = to_f64(-(fp[v] + fm[v]) * T(0.5) * tidx + F[v] * tidx);
-#pragma unroll
-    for (int m = 0; m < 2; ++m) {
-      const long long si = (long long)(v * 2 + m) * P.plane + i;
-      const double uin = uinc[v * 2 + m];
-      if (S.Lout) {
-        S.Lout[si] = L[m];
-        if (S.Umod) S.Umod[si] = uin;
-        continue;
-      }
-      double r;
-      if (first) {
-        r = fma(S.dt, L[m], uin);
-      } else {
-        const double un = (m == 1 && fn) ? S.ModN[(long long)v * P.plane + i] : S.Un[si];
-        r = S.cA * un + S.cB * (uin + S.dt * L[m]);
-      }
-      S.Uout[si] = r;
-      if (m == 0) newavg[v] = r;
-      // non-finite by the exponent field (integer work, no FP64 compare)
-      finite = finite && ((__double_as_longlong(r) >> 52) & 0x7FF) != 0x7FF;
+  for (int m = 0; m < 2; ++m) {
+    const long long si = (long long)(v * 2 + m) * P.plane + i;
+    const double uin = m ? uin1 : uin0;
+    if (S.Lout) {
+      S.Lout[si] = L[m];
+      if (S.Umod) S.Umod[si] = uin;
+      continue;
     }
+    double r;
+    if (S.cA == 0.0) {
+      r = fma(S.dt, L[m], uin);
+    } else {
+      const bool fn = m == 1 && P.persist && S.maskN && S.maskN[i] != 0;
+      const double un = fn ? S.ModN[(long long)v * P.plane + i] : S.Un[si];
+      r = fma(S.cA, un, S.cB * fma(S.dt, L[m], uin));
+    }
+    S.Uout[si] = r;
+    if (m == 0) avg = r;
+    // non-finite by the exponent field (integer work, no FP64 compare)
+    finite = finite && ((__double_as_longlong(r) >> 52) & 0x7FF) != 0x7FF;
   }
-  if (S.Lout) return;
-  if (!finite) atomicOr(S.status, ST_NONFINITE);
-  if (NV == 3) {
-    // rho > 0 and p = (gamma - 1)(E - m^2 / (2 rho)) > 0, the latter as 2 E rho > m^2 (no division)
-    const double rho = newavg[0];
-    if (!(rho > 0.0) || !(2.0 * newavg[NV - 1] * rho > newavg[1] * newavg[1])) atomicOr(S.status, ST_NONPOSITIVE);
-  }
+  return avg;
+}
+
+// The checks of a cell's new averages.
+template <int NV>
+__device__ __forceinline__ void check1(const Rk1& S, const double (&avg)[NV]) {
+  if (NV == 3 && nonphysical(avg[0], avg[1], 0.0, avg[NV - 1])) atomicOr(S.status, ST_NONPOSITIVE);
 }
 
 template <typename T, int NV>
@@ -332,16 +342,22 @@ __global__ void __launch_bounds__(UB) update1d_kernel(Prob P, const T* __restric
   T u[4][NV], F[NV];
 #pragma unroll
   for (int k = 0; k < 4; ++k) gl1<T, NV>(P, G, self, k, u[k]);
-  quad1<T, NV>(P, u, F);
+  double ub[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) ub[v] = S.Uin[(long long)(2 * v) * P.plane + i];
+  quad1<T, NV>(P, u, ub, F);
   // modified first moments in the combination (persist), and always in the Umod output of Lout
   const bool fk = S.mask[i] != 0 && (P.persist || S.Lout);
-  double uin[2 * NV];
+  double avg[NV];
+  bool finite = true;
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
-    uin[2 * v] = S.Uin[(long long)(2 * v) * P.plane + i];
-    uin[2 * v + 1] = fk ? S.Mod[(long long)v * P.plane + i] : S.Uin[(long long)(2 * v + 1) * P.plane + i];
+    const double u1 = fk ? S.Mod[(long long)v * P.plane + i] : S.Uin[(long long)(2 * v + 1) * P.plane + i];
+    avg[v] = rk1_var<T>(P, S, i, v, fx[t + 1][v], fx[t][v], F[v], ub[v], u1, finite);
   }
-  rk1_cell<T, NV>(P, S, i, fx[t + 1], fx[t], F, uin);
+  if (S.Lout) return;
+  if (!finite) atomicOr(S.status, ST_NONFINITE);
+  check1<NV>(S, avg);
 }
 
 }  // namespace

@@ -560,9 +560,7 @@ __device__ __forceinline__ void update_cell_lean(const Prob& P, const Src& src, 
   }
   if (S.Lout || !owned) return;
   if (!finite) atomicOr(S.status, ST_NONFINITE);
-  // rho > 0 and p = (gamma - 1)(E - |m|^2 / (2 rho)) > 0, the latter as 2 E rho > |m|^2 (no division)
-  const double m2 = newavg[1] * newavg[1] + newavg[2] * newavg[2];
-  if (!(newavg[0] > 0.0) || !(2.0 * newavg[3] * newavg[0] > m2)) atomicOr(S.status, ST_NONPOSITIVE);
+  if (nonphysical(newavg[0], newavg[1], newavg[2], newavg[3])) atomicOr(S.status, ST_NONPOSITIVE);
 }
 
 // Step 3 for the TXV x TYV tile at (i0, j0): face fluxes into shared memory, then
@@ -767,11 +765,9 @@ __device__ __forceinline__ void update2d_tile(const Prob& P, const Src& src, con
     }
   }
   if (!S.Lout && !finite && owned) atomicOr(S.status, ST_NONFINITE);
-  if (!S.Lout && P.eq == EQ_EULER && NV == 4 && owned) {
-    // rho > 0 and p = (gamma - 1)(E - |m|^2 / (2 rho)) > 0, the latter as 2 E rho > |m|^2 (no division)
-    const double rho = newavg[0];
-    const double m2 = newavg[1] * newavg[1] + newavg[2] * newavg[2];
-    if (!(rho > 0.0) || !(2.0 * newavg[NV - 1] * rho > m2)) atomicOr(S.status, ST_NONPOSITIVE);
+  if constexpr (NV == 4) {
+    if (!S.Lout && P.eq == EQ_EULER && owned && nonphysical(newavg[0], newavg[1], newavg[2], newavg[3]))
+      atomicOr(S.status, ST_NONPOSITIVE);
   }
   }
 }

@@ -431,6 +431,7 @@ hweno_status hweno_create(const hweno_grid* grid, const hweno_bc* bc, double gam
   }
   cudaMemset(h->B.status, 0, sizeof(unsigned));
   cudaMemset(h->mask3, 0, 3 * nc);
+  cudaMemset(h->red_part, 0, hw::reduce_partials_len(P) * sizeof(double));
   cudaMemset(h->B.count, 0, 4 * sizeof(int));
   cudaMemset(h->B.rerec, 0, sizeof(unsigned long long));
   for (int k = 0; k < 3; ++k) cudaMemset(h->U[k], 0, sbytes);
@@ -645,7 +646,7 @@ hweno_status hweno_wave_speeds(hweno_t h, double* ax_ay) {
   if (!h->have_state) return fail(h, HWENO_ESTATE, "wave_speeds: no moments set");
   hweno_status s = check_status(h);
   if (s != HWENO_OK) return s;
-  hw::run_wavespeed(h->P, h->U[h->cur], h->red_part, h->red_out, h->stream);
+  hw::run_wavespeed(h->P, h->U[h->cur], h->red_part, h->red_out, nullptr, nullptr, nullptr, h->stream);
   CK(h, cudaMemcpyAsync(h->host_buf, h->red_out, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   CK(h, cudaStreamSynchronize(h->stream));
   ax_ay[0] = h->host_buf[0];
@@ -669,8 +670,7 @@ cudaError_t advance_steps(hweno_t h, int a, cudaStream_t st) {
   double* stt = h->adv + 3;
   for (int k = 0; k < ADV_K; ++k) {
     const int b = (a + 1) % 3, c = (a + 2) % 3;
-    hw::run_wavespeed(h->P, h->U[a], h->red_part, h->red_out, st);
-    hw::run_advance_dt(h->P, h->red_out, par, stt, h->B.status, st);
+    hw::run_wavespeed(h->P, h->U[a], h->red_part, h->red_out, par, stt, h->B.status, st);
     auto run = [&](const hw::StageCall& S) {
       if (h->P.fixtab) {   // stage time from the device: t_n + c dt, c = 0, 1, 1/2
         const double cst[3] = {0.0, 1.0, 0.5};
@@ -767,7 +767,7 @@ hweno_status hweno_max_dt(hweno_t h, double cfl, double* dt_out) {
   if (!(cfl > 0.0)) return fail(h, HWENO_EINVAL, "max_dt: cfl must be positive");
   hweno_status s = check_status(h);
   if (s != HWENO_OK) return s;
-  hw::run_wavespeed(h->P, h->U[h->cur], h->red_part, h->red_out, h->stream);
+  hw::run_wavespeed(h->P, h->U[h->cur], h->red_part, h->red_out, nullptr, nullptr, nullptr, h->stream);
   CK(h, cudaMemcpyAsync(h->host_buf, h->red_out, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   CK(h, cudaStreamSynchronize(h->stream));
   const double ax = h->host_buf[0], ay = h->host_buf[1];

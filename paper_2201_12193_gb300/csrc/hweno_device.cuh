@@ -268,6 +268,10 @@ template <> __device__ __forceinline__ fx64 rcp<fx64>(fx64 a) {
 
 __device__ __forceinline__ double rcp64(double x) { return rcp<fx64>(x).v; }
 
+// a + b never contracted into an FMA (operands that are products)
+template <typename T> __device__ __forceinline__ T addrn(T a, T b) { return a + b; }
+template <> __device__ __forceinline__ fx64 addrn<fx64>(fx64 a, fx64 b) { return __dadd_rn(a.v, b.v); }
+
 template <typename T, int NV>
 __device__ __forceinline__ void phys_flux(const Prob& P, const T* u, int dir, T* f) {
   if constexpr (NV == 1) {
@@ -713,8 +717,6 @@ __device__ __forceinline__ void recon1d(const Weights<T>& W, const Beta1<T>& B, 
 // b^2 + h^2, b^2 + g^2, a^2 + g^2; their six unordered differences are +-A twice,
 // +-B twice, +-(A + B) and +-(A - B), A = a^2 - b^2, B = h^2 - g^2, so that
 // tau_1 = ((|A| + |B| + max(|A|, |B|)) / 3)^2.
-template <typename T> __device__ __forceinline__ T addrn(T a, T b) { return a + b; }
-template <> __device__ __forceinline__ fx64 addrn<fx64>(fx64 a, fx64 b) { return __dadd_rn(a.v, b.v); }
 template <typename T>
 __device__ __forceinline__ T beta1_2d(const Weights<T>& W, T a, T b, T g, T h) {
   const T A = tabs(fma(a, a, -(b * b))), Bq = tabs(fma(h, h, -(g * g)));
@@ -989,6 +991,28 @@ __device__ __forceinline__ T kxrcf2d(const Prob& P, const T* __restrict__ G, con
   const T nrm = aux[4 * P.gplane + o];
   if (len == T(0) || nrm == T(0)) return T(0);
   return tabs(s) / len / (pc<T>(P.cdx2) * nrm);   // h^{(l+1)/3}, l = 5, h = dx
+}
+
+// ---------------------------------------------------------------- step checks
+// A double truncated to FP32 by integer work, magnitudes outside its normal range as 0 or infinity.
+__device__ __forceinline__ float f32_trunc(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int e = (int)((hi >> 20) & 0x7FFu) - (1023 - 127);
+  if (e <= 0) return 0.0f;
+  if (e >= 255) return __uint_as_float((hi & 0x80000000u) | 0x7F800000u);
+  return __uint_as_float((hi & 0x80000000u) | ((unsigned)e << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29));
+}
+
+// Whether an Euler cell average is outside the physical set: not rho > 0, or not
+// p = (gamma - 1)(E - |m|^2 / (2 rho)) > 0, i.e. 2 E rho > |m|^2 (no division).
+// Cells that are inside by more than FP32's rounding are passed on FP32 copies;
+// only the others take the FP64 test.
+__device__ __forceinline__ bool nonphysical(double rho, double m, double n, double E) {
+  const float r = f32_trunc(rho), a = f32_trunc(m), b = f32_trunc(n), e = f32_trunc(E);
+  const float x = 2.0f * e * r, y = a * a + b * b;
+  if (r > 0.0f && x > 1.00001f * y && x > 1e-30f && x < 1e30f) return false;
+  const double m2 = m * m + n * n;
+  return !(rho > 0.0) || !(2.0 * E * rho > m2);
 }
 
 // ---------------------------------------------------------------- TVB indicator

@@ -30,7 +30,8 @@ template <typename T, int NV, int S>
 struct Fused1dSmem {
   static constexpr int W = S + 8;   // window: owned + 4 each side
   double U[2 * NV][W];   // moments with the image signs applied (FP64: eq. (vi) and the state)
-  T UT[2 * NV][W];       // the same in the compute precision (the reconstruction's input)
+  T UT[2 * NV][W];       // the same in the compute precision (the reconstruction's input);
+                         //    after Step 2.3 the owned cells' quadratures, [v][4 + c]
   T G[4 * NV][W];        // point values
   T V[2][W];             // KXRCF velocities at the left and right end points
   double Mod[NV][W];     // modified first moments of flagged positions
@@ -149,7 +150,7 @@ __global__ void __launch_bounds__(NT) fused1d_kernel(const __grid_constant__ Pro
       for (int s = 0; s < 2; ++s) {
         const int k = s ? 3 : 0;
         if constexpr (NV == 1) sm.V[s][p] = scalar_velocity(P, sm.G[k][p], 0);
-        else sm.V[s][p] = sm.G[4 + k][p] / sm.G[k][p];
+        else sm.V[s][p] = vel1(sm.G[4 + k][p], sm.G[k][p]);
       }
     }
     __syncthreads();
@@ -168,19 +169,23 @@ __global__ void __launch_bounds__(NT) fused1d_kernel(const __grid_constant__ Pro
       T nrm = T(0);
 #pragma unroll
       for (int k = 0; k < 4; ++k) nrm = tmax(nrm, tabs(sm.G[k][p]));
-      const T a = kxrcf1<T>(P, jl, jr, vl, vr, nrm);
-      if (aleph && p >= 4 && p < 4 + S && i < P.nx) aleph[i] = double(a);
-      flag = a > T(1);
+      flag = kxrcf1<T>(P, jl, jr, vl, vr, nrm, aleph && p >= 4 && p < 4 + S && i < P.nx ? aleph + i : nullptr);
     }
-    sm.F[p] = flag ? 1 : 0;
-    if (flag) {
-#pragma unroll
-      for (int v = 0; v < NV; ++v)
-        sm.Mod[v][p] = mod1(sm.U[2 * v][p - 1], sm.U[2 * v][p + 1], sm.U[2 * v + 1][p - 1], sm.U[2 * v + 1][p + 1]);
-    }
+    if (!flag) continue;
+    sm.F[p] = 1;
+    sm.list[atomicAdd(&sm.nlist, 1)] = (short)p;
+    if (p >= 4 && p < 4 + S && i < P.nx) atomicAdd(&sm.nown, 1);
   }
   __syncthreads();
   if (P.indicator != IND_NONE) {
+    // eq. (vi) of the flagged positions, from their list: spread over the warps by
+    // flags rather than by positions (FP64 work, issued per warp)
+    const int nl = sm.nlist;
+    for (int t = tid; t < nl * NV; t += NT) {
+      const int v = t / nl, p = sm.list[t - v * nl];
+      sm.Mod[v][p] = mod1(sm.U[2 * v][p - 1], sm.U[2 * v][p + 1], sm.U[2 * v + 1][p - 1], sm.U[2 * v + 1][p + 1]);
+    }
+    if (nl) __syncthreads();   // block-uniform
     // mirrored ghosts take their image's flag and modified moments (load_mom1<true> of the pipeline)
     for (int p = 2 + tid; p < WN - 2; p += NT) {
       const int i = i0 - 4 + p;
@@ -198,16 +203,9 @@ __global__ void __launch_bounds__(NT) fused1d_kernel(const __grid_constant__ Pro
     }
     __syncthreads();
     // ---- Step 2.3: flagged positions 3 .. WN - 4 (cells -1 .. S) again, from the modified moments
-    for (int p = 3 + tid; p < WN - 3; p += NT) {
-      const int i = i0 - 4 + p;
-      if (!sm.F[p] || f1_mirror(P, i)) continue;
-      sm.list[atomicAdd(&sm.nlist, 1)] = (short)p;
-      if (p >= 4 && p < 4 + S && i < P.nx) atomicAdd(&sm.nown, 1);
-    }
-    __syncthreads();
-    const int nl = sm.nlist;
     for (int t = tid; t < nl * NV; t += NT) {
-      const int v = t / nl, p = sm.list[t % nl];
+      const int v = t / nl, p = sm.list[t - v * nl];
+      if (p < 3 || p >= WN - 3) continue;
       T d[6];
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
@@ -227,41 +225,60 @@ __global__ void __launch_bounds__(NT) fused1d_kernel(const __grid_constant__ Pro
     }
     if (tid == 0 && rerec && sm.nown) atomicAdd(rerec, (unsigned long long)sm.nown);
   }
-  // ---- Step 3: the face fluxes (face c left of owned cell c; one call site as in the pipeline)
-  for (int c = tid; c <= S; c += NT) {
-    if (i0 + c - 1 >= P.nx) continue;
-    T uL[NV], uR[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      uL[v] = sm.G[v * 4 + 3][3 + c];
-      uR[v] = sm.G[v * 4][4 + c];
-    }
-    num_flux<T, NV>(P, uL, uR, 0, sm.FX[c]);
-  }
-  __syncthreads();
-  for (int c = tid; c < S; c += NT) {
-    const int i = i0 + c, p = 4 + c;
-    if (i >= P.nx) return;
-    T u[4][NV], Fq[NV];
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-#pragma unroll
-      for (int v = 0; v < NV; ++v) u[k][v] = sm.G[v * 4 + k][p];
-    quad1<T, NV>(P, u, Fq);
-    const bool flagged = sm.F[p] != 0;
-    mask[i] = flagged ? 1 : 0;
-    double uin[2 * NV];   // the stage input (an owned cell's moments carry no sign)
-#pragma unroll
-    for (int q = 0; q < 2 * NV; ++q) uin[q] = sm.U[q][p];
-    if (flagged) {
+  // ---- Step 3: the face fluxes (face c left of owned cell c; one call site as in
+  // the pipeline) and the quadratures, on different warps where the block has room
+  constexpr int QF = (S + 1 + 31) / 32 * 32;
+  for (int t = tid; t < QF + S; t += NT) {
+    if (t < QF) {
+      const int c = t;
+      if (c > S || i0 + c - 1 >= P.nx) continue;
+      T uL[NV], uR[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        const double mv = sm.Mod[v][p];
-        if (R.Lout || P.persist) uin[2 * v + 1] = mv;
-        if (ModOut) ModOut[(long long)v * P.plane + i] = mv;
+        uL[v] = sm.G[v * 4 + 3][3 + c];
+        uR[v] = sm.G[v * 4][4 + c];
       }
+      num_flux<T, NV>(P, uL, uR, 0, sm.FX[c]);
+    } else {
+      const int c = t - QF, p = 4 + c;
+      if (i0 + c >= P.nx) continue;
+      T u[4][NV], Fq[NV];
+      double ub[NV];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        ub[v] = sm.U[2 * v][p];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) u[k][v] = sm.G[v * 4 + k][p];
+      }
+      quad1<T, NV>(P, u, ub, Fq);
+#pragma unroll
+      for (int v = 0; v < NV; ++v) sm.UT[v][p] = Fq[v];
     }
-    rk1_cell<T, NV>(P, R, i, sm.FX[c + 1], sm.FX[c], Fq, uin);
+  }
+  __syncthreads();
+  // ---- L and the Runge-Kutta combination, one variable of a cell per thread
+  bool finite = true;
+  for (int t = tid; t < S * NV; t += NT) {
+    const int v = t / S, c = t - v * S, i = i0 + c, p = 4 + c;
+    if (i >= P.nx) continue;
+    const bool flagged = sm.F[p] != 0;
+    double u1 = sm.U[2 * v + 1][p];   // the stage input (an owned cell's moments carry no sign)
+    if (flagged) {
+      const double mv = sm.Mod[v][p];
+      if (R.Lout || P.persist) u1 = mv;
+      if (ModOut) ModOut[(long long)v * P.plane + i] = mv;
+    }
+    if (v == 0) mask[i] = flagged ? 1 : 0;
+    const double a = rk1_var<T>(P, R, i, v, sm.FX[c + 1][v], sm.FX[c][v], sm.UT[v][p], sm.U[2 * v][p], u1, finite);
+    sm.U[2 * v][p] = a;   // (this thread's own entry: the new average for the checks)
+  }
+  if (R.Lout) return;
+  if (!finite) atomicOr(R.status, ST_NONFINITE);
+  if constexpr (NV == 3) {
+    __syncthreads();
+    for (int c = tid; c < S; c += NT)
+      if (i0 + c < P.nx && nonphysical(sm.U[0][4 + c], sm.U[2][4 + c], 0.0, sm.U[4][4 + c]))
+        atomicOr(R.status, ST_NONPOSITIVE);
   }
 }
 

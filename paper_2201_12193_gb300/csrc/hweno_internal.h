@@ -178,11 +178,11 @@ cudaError_t run_batch_stage_df64(const HostTabs& T, int tile_variant, const Batc
 
 // Reductions over the cell averages (FP64): maximum wave speeds per direction
 // and totals sum(ubar) per variable.  partials needs reduce_partials_len(P)
-// doubles; out gets {ax, ay} or the nvar totals (unscaled sums).
+// doubles, zeroed once; out gets {ax, ay} or the nvar totals (unscaled sums).
+// With par and st set (hweno_advance) the step length follows from {ax, ay}.
 int reduce_partials_len(const Prob& P);
-void run_wavespeed(const Prob& P, const double* U, double* partials, double* out, cudaStream_t st);
-void run_advance_dt(const Prob& P, const double* speeds, const double* par, double* st, unsigned* status,
-                    cudaStream_t s);
+void run_wavespeed(const Prob& P, const double* U, double* partials, double* out, const double* par, double* st,
+                   unsigned* status, cudaStream_t s);
 void run_totals(const Prob& P, const double* U, double* partials, double* out, cudaStream_t st);
 // FP32 form: rows [j0, j0 + nrows) of the float copy of state U, rounded to nearest.
 void run_shadow32(const Prob& P, const double* U, float* U32, int j0, int nrows, cudaStream_t st);

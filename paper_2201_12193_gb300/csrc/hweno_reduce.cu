@@ -10,11 +10,11 @@
 namespace hw {
 namespace {
 
-constexpr int RT = 256;       // threads per block
+constexpr int RT = 256;       // threads per block (64 in the wave speeds of small grids)
 constexpr int MAXB = 1024;    // blocks of the first pass (partials per quantity)
 
-template <int K>
-__device__ __forceinline__ void block_reduce(double (&v)[K], bool is_max, double (*sm)[RT / 32]) {
+template <int K, int NT = RT>
+__device__ __forceinline__ void block_reduce(double (&v)[K], bool is_max, double (*sm)[NT / 32]) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
   for (int k = 0; k < K; ++k)
@@ -30,7 +30,7 @@ __device__ __forceinline__ void block_reduce(double (&v)[K], bool is_max, double
   if (wid == 0) {
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-      double x = lane < RT / 32 ? sm[k][lane] : 0.0;   // 0 is neutral for sums and for max of speeds
+      double x = lane < NT / 32 ? sm[k][lane] : 0.0;   // 0 is neutral for sums and for max of speeds
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
         const double w = __shfl_down_sync(0xffffffffu, x, o);
@@ -41,14 +41,50 @@ __device__ __forceinline__ void block_reduce(double (&v)[K], bool is_max, double
   }
 }
 
+// The step length of hweno_advance on the device, from the wave-speed maxima:
+// the CFL rule of the host's hweno_max_dt (same expressions), clipped to the
+// remaining time; st[0] = t, st[1] = dt, st[2] = steps taken, st[3] = the time at
+// the start of the step, par = {T, cfl, max_steps}.  dt = -1 marks a step to skip
+// (done, step budget spent, or a non-physical average, which also sets
+// ST_NONPOSITIVE and ST_NODT; the latter fails the call whatever the positivity switch).
+__device__ __forceinline__ void advance_dt(const Prob& P, double ax, double ay, const double* __restrict__ par,
+                                           double* __restrict__ st, unsigned* __restrict__ status) {
+  const double T = par[0], cfl = par[1], maxs = par[2];
+  double dtc;
+  if (P.nmom == 2) dtc = ax > 0.0 ? cfl * P.dx / ax : INFINITY;
+  else {
+    const double r = ax / P.dx + ay / P.dy;
+    dtc = r > 0.0 ? cfl / r : INFINITY;
+  }
+  const double t = st[0], rem = T - t;
+  st[3] = t;
+  double dt = -1.0;
+  if (!(dtc > 0.0) || isnan(dtc)) {
+    atomicOr(status, ST_NONPOSITIVE | ST_NODT);
+  } else if (st[2] < maxs && rem > 1e-14 * fmax(1.0, fabs(T))) {
+    dt = fmin(dtc, rem);
+    st[0] = dtc >= rem ? T : t + dt;
+    st[2] += 1.0;
+  }
+  st[1] = dt;
+}
+
 // Largest |f'| (scalars) or |velocity| + sound speed (Euler) per direction,
 // from cell averages.  A non-physical average yields +inf (dt = 0).  With the
 // positivity check off the sound speed uses max(p, 0).
-__global__ void __launch_bounds__(RT) wavespeed_kernel(Prob P, const double* __restrict__ U, double* __restrict__ part) {
-  __shared__ double sm[2][RT / 32];
+// The last block to arrive (part[4 MAXB] counts them and returns to 0) reduces the
+// blocks' partials to out[0..1] and, with par set, forms hweno_advance's step
+// length: one launch where the partials, their reduction and the step length took
+// three (each about 2 us of a small grid's step; a maximum is the same in any order).
+template <int NT>
+__global__ void __launch_bounds__(NT) wavespeed_kernel(Prob P, const double* __restrict__ U, double* __restrict__ part,
+                                                       double* __restrict__ out, const double* __restrict__ par,
+                                                       double* __restrict__ st, unsigned* __restrict__ status) {
+  __shared__ double sm[2][NT / 32];
+  __shared__ bool last;
   double v[2] = {0.0, 0.0};
   const long long n = (long long)P.nx * (P.jhi - P.jlo);   // owned rows
-  for (long long t = (long long)blockIdx.x * RT + threadIdx.x; t < n; t += (long long)gridDim.x * RT) {
+  for (long long t = (long long)blockIdx.x * NT + threadIdx.x; t < n; t += (long long)gridDim.x * NT) {
     const int i = (int)(t % P.nx), j = P.jlo + (int)(t / P.nx);
     if (P.sol_j > 0 && is_solid(P, i, j)) continue;    // the step's block takes no part
     double sx, sy;
@@ -65,8 +101,28 @@ __global__ void __launch_bounds__(RT) wavespeed_kernel(Prob P, const double* __r
     v[0] = fmax(v[0], sx);
     v[1] = fmax(v[1], sy);
   }
-  block_reduce<2>(v, true, sm);
-  if (threadIdx.x == 0) { part[blockIdx.x] = v[0]; part[MAXB + blockIdx.x] = v[1]; }
+  block_reduce<2, NT>(v, true, sm);
+  if (threadIdx.x == 0) {
+    part[blockIdx.x] = v[0];
+    part[MAXB + blockIdx.x] = v[1];
+    __threadfence();
+    last = atomicInc(reinterpret_cast<unsigned*>(part + 4 * MAXB), gridDim.x - 1) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double w[2] = {0.0, 0.0};
+  for (int b = threadIdx.x; b < gridDim.x; b += NT) {
+    w[0] = fmax(w[0], __ldcg(part + b));
+    w[1] = fmax(w[1], __ldcg(part + MAXB + b));
+  }
+  __syncthreads();   // sm is free again
+  block_reduce<2, NT>(w, true, sm);
+  if (threadIdx.x == 0) {
+    out[0] = w[0];
+    out[1] = w[1];
+    if (par) advance_dt(P, w[0], w[1], par, st, status);
+  }
 }
 
 __global__ void __launch_bounds__(RT) totals_kernel(Prob P, const double* __restrict__ U, double* __restrict__ part) {
@@ -86,18 +142,17 @@ __global__ void __launch_bounds__(RT) totals_kernel(Prob P, const double* __rest
     for (int k = 0; k < 4; ++k) part[k * MAXB + blockIdx.x] = v[k];
 }
 
-// Single block: reduce K rows of nb partials each into out[K].
+// Single block: sum K rows of nb partials each into out[K].
 template <int K>
-__global__ void __launch_bounds__(RT) finish_kernel(const double* __restrict__ part, int nb, bool is_max,
-                                                    double* __restrict__ out) {
+__global__ void __launch_bounds__(RT) finish_kernel(const double* __restrict__ part, int nb, double* __restrict__ out) {
   __shared__ double sm[K][RT / 32];
   double v[K];
 #pragma unroll
   for (int k = 0; k < K; ++k) {
     v[k] = 0.0;
-    for (int b = threadIdx.x; b < nb; b += RT) v[k] = is_max ? fmax(v[k], part[k * MAXB + b]) : v[k] + part[k * MAXB + b];
+    for (int b = threadIdx.x; b < nb; b += RT) v[k] += part[k * MAXB + b];
   }
-  block_reduce<K>(v, is_max, sm);
+  block_reduce<K>(v, false, sm);
   if (threadIdx.x == 0)
 #pragma unroll
     for (int k = 0; k < K; ++k) out[k] = v[k];
@@ -106,35 +161,6 @@ __global__ void __launch_bounds__(RT) finish_kernel(const double* __restrict__ p
 int first_pass_blocks(const Prob& P) {
   const long long n = (long long)P.nx * (P.jhi - P.jlo);
   return (int)std::min<long long>(MAXB, (n + RT - 1) / RT);
-}
-
-// The step length of hweno_advance on the device, from the wave-speed maxima in
-// sp[0..1]: the CFL rule of the host's hweno_max_dt (same expressions), clipped
-// to the remaining time; st[0] = t, st[1] = dt, st[2] = steps taken,
-// st[3] = the time at the start of the step, par = {T, cfl, max_steps}.  dt = -1 marks a step to skip (done, step budget
-// spent, or a non-physical average, which also sets ST_NONPOSITIVE and
-// ST_NODT; the latter fails the call whatever the positivity switch).
-__global__ void advance_dt_kernel(Prob P, const double* __restrict__ sp, const double* __restrict__ par,
-                                  double* __restrict__ st, unsigned* __restrict__ status) {
-  const double ax = sp[0], ay = sp[1];
-  const double T = par[0], cfl = par[1], maxs = par[2];
-  double dtc;
-  if (P.nmom == 2) dtc = ax > 0.0 ? cfl * P.dx / ax : INFINITY;
-  else {
-    const double r = ax / P.dx + ay / P.dy;
-    dtc = r > 0.0 ? cfl / r : INFINITY;
-  }
-  const double t = st[0], rem = T - t;
-  st[3] = t;
-  double dt = -1.0;
-  if (!(dtc > 0.0) || isnan(dtc)) {
-    atomicOr(status, ST_NONPOSITIVE | ST_NODT);
-  } else if (st[2] < maxs && rem > 1e-14 * fmax(1.0, fabs(T))) {
-    dt = fmin(dtc, rem);
-    st[0] = dtc >= rem ? T : t + dt;
-    st[2] += 1.0;
-  }
-  st[1] = dt;
 }
 
 // Fixed-state ghost table for the stage at time t (or, with dtp set, at
@@ -189,23 +215,23 @@ void run_fixfill(const FixSpec& F, double* tab, double t, const double* tn, cons
   fixfill_kernel<<<(n + 127) / 128, 128, 0, st>>>(F, tab, t, tn, dtp, c);
 }
 
-void run_advance_dt(const Prob& P, const double* speeds, const double* par, double* st, unsigned* status,
-                    cudaStream_t s) {
-  advance_dt_kernel<<<1, 1, 0, s>>>(P, speeds, par, st, status);
-}
+int reduce_partials_len(const Prob&) { return 4 * MAXB + 1; }
 
-int reduce_partials_len(const Prob&) { return 4 * MAXB; }
-
-void run_wavespeed(const Prob& P, const double* U, double* partials, double* out, cudaStream_t st) {
-  const int nb = first_pass_blocks(P);
-  wavespeed_kernel<<<nb, RT, 0, st>>>(P, U, partials);
-  finish_kernel<2><<<1, RT, 0, st>>>(partials, nb, true, out);
+void run_wavespeed(const Prob& P, const double* U, double* partials, double* out, const double* par, double* st,
+                   unsigned* status, cudaStream_t s) {
+  const long long n = (long long)P.nx * (P.jhi - P.jlo);
+  // few cells: 64-thread blocks, one warp per scheduler of more SMs (the cells' FP64
+  // divisions and roots issue at 2 per clock and SM)
+  if (n <= 256LL * P.nsm)
+    wavespeed_kernel<64><<<(int)std::min<long long>(MAXB, (n + 63) / 64), 64, 0, s>>>(P, U, partials, out, par, st, status);
+  else
+    wavespeed_kernel<RT><<<first_pass_blocks(P), RT, 0, s>>>(P, U, partials, out, par, st, status);
 }
 
 void run_totals(const Prob& P, const double* U, double* partials, double* out, cudaStream_t st) {
   const int nb = first_pass_blocks(P);
   totals_kernel<<<nb, RT, 0, st>>>(P, U, partials);
-  finish_kernel<4><<<1, RT, 0, st>>>(partials, nb, false, out);
+  finish_kernel<4><<<1, RT, 0, st>>>(partials, nb, out);
 }
 
 }  // namespace hw
