@@ -1015,12 +1015,11 @@ void stage_t(const Prob& P, const HostTabs& HT, const Weights<T>& W, const Beta2
 
 // ---------------------------------------------------------------- batched problems
 //
-// One persistent cooperative launch per Runge-Kutta stage advances every problem
-// of a batch.  Work items of all problems form one list per phase (128-cell rows
-// for the per-cell phases, update tiles for the flux phase); the resident blocks
-// stride over it.  Phases are separated by a grid barrier whose wait is bounded:
-// past the limit the block records ST_TIMEOUT and continues (the host reports
-// HWENO_ETIMEOUT), so no wait can hang the GPU.
+// Work items of all problems form one list per phase (128-cell rows for the
+// per-cell phases, update tiles for the flux phase).  A stage runs a launch per
+// phase, or one persistent cooperative launch whose resident blocks stride over
+// the lists, phases separated by a grid barrier.  The barrier's wait is bounded: past the limit the block records ST_TIMEOUT and continues (the host
+// reports HWENO_ETIMEOUT), so no wait can hang the GPU.
 
 // nblocks: arrivals that release the barrier; limit: polls before the wait gives up.
 __device__ __forceinline__ void grid_barrier(unsigned* bar, unsigned nblocks, unsigned* status,
@@ -1050,119 +1049,240 @@ __device__ __forceinline__ void grid_barrier(unsigned* bar, unsigned nblocks, un
   __syncthreads();
 }
 
-// problem owning work item it (first[] ascending)
-template <int FIELD>
-__device__ __forceinline__ int owner(const BProb* __restrict__ probs, int n, int it) {
-  int lo = 0, hi = n - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    const int f = FIELD == 0 ? probs[mid].rec_first : probs[mid].upd_first;
-    if (f <= it) lo = mid; else hi = mid - 1;
+// One work item of each phase; tid 0 .. RB - 1.  P: the problem's description
+// (shared memory), Q its entry.
+__device__ __forceinline__ void batch_speeds_item(const BatchStage& A, const Prob& P, const BProb& Q, int p, int it,
+                                                  int tid, bool filter) {
+  const double* U = A.Uin + Q.uoff;
+  const int cell = (it - Q.rec_first) * RB + tid;
+  double sx = 0.0, sy = 0.0;
+  bool take = cell < P.nx * P.ny;
+  const int i = cell % P.nx, j = cell / P.nx;
+  if (take && filter) {   // only cells whose FP32 upper bound reaches the largest lower bound
+    float lo[2], hi[2];
+    speed_bounds(P, U, i, j, lo, hi);
+    take = !(hi[0] < __uint_as_float(A.bounds[2 * p]) && hi[1] < __uint_as_float(A.bounds[2 * p + 1]));
   }
-  return lo;
+  if (take) {
+    const double rho = U[sidx(P, 0, 0, i, j)];
+    const double mu = U[sidx(P, 1, 0, i, j)] / rho, nu = U[sidx(P, 2, 0, i, j)] / rho;
+    const double pr = (P.gamma - 1.0) * (U[sidx(P, 3, 0, i, j)] - 0.5 * rho * (mu * mu + nu * nu));
+    cell_speeds(P, rho, mu, nu, pr, sx, sy);
+  }
+  if (!__any_sync(0xffffffffu, take)) return;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    sx = fmax(sx, __shfl_down_sync(0xffffffffu, sx, o));
+    sy = fmax(sy, __shfl_down_sync(0xffffffffu, sy, o));
+  }
+  if ((tid & 31) == 0) {   // non-negative doubles order like their bit patterns
+    atomicMax(A.speeds + 2 * p, (unsigned long long)__double_as_longlong(sx));
+    atomicMax(A.speeds + 2 * p + 1, (unsigned long long)__double_as_longlong(sy));
+  }
+}
+
+__device__ __forceinline__ double batch_dt(const BatchStage& A, const Prob& P, int p) {
+  if (A.dt_in) return A.dt_in[p];
+  const double ax = __longlong_as_double((long long)A.speeds[2 * p]);
+  const double ay = __longlong_as_double((long long)A.speeds[2 * p + 1]);
+  const double r = ax / P.dx + ay / P.dy;
+  return (r > 0.0 && isfinite(r)) ? A.cfl / r : 0.0;
+}
+
+template <typename T>
+__device__ __forceinline__ void batch_rec_item(const BatchStage& A, const Prob& P, const BProb& Q, int it, int tid,
+                                               const Weights<T>& W, const typename rows2d<T>::type& B) {
+  constexpr bool S32 = std::is_same<T, float>::value;
+  const int cell = (it - Q.rec_first) * RB + tid;
+  if (cell < P.nx * P.ny)
+    rec2d_cell<T, 4, REC_PLAIN, false, S32>(P, W, B, A.Uin + Q.uoff, nullptr, nullptr, cell % P.nx, cell / P.nx,
+                                            (T*)A.G + Q.goff, (T*)A.aux + Q.aoff, S32 ? A.U32in + Q.uoff : nullptr);
+}
+
+template <typename T>
+__device__ __forceinline__ void batch_flag_item(const BatchStage& A, const Prob& P, const BProb& Q, int p, int it,
+                                                int tid) {
+  const int cell = (it - Q.rec_first) * RB + tid;
+  const bool valid = cell < P.nx * P.ny;
+  const int i = cell % P.nx, j = cell / P.nx;
+  const bool flag =
+      valid && flag2d_cell<T>(P, A.Uin + Q.uoff, (const T*)A.G + Q.goff, (const T*)A.aux + Q.aoff, i, j, nullptr);
+  warp_append<unsigned long long>(flag, ((unsigned long long)p << 32) | (unsigned)cell, A.list, A.count);
+  if (valid) {
+    A.mask[Q.coff + cell] = flag ? 1 : 0;
+    if (flag) modify2d_cell<4>(P, A.Uin + Q.uoff, A.Mod + Q.moff, i, j);
+  }
+}
+
+template <typename T>
+__device__ __forceinline__ void batch_rerec(const BatchStage& A, const Weights<T>& W,
+                                            const typename rows2d<T>::type& B) {
+  constexpr bool S32 = std::is_same<T, float>::value;
+  const int n = *(volatile int*)A.count;
+  for (int t = blockIdx.x * RB + threadIdx.x; t < n; t += gridDim.x * RB) {
+    const unsigned long long e = A.list[t];
+    const int p = (int)(e >> 32), cell = (int)(e & 0xffffffffu);
+    // after a barrier wait that gave up, an entry may not be written yet
+    if (p < 0 || p >= A.nprob || cell < 0 || cell >= A.probs[p].P.nx * A.probs[p].P.ny) continue;
+    const BProb& Q = A.probs[p];
+    rec2d_cell<T, 4, REC_FLAGGED, false, S32>(Q.P, W, B, A.Uin + Q.uoff, A.mask + Q.coff, A.Mod + Q.moff,
+                                              cell % Q.P.nx, cell / Q.P.nx, (T*)A.G + Q.goff, nullptr,
+                                              S32 ? A.U32in + Q.uoff : nullptr);
+  }
 }
 
 template <typename T, int TXV, int TYV>
-__global__ void __launch_bounds__(TXV * TYV) batch_stage_kernel(const __grid_constant__ BatchStage A, const __grid_constant__ Weights<T> W,
+__device__ __forceinline__ void batch_update_item(const BatchStage& A, const Prob& P, const BProb& Q, int p, int it,
+                                                  int tid, double dt, T (&xf)[TYV][TXV + 1][4][4],
+                                                  T (&yf)[TYV + 1][TXV][4][4]) {
+  const int t = it - Q.upd_first;
+  Rk S{A.Uin + Q.uoff, A.Un + Q.uoff, A.Uout + Q.uoff, A.mask + Q.coff, A.Mod + Q.moff,
+       A.maskN ? A.maskN + Q.coff : nullptr, A.ModN ? A.ModN + Q.moff : nullptr, dt, A.cA, A.cB,
+       nullptr, nullptr, A.pstatus + p, nullptr, std::is_same<T, float>::value ? A.U32out + Q.uoff : nullptr};
+  update2d_tile<T, 4, TXV, TYV>(P, GlobalSrc<T>{(const T*)A.G + Q.goff}, S, (t % Q.tiles_x) * TXV,
+                                (t / Q.tiles_x) * TYV, tid, xf, yf);
+}
+
+// The block's problem description in shared memory (the kernels' stores could
+// alias a description in global memory, so its fields would be loaded again and again).
+__device__ __forceinline__ void stage_prob(const BProb& Q, Prob* sp, int tid) {
+  static_assert(sizeof(Prob) % 4 == 0, "copied by words");
+  const int* src = reinterpret_cast<const int*>(&Q.P);
+  for (int k = tid; k < (int)(sizeof(Prob) / 4); k += RB) reinterpret_cast<int*>(sp)[k] = src[k];
+  __syncthreads();
+}
+
+// ---- a launch per phase
+__global__ void __launch_bounds__(RB) batch_bounds_kernel(const __grid_constant__ BatchStage A) {
+  const int it = blockIdx.x, p = A.rec_owner[it], tid = threadIdx.x;
+  const BProb& Q = A.probs[p];
+  const Prob& P = Q.P;
+  const int cell = (it - Q.rec_first) * RB + tid;
+  float lo[2] = {0.0f, 0.0f}, hi[2];
+  if (cell < P.nx * P.ny) speed_bounds(P, A.Uin + Q.uoff, cell % P.nx, cell / P.nx, lo, hi);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {   // non-negative floats order like their bit patterns
+    const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(lo[k]));
+    if ((tid & 31) == 0) atomicMax(A.bounds + 2 * p + k, m);
+  }
+}
+
+__global__ void __launch_bounds__(RB) batch_speeds_kernel(const __grid_constant__ BatchStage A) {
+  const int it = blockIdx.x, p = A.rec_owner[it];
+  batch_speeds_item(A, A.probs[p].P, A.probs[p], p, it, threadIdx.x, true);
+}
+
+__global__ void batch_dt_kernel(const __grid_constant__ BatchStage A) {
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p < A.nprob) A.dt_out[p] = batch_dt(A, A.probs[p].P, p);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(RB, (is_df64<T>::value ? 4 : std::is_same<T, float>::value ? 8 : 5))
+    batch_rec_kernel(const __grid_constant__ BatchStage A, const __grid_constant__ Weights<T> W,
+                     const __grid_constant__ typename rows2d<T>::type B) {
+  __shared__ Prob sp;
+  const int it = blockIdx.x;
+  const BProb& Q = A.probs[A.rec_owner[it]];
+  stage_prob(Q, &sp, threadIdx.x);
+  batch_rec_item<T>(A, sp, Q, it, threadIdx.x, W, B);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(RB) batch_flag_kernel(const __grid_constant__ BatchStage A) {
+  __shared__ Prob sp;
+  const int it = blockIdx.x, p = A.rec_owner[it];
+  const BProb& Q = A.probs[p];
+  stage_prob(Q, &sp, threadIdx.x);
+  batch_flag_item<T>(A, sp, Q, p, it, threadIdx.x);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(RB) batch_rerec_kernel(const __grid_constant__ BatchStage A,
+                                                         const __grid_constant__ Weights<T> W,
+                                                         const __grid_constant__ typename rows2d<T>::type B) {
+  batch_rerec<T>(A, W, B);
+}
+
+template <typename T, int TXV, int TYV>
+__global__ void __launch_bounds__(TXV * TYV, (std::is_same<T, float>::value ? 7 : 4))
+    batch_update_kernel(const __grid_constant__ BatchStage A) {
+  __shared__ T xf[TYV][TXV + 1][4][4];
+  __shared__ T yf[TYV + 1][TXV][4][4];
+  __shared__ Prob sp;
+  const int it = blockIdx.x, p = A.upd_owner[it];
+  const BProb& Q = A.probs[p];
+  stage_prob(Q, &sp, threadIdx.x);
+  batch_update_item<T, TXV, TYV>(A, sp, Q, p, it, threadIdx.x, A.dt_out[p], xf, yf);
+}
+
+// ---- one persistent launch
+template <typename T, int TXV, int TYV>
+__global__ void __launch_bounds__(TXV * TYV) batch_stage_kernel(const __grid_constant__ BatchStage A,
+                                                                const __grid_constant__ Weights<T> W,
                                                                 const __grid_constant__ typename rows2d<T>::type B) {
   static_assert(TXV * TYV == RB, "tiles and rows use the same block");
   __shared__ T xf[TYV][TXV + 1][4][4];
   __shared__ T yf[TYV + 1][TXV][4][4];
   const int tid = threadIdx.x;
   const unsigned nb = gridDim.x;
-  T* G = (T*)A.G;
-  T* aux = (T*)A.aux;
   // CFL wave speeds of U^n (first stage, when the caller gives no dt)
   if (A.stage == 0 && !A.dt_in) {
     for (int it = blockIdx.x; it < A.n_rec; it += nb) {
-      const int p = owner<0>(A.probs, A.nprob, it);
-      const Prob P = A.probs[p].P;
-      const double* U = A.Uin + A.probs[p].uoff;
-      const int cell = (it - A.probs[p].rec_first) * RB + tid;
-      double sx = 0.0, sy = 0.0;
-      if (cell < P.nx * P.ny) {
-        const int i = cell % P.nx, j = cell / P.nx;
-        const double rho = U[sidx(P, 0, 0, i, j)];
-        const double mu = U[sidx(P, 1, 0, i, j)] / rho, nu = U[sidx(P, 2, 0, i, j)] / rho;
-        const double pr = (P.gamma - 1.0) * (U[sidx(P, 3, 0, i, j)] - 0.5 * rho * (mu * mu + nu * nu));
-        cell_speeds(P, rho, mu, nu, pr, sx, sy);
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        sx = fmax(sx, __shfl_down_sync(0xffffffffu, sx, o));
-        sy = fmax(sy, __shfl_down_sync(0xffffffffu, sy, o));
-      }
-      if ((tid & 31) == 0) {   // non-negative doubles order like their bit patterns
-        atomicMax(A.speeds + 2 * p, (unsigned long long)__double_as_longlong(sx));
-        atomicMax(A.speeds + 2 * p + 1, (unsigned long long)__double_as_longlong(sy));
-      }
+      const int p = A.rec_owner[it];
+      batch_speeds_item(A, A.probs[p].P, A.probs[p], p, it, tid, false);
     }
     grid_barrier(A.bar, nb + A.bar_extra, A.status, A.spin_limit);
   }
   // Step 1: every cell
   for (int it = blockIdx.x; it < A.n_rec; it += nb) {
-    const int p = owner<0>(A.probs, A.nprob, it);
-    const BProb& Q = A.probs[p];
-    const int cell = (it - Q.rec_first) * RB + tid;
-    if (cell < Q.P.nx * Q.P.ny)
-      rec2d_cell<T, 4, REC_PLAIN>(Q.P, W, B, A.Uin + Q.uoff, nullptr, nullptr, cell % Q.P.nx, cell / Q.P.nx, G + Q.goff,
-                              aux + Q.aoff);
+    const BProb& Q = A.probs[A.rec_owner[it]];
+    batch_rec_item<T>(A, Q.P, Q, it, tid, W, B);
   }
   grid_barrier(A.bar, nb + A.bar_extra, A.status, A.spin_limit);
   // Steps 2.1-2.2
   for (int it = blockIdx.x; it < A.n_rec; it += nb) {
-    const int p = owner<0>(A.probs, A.nprob, it);
-    const BProb& Q = A.probs[p];
-    const int cell = (it - Q.rec_first) * RB + tid;
-    const bool valid = cell < Q.P.nx * Q.P.ny;
-    const int i = cell % Q.P.nx, j = cell / Q.P.nx;
-    const bool flag = valid && flag2d_cell<T>(Q.P, A.Uin + Q.uoff, G + Q.goff, aux + Q.aoff, i, j, nullptr);
-    warp_append<unsigned long long>(flag, ((unsigned long long)p << 32) | (unsigned)cell, A.list, A.count);
-    if (valid) {
-      A.mask[Q.coff + cell] = flag ? 1 : 0;
-      if (flag) modify2d_cell<4>(Q.P, A.Uin + Q.uoff, A.Mod + Q.moff, i, j);
-    }
+    const int p = A.rec_owner[it];
+    batch_flag_item<T>(A, A.probs[p].P, A.probs[p], p, it, tid);
   }
   grid_barrier(A.bar, nb + A.bar_extra, A.status, A.spin_limit);
   // Step 2.3: troubled cells
-  {
-    const int n = *(volatile int*)A.count;
-    for (int t = blockIdx.x * RB + tid; t < n; t += nb * RB) {
-      const unsigned long long e = A.list[t];
-      const int p = (int)(e >> 32), cell = (int)(e & 0xffffffffu);
-      // after a barrier wait that gave up, an entry may not be written yet
-      if (p < 0 || p >= A.nprob || cell < 0 || cell >= A.probs[p].P.nx * A.probs[p].P.ny) continue;
-      const BProb& Q = A.probs[p];
-      rec2d_cell<T, 4, REC_FLAGGED>(Q.P, W, B, A.Uin + Q.uoff, A.mask + Q.coff, A.Mod + Q.moff, cell % Q.P.nx,
-                             cell / Q.P.nx, G + Q.goff, nullptr);
-    }
-  }
+  batch_rerec<T>(A, W, B);
   grid_barrier(A.bar, nb + A.bar_extra, A.status, A.spin_limit);
   // Step 3: fluxes, quadrature, L, Runge-Kutta
   for (int it = blockIdx.x; it < A.n_upd; it += nb) {
-    const int p = owner<1>(A.probs, A.nprob, it);
+    const int p = A.upd_owner[it];
     const BProb& Q = A.probs[p];
-    double dt;
-    if (A.dt_in) {
-      dt = A.dt_in[p];
-    } else {
-      const double ax = __longlong_as_double((long long)A.speeds[2 * p]);
-      const double ay = __longlong_as_double((long long)A.speeds[2 * p + 1]);
-      const double r = ax / Q.P.dx + ay / Q.P.dy;
-      dt = (r > 0.0 && isfinite(r)) ? A.cfl / r : 0.0;
-    }
-    const int t = it - Q.upd_first;
-    if (A.stage == 0 && t == 0 && tid == 0) A.dt_out[p] = dt;
-    Rk S{A.Uin + Q.uoff, A.Un + Q.uoff, A.Uout + Q.uoff, A.mask + Q.coff, A.Mod + Q.moff,
-         A.maskN ? A.maskN + Q.coff : nullptr, A.ModN ? A.ModN + Q.moff : nullptr, dt, A.cA, A.cB,
-         nullptr, nullptr, A.pstatus + p};
-    update2d_tile<T, 4, TXV, TYV>(Q.P, GlobalSrc<T>{G + Q.goff}, S, (t % Q.tiles_x) * TXV, (t / Q.tiles_x) * TYV, tid,
-                                  xf, yf);
+    const double dt = batch_dt(A, Q.P, p);
+    if (A.stage == 0 && it == Q.upd_first && tid == 0) A.dt_out[p] = dt;
+    batch_update_item<T, TXV, TYV>(A, Q.P, Q, p, it, tid, dt, xf, yf);
   }
 }
 
+// The persistent kernel holds every phase to the registers and shared memory of the
+// largest and pays four grid barriers; a launch per phase measured faster at every
+// size (ms per step, persistent / per phase: 4 problems of 13 k cells FP32
+// 0.29 / 0.20, FP64 1.03 / 0.57; 64 problems of 3.8 M cells FP32 8.3 / 5.5, FP64
+// 44 / 41; FP32 9.0 with its moments converted per gather).  The persistent form
+// remains where the caller sets the barrier up (hweno_batch_set_barrier with extra
+// arrivals).
 template <typename T, int TXV, int TYV>
-cudaError_t launch_batch(const Weights<T>& W, const typename rows2d<T>::type& Bt, const BatchStage& S, int nsm, cudaStream_t st) {
+cudaError_t launch_batch(const Weights<T>& W, const typename rows2d<T>::type& Bt, const BatchStage& S, int nsm,
+                         cudaStream_t st) {
+  if (S.bar_extra == 0) {
+    if (S.stage == 0) {
+      if (!S.dt_in) {
+        batch_bounds_kernel<<<S.n_rec, RB, 0, st>>>(S);
+        batch_speeds_kernel<<<S.n_rec, RB, 0, st>>>(S);
+      }
+      batch_dt_kernel<<<(S.nprob + 127) / 128, 128, 0, st>>>(S);
+    }
+    batch_rec_kernel<T><<<S.n_rec, RB, 0, st>>>(S, W, Bt);
+    batch_flag_kernel<T><<<S.n_rec, RB, 0, st>>>(S);
+    batch_rerec_kernel<T><<<nsm * 8, RB, 0, st>>>(S, W, Bt);
+    batch_update_kernel<T, TXV, TYV><<<S.n_upd, RB, 0, st>>>(S);
+    return cudaGetLastError();
+  }
   auto kern = batch_stage_kernel<T, TXV, TYV>;
   int per_sm = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, RB, 0);

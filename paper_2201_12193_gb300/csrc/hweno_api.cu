@@ -58,7 +58,8 @@ struct hweno_s {
   int n_rec = 0, n_upd = 0;
   int tile_variant = 0;
   unsigned long long* blist = nullptr;
-  unsigned long long* speeds = nullptr;
+  unsigned long long* speeds = nullptr;   // per problem {max a_x, max a_y}, then their FP32 bounds (one pair of words each)
+  int* owner = nullptr;          // problem of each 128-cell row [n_rec], then of each update tile
   double* dt_out = nullptr;
   unsigned* bar = nullptr;
   unsigned* pstatus = nullptr;   // per-problem status bits (device)
@@ -270,6 +271,7 @@ void free_all(hweno_s* h) {
   cudaFree(h->dprobs);
   cudaFree(h->blist);
   cudaFree(h->speeds);
+  cudaFree(h->owner);
   cudaFree(h->dt_out);
   cudaFree(h->bar);
   cudaFree(h->pstatus);
@@ -1077,12 +1079,27 @@ void layout_batch(hweno_t h) {
   h->n_upd = upd;
 }
 
+// The device copies of the layout; owner is allocated for the variant with the most tiles.
+cudaError_t upload_layout(hweno_t h) {
+  std::vector<int> own(h->n_rec + h->n_upd);
+  for (int k = 0; k < h->nprob; ++k) {
+    const bool end = k + 1 == h->nprob;
+    std::fill(own.begin() + h->probs[k].rec_first, own.begin() + (end ? h->n_rec : h->probs[k + 1].rec_first), k);
+    std::fill(own.begin() + h->n_rec + h->probs[k].upd_first,
+              own.begin() + h->n_rec + (end ? h->n_upd : h->probs[k + 1].upd_first), k);
+  }
+  const cudaError_t e = cudaMemcpy(h->owner, own.data(), own.size() * sizeof(int), cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) return e;
+  return cudaMemcpy(h->dprobs, h->probs.data(), h->nprob * sizeof(hw::BProb), cudaMemcpyHostToDevice);
+}
+
 size_t batch_count(const hweno_s* h, int k) {
   const Prob& P = h->probs[k].P;
   return (size_t)P.nvar * P.nmom * P.nx * P.ny;
 }
 
 hweno_status batch_graph(hweno_t h, int a, const double* dt_in, double cfl, cudaGraphExec_t* out);
+cudaError_t batch_enqueue(hweno_t h, int a, const double* dt_in, double cfl, cudaStream_t st);
 
 }  // namespace
 
@@ -1144,7 +1161,6 @@ hweno_status hweno_create_batch(const hweno_grid* grids, const hweno_bc* bcs, in
   h->tot_cells = tc;
   h->P = h->probs[0].P;
   build_tables(h);
-  layout_batch(h);
   const size_t esz = h->fp32 == hw::PREC_FP32 ? sizeof(float) : sizeof(double);   // df64 is 8 bytes
   bool ok = true;
   for (int k = 0; k < 3; ++k) ok = ok && cudaMalloc(&h->U[k], tu * sizeof(double)) == cudaSuccess;
@@ -1156,7 +1172,18 @@ hweno_status hweno_create_batch(const hweno_grid* grids, const hweno_bc* bcs, in
   ok = ok && cudaMalloc(&h->blist, tc * sizeof(unsigned long long)) == cudaSuccess;
   ok = ok && cudaMalloc(&h->B.count, 4 * sizeof(int)) == cudaSuccess;
   ok = ok && cudaMalloc(&h->B.status, sizeof(unsigned)) == cudaSuccess;
-  ok = ok && cudaMalloc(&h->speeds, 2 * n * sizeof(unsigned long long)) == cudaSuccess;
+  ok = ok && cudaMalloc(&h->speeds, 3 * n * sizeof(unsigned long long)) == cudaSuccess;
+  size_t most = 0;               // update tiles of the variant with the most
+  for (int v = 0; v < 3; ++v) {
+    h->tile_variant = v;
+    layout_batch(h);
+    most = std::max(most, (size_t)h->n_upd);
+  }
+  h->tile_variant = 0;
+  layout_batch(h);
+  ok = ok && cudaMalloc(&h->owner, (h->n_rec + most) * sizeof(int)) == cudaSuccess;
+  for (int k = 0; k < 3 && h->fp32 == hw::PREC_FP32; ++k)
+    ok = ok && cudaMalloc(&h->U32[k], tu * sizeof(float)) == cudaSuccess;
   ok = ok && cudaMalloc(&h->dt_out, n * sizeof(double)) == cudaSuccess;
   ok = ok && cudaMalloc(&h->bar, 2 * sizeof(unsigned)) == cudaSuccess;
   ok = ok && cudaMalloc(&h->pstatus, n * sizeof(unsigned)) == cudaSuccess;
@@ -1169,7 +1196,7 @@ hweno_status hweno_create_batch(const hweno_grid* grids, const hweno_bc* bcs, in
     fprintf(stderr, "hweno_create_batch: device allocation failed\n");
     return HWENO_ENOMEM;
   }
-  cudaMemcpy(h->dprobs, h->probs.data(), n * sizeof(hw::BProb), cudaMemcpyHostToDevice);
+  upload_layout(h);
   cudaMemset(h->B.status, 0, sizeof(unsigned));
   cudaMemset(h->mask3, 0, 3 * tc);
   cudaMemset(h->bar, 0, 2 * sizeof(unsigned));
@@ -1177,6 +1204,7 @@ hweno_status hweno_create_batch(const hweno_grid* grids, const hweno_bc* bcs, in
   cudaMemset(h->pstatus, 0, n * sizeof(unsigned));
   cudaMemset(h->dt_out, 0, n * sizeof(double));
   for (int k = 0; k < 3; ++k) cudaMemset(h->U[k], 0, tu * sizeof(double));
+  for (int k = 0; k < 3 && h->U32[k]; ++k) cudaMemset(h->U32[k], 0, tu * sizeof(float));
   if (cudaDeviceSynchronize() != cudaSuccess) { free_all(h); delete h; return HWENO_ECUDA; }
   *out = h;
   return HWENO_OK;
@@ -1188,7 +1216,7 @@ hweno_status hweno_batch_set_tile(hweno_t h, int variant) {
   CK(h, cudaStreamSynchronize(h->stream));
   h->tile_variant = variant;
   layout_batch(h);
-  CK(h, cudaMemcpy(h->dprobs, h->probs.data(), h->nprob * sizeof(hw::BProb), cudaMemcpyHostToDevice));
+  CK(h, upload_layout(h));
   drop_graphs(h);
   return HWENO_OK;
 }
@@ -1200,6 +1228,8 @@ hweno_status hweno_batch_set_moments(hweno_t h, int k, const double* m, size_t c
   CK(h, cudaMemcpy2DAsync(h->U[h->cur] + h->probs[k].uoff, P.pitch * sizeof(double), m, P.nx * sizeof(double),
                           P.nx * sizeof(double), (size_t)12 * P.ny,
                           on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->stream));
+  if (h->U32[h->cur])
+    hw::run_shadow32(P, h->U[h->cur] + h->probs[k].uoff, h->U32[h->cur] + h->probs[k].uoff, 0, P.ny, h->stream);
   CK(h, cudaMemsetAsync(h->B.status, 0, sizeof(unsigned), h->stream));
   h->have_state = true;
   h->stepped = false;
@@ -1283,27 +1313,7 @@ hweno_status hweno_step_batch(hweno_t h, const double* dt_device, double cfl) {
   if (h->use_graph && h->graphs[a]) {
     CK(h, cudaGraphLaunch(h->graphs[a], h->stream));
   } else {
-    hw::BatchStage S{};
-    const int b = (a + 1) % 3, c = (a + 2) % 3;
-    const long long T = h->tot_cells;
-    CK(h, cudaMemsetAsync(h->speeds, 0, 2 * h->nprob * sizeof(unsigned long long), h->stream));
-    CK(h, cudaMemsetAsync(h->B.count, 0, 4 * sizeof(int), h->stream));
-    for (int st = 0; st < 3; ++st) {
-      S.probs = h->dprobs; S.nprob = h->nprob; S.n_rec = h->n_rec; S.n_upd = h->n_upd;
-      S.G = h->B.G; S.aux = h->B.aux; S.list = h->blist; S.count = h->B.count + st;
-      S.speeds = h->speeds; S.dt_in = dt_device; S.dt_out = h->dt_out; S.cfl = cfl;
-      S.status = h->B.status; S.pstatus = h->pstatus; S.bar = h->bar; S.stage = st;
-      S.spin_limit = h->spin_limit; S.bar_extra = h->bar_extra;
-      S.Un = h->U[a];
-      if (st == 0) { S.Uin = h->U[a]; S.Uout = h->U[b]; S.cA = 0.0; S.cB = 1.0; S.Mod = h->ModN; S.ModN = nullptr;
-                     S.mask = h->mask3; S.maskN = nullptr; }
-      if (st == 1) { S.Uin = h->U[b]; S.Uout = h->U[c]; S.cA = 0.75; S.cB = 0.25; S.Mod = h->ModK; S.ModN = h->ModN;
-                     S.mask = h->mask3 + T; S.maskN = h->mask3; }
-      if (st == 2) { S.Uin = h->U[c]; S.Uout = h->U[b]; S.cA = 1.0 / 3.0; S.cB = 2.0 / 3.0; S.Mod = h->ModK;
-                     S.ModN = h->ModN; S.mask = h->mask3 + 2 * T; S.maskN = h->mask3; }
-      CK(h, cudaMemsetAsync(h->bar, 0, sizeof(unsigned), h->stream));
-      CK(h, hw::run_batch_stage(h->T, h->fp32, h->tile_variant, S, h->P.nsm, h->stream));
-    }
+    CK(h, batch_enqueue(h, a, dt_device, cfl, h->stream));
   }
   h->prev = a;
   h->cur = (a + 1) % 3;
@@ -1315,34 +1325,41 @@ hweno_status hweno_step_batch(hweno_t h, const double* dt_device, double cfl) {
 
 namespace {
 
-// Capture one batched step (memsets + three cooperative stage launches) for the
-// state rotation starting at buffer a.
+// One batched step from the state rotation starting at buffer a: memsets and three stages.
+cudaError_t batch_enqueue(hweno_t h, int a, const double* dt_in, double cfl, cudaStream_t st) {
+  const int b = (a + 1) % 3, c = (a + 2) % 3;
+  const long long T = h->tot_cells;
+  cudaMemsetAsync(h->speeds, 0, 3 * h->nprob * sizeof(unsigned long long), st);
+  cudaMemsetAsync(h->B.count, 0, 4 * sizeof(int), st);
+  cudaError_t e = cudaGetLastError();
+  for (int k = 0; k < 3 && e == cudaSuccess; ++k) {
+    hw::BatchStage S{};
+    S.probs = h->dprobs; S.nprob = h->nprob; S.n_rec = h->n_rec; S.n_upd = h->n_upd;
+    S.rec_owner = h->owner; S.upd_owner = h->owner + h->n_rec;
+    S.G = h->B.G; S.aux = h->B.aux; S.list = h->blist; S.count = h->B.count + k;
+    S.speeds = h->speeds; S.bounds = reinterpret_cast<unsigned*>(h->speeds + 2 * h->nprob);
+    S.dt_in = dt_in; S.dt_out = h->dt_out; S.cfl = cfl;
+    S.status = h->B.status; S.pstatus = h->pstatus; S.bar = h->bar; S.stage = k;
+    S.spin_limit = h->spin_limit; S.bar_extra = h->bar_extra; S.Un = h->U[a];
+    const int in = k == 0 ? a : (k == 1 ? b : c), out = k == 1 ? c : b;
+    S.Uin = h->U[in]; S.Uout = h->U[out]; S.U32in = h->U32[in]; S.U32out = h->U32[out];
+    S.cA = k == 0 ? 0.0 : (k == 1 ? 0.75 : 1.0 / 3.0); S.cB = k == 0 ? 1.0 : (k == 1 ? 0.25 : 2.0 / 3.0);
+    S.Mod = k == 0 ? h->ModN : h->ModK; S.ModN = k == 0 ? nullptr : h->ModN;
+    S.mask = h->mask3 + k * T; S.maskN = k == 0 ? nullptr : h->mask3;
+    cudaMemsetAsync(h->bar, 0, sizeof(unsigned), st);
+    e = hw::run_batch_stage(h->T, h->fp32, h->tile_variant, S, h->P.nsm, st);
+  }
+  return e;
+}
+
+// Capture it.
 hweno_status batch_graph(hweno_t h, int a, const double* dt_in, double cfl, cudaGraphExec_t* out) {
   cudaStream_t cs;
   if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) return HWENO_ECUDA;
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
-  const int b = (a + 1) % 3, c = (a + 2) % 3;
-  const long long T = h->tot_cells;
   if (e == cudaSuccess) {
-    cudaMemsetAsync(h->speeds, 0, 2 * h->nprob * sizeof(unsigned long long), cs);
-    cudaMemsetAsync(h->B.count, 0, 4 * sizeof(int), cs);
-    for (int st = 0; st < 3 && e == cudaSuccess; ++st) {
-      hw::BatchStage S{};
-      S.probs = h->dprobs; S.nprob = h->nprob; S.n_rec = h->n_rec; S.n_upd = h->n_upd;
-      S.G = h->B.G; S.aux = h->B.aux; S.list = h->blist; S.count = h->B.count + st;
-      S.speeds = h->speeds; S.dt_in = dt_in; S.dt_out = h->dt_out; S.cfl = cfl;
-      S.status = h->B.status; S.pstatus = h->pstatus; S.bar = h->bar; S.stage = st;
-      S.spin_limit = h->spin_limit; S.bar_extra = h->bar_extra; S.Un = h->U[a];
-      if (st == 0) { S.Uin = h->U[a]; S.Uout = h->U[b]; S.cA = 0.0; S.cB = 1.0; S.Mod = h->ModN; S.ModN = nullptr;
-                     S.mask = h->mask3; S.maskN = nullptr; }
-      if (st == 1) { S.Uin = h->U[b]; S.Uout = h->U[c]; S.cA = 0.75; S.cB = 0.25; S.Mod = h->ModK; S.ModN = h->ModN;
-                     S.mask = h->mask3 + T; S.maskN = h->mask3; }
-      if (st == 2) { S.Uin = h->U[c]; S.Uout = h->U[b]; S.cA = 1.0 / 3.0; S.cB = 2.0 / 3.0; S.Mod = h->ModK;
-                     S.ModN = h->ModN; S.mask = h->mask3 + 2 * T; S.maskN = h->mask3; }
-      cudaMemsetAsync(h->bar, 0, sizeof(unsigned), cs);
-      e = hw::run_batch_stage(h->T, h->fp32, h->tile_variant, S, h->P.nsm, cs);
-    }
+    e = batch_enqueue(h, a, dt_in, cfl, cs);
     const cudaError_t e2 = cudaStreamEndCapture(cs, &g);
     if (e == cudaSuccess) e = e2;
   }

@@ -130,6 +130,8 @@ struct BProb {
 // Buffers and coefficients of one batched stage launch.
 struct BatchStage {
   const BProb* probs;     // device array
+  const int* rec_owner;   // problem of each 128-cell row, of each update tile
+  const int* upd_owner;
   int nprob, n_rec, n_upd;
   const double* Uin; const double* Un; double* Uout;
   void* G; void* aux;
@@ -140,6 +142,8 @@ struct BatchStage {
   unsigned long long* list;   // troubled (problem << 32 | cell)
   int* count;
   unsigned long long* speeds; // per problem: max a_x, max a_y as FP64 bit patterns
+  unsigned* bounds;       // per problem: their largest FP32 lower bounds, as bit patterns (launch per phase)
+  const float* U32in; float* U32out;   // FP32: float copies of Uin and Uout
   const double* dt_in;    // per-problem dt from the caller, or nullptr (CFL)
   double* dt_out;         // per-problem dt used (written in the first stage)
   double cfl, cA, cB;
@@ -155,8 +159,8 @@ struct BatchStage {
 // Default bound of a grid-barrier wait: 2^26 polls with 64 ns sleeps, seconds.
 constexpr unsigned long long BARRIER_SPIN_DEFAULT = 1ull << 26;
 
-// Launch one batched stage as a single persistent cooperative kernel (grid =
-// resident blocks); returns the CUDA error of the launch.
+// Launch one batched stage (a launch per phase, or one persistent cooperative
+// kernel with grid = resident blocks); returns the CUDA error of the launch.
 cudaError_t run_batch_stage(const HostTabs& T, int fp32, int tile_variant, const BatchStage& S, int nsm,
                             cudaStream_t st);
 constexpr unsigned ST_TIMEOUT = 4u;   // a bounded grid-barrier wait gave up
