@@ -119,12 +119,37 @@ __device__ __forceinline__ float load_mom32(const Prob& P, const float* __restri
   return __uint_as_float(__float_as_uint(v) ^ (flip << 31));
 }
 
+// KXRCF face-velocity partials of faces [f0, f1) (x-lo, x-hi, y-lo, y-hi) of the cell
+// at offset o from its point values: point indices p0 + q dp, velocity
+// (rho mu)/rho, (rho nu)/rho or u.  (G was written by this block: no read-only loads.)
+template <typename T, int NV>
+__device__ __forceinline__ void face_partials(const Prob& P, T* G, T* aux, long long o, int f0, int f1) {
+#pragma unroll 1
+  for (int f = f0; f < f1; ++f) {
+    const int p0 = f == 1 ? 12 : f == 3 ? 3 : 0, dp = f < 2 ? 1 : 4, v = NV == 4 ? (f < 2 ? 1 : 2) : 0;
+    T s = T(0);
+    if (P.eq == EQ_ADV) {
+      s = T(f < 2 ? P.adv_a : P.adv_b);
+    } else {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const T m = G[(long long)(v * 16 + p0 + q * dp) * P.gplane + o];
+        s = fma(gl_w<T>(q), NV == 4 ? m * rcp(G[(long long)(p0 + q * dp) * P.gplane + o]) : m, s);
+      }
+    }
+    aux[(long long)f * P.gplane + o] = s;
+  }
+}
+
+// Variables [v0, v1) of cell (i, j).  The fixed-point precisions leave the face
+// partials to face_partials.
 template <typename T, int NV, int MODE, bool FIX = false, bool S32 = false>
 __device__ __forceinline__ void rec2d_cell(const Prob& P, const Weights<T>& W,
                                            const typename rows2d<T>::type& B, const double* __restrict__ U,
                                            const uint8_t* __restrict__ mask,
                                            const double* __restrict__ Mod, int i, int j, T* __restrict__ G,
-                                           T* __restrict__ aux, const float* __restrict__ U32 = nullptr) {
+                                           T* __restrict__ aux, const float* __restrict__ U32 = nullptr, int v0 = 0,
+                                           int v1 = NV) {
   constexpr bool FLAGGED = MODE == REC_FLAGGED;
   const bool usemod = MODE == REC_FLAGGED || (MODE == REC_MIXED && mask[(long long)j * P.nx + i] == 1);
   const Nbr nb = neighbours<FIX>(P, i, j);
@@ -143,7 +168,7 @@ __device__ __forceinline__ void rec2d_cell(const Prob& P, const Weights<T>& W,
   T pxl = T(0), pxr = T(0), pyb = T(0), pyt = T(0), nrm = T(0);
   [[maybe_unused]] long long nrmb = 0;   // fx64: the norm's bits (non-negative doubles order like them)
 #pragma unroll 1
-  for (int v = 0; v < NV; ++v) {
+  for (int v = v0; v < v1; ++v) {
     D d[23];
     if (inner) {
 #pragma unroll
@@ -175,6 +200,10 @@ __device__ __forceinline__ void rec2d_cell(const Prob& P, const Weights<T>& W,
           else nrmb = max(nrmb, __double_as_longlong(x.v) & 0x7FFFFFFFFFFFFFFFLL);
         }
       });
+      if (!FLAGGED && v == 0) {
+        if constexpr (!is_df64<T>::value) nrm = __longlong_as_double(nrmb);
+        aux[4 * P.gplane + o] = nrm;
+      }
     } else {
       recon2d<T>(W, B, d, [&](int p, T x) { out[p] = x; });
 #pragma unroll
@@ -225,28 +254,7 @@ __device__ __forceinline__ void rec2d_cell(const Prob& P, const Weights<T>& W,
       }
     }
   }
-  if constexpr (FXD && !FLAGGED) {
-    if constexpr (!is_df64<T>::value) nrm = __longlong_as_double(nrmb);
-    if (P.eq == EQ_ADV) {
-      pxl = pxr = T(P.adv_a);
-      pyb = pyt = T(P.adv_b);
-    } else {
-      // faces x-lo, x-hi, y-lo, y-hi: point indices p0 + q dp, velocity (rho mu)/rho, (rho nu)/rho or u
-      const T* Gr = G + o;
-#pragma unroll
-      for (int f = 0; f < 4; ++f) {
-        const int p0 = f == 0 ? 0 : f == 1 ? 12 : f == 2 ? 0 : 3, dp = f < 2 ? 1 : 4, v = NV == 4 ? (f < 2 ? 1 : 2) : 0;
-        T s = T(0);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const T m = Gr[(long long)(v * 16 + p0 + q * dp) * P.gplane];
-          s += gl_w<T>(q) * (NV == 4 ? m * rcp(Gr[(long long)(p0 + q * dp) * P.gplane]) : m);
-        }
-        (f == 0 ? pxl : f == 1 ? pxr : f == 2 ? pyb : pyt) = s;
-      }
-    }
-  }
-  if (!FLAGGED) {
+  if (!FLAGGED && !FXD) {
     aux[0 * P.gplane + o] = pxl;
     aux[1 * P.gplane + o] = pxr;
     aux[2 * P.gplane + o] = pyb;
@@ -256,18 +264,11 @@ __device__ __forceinline__ void rec2d_cell(const Prob& P, const Weights<T>& W,
 }
 
 // rerec (REC_FLAGGED only, may be null) accumulates the number of cells
-// reconstructed a second time.
-// Double-float: 4 resident blocks per SM 5.41 ms per 2048^2 launch, 3 5.72, 5 5.79
-// (all in pairs: 7.6; 30 k instructions per cell, the ALU 45 % busy; its weights in
-// FP64 beside the integers measured alike, 5.6).  FP32 with
-// the float copy: 8 blocks (64 registers, 164 B of spills) measured 0.545 ms per
-// 2048^2 launch against 0.685 at 4 blocks (119 registers).  FP64: 5 blocks (96
-// registers, 20 spilled) 5.52 ms per 2048^2 launch, 4 blocks 5.71, 2 blocks 6.34;
-// the linear part in integers took it there from 18.1 ms (all in FP64): 696 FP64
-// operations per cell instead of 2330, the FP64 pipe 80 % busy beside 20 k
-// integer instructions per cell.
+// reconstructed a second time.  A thread per cell: FP32, plain double and the
+// scalar laws.  FP32 with the float copy: 8 blocks (64 registers, 164 B of spills)
+// measured 0.545 ms per 2048^2 launch against 0.685 at 4 blocks (119 registers).
 template <typename T, int NV, int MODE, bool FIX = false, bool S32 = false>
-__global__ void __launch_bounds__(RB, (is_df64<T>::value ? 4 : std::is_same<T, float>::value ? 8 : std::is_same<T, fx64>::value ? 5 : 1)) rec2d_kernel(
+__global__ void __launch_bounds__(RB, (std::is_same<T, float>::value ? 8 : fixed2d<T>::value ? 4 : 1)) rec2d_kernel(
     const __grid_constant__ Prob P, const __grid_constant__ Weights<T> W,
     const __grid_constant__ typename rows2d<T>::type B, const double* __restrict__ U,
                                                   const uint8_t* __restrict__ mask, const double* __restrict__ Mod,
@@ -283,6 +284,38 @@ __global__ void __launch_bounds__(RB, (is_df64<T>::value ? 4 : std::is_same<T, f
     const int cell = FLAGGED ? list[t] : (int)t;
     if (FIX && is_solid(P, cell % P.nx, cell / P.nx)) continue;   // solid cells are images, never read
     rec2d_cell<T, NV, MODE, FIX, S32>(P, W, B, U, mask, Mod, cell % P.nx, cell / P.nx, G, aux, U32);
+    if constexpr (fixed2d<T>::value && !FLAGGED) face_partials<T, NV>(P, G, aux, goff(P, cell % P.nx, cell / P.nx), 0, 4);
+  }
+}
+
+// 2D Euler in the fixed-point precisions: 32 cells a block, a warp per variable and
+// then per face, so that a thread's chain is a quarter of the cell's and the code
+// between the barriers is shared by the block.  Measured against a thread per cell
+// (ms per launch, FP64): 64^2 0.065 -> 0.021, 256^2 0.123 -> 0.105, 2048^2
+// 5.67 -> 5.52 (18.1 with the linear part in FP64), troubled cells 0.13 -> 0.11;
+// double-float 2048^2 5.44 -> 5.24 (7.6 in pairs).  FP64: 5 resident blocks per SM;
+// 690 FP64 operations per cell (2330 before), that pipe 80 % busy beside 20 k
+// integer instructions.  Double-float: 4 blocks, 30 k instructions per cell, the
+// ALU 45 % busy; weights in FP64 beside the integers measured alike.
+template <typename T, int MODE, bool FIX = false>
+__global__ void __launch_bounds__(RB, (is_df64<T>::value ? 4 : 5)) rec2d_split_kernel(
+    const __grid_constant__ Prob P, const __grid_constant__ Weights<T> W,
+    const __grid_constant__ typename rows2d<T>::type B, const double* __restrict__ U,
+    const uint8_t* __restrict__ mask, const double* __restrict__ Mod, const int* __restrict__ list,
+    const int* __restrict__ count, T* __restrict__ G, T* __restrict__ aux, unsigned long long* __restrict__ rerec) {
+  constexpr bool FLAGGED = MODE == REC_FLAGGED;
+  const int n = FLAGGED ? *count : P.nx * P.ny;
+  if (FLAGGED && rerec && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(rerec, (unsigned long long)n);
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int t0 = blockIdx.x * 32; t0 < n; t0 += gridDim.x * 32) {   // (block-uniform)
+    const int t = t0 + lane, cell = t < n ? (FLAGGED ? list[t] : t) : -1;
+    const int i = cell % P.nx, j = cell / P.nx;
+    const bool take = cell >= 0 && !(FIX && is_solid(P, i, j));
+    if (take) rec2d_cell<T, 4, MODE, FIX>(P, W, B, U, mask, Mod, i, j, G, aux, nullptr, w, w + 1);
+    if constexpr (!FLAGGED) {
+      __syncthreads();
+      if (take) face_partials<T, 4>(P, G, aux, goff(P, i, j), w, w + 1);
+    }
   }
 }
 
@@ -298,9 +331,7 @@ __device__ __forceinline__ bool flag2d_cell(const Prob& P, const double* __restr
   if (P.indicator == IND_ALL) return true;
   if (P.indicator == IND_TVB) return tvb_cell(P, U, i, j);
   if (P.indicator != IND_KXRCF) return false;
-  const T a = kxrcf2d<T>(P, G, aux, i, j);
-  if (aleph) aleph[(long long)j * P.nx + i] = double(a);
-  return a > T(1);
+  return kxrcf2d<T>(P, G, aux, i, j, aleph ? aleph + ((long long)j * P.nx + i) : nullptr);
 }
 
 // Step 2.2 for one troubled cell (dimension by dimension): modified first
@@ -315,8 +346,10 @@ __device__ __forceinline__ void modify2d_cell(const Prob& P, const double* __res
   // ghost has its state as average and zero first moments
   auto mom = [&](const Img& m, int v, int kind) -> double {
     if (m.fs >= 0) return kind == 0 ? fixed_val(P, m, v) : 0.0;
-    const int g = vsign(m, v) * (kind == 1 ? m.sx : kind == 2 ? m.sy : 1);
-    return g * U[sidx(P, v, kind, m.i, m.j)];
+    // the image's sign as a bit (a product with an integer sign is a conversion and
+    // a multiplication on the FP64 pipe: 70 % of this kernel's cycles in FP32)
+    const int neg = ((m.neg >> v) ^ ((kind == 1 ? m.sx : kind == 2 ? m.sy : 1) >> 31)) & 1;
+    return __longlong_as_double(__double_as_longlong(U[sidx(P, v, kind, m.i, m.j)]) ^ ((long long)neg << 63));
   };
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
@@ -374,9 +407,7 @@ __global__ void __launch_bounds__(RB) fallback2d_kernel(const __grid_constant__ 
     if (t < n) {
       cell = und[t];
       const int i = cell % P.nx, j = cell / P.nx;
-      const T a = kxrcf2d<T>(P, G, aux, i, j);
-      if (aleph) aleph[cell] = double(a);
-      flag = a > T(1);
+      flag = kxrcf2d<T>(P, G, aux, i, j, aleph ? aleph + cell : nullptr);
       mask[cell] = flag ? 1 : 0;
       if (flag) modify2d_cell<NV>(P, U, Mod, i, j);
     }
@@ -800,7 +831,7 @@ __global__ void __launch_bounds__(TX * TY, (std::is_same<T, float>::value ? 8 : 
     }
   }
   const int tid = threadIdx.y * TX + threadIdx.x;
-  if constexpr (lean<T>::value) {
+  if constexpr (!std::is_same<T, float>::value) {
 #pragma unroll 1
     for (int j0 = ja; j0 < jb; j0 += TY)
       update2d_tile<T, NV, TX, TY, SOLID>(P, GlobalSrc<T>{G}, S, i0, j0, tid, xf, yf, j0 > ja);
@@ -813,7 +844,7 @@ __global__ void __launch_bounds__(TX * TY, (std::is_same<T, float>::value ? 8 : 
 // most 16; small grids keep one, their blocks must reach every SM first.
 template <typename T>
 inline int update_sweep(const Prob& P) {
-  if (!lean<T>::value) return 1;
+  if (std::is_same<T, float>::value) return 1;
   const long long tiles = (long long)((P.nx + TX - 1) / TX) * ((P.ny + TY - 1) / TY);
   return (int)std::max<long long>(1, std::min<long long>(16, tiles / (6LL * P.nsm * 4)));
 }
@@ -923,13 +954,18 @@ void launch_rec2d(int blocks, cudaStream_t st, const Prob& P, const Weights<T>& 
       return;
     }
   }
-  if constexpr (NV == 4 && std::is_same<T, fx64>::value) {
-    if (P.fixtab || P.sol_j > 0) {
-      rec2d_kernel<T, NV, MODE, true><<<blocks, RB, 0, st>>>(P, W, Bt, U, mask, Mod, list, count, G, aux, rerec);
-      return;
+  if constexpr (NV == 4 && fixed2d<T>::value) {
+    const int sb = MODE == REC_FLAGGED ? blocks : (int)(((long long)P.nx * P.ny + 31) / 32);
+    if constexpr (std::is_same<T, fx64>::value && MODE != REC_MIXED) {
+      if (P.fixtab || P.sol_j > 0) {
+        rec2d_split_kernel<T, MODE, true><<<sb, RB, 0, st>>>(P, W, Bt, U, mask, Mod, list, count, G, aux, rerec);
+        return;
+      }
     }
+    rec2d_split_kernel<T, MODE><<<sb, RB, 0, st>>>(P, W, Bt, U, mask, Mod, list, count, G, aux, rerec);
+  } else {
+    rec2d_kernel<T, NV, MODE><<<blocks, RB, 0, st>>>(P, W, Bt, U, mask, Mod, list, count, G, aux, rerec);
   }
-  rec2d_kernel<T, NV, MODE><<<blocks, RB, 0, st>>>(P, W, Bt, U, mask, Mod, list, count, G, aux, rerec);
 }
 
 template <typename T, int NV>
@@ -969,8 +1005,8 @@ void stage_t(const Prob& P, const HostTabs& HT, const Weights<T>& W, const Beta2
       run_mlpre2d(P, B.mlp, B.mlp_conf, S.Uin, S.mask, S.Mod, B.und, ucnt, B.mlp_stats, B.mlp_prob, st);
       if (B.prof) B.prof->end(st);
       if (B.prof) B.prof->begin(0, st);
-      rec2d_kernel<T, NV, REC_MIXED><<<rblocks, RB, 0, st>>>(P, W, Bt, S.Uin, S.mask, S.Mod, nullptr, nullptr,
-                                                             (T*)B.G, (T*)B.aux, nullptr);
+      launch_rec2d<T, NV, REC_MIXED>(rblocks, st, P, W, Bt, S.Uin, S.mask, S.Mod, nullptr, nullptr, (T*)B.G,
+                                     (T*)B.aux, nullptr);
       if (B.prof) B.prof->end(st);
       if (B.prof) B.prof->begin(1, st);
       fallback2d_kernel<T, NV><<<fblocks, RB, 0, st>>>(P, S.Uin, (const T*)B.G, (const T*)B.aux, B.und, ucnt,
@@ -1089,14 +1125,29 @@ __device__ __forceinline__ double batch_dt(const BatchStage& A, const Prob& P, i
   return (r > 0.0 && isfinite(r)) ? A.cfl / r : 0.0;
 }
 
+// Quarters [q0, q1) of the item's 128 cells (fixed-point precisions: 32 cells at a
+// time, a warp per variable and then per face).
 template <typename T>
 __device__ __forceinline__ void batch_rec_item(const BatchStage& A, const Prob& P, const BProb& Q, int it, int tid,
-                                               const Weights<T>& W, const typename rows2d<T>::type& B) {
-  constexpr bool S32 = std::is_same<T, float>::value;
-  const int cell = (it - Q.rec_first) * RB + tid;
-  if (cell < P.nx * P.ny)
-    rec2d_cell<T, 4, REC_PLAIN, false, S32>(P, W, B, A.Uin + Q.uoff, nullptr, nullptr, cell % P.nx, cell / P.nx,
-                                            (T*)A.G + Q.goff, (T*)A.aux + Q.aoff, S32 ? A.U32in + Q.uoff : nullptr);
+                                               const Weights<T>& W, const typename rows2d<T>::type& B, int q0 = 0,
+                                               int q1 = 4) {
+  T* G = (T*)A.G + Q.goff;
+  T* aux = (T*)A.aux + Q.aoff;
+  if constexpr (fixed2d<T>::value) {
+    const int w = tid >> 5;
+    for (int q = q0; q < q1; ++q) {
+      const int cell = (it - Q.rec_first) * RB + q * 32 + (tid & 31), i = cell % P.nx, j = cell / P.nx;
+      if (cell < P.nx * P.ny)
+        rec2d_cell<T, 4, REC_PLAIN>(P, W, B, A.Uin + Q.uoff, nullptr, nullptr, i, j, G, aux, nullptr, w, w + 1);
+      __syncthreads();
+      if (cell < P.nx * P.ny) face_partials<T, 4>(P, G, aux, goff(P, i, j), w, w + 1);
+    }
+  } else {
+    const int cell = (it - Q.rec_first) * RB + tid;
+    if (cell < P.nx * P.ny)
+      rec2d_cell<T, 4, REC_PLAIN, false, true>(P, W, B, A.Uin + Q.uoff, nullptr, nullptr, cell % P.nx, cell / P.nx, G,
+                                               aux, A.U32in + Q.uoff);
+  }
 }
 
 template <typename T>
@@ -1117,9 +1168,11 @@ __device__ __forceinline__ void batch_flag_item(const BatchStage& A, const Prob&
 template <typename T>
 __device__ __forceinline__ void batch_rerec(const BatchStage& A, const Weights<T>& W,
                                             const typename rows2d<T>::type& B) {
-  constexpr bool S32 = std::is_same<T, float>::value;
+  constexpr bool S32 = std::is_same<T, float>::value, FXD = fixed2d<T>::value;
   const int n = *(volatile int*)A.count;
-  for (int t = blockIdx.x * RB + threadIdx.x; t < n; t += gridDim.x * RB) {
+  // a thread per cell, or (fixed-point precisions) a warp per variable of 32 cells
+  const int per = FXD ? 32 : RB, w = threadIdx.x >> 5;
+  for (int t = blockIdx.x * per + (FXD ? threadIdx.x & 31 : threadIdx.x); t < n; t += gridDim.x * per) {
     const unsigned long long e = A.list[t];
     const int p = (int)(e >> 32), cell = (int)(e & 0xffffffffu);
     // after a barrier wait that gave up, an entry may not be written yet
@@ -1127,7 +1180,7 @@ __device__ __forceinline__ void batch_rerec(const BatchStage& A, const Weights<T
     const BProb& Q = A.probs[p];
     rec2d_cell<T, 4, REC_FLAGGED, false, S32>(Q.P, W, B, A.Uin + Q.uoff, A.mask + Q.coff, A.Mod + Q.moff,
                                               cell % Q.P.nx, cell / Q.P.nx, (T*)A.G + Q.goff, nullptr,
-                                              S32 ? A.U32in + Q.uoff : nullptr);
+                                              S32 ? A.U32in + Q.uoff : nullptr, FXD ? w : 0, FXD ? w + 1 : 4);
   }
 }
 
@@ -1182,10 +1235,10 @@ __global__ void __launch_bounds__(RB, (is_df64<T>::value ? 4 : std::is_same<T, f
     batch_rec_kernel(const __grid_constant__ BatchStage A, const __grid_constant__ Weights<T> W,
                      const __grid_constant__ typename rows2d<T>::type B) {
   __shared__ Prob sp;
-  const int it = blockIdx.x;
+  const int it = fixed2d<T>::value ? blockIdx.x >> 2 : blockIdx.x, q = blockIdx.x & 3;
   const BProb& Q = A.probs[A.rec_owner[it]];
   stage_prob(Q, &sp, threadIdx.x);
-  batch_rec_item<T>(A, sp, Q, it, threadIdx.x, W, B);
+  batch_rec_item<T>(A, sp, Q, it, threadIdx.x, W, B, q, q + 1);
 }
 
 template <typename T>
@@ -1277,7 +1330,7 @@ cudaError_t launch_batch(const Weights<T>& W, const typename rows2d<T>::type& Bt
       }
       batch_dt_kernel<<<(S.nprob + 127) / 128, 128, 0, st>>>(S);
     }
-    batch_rec_kernel<T><<<S.n_rec, RB, 0, st>>>(S, W, Bt);
+    batch_rec_kernel<T><<<fixed2d<T>::value ? 4 * S.n_rec : S.n_rec, RB, 0, st>>>(S, W, Bt);
     batch_flag_kernel<T><<<S.n_rec, RB, 0, st>>>(S);
     batch_rerec_kernel<T><<<nsm * 8, RB, 0, st>>>(S, W, Bt);
     batch_update_kernel<T, TXV, TYV><<<S.n_upd, RB, 0, st>>>(S);

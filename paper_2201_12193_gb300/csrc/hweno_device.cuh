@@ -940,11 +940,12 @@ __device__ __forceinline__ int mpt(const Img& m, int k, int l) {
 
 __device__ __forceinline__ long long goff(const Prob& P, int i, int j) { return (long long)j * P.gpitch + i; }
 
-// KXRCF value of eq. (KXRCF_) with eq. (line-integral-average_): inflow faces by
+// KXRCF decision (and, where asked for, the value) of eq. (KXRCF_) with eq. (line-integral-average_): inflow faces by
 // the sign of the GL-weighted face velocity (average of both sides), jumps of
 // the indicator variable (variable 0) weighted by dy w_l or dx w_k.
 template <typename T>
-__device__ __forceinline__ T kxrcf2d(const Prob& P, const T* __restrict__ G, const T* __restrict__ aux, int i, int j) {
+__device__ __forceinline__ bool kxrcf2d(const Prob& P, const T* __restrict__ G, const T* __restrict__ aux, int i, int j,
+                                        double* __restrict__ aleph) {
   const long long o = goff(P, i, j);
   const Img L = image(P, i - 1, j, i, j), R = image(P, i + 1, j, i, j), Bo = image(P, i, j - 1, i, j),
             Tp = image(P, i, j + 1, i, j);
@@ -955,10 +956,6 @@ __device__ __forceinline__ T kxrcf2d(const Prob& P, const T* __restrict__ G, con
   const T axr = R.fs >= 0 ? from_double<T>(P.fixtab[4 * R.fs + 1] / P.fixtab[4 * R.fs]) : aux[(R.sx < 0 ? 1 : 0) * P.gplane + oR];
   const T ayb = Bo.fs >= 0 ? from_double<T>(P.fixtab[4 * Bo.fs + 2] / P.fixtab[4 * Bo.fs]) : aux[(Bo.sy < 0 ? 2 : 3) * P.gplane + oB];
   const T ayt = Tp.fs >= 0 ? from_double<T>(P.fixtab[4 * Tp.fs + 2] / P.fixtab[4 * Tp.fs]) : aux[(Tp.sy < 0 ? 3 : 2) * P.gplane + oT];
-  const T vxl = T(0.5) * ((L.neg & 2 ? -axl : axl) + aux[0 * P.gplane + o]);
-  const T vxr = T(0.5) * (aux[1 * P.gplane + o] + (R.neg & 2 ? -axr : axr));
-  const T vyb = T(0.5) * ((Bo.neg & 4 ? -ayb : ayb) + aux[2 * P.gplane + o]);
-  const T vyt = T(0.5) * (aux[3 * P.gplane + o] + (Tp.neg & 4 ? -ayt : ayt));
   // the indicator variable (density) of a neighbour at its point (k, l)
   auto rho_at = [&](const Img& m, long long om, int k, int l) -> T {
     return m.fs >= 0 ? from_double<T>(P.fixtab[4 * m.fs]) : G[(long long)mpt(m, k, l) * P.gplane + om];
@@ -968,6 +965,38 @@ __device__ __forceinline__ T kxrcf2d(const Prob& P, const T* __restrict__ G, con
   // a face shared with a solid cell (the forward step's block) is a wall, never an inflow face
   const bool wl = P.sol_j > 0 && is_solid(P, i - 1, j), wr = P.sol_j > 0 && is_solid(P, i + 1, j);
   const bool wb = P.sol_j > 0 && is_solid(P, i, j - 1), wt = P.sol_j > 0 && is_solid(P, i, j + 1);
+  const T nrm = aux[4 * P.gplane + o];
+  if constexpr (std::is_same<T, fx64>::value) {
+    // FP64: no halving, halves of the weights, division or compare on the FP64 pipe
+    // (about 50 operations against 90)
+    auto inflow = [](fx64 a, fx64 b) {               // (a + b) / 2 > KX_VDEAD (positive doubles order like
+      const long long x = __double_as_longlong(a.v + b.v);   //    their bits; not a NaN)
+      return x > __double_as_longlong(2.0 * KX_VDEAD) && x < 0x7FF0000000000000LL;
+    };
+    const bool il = inflow(L.neg & 2 ? -axl : axl, aux[0 * P.gplane + o]) && !wl;
+    const bool ir = inflow(-aux[1 * P.gplane + o], R.neg & 2 ? axr : -axr) && !wr;
+    const bool ib = inflow(Bo.neg & 4 ? -ayb : ayb, aux[2 * P.gplane + o]) && !wb;
+    const bool it = inflow(-aux[3 * P.gplane + o], Tp.neg & 4 ? ayt : -ayt) && !wt;
+    auto jump = [&](int p0, int dp, const Img& m, long long om, bool xd, int e) {
+      T q[4];
+#pragma unroll
+      for (int l = 0; l < 4; ++l)
+        q[l] = G[(long long)(p0 + l * dp) * P.gplane + o] - (xd ? rho_at(m, om, e, l) : rho_at(m, om, l, e));
+      return fma(T(5.0 / 12.0), addrn(q[1], q[2]), T(1.0 / 12.0) * addrn(q[0], q[3]));
+    };
+    if (il) { s = dy * jump(0, 1, L, oL, true, 3); len = dy; }
+    if (ir) { s = fma(dy, jump(12, 1, R, oR, true, 0), s); len += dy; }
+    if (ib) { s = fma(dx, jump(0, 4, Bo, oB, false, 3), s); len += dx; }
+    if (it) { s = fma(dx, jump(3, 4, Tp, oT, false, 0), s); len += dx; }
+    const T d = len * (pc<T>(P.cdx2) * nrm);
+    if (aleph) *aleph = d == T(0) ? 0.0 : double(tabs(s) / d);
+    const long long bs = __double_as_longlong(tabs(s).v), bd = __double_as_longlong(d.v);
+    return bs > bd && bd > 0 && bs <= 0x7FF0000000000000LL;
+  }
+  const T vxl = T(0.5) * ((L.neg & 2 ? -axl : axl) + aux[0 * P.gplane + o]);
+  const T vxr = T(0.5) * (aux[1 * P.gplane + o] + (R.neg & 2 ? -axr : axr));
+  const T vyb = T(0.5) * ((Bo.neg & 4 ? -ayb : ayb) + aux[2 * P.gplane + o]);
+  const T vyt = T(0.5) * (aux[3 * P.gplane + o] + (Tp.neg & 4 ? -ayt : ayt));
   if (vxl > T(KX_VDEAD) && !wl) {
 #pragma unroll
     for (int l = 0; l < 4; ++l) s += dy * gl_w<T>(l) * (G[(long long)(l)*P.gplane + o] - rho_at(L, oL, 3, l));
@@ -988,9 +1017,9 @@ __device__ __forceinline__ T kxrcf2d(const Prob& P, const T* __restrict__ G, con
     for (int k = 0; k < 4; ++k) s += dx * gl_w<T>(k) * (G[(long long)(k * 4 + 3) * P.gplane + o] - rho_at(Tp, oT, k, 0));
     len += dx;
   }
-  const T nrm = aux[4 * P.gplane + o];
-  if (len == T(0) || nrm == T(0)) return T(0);
-  return tabs(s) / len / (pc<T>(P.cdx2) * nrm);   // h^{(l+1)/3}, l = 5, h = dx
+  const T a = len == T(0) || nrm == T(0) ? T(0) : tabs(s) / len / (pc<T>(P.cdx2) * nrm);   // h^{(l+1)/3}, l = 5, h = dx
+  if (aleph) *aleph = double(a);
+  return a > T(1);
 }
 
 // ---------------------------------------------------------------- step checks
