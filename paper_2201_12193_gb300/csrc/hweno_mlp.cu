@@ -141,14 +141,41 @@ struct WSmem {
   float b1[NH], b2[NH], w3[NH], b3;
 };
 
-__device__ void load_weights(const float* __restrict__ th, WSmem& S) {
-  for (int q = threadIdx.x; q < NH * S1; q += blockDim.x) {
-    const int o = q / S1, k = q % S1;
-    S.w1[q] = __float2bfloat16_rn(k < NIN ? th[OFF_W1 + o * NIN + k] : 0.0f);
+// Four consecutive floats, as one 16-byte load where the base allows it.
+__device__ __forceinline__ float4 load4(const float* __restrict__ p, bool vec) {
+  if (vec) return *reinterpret_cast<const float4*>(p);
+  return make_float4(p[0], p[1], p[2], p[3]);
+}
+__device__ __forceinline__ bool aligned16(const void* p) { return (reinterpret_cast<unsigned long long>(p) & 15) == 0; }
+
+// Four BF16 values to an even element of a row (4-byte aligned).
+__device__ __forceinline__ void store4(__nv_bfloat16* q, float4 v) {
+  reinterpret_cast<unsigned*>(q)[0] = pack_bf16(v.x, v.y);
+  reinterpret_cast<unsigned*>(q)[1] = pack_bf16(v.z, v.w);
+}
+
+// w2t: W2^T too (training), or null.  Rows of 27 (W1) and 16 (W2) quadruples; every
+// offset of the flat parameters is a multiple of 16 bytes.
+__device__ __forceinline__ void load_weights(const float* __restrict__ th, WSmem& S, __nv_bfloat16* w2t = nullptr) {
+  static_assert(NIN % 4 == 0 && OFF_W2 % 4 == 0, "quadruples");
+  const bool vec = aligned16(th);
+#pragma unroll 4
+  for (int q = threadIdx.x; q < NH * (NIN / 4); q += blockDim.x) {
+    const int o = q / (NIN / 4), k = q % (NIN / 4) * 4;
+    store4(S.w1 + o * S1 + k, load4(th + OFF_W1 + o * NIN + k, vec));
   }
-  for (int q = threadIdx.x; q < NH * S2; q += blockDim.x) {
-    const int o = q / S2, k = q % S2;
-    S.w2[q] = __float2bfloat16_rn(k < NH ? th[OFF_W2 + o * NH + k] : 0.0f);
+  for (int o = threadIdx.x; o < NH; o += blockDim.x) store4(S.w1 + o * S1 + NIN, make_float4(0.f, 0.f, 0.f, 0.f));
+#pragma unroll 4
+  for (int q = threadIdx.x; q < NH * (NH / 4); q += blockDim.x) {
+    const int o = q / (NH / 4), k = q % (NH / 4) * 4;
+    const float4 v = load4(th + OFF_W2 + o * NH + k, vec);
+    store4(S.w2 + o * S2 + k, v);
+    if (w2t) {
+      w2t[k * S2 + o] = __float2bfloat16_rn(v.x);
+      w2t[(k + 1) * S2 + o] = __float2bfloat16_rn(v.y);
+      w2t[(k + 2) * S2 + o] = __float2bfloat16_rn(v.z);
+      w2t[(k + 3) * S2 + o] = __float2bfloat16_rn(v.w);
+    }
   }
   for (int q = threadIdx.x; q < NH; q += blockDim.x) {
     S.b1[q] = th[OFF_B1 + q];
@@ -273,7 +300,7 @@ struct TSmem {
   __nv_bfloat16 h1t[NH * S2];     // h1^T
   __nv_bfloat16 da2t[NH * S2];    // (dL/da2)^T
   __nv_bfloat16 da1t[NH * S2];    // (dL/da1)^T
-  float gw1[NH * NINP];
+  alignas(16) float gw1[NH * NINP];   // (read and written in pairs)
   float gw2[NH * NH];
   // per-warp sums (one writer each), combined in warp order at the end
   float gb1[TT / 32][NH], gb2[TT / 32][NH], gw3[TT / 32][NH], gb3[TT / 32], loss[TT / 32];
@@ -292,26 +319,40 @@ __global__ void __launch_bounds__(TT) mlp_train_kernel(const float* __restrict__
                                                        int n, float inv_n, float* __restrict__ part) {
   extern __shared__ __align__(16) unsigned char smem[];
   TSmem& S = *reinterpret_cast<TSmem*>(smem);
-  load_weights(th, S.W);
-  for (int q = threadIdx.x; q < NH * S2; q += TT) {
-    const int o = q / S2, k = q % S2;
-    S.w2t[q] = __float2bfloat16_rn(k < NH ? th[OFF_W2 + k * NH + o] : 0.0f);
-  }
-  for (int q = threadIdx.x; q < NH * NINP; q += TT) S.gw1[q] = 0.f;
-  for (int q = threadIdx.x; q < NH * NH; q += TT) S.gw2[q] = 0.f;
+  // the block's first rows travel while the weights are staged: a thread holds one
+  // row's quadruples tid / 64, + 2, ... (consecutive lanes, consecutive rows: the
+  // stores to both layouts of the tile meet no bank conflict)
+  constexpr int NQ = (NIN / 4 + 1) / 2;
+  const bool vec = aligned16(X);
+  const int xr = threadIdx.x & (TR - 1), xk = threadIdx.x / TR;
+  float4 xq[NQ];
+  auto fetch = [&](int base) {
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) {
+      const int k = xk + 2 * i;
+      xq[i] = k < NIN / 4 && base + xr < n ? load4(X + (long long)(base + xr) * NIN + 4 * k, vec)
+                                           : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  };
+  fetch(blockIdx.x * TR);
+  load_weights(th, S.W, S.w2t);
   for (int q = threadIdx.x; q < (TT / 32) * NH; q += TT) {
     (&S.gb1[0][0])[q] = 0.f; (&S.gb2[0][0])[q] = 0.f; (&S.gw3[0][0])[q] = 0.f;
   }
   if (threadIdx.x < TT / 32) { S.gb3[threadIdx.x] = 0.f; S.loss[threadIdx.x] = 0.f; }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   for (int base = blockIdx.x * TR; base < n; base += gridDim.x * TR) {
+    const bool first = base == blockIdx.x * TR;
     __syncthreads();
-    for (int q = threadIdx.x; q < TR * NINP; q += TT) {
-      const int r = q / NINP, k = q % NINP;
-      const int row = base + r;
-      const __nv_bfloat16 v = __float2bfloat16_rn((row < n && k < NIN) ? X[(long long)row * NIN + k] : 0.0f);
-      S.xs[r * S1 + k] = v;
-      S.xt[k * S2 + r] = v;
+    if (!first) fetch(base);
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) {
+      const int k = 4 * (xk + 2 * i);             // (the quadruple past the row's end holds the padding zeros)
+      store4(S.xs + xr * S1 + k, xq[i]);
+      S.xt[k * S2 + xr] = __float2bfloat16_rn(xq[i].x);
+      S.xt[(k + 1) * S2 + xr] = __float2bfloat16_rn(xq[i].y);
+      S.xt[(k + 2) * S2 + xr] = __float2bfloat16_rn(xq[i].z);
+      S.xt[(k + 3) * S2 + xr] = __float2bfloat16_rn(xq[i].w);
     }
     __syncthreads();
     // ---- per warp: rows r0 .. r0+15 of the tile
@@ -429,10 +470,11 @@ __global__ void __launch_bounds__(TT) mlp_train_kernel(const float* __restrict__
 #pragma unroll
       for (int nb = 0; nb < 8; ++nb) {
         const int c = nb * 8 + 2 * t;
-        S.gw2[(o0 + g) * NH + c] += acc[nb][0];
-        S.gw2[(o0 + g) * NH + c + 1] += acc[nb][1];
-        S.gw2[(o0 + g + 8) * NH + c] += acc[nb][2];
-        S.gw2[(o0 + g + 8) * NH + c + 1] += acc[nb][3];
+        float2* ga = reinterpret_cast<float2*>(&S.gw2[(o0 + g) * NH + c]);
+        float2* gb = reinterpret_cast<float2*>(&S.gw2[(o0 + g + 8) * NH + c]);
+        const float2 z2 = make_float2(0.f, 0.f), a0 = first ? z2 : *ga, b0 = first ? z2 : *gb;
+        *ga = make_float2(a0.x + acc[nb][0], a0.y + acc[nb][1]);
+        *gb = make_float2(b0.x + acc[nb][2], b0.y + acc[nb][3]);
       }
       float acc1[14][4];
 #pragma unroll
@@ -453,10 +495,11 @@ __global__ void __launch_bounds__(TT) mlp_train_kernel(const float* __restrict__
 #pragma unroll
       for (int nb = 0; nb < 14; ++nb) {
         const int c = nb * 8 + 2 * t;
-        S.gw1[(o0 + g) * NINP + c] += acc1[nb][0];
-        S.gw1[(o0 + g) * NINP + c + 1] += acc1[nb][1];
-        S.gw1[(o0 + g + 8) * NINP + c] += acc1[nb][2];
-        S.gw1[(o0 + g + 8) * NINP + c + 1] += acc1[nb][3];
+        float2* ga = reinterpret_cast<float2*>(&S.gw1[(o0 + g) * NINP + c]);
+        float2* gb = reinterpret_cast<float2*>(&S.gw1[(o0 + g + 8) * NINP + c]);
+        const float2 z2 = make_float2(0.f, 0.f), a0 = first ? z2 : *ga, b0 = first ? z2 : *gb;
+        *ga = make_float2(a0.x + acc1[nb][0], a0.y + acc1[nb][1]);
+        *gb = make_float2(b0.x + acc1[nb][2], b0.y + acc1[nb][3]);
       }
     }
   }
@@ -489,6 +532,7 @@ __global__ void train_sum_kernel(const float* __restrict__ part, int nblocks, fl
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q > NPARAM) return;
   float s = 0.f;
+#pragma unroll 16
   for (int b = 0; b < nblocks; ++b) s += part[(long long)b * (NPARAM + 1) + q];
   if (q < NPARAM) grad[q] += s;
   else *loss += s;
@@ -636,7 +680,7 @@ cudaError_t run_mlp_train(const float* th, const float* X, const float* y, const
     cap = need;
   }
   mlp_train_kernel<<<blocks, TT, sm, st>>>(th, X, y, w, n, 1.0f / (float)n, part);
-  train_sum_kernel<<<(NPARAM + 1 + 255) / 256, 256, 0, st>>>(part, blocks, grad, loss);
+  train_sum_kernel<<<(NPARAM + 1 + 63) / 64, 64, 0, st>>>(part, blocks, grad, loss);
   return cudaGetLastError();
 }
 
