@@ -322,6 +322,17 @@ hweno_status check_status(hweno_t h) {
   return HWENO_OK;
 }
 
+// The CFL wave speeds of the current state in host_buf[0..1], and the status check:
+// one read and one wait for both, where two of each left the device idle between them
+// (a max_dt + step loop over 200 cells in 1D, 16 steps: 365 -> 310 us).  A bad status
+// takes check_status's path, and the speeds of that state are dropped.
+hweno_status read_speeds(hweno_t h) {
+  hw::run_wavespeed(h->P, h->U[h->cur], h->red_part, h->red_out, nullptr, nullptr, h->B.status, h->stream);
+  CK(h, cudaMemcpyAsync(h->host_buf, h->red_out, 3 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+  CK(h, cudaStreamSynchronize(h->stream));
+  return h->host_buf[2] != 0.0 || h->batch ? check_status(h) : HWENO_OK;
+}
+
 // every inflow side has its fixed states
 bool fix_ready(const hweno_s* h) {
   const int k[4] = {h->bc.xlo, h->bc.xhi, h->bc.ylo, h->bc.yhi};
@@ -646,11 +657,8 @@ hweno_status hweno_wave_speeds(hweno_t h, double* ax_ay) {
   if (!h || !ax_ay) return HWENO_EINVAL;
   if (h->batch) return fail(h, HWENO_ESTATE, "wave_speeds: single-problem handles only");
   if (!h->have_state) return fail(h, HWENO_ESTATE, "wave_speeds: no moments set");
-  hweno_status s = check_status(h);
+  const hweno_status s = read_speeds(h);
   if (s != HWENO_OK) return s;
-  hw::run_wavespeed(h->P, h->U[h->cur], h->red_part, h->red_out, nullptr, nullptr, nullptr, h->stream);
-  CK(h, cudaMemcpyAsync(h->host_buf, h->red_out, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-  CK(h, cudaStreamSynchronize(h->stream));
   ax_ay[0] = h->host_buf[0];
   ax_ay[1] = h->host_buf[1];
   return HWENO_OK;
@@ -767,11 +775,8 @@ hweno_status hweno_max_dt(hweno_t h, double cfl, double* dt_out) {
   if (!h || !dt_out) return HWENO_EINVAL;
   if (!h->have_state) return fail(h, HWENO_ESTATE, "max_dt: no moments set");
   if (!(cfl > 0.0)) return fail(h, HWENO_EINVAL, "max_dt: cfl must be positive");
-  hweno_status s = check_status(h);
+  const hweno_status s = read_speeds(h);
   if (s != HWENO_OK) return s;
-  hw::run_wavespeed(h->P, h->U[h->cur], h->red_part, h->red_out, nullptr, nullptr, nullptr, h->stream);
-  CK(h, cudaMemcpyAsync(h->host_buf, h->red_out, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-  CK(h, cudaStreamSynchronize(h->stream));
   const double ax = h->host_buf[0], ay = h->host_buf[1];
   if (!isfinite(ax) || !isfinite(ay)) return fail(h, HWENO_ENONPHYSICAL, "max_dt: non-physical cell average");
   double dt;

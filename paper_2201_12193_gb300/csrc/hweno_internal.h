@@ -182,7 +182,7 @@ cudaError_t run_batch_stage_df64(const HostTabs& T, int tile_variant, const Batc
 
 // Reductions over the cell averages (FP64): maximum wave speeds per direction
 // and totals sum(ubar) per variable.  partials needs reduce_partials_len(P)
-// doubles, zeroed once; out gets {ax, ay} or the nvar totals (unscaled sums).
+// doubles, zeroed once; out gets {ax, ay, status word} or the nvar totals (unscaled sums).
 // With par and st set (hweno_advance) the step length follows from {ax, ay}.
 int reduce_partials_len(const Prob& P);
 void run_wavespeed(const Prob& P, const double* U, double* partials, double* out, const double* par, double* st,

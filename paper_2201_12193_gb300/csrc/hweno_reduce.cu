@@ -87,7 +87,8 @@ __device__ __forceinline__ void speeds_of(const Prob& P, const double* __restric
 }
 
 // The last block to arrive (part[4 MAXB] counts them and returns to 0) reduces the
-// blocks' partials to out[0..1] and, with par set, forms hweno_advance's step
+// blocks' partials to out[0..1], copies the status word to out[2] (the host then reads
+// speeds and status at once) and, with par set, forms hweno_advance's step
 // length: one launch where the partials, their reduction and the step length took
 // three (each about 2 us of a small grid's step; a maximum is the same in any order).
 // FILTER (Euler, large grids): a block first takes the largest lower bound of its
@@ -159,6 +160,7 @@ __global__ void __launch_bounds__(NT) wavespeed_kernel(const __grid_constant__ P
   if (threadIdx.x == 0) {
     out[0] = w[0];
     out[1] = w[1];
+    out[2] = (double)*status;
     if (par) advance_dt(P, w[0], w[1], par, st, status);
   }
 }
