@@ -1,13 +1,15 @@
 // The compute precision of the FP64 forms: a double whose every operation is
 // FP64, as a type of its own because the functions that carry the work have
 // versions for it that GB300's scarce FP64 pipe needs (recon1d / recon2d in
-// block fixed point, rcp).  Plain double keeps the plain versions (all in FP64,
+// block fixed point, rcp and sqrt in integers).  Plain double keeps the plain versions (all in FP64,
 // IEEE reciprocals): the learned indicator's stages use it.  Its network
 // decides by a threshold on BF16-rounded features, which are noise-sized
 // wherever the data hardly vary, so a last-bit change of the point values
 // moves decisions (measured with fx64 there: one to three cells of 1024^2
 // change sides per step on blast data).
 #pragma once
+
+#include "fx64_roots.h"
 
 namespace hw {
 
@@ -32,19 +34,34 @@ __device__ __forceinline__ bool operator<=(fx64 a, fx64 b) { return a.v <= b.v; 
 __device__ __forceinline__ bool operator>=(fx64 a, fx64 b) { return a.v >= b.v; }
 __device__ __forceinline__ bool operator==(fx64 a, fx64 b) { return a.v == b.v; }
 __device__ __forceinline__ fx64 fma(fx64 a, fx64 b, fx64 c) { return ::fma(a.v, b.v, c.v); }
-// Square root: the hardware's approximation y of 1/sqrt(x) (2^-20) and one
-// third-order step of Householder's iteration on g = x y, g (1 + r/2 + 3/8 r^2)
-// with r = 1 - g y: within 0.75 units in the last place (half of g's rounding and
-// the last one), five FP64 operations where the IEEE root takes nine (measured
-// rates).  Zero gives zero, a negative argument NaN, infinity NaN.
+// Square root and reciprocal in integers (fx64_roots.h), where the FP64 steps held
+// the FP64 pipe for five and three operations.  At 2048^2: Step 3 8.0 -> 5.8 ms per
+// launch, the reconstruction 5.5 -> 5.1.  Root: zero gives zero; a negative
+// argument, a subnormal one, infinity and NaN give NaN.  Reciprocal: zero, a
+// subnormal argument, infinity and NaN give NaN; results below 2^-1022 become 0.
 __device__ __forceinline__ fx64 sqrt(fx64 a) {
-  const double x = a.v;
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double g = x * y;
-  const double r = ::fma(-g, y, 1.0);
-  const double s = ::fma(g, ::fma(r, 0.375, 0.5) * r, g);
-  return ((__double2hiint(x) << 1) | __double2loint(x)) == 0 ? x : s;
+  const unsigned h = (unsigned)__double2hiint(a.v), l = (unsigned)__double2loint(a.v);
+  const unsigned odd = ~(h >> 20) & 1u;              // the mantissa in [1, 4), the exponent left even
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(__uint_as_float(fxr::seed_bits(h, l) + (odd << 23))));
+  const unsigned mh = (h & 0xFFFFFu) | 0x100000u;
+  const unsigned long long s =
+      fxr::sqrt_mantissa(odd ? __funnelshift_l(l, mh, 1) : mh, l << odd,
+                         fxr::seed_fixed(__float_as_uint(__fadd_rz(y, fxr::ROOT_ONE)))) +
+      ((unsigned long long)((((h >> 20) + 1023u) >> 1) - 1u) << 52);
+  if (h - 0x00100000u < 0x7FE00000u) return __longlong_as_double((long long)s);
+  return ((h << 1) | l) == 0u ? a.v : __longlong_as_double(0x7FF8000000000000LL);
+}
+__device__ __forceinline__ fx64 reciprocal(fx64 a) {
+  const unsigned h = (unsigned)__double2hiint(a.v), l = (unsigned)__double2loint(a.v);
+  const unsigned e = (h >> 20) & 0x7FFu;
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(__uint_as_float(fxr::seed_bits(h, l))));
+  const unsigned long long s = fxr::rcp_mantissa((h & 0xFFFFFu) | 0x100000u, l,
+                                                 fxr::seed_fixed(__float_as_uint(__fadd_rz(y, fxr::RCP_ONE)))) +
+                               ((unsigned long long)((2044u - e) | ((h >> 20) & 0x800u)) << 52);
+  if (e - 1u < 2044u) return __longlong_as_double((long long)s);
+  return e == 0x7FFu || e == 0u ? __longlong_as_double(0x7FF8000000000000LL) : 0.0;
 }
 
 // Comparisons and halving by integer work: an FP64 compare takes the FP64 pipe's

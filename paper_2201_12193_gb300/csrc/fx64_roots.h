@@ -1,0 +1,78 @@
+// Reciprocal and square root of a double in 32-bit integer steps, for fx64.
+//
+// An FP64 instruction holds a scheduler's FP64 pipe for 64 clocks, an integer
+// one for 1 or 2, so a Newton correction of three to five FP64 operations (192
+// to 320 clocks) costs more than the same correction in some 35 to 50 integer
+// instructions.  Both start from the FP32 approximation of the mantissa's
+// reciprocal (or reciprocal root), lowered so that it lies below the true
+// value (the residual is then never negative), and add the first terms of the
+// binomial series of the residual (Householder's iteration):
+//   1/m     = y (1 + e + e^2 + ...),              e = 1 - m y   < 2^-19.8
+//   sqrt(m) = m y (1 + r/2 + 3/8 r^2 + ...),      r = 1 - m y^2 < 2^-19
+// The residual comes from the low words of a product whose high words cancel.
+// What the series leaves out is below 2^-58 relative, the truncations of the
+// fixed point below 2^-59; the result is rounded to 53 bits once, to within 0.52
+// units in the last place (the FP64 steps had 0.75).  Plain C++: also compiled
+// for the host.
+#pragma once
+
+#include <stdint.h>
+
+#ifdef __CUDACC__
+#define FXR_HD __host__ __device__ __forceinline__
+#else
+#define FXR_HD inline
+#endif
+
+namespace fxr {
+
+FXR_HD uint64_t wide(uint32_t a, uint32_t b) { return (uint64_t)a * b; }
+
+// The 32-bit halves (through an empty asm on the device: products of halves the
+// compiler recognises are multiplied as 64 x 64 bits).
+FXR_HD void split(uint64_t x, uint32_t& h, uint32_t& l) {
+  h = (uint32_t)(x >> 32);
+  l = (uint32_t)x;
+#ifdef __CUDA_ARCH__
+  asm("" : "+r"(h), "+r"(l));
+#endif
+}
+
+// The leading 24 bits of the mantissa of a double (high word h, low word l) as the bits of a float in [1, 2).
+FXR_HD uint32_t seed_bits(uint32_t h, uint32_t l) { return (((h << 3) | (l >> 29)) & 0x7FFFFFu) | 0x3F800000u; }
+
+// y - D 2^-24 in units of 2^-23 from the bits of 1 - D 2^-24 + y (rounded towards zero), 0.49 < y < 1.0000003
+FXR_HD uint32_t seed_fixed(uint32_t bits_1py) { return bits_1py & 0x7FFFFFu; }
+constexpr float RCP_ONE = 1.0f - 5.0f / 16777216.0f;    // D = 5: the approximation's 2^-23 and the mantissa's truncation
+constexpr float ROOT_ONE = 1.0f - 4.0f / 16777216.0f;   // D = 4: 2^-22.9 and half the truncation
+
+// 2^62 / m for the mantissa M = mh:ml (2^52 <= M < 2^53, m = M 2^-52) from y in
+// units of 2^-23: as the mantissa rounded to [2^52, 2^53] of 1/m = it / 2^53.
+FXR_HD uint64_t rcp_mantissa(uint32_t mh, uint32_t ml, uint32_t y) {
+  const uint64_t t = wide(ml, y) + ((uint64_t)(uint32_t)(mh * y) << 32);   // m y, units 2^-75, less 1
+  const uint64_t r = 0 - t;                                                // e
+  uint32_t rh, rl;
+  split(r, rh, rl);
+  const uint64_t e = r + (wide(rh, rh) >> 11);                             // e + e^2
+  split(e, rh, rl);
+  const uint64_t c = wide(y, rh) + (wide(y, rl) >> 32);                    // y (e + e^2), units 2^-66
+  return (((uint64_t)(y << 7) << 32) + (c >> 4) + 256) >> 9;
+}
+
+// sqrt(m) 2^52, rounded, for m = M 2^-52 in [1, 4) (M = mh:ml below 2^54) from y in units of 2^-23.
+FXR_HD uint64_t sqrt_mantissa(uint32_t mh, uint32_t ml, uint32_t y) {
+  uint32_t h, l;
+  split(wide(y, y), h, l);                                                 // y^2, units 2^-46
+  const uint64_t s = (wide(ml, l) >> 32) + wide(ml, h) + wide(mh, l) + ((uint64_t)(uint32_t)(mh * h) << 32);
+  const uint64_t r = 0 - s;                                                // r, units 2^-66
+  const uint32_t q = (uint32_t)(r >> 24);
+  const uint64_t c = r + (wide(q, 3 * q) >> 20);                           // r/2 + 3/8 r^2, units 2^-67
+  const uint64_t g = wide(mh << 10, y << 9) + (wide(ml, y) >> 13);         // m y, units 2^-62
+  uint32_t gh, gl, ch, cl;
+  split(g, gh, gl);
+  split(c, ch, cl);
+  const uint64_t d = wide(gh, ch) + ((wide(gh, cl) + wide(gl, ch)) >> 32); // m y c, units 2^-65
+  return (g + (d >> 3) + 512) >> 10;
+}
+
+}  // namespace fxr

@@ -249,22 +249,12 @@ __device__ __forceinline__ double avg_img(const Prob& P, const double* __restric
 // ---------------------------------------------------------------- physics
 // Physical flux of eq. (1D-Euler) / (2D-Euler) or of the scalar laws in
 // direction dir (0 = x, 1 = y); NV = 1 (scalar), 3 (1D Euler), 4 (2D Euler).
-// 1/x.  FP32, double: correctly rounded.  fx64: the hardware's approximation y (2^-20) and
-// one third-order step of Householder's iteration, y (1 + e + e^2) with e = 1 - x y:
-// the truncation is e^3 (2^-60), the result within 0.5 + 2^-7 units in the last
-// place, and three FP64 operations where the IEEE reciprocal takes 5.4 (measured
-// rates; FP64 issues at 2 per clock and SM).  0 and infinity give NaN.
+// 1/x.  FP32, double: correctly rounded.  fx64: in integers, within 0.52 units in the
+// last place.
 template <typename T> __device__ __forceinline__ T rcp(T x) { return T(1) / x; }
 template <> __device__ __forceinline__ float rcp<float>(float x) { return __frcp_rn(x); }
 template <> __device__ __forceinline__ double rcp<double>(double x) { return __drcp_rn(x); }
-template <> __device__ __forceinline__ fx64 rcp<fx64>(fx64 a) {
-  const double x = a.v;
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  double e = fma(-x, y, 1.0);
-  e = fma(e, e, e);
-  return fma(y, e, y);
-}
+template <> __device__ __forceinline__ fx64 rcp<fx64>(fx64 x) { return reciprocal(x); }
 
 __device__ __forceinline__ double rcp64(double x) { return rcp<fx64>(x).v; }
 

@@ -1,0 +1,75 @@
+"""Host check of the integer reciprocal and square root of the FP64 forms.
+
+The hardware's starting values may be off by its stated error either way; the
+results have to be within 0.52 units in the last place for every start allowed,
+and exact where the true value is representable.
+"""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(__file__), "..", "paper_2201_12193_gb300", "csrc")
+
+SOURCE = r"""
+#include "fx64_roots.h"
+#include <cmath>
+#include <cstdio>
+#include <cstring>
+#include <random>
+static uint32_t bits(float f) { uint32_t b; memcpy(&b, &f, 4); return b; }
+static float flt(uint32_t b) { float f; memcpy(&f, &b, 4); return f; }
+static uint32_t seed(float y, float one) {          // the sum rounded towards zero
+  const double s = (double)y + one;
+  float f = (float)s;
+  if (f > s) f = nextafterf(f, -1.0f);
+  return fxr::seed_fixed(bits(f));
+}
+// units of the last place from n / 2^52 to sqrt(m / 2^52), m < 2^54
+static double root_error(uint64_t n, uint64_t m) {
+  const __int128 d = (__int128)m * ((__int128)1 << 52) - (__int128)n * n;
+  return std::fabs((double)d / (2.0 * (double)n));
+}
+int main() {
+  std::mt19937_64 g(7);
+  double er = 0, es = 0;
+  for (long k = 0; k < 600000; ++k) {
+    uint64_t M = (1ull << 52) | (g() >> 12);
+    if (k < 300) M = (1ull << 52) + k / 3;                                   // just above 1
+    else if (k < 600) M = (1ull << 53) - 1 - (k - 300) / 3;                  // just below 2
+    else if (k % 4 == 1) M &= ~((1ull << (g() % 53)) - 1);                   // few bits
+    else if (k % 4 == 2) M |= (1ull << (g() % 52)) - 1;
+    const double p = k % 3 - 1;                                              // the start's error: least, none, most
+    const uint32_t h = M >> 32, l = (uint32_t)M, sb = fxr::seed_bits(h, l);
+    const float m = flt(sb);
+    const uint64_t q = fxr::rcp_mantissa(h, l, seed((float)((1.0 / m) * (1 + p * std::ldexp(1.0, -23))), fxr::RCP_ONE));
+    // q / 2^53 against 2^52 / M: (2^105 - q M) / M
+    const __int128 d = ((__int128)1 << 105) - (__int128)q * M;
+    er = std::fmax(er, std::fabs((double)d / (double)M));
+    if ((M & (M - 1)) == 0 && q != 1ull << 53) { printf("2^k\n"); return 1; }
+    for (int odd = 0; odd < 2; ++odd) {
+      const uint64_t N = M << odd;
+      const float z = flt(sb + ((uint32_t)odd << 23));
+      const float y = (float)((1.0 / std::sqrt((double)z)) * (1 + p * std::exp2(-22.9)));
+      es = std::fmax(es, root_error(fxr::sqrt_mantissa(N >> 32, (uint32_t)N, seed(y, fxr::ROOT_ONE)), N));
+    }
+    const uint64_t a = (1u << 26) + g() % (1u << 26);                        // a square: a^2, a < 2^27
+    const uint64_t S = a * a;                                                // m = S / 2^52 in [1, 4)
+    const float sf = flt(bits((float)1.0f) + (uint32_t)((S >> 53) << 23) | (uint32_t)((S << (S >> 53 ? 11 : 12)) >> 41));
+    const uint64_t r = fxr::sqrt_mantissa(S >> 32, (uint32_t)S, seed((float)(1.0 / std::sqrt((double)sf)), fxr::ROOT_ONE));
+    if (r != a << 26) { printf("square %llu\n", (unsigned long long)a); return 1; }
+  }
+  printf("%.4f %.4f\n", er, es);
+  return er <= 0.52 && es <= 0.52 ? 0 : 1;
+}
+"""
+
+
+@pytest.mark.skipif(shutil.which("g++") is None, reason="needs g++")
+def test_reciprocal_and_root_within_half_a_unit(tmp_path):
+    src = tmp_path / "roots.cpp"
+    src.write_text(SOURCE)
+    subprocess.check_call(["g++", "-O2", "-I", CSRC, "-o", str(tmp_path / "roots"), str(src)])
+    out = subprocess.run([str(tmp_path / "roots")], capture_output=True, text=True)
+    assert out.returncode == 0, out.stdout
