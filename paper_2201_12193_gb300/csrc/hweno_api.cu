@@ -5,6 +5,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <initializer_list>
 #include <string>
 
 #define HWP_HOST_TABLES
@@ -168,24 +169,29 @@ void build_tables(hweno_s* h) {
       if (outl) outl[k] = (double)v;
     }
   };
-  // FP64: the rows of a parity class in fixed point, the sum of each one's |coefficients|
-  // between 2^61.9 and 2^62.9 units; first[]: its rows of levels 2, 3, 4
-  auto fill_fx = [&](int (*first)(int), int nc, const double* rl, const double* rm, int2* out, int* f) {
-    for (int r = 0; r < first(3); ++r) {
-      coef(r < first(1) ? 2 : r < first(2) ? 3 : 4, a, b);
-      std::vector<long double> v(nc);
-      long double sum = 0.0L;
-      for (int k = 0; k < nc; ++k) {
-        v[k] = a * rl[r * nc + k] + b * rm[r * nc + k];
-        sum += fabsl(v[k]);
-      }
-      const int F = sum > 0.0L ? (int)floorl(62.9L - log2l(sum)) : 60;
-      f[r] = 60 - F;
-      for (int k = 0; k < nc; ++k) {
-        const long long c = llrintl(ldexpl(v[k], F));
-        const int lo = (int)(unsigned)(unsigned long long)c;
-        out[r * nc + k] = make_int2((int)((c - lo) >> 32), lo);
-      }
+  // FP64: the rows in fixed point, one unit 2^-F a level: the root of the sum of
+  // squares of its rows' |coefficient| sums lies between 2^61.9 and 2^62.9 units (f = 61 - F: the
+  // exponent of a row's value times 2^-61).  first[]: a class's rows of levels 2, 3, 4;
+  // times: its data sets (the odd class of 2D has two).
+  struct FxClass { int (*first)(int); int nc, times; const double *rl, *rm; int2* out; };
+  auto fill_fx = [&](std::initializer_list<FxClass> cls, int* f) {
+    for (int l = 0; l < 3; ++l) {
+      coef(l + 2, a, b);
+      long double sq = 0.0L;
+      for (const FxClass& c : cls)
+        for (int r = c.first(l); r < c.first(l + 1); ++r) {
+          long double sum = 0.0L;
+          for (int k = 0; k < c.nc; ++k) sum += fabsl(a * c.rl[r * c.nc + k] + b * c.rm[r * c.nc + k]);
+          sq += c.times * sum * sum;
+        }
+      const int F = sq > 0.0L ? (int)floorl(62.9L - 0.5L * log2l(sq)) : 60;
+      f[l] = 61 - F;
+      for (const FxClass& c : cls)
+        for (int q = c.first(l) * c.nc; q < c.first(l + 1) * c.nc; ++q) {
+          const long long x = llrintl(ldexpl(a * c.rl[q] + b * c.rm[q], F));
+          const int lo = (int)(unsigned)(unsigned long long)x;
+          c.out[q] = make_int2((int)((x - lo) >> 32), lo);
+        }
     }
   };
   if (h->g.dim == 1) {
@@ -193,16 +199,16 @@ void build_tables(hweno_s* h) {
     fill(3, hwp::D1P_RC3_3, hwp::D1P_RC3_2, hwp::D1_NB3, h->T.b1f.B3, h->T.b1x.B3, nullptr);
     fill(4, hwp::D1P_RC4_4, hwp::D1P_RC4_3, hwp::D1_NB4, h->T.b1f.B4, h->T.b1x.B4, nullptr);
     auto& B = h->T.b1d;
-    fill_fx(hwp::D1_RA, hwp::D1_NCA, &hwp::D1P_AL[0][0], &hwp::D1P_AM[0][0], &B.a[0][0], B.fa);
-    fill_fx(hwp::D1_RB, hwp::D1_NCB, &hwp::D1P_BL[0][0], &hwp::D1P_BM[0][0], &B.b[0][0], B.fb);
+    fill_fx({{hwp::D1_RA, hwp::D1_NCA, 1, &hwp::D1P_AL[0][0], &hwp::D1P_AM[0][0], &B.a[0][0]},
+             {hwp::D1_RB, hwp::D1_NCB, 1, &hwp::D1P_BL[0][0], &hwp::D1P_BM[0][0], &B.b[0][0]}}, B.f);
   } else {
     fill(2, hwp::D2P_RC2_2, nullptr, hwp::D2_NB2, h->T.b2f.B2, h->T.b2x.B2, h->T.b2l.B2);
     fill(3, hwp::D2P_RC3_3, hwp::D2P_RC3_2, hwp::D2_NB3, h->T.b2f.B3, h->T.b2x.B3, h->T.b2l.B3);
     fill(4, hwp::D2P_RC4_4, hwp::D2P_RC4_3, hwp::D2_NB4, h->T.b2f.B4, h->T.b2x.B4, h->T.b2l.B4);
     auto& B = h->T.b2d;
-    fill_fx(hwp::D2_RA, hwp::D2_NCA, &hwp::D2P_AL[0][0], &hwp::D2P_AM[0][0], &B.a[0][0], B.fa);
-    fill_fx(hwp::D2_RB, hwp::D2_NCB, &hwp::D2P_BL[0][0], &hwp::D2P_BM[0][0], &B.b[0][0], B.fb);
-    fill_fx(hwp::D2_RE, hwp::D2_NCE, &hwp::D2P_EL[0][0], &hwp::D2P_EM[0][0], &B.e[0][0], B.fe);
+    fill_fx({{hwp::D2_RA, hwp::D2_NCA, 1, &hwp::D2P_AL[0][0], &hwp::D2P_AM[0][0], &B.a[0][0]},
+             {hwp::D2_RB, hwp::D2_NCB, 2, &hwp::D2P_BL[0][0], &hwp::D2P_BM[0][0], &B.b[0][0]},
+             {hwp::D2_RE, hwp::D2_NCE, 1, &hwp::D2P_EL[0][0], &hwp::D2P_EM[0][0], &B.e[0][0]}}, B.f);
   }
 }
 

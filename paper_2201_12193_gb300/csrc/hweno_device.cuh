@@ -111,7 +111,7 @@ template <typename T> struct Beta2 { T B2[hwp::D2_NB2]; T B3[hwp::D2_NB3]; T B4[
 template <int RA, int CA, int RB, int CB, int RE, int CE>
 struct FxRows {
   int2 a[RA][CA], b[RB][CB], e[RE][CE];
-  int fa[RA], fb[RB], fe[RE];
+  int f[3];           // the unit of a level's rows is 2^f
 };
 template <> struct Beta1<fx64> : FxRows<hwp::D1_NRA, hwp::D1_NCA, hwp::D1_NRB, hwp::D1_NCB, 1, 1> {};
 template <> struct Beta2<fx64>
@@ -590,13 +590,22 @@ template <> __device__ __forceinline__ df64 from_fixed<df64>(long long x, int eb
   return df64(r.x, r.y);
 }
 
-// sum_k c[k] s[k] of a beta row: the row's units are 2^ef.
-template <typename T, int N>
-__device__ __forceinline__ T fx_row(const hwfx::Half2 (&s)[N], const int2 (&c)[N], int ef) {
+template <typename T> __device__ __forceinline__ T from_squares(const hwfx::Squares& s, int e);
+template <> __device__ __forceinline__ fx64 from_squares<fx64>(const hwfx::Squares& s, int e) { return hwfx::sum_of(s, e); }
+template <> __device__ __forceinline__ df64 from_squares<df64>(const hwfx::Squares& s, int e) {
+  const float2 r = hwfx::sum_of_pair(s, e);
+  return df64(r.x, r.y);
+}
+
+// Adds (sum_k c[k] s[k])^2 of a beta row.  The class data are sums of up to four
+// 57-bit data, the level's coefficients below 2^62.9 (root of the sum of squares of the
+// rows' sums): with 2^-61 of the product the squares sum below 2^122.
+template <int N>
+__device__ __forceinline__ void fx_row(const hwfx::Half2 (&s)[N], const int2 (&c)[N], hwfx::Squares& q) {
   hwfx::Acc t = hwfx::prod(s[0], c[0].x, c[0].y);
 #pragma unroll
   for (int k = 1; k < N; ++k) hwfx::mac(t, s[k], c[k].x, c[k].y);
-  return from_fixed<T>(hwfx::scaled<60>(t), ef);
+  hwfx::add_square(q, hwfx::scaled<61>(t));
 }
 
 // The weights c_2, c_3, c_4, c_2 + c_3 as fixed-point integers of one exponent;
@@ -640,12 +649,12 @@ __device__ __forceinline__ void recon1d_fp64(const Weights<fx64>& W, const Beta1
   const int e0 = e - (1022 + hwfx::BITS);
 #pragma unroll
   for (int l = 0; l < 3; ++l) {
-    fx64 bl = 0.0;
+    hwfx::Squares bl{0, 0, 0};
 #pragma unroll
-    for (int r = hwp::D1_RA(l); r < hwp::D1_RA(l + 1); ++r) { const fx64 x = fx_row<fx64>(sa, B.a[r], e0 + B.fa[r]); bl = fma(x, x, bl); }
+    for (int r = hwp::D1_RA(l); r < hwp::D1_RA(l + 1); ++r) fx_row(sa, B.a[r], bl);
 #pragma unroll
-    for (int r = hwp::D1_RB(l); r < hwp::D1_RB(l + 1); ++r) { const fx64 x = fx_row<fx64>(sb, B.b[r], e0 + B.fb[r]); bl = fma(x, x, bl); }
-    beta[l + 1] = bl;
+    for (int r = hwp::D1_RB(l); r < hwp::D1_RB(l + 1); ++r) fx_row(sb, B.b[r], bl);
+    beta[l + 1] = from_squares<fx64>(bl, 2 * (e0 + B.f[l]));
   }
   // beta_1: eqs. (beta1-LR), (tau1), (w1_-LR), (w1-LR), (beta1) over a common denominator
   {
@@ -766,16 +775,17 @@ __device__ __forceinline__ void recon2d_fx(const Weights<T>& W, const Beta2<fx64
       const int na = l == 0 ? hwp::D2_RA(1) : l == 1 ? hwp::D2_RA(2) : hwp::D2_RA(3);
       const int nb = l == 0 ? hwp::D2_RB(1) : l == 1 ? hwp::D2_RB(2) : hwp::D2_RB(3);
       const int ne = l == 0 ? hwp::D2_RE(1) : l == 1 ? hwp::D2_RE(2) : hwp::D2_RE(3);
-      T bl = T(0);
+      hwfx::Squares q{0, 0, 0};
 #pragma unroll 1
-      for (; ra < na; ++ra) { const T x = fx_row<T>(sa, B.a[ra], e0 + B.fa[ra]); bl = fma(x, x, bl); }
+      for (; ra < na; ++ra) fx_row(sa, B.a[ra], q);
 #pragma unroll 1
       for (; rb < nb; ++rb) {   // the same rows for both odd classes (x <-> y images)
-        const T x = fx_row<T>(sb, B.b[rb], e0 + B.fb[rb]), y = fx_row<T>(sc, B.b[rb], e0 + B.fb[rb]);
-        bl = fma(x, x, fma(y, y, bl));
+        fx_row(sb, B.b[rb], q);
+        fx_row(sc, B.b[rb], q);
       }
 #pragma unroll 1
-      for (; re < ne; ++re) { const T x = fx_row<T>(se, B.e[re], e0 + B.fe[re]); bl = fma(x, x, bl); }
+      for (; re < ne; ++re) fx_row(se, B.e[re], q);
+      const T bl = from_squares<T>(q, 2 * (e0 + B.f[l]));
       if (l == 0) beta[1] = bl; else if (l == 1) beta[2] = bl; else beta[3] = bl;
     }
   }

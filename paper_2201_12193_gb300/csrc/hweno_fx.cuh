@@ -67,6 +67,40 @@ __device__ __forceinline__ long long to_fx(double x, int e) {
   return ((long long)m ^ s) - s;
 }
 
+// A sum of squares, exact: x = h 2^30 + l with |l| <= 2^29, |x| < 2^61; the sum
+// below 2^122 and at most 32 terms.  A square is four additions and shifts and
+// three multiply-adds; in FP64 it took a conversion to double (15 instructions)
+// and one FP64 operation, which holds its pipe for 64 clocks.
+struct Squares { long long hh, hl, ll; };
+
+__device__ __forceinline__ void add_square(Squares& s, long long x) {
+  int h = (int)((x + (1LL << 29)) >> 30), l = (int)((unsigned)x - ((unsigned)h << 30));
+  asm("" : "+r"(h), "+r"(l));
+  s.hh += (long long)h * h;
+  s.hl += (long long)h * l;
+  s.ll += (long long)l * l;
+}
+// The sum's leading 64 bits; their unit is 2^k.
+__device__ __forceinline__ unsigned long long leading(const Squares& s, int& k) {
+  const unsigned __int128 t = ((unsigned __int128)(__int128)s.hh << 60) + ((unsigned __int128)(__int128)s.hl << 31) +
+                              (unsigned long long)s.ll;
+  unsigned long long hi = (unsigned long long)(t >> 64), lo = (unsigned long long)t;
+  const bool one = hi == 0;
+  if (one) { hi = lo; lo = 0; }
+  const int n = __clzll((long long)hi);
+  k = (one ? 0 : 64) - n;
+  return (hi << (n & 63)) | (n & 63 ? lo >> (64 - n) : 0ull);
+}
+// The sum times 2^e as a double; results below 2^-1022 become 0, above the range infinity.
+__device__ __forceinline__ double sum_of(const Squares& s, int e) {
+  int k;
+  const unsigned long long m = leading(s, k);
+  const int f = k + e + 1085;                        // the biased exponent less 1
+  const unsigned long long r = (((m >> 10) + 1) >> 1) + ((unsigned long long)(unsigned)f << 52);
+  if (m == 0 || f < 0) return 0.0;
+  return __longlong_as_double(f >= 2046 ? 0x7FF0000000000000LL : (long long)r);
+}
+
 // x 2^eb as a double (integer work; rounded to 53 bits, halves up).  The caller keeps the exponent in range.
 __device__ __forceinline__ double from_fx(long long x, int eb) {
   const long long s = x >> 63;
@@ -91,6 +125,14 @@ __device__ __forceinline__ float2 from_fx_pair(long long x, int eb) {
   const float unit = __uint_as_float((unsigned)max(fe - 54, 0) << 23);
   const float lo = __fmul_rn(__uint2float_rn((unsigned)(m >> 8)), unit);
   return make_float2(hi, __uint_as_float(__float_as_uint(lo) ^ sg));
+}
+
+// The sum of squares times 2^e as a pair; above FP32's range infinity.
+__device__ __forceinline__ float2 sum_of_pair(const Squares& s, int e) {
+  int k;
+  const unsigned long long m = leading(s, k);
+  if (k + e > 64) return make_float2(__int_as_float(0x7F800000), 0.0f);
+  return from_fx_pair((long long)(m >> 1), k + e + 1);
 }
 
 // A float in the units of to_fx<B> at biased (FP64) exponent e.
