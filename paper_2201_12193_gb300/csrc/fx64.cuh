@@ -64,6 +64,12 @@ __device__ __forceinline__ fx64 reciprocal(fx64 a) {
   return e == 0x7FFu || e == 0u ? __longlong_as_double(0x7FF8000000000000LL) : 0.0;
 }
 
+// a b in integers: the same bits as a * b where operands and result are normal.
+__device__ __forceinline__ fx64 product(fx64 a, fx64 b) {
+  return __longlong_as_double((long long)fxr::product((unsigned)__double2hiint(a.v), (unsigned)__double2loint(a.v),
+                                                      (unsigned)__double2hiint(b.v), (unsigned)__double2loint(b.v)));
+}
+
 // Comparisons and halving by integer work: an FP64 compare takes the FP64 pipe's
 // full issue slot.  NaN compares false; -0 counts as negative.
 __device__ __forceinline__ bool nonneg(fx64 a) { return (unsigned)__double2hiint(a.v) < 0x7FF00000u; }   // 0 <= a, finite

@@ -75,4 +75,29 @@ FXR_HD uint64_t sqrt_mantissa(uint32_t mh, uint32_t ml, uint32_t y) {
   return (g + (d >> 3) + 512) >> 10;
 }
 
+// a b for the doubles ah:al and bh:bl, rounded to nearest even as the FP64
+// product is, bit for bit, where operands and result are normal.  Subnormal
+// operands and results become 0, an infinite operand gives NaN.
+FXR_HD uint64_t product(uint32_t ah, uint32_t al, uint32_t bh, uint32_t bl) {
+  const uint32_t ea = (ah >> 20) & 0x7FFu, eb = (bh >> 20) & 0x7FFu, sg = (ah ^ bh) & 0x80000000u;
+  const uint32_t mh = (ah & 0xFFFFFu) | 0x100000u, nh = (bh & 0xFFFFFu) | 0x100000u;
+  uint32_t w0, w1, w2, w3, x;                        // the 106-bit product w3:w2:w1:w0
+  split(wide(al, bl), x, w0);
+  split(wide(mh, bl) + (wide(al, nh) + x), x, w1);
+  split(wide(mh, nh) + x, w3, w2);                   // w3:w2 in [2^40, 2^42)
+  const uint32_t n = w3 >> 9, k = 20u + n;           // the mantissa is the product times 2^-(32 + k)
+  uint32_t h = (w3 << (32u - k)) | (w2 >> k), l = (w2 << (32u - k)) | (w1 >> k);
+  const uint32_t rest = (w1 << (32u - k)) | (w0 != 0u ? 1u : 0u);
+  const uint64_t q = (((uint64_t)h << 32) | l) + (rest + (l & 1u) > 0x80000000u ? 1u : 0u);
+  const int e = (int)(ea + eb + n) - 1024;           // biased exponent less 1: a carry of the rounding raises it
+  split(q, h, l);
+  uint32_t rh = (h + ((uint32_t)e << 20)) | sg;
+  const uint32_t lo = ea < eb ? ea : eb, hi = ea < eb ? eb : ea;
+  if (lo == 0u || (uint32_t)e >= 2046u || hi == 0x7FFu) {
+    l = 0u;
+    rh = hi == 0x7FFu ? 0x7FF80000u : sg | (lo != 0u && e >= 2046 ? 0x7FF00000u : 0u);
+  }
+  return ((uint64_t)rh << 32) | l;
+}
+
 }  // namespace fxr

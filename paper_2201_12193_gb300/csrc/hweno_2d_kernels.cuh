@@ -435,7 +435,7 @@ __device__ __forceinline__ void gl_state(const Prob& P, const T* __restrict__ G,
 // directions: a y face is an x face with the two momentum components
 // exchanged (the HLLC expressions are the same, term for term); at a wall
 // face the star branch is taken.
-template <typename T, int NV>
+template <typename T, int NV, bool SOFT = true>
 __device__ __forceinline__ void face_flux(const Prob& P, T (&uL)[NV], T (&uR)[NV], bool xd, bool wall, T* out) {
   if constexpr (NV == 4) {
     if (!xd) {
@@ -444,7 +444,7 @@ __device__ __forceinline__ void face_flux(const Prob& P, T (&uL)[NV], T (&uR)[NV
       uR[1] = uR[2]; uR[2] = b;
     }
     T F[4];
-    if constexpr (lean<T>::value) hllc_lean<T, 4>(P, uL, uR, 0, F, wall);
+    if constexpr (lean<T>::value) hllc_lean<T, 4, SOFT>(P, uL, uR, 0, F, wall);
     else hllc<T, 4>(P, uL, uR, 0, F, wall);
     out[0] = F[0];
     out[1] = xd ? F[1] : F[2];
@@ -506,21 +506,17 @@ struct StagedSrc {
   }
 };
 
-// Quadrature, L(U) and the Runge-Kutta combination of one cell (2D Euler, the
-// lean precisions), from the integrals of its faces (slot 0 the mean, 1 the first
-// moment; xm left, xp right, ym below, yp above).  The 16 points fall into three
-// groups of one weight (corners 1, edges 5, centre 25, over 144), summed without
-// weights.  With the kinetic terms A = sum w m^2/rho and S = sum w (m^2 + n^2)/rho
-// the momentum fluxes need no pressure per point: sum w p = (gamma - 1)(E - S/2),
-// and the sums of m, n and E are the cell's averages (every q_l has them, and the
-// quadrature is exact for degree 5).
+// Quadrature of one cell (2D Euler, the lean precisions).  The 16 points fall into
+// three groups of one weight (corners 1, edges 5, centre 25, over 144), summed
+// without weights.  With the kinetic terms A = sum w m^2/rho and
+// S = sum w (m^2 + n^2)/rho the momentum fluxes need no pressure per point:
+// sum w p = (gamma - 1)(E - S/2), and the sums of m, n and E are the cell's averages
+// (every q_l has them, and the quadrature is exact for degree 5).
+template <typename T> struct Quad { T A, C, K, X, Y; };
+
 template <typename T, typename Src>
-__device__ __forceinline__ void update_cell_lean(const Prob& P, const Src& src, const Rk& S, int i, int j,
-                                                 const T (&xm)[4][4], const T (&xp)[4][4], const T (&ym)[4][4],
-                                                 const T (&yp)[4][4]) {
-  const long long so = (long long)j * P.pitch + i;
-  const long long cell = (long long)j * P.nx + i;
-  const T g = pc<T>(P.cgamma), gm1 = pc<T>(P.cgm1), kap = pc<T>(P.chg);
+__device__ __forceinline__ Quad<T> quad_lean(const Prob& P, const Src& src, int i, int j) {
+  const T kap = pc<T>(P.chg);
   T A, C, K, X, Y;
   A = C = K = X = Y = T(0);
 #pragma unroll
@@ -545,6 +541,21 @@ __device__ __forceinline__ void update_cell_lean(const Prob& P, const Src& src, 
         Y = fma(nu, H, Y);
       }
   }
+  return Quad<T>{A, C, K, X, Y};
+}
+
+// L(U) and the Runge-Kutta combination of variables [v0, v1) of one cell, from its
+// quadrature and the integrals of its faces (slot 0 the mean, 1 the first moment; xm
+// left, xp right, ym below, yp above).  The new averages go to newavg; returns
+// whether every new moment is finite.
+template <typename T, typename Src>
+__device__ __forceinline__ bool combine_lean(const Prob& P, const Src& src, const Rk& S, int i, int j, const Quad<T>& q,
+                                             const T (&xm)[4][4], const T (&xp)[4][4], const T (&ym)[4][4],
+                                             const T (&yp)[4][4], int v0, int v1, double* newavg) {
+  const long long so = (long long)j * P.pitch + i;
+  const long long cell = (long long)j * P.nx + i;
+  const T g = pc<T>(P.cgamma), gm1 = pc<T>(P.cgm1);
+  const T A = q.A, C = q.C, K = q.K, X = q.X, Y = q.Y;
   // (every product that meets a sum is a written fma: what the compiler would
   // contract could differ between the kernels that share this, which agree bit for bit)
   const T w = T(1.0 / 144.0);
@@ -558,11 +569,10 @@ __device__ __forceinline__ void update_cell_lean(const Prob& P, const Src& src, 
   const bool fk = S.mask[cell] != 0 && (P.persist || S.Lout);
   const bool fn = P.persist && S.maskN && S.maskN[cell] != 0;
   const bool first = S.cA == 0.0;                    // U^(1) = U' + dt L: no U^n term
-  const bool owned = j >= P.jlo && j < P.jhi;
-  double newavg[4];
   bool finite = true;
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
+    if (v < v0 || v >= v1) continue;
     double L[3];
     const T Fp = xp[0][v], Fm = xm[0][v], Gp = yp[0][v], Gm = ym[0][v];
     L[0] = -fma(to_f64(Fp) - to_f64(Fm), idx, (to_f64(Gp) - to_f64(Gm)) * idy);
@@ -589,37 +599,37 @@ __device__ __forceinline__ void update_cell_lean(const Prob& P, const Src& src, 
       finite = finite && ((__double_as_longlong(r) >> 52) & 0x7FF) != 0x7FF;
     }
   }
-  if (S.Lout || !owned) return;
+  return finite;
+}
+
+template <typename T, typename Src>
+__device__ __forceinline__ void update_cell_lean(const Prob& P, const Src& src, const Rk& S, int i, int j,
+                                                 const T (&xm)[4][4], const T (&xp)[4][4], const T (&ym)[4][4],
+                                                 const T (&yp)[4][4]) {
+  double newavg[4];
+  const bool finite = combine_lean<T>(P, src, S, i, j, quad_lean<T>(P, src, i, j), xm, xp, ym, yp, 0, 4, newavg);
+  if (S.Lout || j < P.jlo || j >= P.jhi) return;
   if (!finite) atomicOr(S.status, ST_NONFINITE);
   if (nonphysical(newavg[0], newavg[1], newavg[2], newavg[3])) atomicOr(S.status, ST_NONPOSITIVE);
 }
 
-// Step 3 for the TXV x TYV tile at (i0, j0): face fluxes into shared memory, then
-// quadrature, L(U) and the Runge-Kutta combination per cell.  tid = ty*TXV + tx.
-// above: the block has just done the tile below (its top faces are reused).
-// SOLID: the handle may have a solid block (FP64 2D Euler only); without it the
-// wall-face code is not compiled in (the batched kernel runs at the register limit).
-template <typename T, int NV, int TXV, int TYV, bool SOLID = false, typename Src = GlobalSrc<T>>
-__device__ __forceinline__ void update2d_tile(const Prob& P, const Src& src, const Rk& S, int i0, int j0,
-                                              int tid, T (&xf)[TYV][TXV + 1][4][NV], T (&yf)[TYV + 1][TXV][4][NV],
-                                              bool above = false) {
-  const int tx = tid % TXV, ty = tid / TXV;
-  const int i = i0 + tx, j = j0 + ty;
-  const bool live = i < P.nx && j < P.ny;
-  // Every face flux of the tile at one Gauss-Lobatto point per iteration, by one
-  // call site, so that a face shared by two tiles gets bitwise the same flux
-  // from both (the flux differences then telescope exactly in FP64).
-  // xf[r][c] is the face left of cell (i0 + c, j0 + r); yf[r][c] the face below it.
-  constexpr int NXP = (TXV + 1) * TYV * 4, NYP = TXV * (TYV + 1) * 4;
+// Face fluxes of the TXV x TYV tile at (i0, j0) into shared memory, points t0,
+// t0 + step, ... below t1 of tile_points.
+// A face flux at one Gauss-Lobatto point per iteration, by one
+// call site, so that a face shared by two tiles gets bitwise the same flux
+// from both (the flux differences then telescope exactly in FP64).
+// xf[r][c] is the face left of cell (i0 + c, j0 + r); yf[r][c] the face below it.
+template <int TXV, int TYV>
+__host__ __device__ constexpr int tile_points(bool above) { return (TXV + 1) * TYV * 4 + TXV * (TYV + 1) * 4 - (above ? TXV * 4 : 0); }
+
+template <typename T, int NV, int TXV, int TYV, bool SOLID, bool SOFT, typename Src>
+__device__ __forceinline__ void tile_fluxes(const Prob& P, const Src& src, int i0, int j0, int t0, int t1, int step,
+                                            T (&xf)[TYV][TXV + 1][4][NV], T (&yf)[TYV + 1][TXV][4][NV], bool above) {
+  constexpr int NXP = (TXV + 1) * TYV * 4;
   // a tile whose faces all join cells inside the grid (no image, no solid cell):
   // the point values at fixed offsets
   const bool tin = Src::staged || ((!SOLID || P.sol_j == 0) && i0 >= 1 && i0 + TXV < P.nx && j0 >= 1 && j0 + TYV < P.ny);
-  __syncthreads();   // the shared arrays may still be read for a previous tile
-  if (above) {       // the tile below was this block's last: its top faces are this one's bottom faces
-    for (int q = tid; q < TXV * 4 * NV; q += TXV * TYV) (&yf[0][0][0][0])[q] = (&yf[TYV][0][0][0])[q];
-    __syncthreads();
-  }
-  for (int t = tid; t < NXP + NYP - (above ? TXV * 4 : 0); t += TXV * TYV) {
+  for (int t = t0; t < t1; t += step) {
     const int f = above && t >= NXP ? t + TXV * 4 : t;
     // the face's GL point q, its slot (c, r) in the tile, its two cells a
     // (left / below) and b (right / above) and their point indices
@@ -659,21 +669,47 @@ __device__ __forceinline__ void update2d_tile(const Prob& P, const Src& src, con
       }
       wall = sa || sb;
     }
-    face_flux<T, NV>(P, uL, uR, xd, wall, xd ? xf[r][c][q] : yf[r][c][q]);
+    face_flux<T, NV, SOFT>(P, uL, uR, xd, wall, xd ? xf[r][c][q] : yf[r][c][q]);
   }
+}
+
+// Face integrals (eq. (integral2), (integral3)), once per face: point slots 0 and 1
+// become the mean and the first moment along the face.
+template <typename T, int TXV, int TYV>
+__device__ __forceinline__ void tile_integrals(int tid, int step, T (&xf)[TYV][TXV + 1][4][4],
+                                               T (&yf)[TYV + 1][TXV][4][4], bool above) {
+  constexpr int NXF = (TXV + 1) * TYV * 4;
+  for (int t = tid; t < NXF + TXV * (TYV + 1) * 4 - (above ? TXV * 4 : 0); t += step) {
+    const int f = above && t >= NXF ? t + TXV * 4 : t;
+    const int g = (f < NXF ? f : f - NXF) >> 2, v = f & 3;
+    T* q = f < NXF ? &xf[0][0][0][0] + g * 16 + v : &yf[0][0][0][0] + g * 16 + v;
+    const T f0 = q[0], f1 = q[4], f2 = q[8], f3 = q[12];
+    q[0] = fma(T(5.0 / 12.0), f1 + f2, T(1.0 / 12.0) * (f0 + f3));
+    q[4] = fma(T(5.0 / 12.0 * 0.22360679774997896964), f2 - f1, T(1.0 / 24.0) * (f3 - f0));
+  }
+}
+
+// Step 3 for the TXV x TYV tile at (i0, j0): face fluxes into shared memory, then
+// quadrature, L(U) and the Runge-Kutta combination per cell.  tid = ty*TXV + tx.
+// above: the block has just done the tile below (its top faces are reused).
+// SOLID: the handle may have a solid block (FP64 2D Euler only); without it the
+// wall-face code is not compiled in (the batched kernel runs at the register limit).
+template <typename T, int NV, int TXV, int TYV, bool SOLID = false, typename Src = GlobalSrc<T>>
+__device__ __forceinline__ void update2d_tile(const Prob& P, const Src& src, const Rk& S, int i0, int j0,
+                                              int tid, T (&xf)[TYV][TXV + 1][4][NV], T (&yf)[TYV + 1][TXV][4][NV],
+                                              bool above = false) {
+  const int tx = tid % TXV, ty = tid / TXV;
+  const int i = i0 + tx, j = j0 + ty;
+  const bool live = i < P.nx && j < P.ny;
+  __syncthreads();   // the shared arrays may still be read for a previous tile
+  if (above) {       // the tile below was this block's last: its top faces are this one's bottom faces
+    for (int q = tid; q < TXV * 4 * NV; q += TXV * TYV) (&yf[0][0][0][0])[q] = (&yf[TYV][0][0][0])[q];
+    __syncthreads();
+  }
+  tile_fluxes<T, NV, TXV, TYV, SOLID, true>(P, src, i0, j0, tid, tile_points<TXV, TYV>(above), TXV * TYV, xf, yf, above);
   __syncthreads();
   if constexpr (NV == 4 && lean<T>::value) {
-    // face integrals (eq. (integral2), (integral3)), once per face: point slots 0
-    // and 1 become the mean and the first moment along the face
-    constexpr int NXF = (TXV + 1) * TYV * 4;
-    for (int t = tid; t < NXF + TXV * (TYV + 1) * 4 - (above ? TXV * 4 : 0); t += TXV * TYV) {
-      const int f = above && t >= NXF ? t + TXV * 4 : t;
-      const int g = (f < NXF ? f : f - NXF) >> 2, v = f & 3;
-      T* q = f < NXF ? &xf[0][0][0][0] + g * 16 + v : &yf[0][0][0][0] + g * 16 + v;
-      const T f0 = q[0], f1 = q[4], f2 = q[8], f3 = q[12];
-      q[0] = fma(T(5.0 / 12.0), f1 + f2, T(1.0 / 12.0) * (f0 + f3));
-      q[4] = fma(T(5.0 / 12.0 * 0.22360679774997896964), f2 - f1, T(1.0 / 24.0) * (f3 - f0));
-    }
+    tile_integrals<T, TXV, TYV>(tid, TXV * TYV, xf, yf, above);
     __syncthreads();
   }
   if (!live) return;
@@ -808,10 +844,13 @@ __device__ __forceinline__ void update2d_tile(const Prob& P, const Src& src, con
 // which waits for loads rather than for its arithmetic, measured 9 % slower so).
 // fx64 at 2048^2: 15.2 ms per launch with hllc and the quadrature per point, 9.6
 // with hllc_lean and update_cell_lean, 8.07 with the integer compares, the 5-operation
-// root and the sweep; bound by the FP64 pipe (87 % busy, 1053 operations per cell,
-// 1915 before).  Double-float 5.2 -> 3.0 ms.
+// root and the sweep, 5.8 with roots and reciprocals and 4.7 with the flux's products
+// in integers (4.8 at 4 blocks per SM): 600 FP64 operations per cell of 1915, the
+// FP64 pipe still 90 % busy.  Double-float 5.2 -> 3.0 ms.
 template <typename T, int NV, bool SOLID = false>
-__global__ void __launch_bounds__(TX * TY, (std::is_same<T, float>::value ? 8 : lean<T>::value ? 4 : 3))
+__global__ void __launch_bounds__(TX * TY, (std::is_same<T, float>::value ? 8
+                                         : std::is_same<T, fx64>::value && NV == 4 && !SOLID ? 5
+                                         : lean<T>::value ? 4 : 3))
     update2d_kernel(const __grid_constant__ Prob P, const T* __restrict__ G, Rk S, int sweep) {
   __shared__ T xf[TY][TX + 1][4][NV];
   __shared__ T yf[TY + 1][TX][4][NV];
@@ -840,7 +879,64 @@ __global__ void __launch_bounds__(TX * TY, (std::is_same<T, float>::value ? 8 : 
   }
 }
 
-// Tiles per block: as many as leave six waves of resident blocks (4 per SM), at
+// Few tiles (at most WIDE_TILES per SM): 256 threads a tile.  A tile's time is
+// then one warp's chain of FP64 operations (64 clocks each, one warp per
+// scheduler), not the pipe's rate, so the second half of the block takes the
+// quadrature while the first does face fluxes, then the rest of these, and a cell's
+// variables are shared by two threads.  The flux's products stay on the FP64
+// pipe: it has room, and an integer product is the longer chain.  Bit for bit
+// update2d_kernel's results.  Per launch, against update2d_kernel: 64^2 55 -> 39 us,
+// 128^2 57 -> 39, 192^2 (1.9 tiles per SM) 72 -> 68; 224^2 (2.6) 89 -> 98, so the
+// line is at two.
+constexpr int WIDE_TILES = 2;
+template <typename T>
+__global__ void __launch_bounds__(2 * TX * TY, 2)
+    update2d_wide_kernel(const __grid_constant__ Prob P, const T* __restrict__ G, Rk S) {
+  constexpr int N = TX * TY;
+  __shared__ T xf[TY][TX + 1][4][4];
+  __shared__ T yf[TY + 1][TX][4][4];
+  __shared__ Quad<T> qs[N];
+  __shared__ double avg[4][N];
+  __shared__ int bad[N];
+  const int tid = threadIdx.x, c = tid % N, part = tid / N;
+  const int i0 = blockIdx.x * TX, j0 = blockIdx.y * TY, i = i0 + c % TX, j = j0 + c / TX;
+  const bool live = i < P.nx && j < P.ny;
+  if (S.dtp) {
+    S.dt = *S.dtp;
+    if (S.dt < 0.0) {   // a skipped step (block-uniform): the state passes through unchanged
+      if (live && !S.Lout)
+        for (int q = part * 6; q < part * 6 + 6; ++q) {
+          const long long si = (long long)q * P.plane + (long long)j * P.pitch + i;
+          S.Uout[si] = S.Uin[si];
+        }
+      return;
+    }
+  }
+  const GlobalSrc<T> src{G};
+  // 9.1 flux points per cell, of which the half with the quadrature takes 3.1
+  constexpr int first = 6 * N;
+  if (part == 1 && live) qs[c] = quad_lean<T>(P, src, i, j);
+  tile_fluxes<T, 4, TX, TY, false, false>(P, src, i0, j0, part * first + c, part ? tile_points<TX, TY>(false) : first, N,
+                                          xf, yf, false);
+  __syncthreads();
+  tile_integrals<T, TX, TY>(tid, 2 * N, xf, yf, false);
+  __syncthreads();
+  bool finite = true;
+  const int x = c % TX, y = c / TX;
+  if (live) {
+    double a[4];
+    finite = combine_lean<T>(P, src, S, i, j, qs[c], xf[y][x], xf[y][x + 1], yf[y][x], yf[y + 1][x], 2 * part,
+                             2 * part + 2, a);
+    if (part) { avg[2][c] = a[2]; avg[3][c] = a[3]; bad[c] = !finite; }
+    else { avg[0][c] = a[0]; avg[1][c] = a[1]; }
+  }
+  __syncthreads();
+  if (part || !live || S.Lout || j < P.jlo || j >= P.jhi) return;
+  if (!finite || bad[c]) atomicOr(S.status, ST_NONFINITE);
+  if (nonphysical(avg[0][c], avg[1][c], avg[2][c], avg[3][c])) atomicOr(S.status, ST_NONPOSITIVE);
+}
+
+// Tiles per block: as many as leave six waves of 4 resident blocks per SM, at
 // most 16; small grids keep one, their blocks must reach every SM first.
 template <typename T>
 inline int update_sweep(const Prob& P) {
@@ -1036,7 +1132,9 @@ void stage_t(const Prob& P, const HostTabs& HT, const Weights<T>& W, const Beta2
   const int sweep = update_sweep<T>(P);
   const dim3 sgrd(grd.x, (grd.y + sweep - 1) / sweep);
   if constexpr (NV == 4 && std::is_same<T, fx64>::value) {
-    if (P.sol_j > 0) update2d_kernel<T, NV, true><<<sgrd, blk, 0, st>>>(P, (const T*)B.G, r, sweep);
+    if (P.sol_j == 0 && (long long)grd.x * grd.y <= (long long)WIDE_TILES * P.nsm)
+      update2d_wide_kernel<T><<<grd, 2 * TX * TY, 0, st>>>(P, (const T*)B.G, r);
+    else if (P.sol_j > 0) update2d_kernel<T, NV, true><<<sgrd, blk, 0, st>>>(P, (const T*)B.G, r, sweep);
     else update2d_kernel<T, NV><<<sgrd, blk, 0, st>>>(P, (const T*)B.G, r, sweep);
   } else if constexpr (NV == 4 && std::is_same<T, float>::value) {
     if (B.tmG && !S.Lout)

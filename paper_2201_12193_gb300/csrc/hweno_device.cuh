@@ -429,8 +429,8 @@ __device__ __forceinline__ void hllc(const Prob& P, const T* uL, const T* uR, in
   for (int v = 0; v < NV; ++v) F[v] = fK[v] + sK * (us[v] - uK[v]);
 }
 
-// fx64 and double-float take the lean form below (fx64: 68 FP64 operations against
-// 150 of hllc); float and plain double keep hllc.
+// fx64 and double-float take the lean form below (fx64: 24 FP64 operations in 2D, the
+// products, roots and reciprocals being integer work, against 150 of hllc); float and plain double keep hllc.
 template <typename T> struct lean { static constexpr bool value = is_df64<T>::value || std::is_same<T, fx64>::value; };
 template <typename T> __device__ __forceinline__ bool nonneg(T a) { return T(0) <= a; }
 template <typename T> __device__ __forceinline__ bool nonpos(T a) { return a <= T(0); }
@@ -444,9 +444,14 @@ template <typename T> __device__ __forceinline__ T half(T a) { return T(0.5) * a
 // w = rho_K (s_K - m_K), p* = p_K + w (s* - m_K) and rho* = w / (s_K - s*) it is
 // (rho* s*, rho* s*^2 + p*, rho* s* t_K, s* (E* + p*)),
 // E* = (E_K (s_K - m_K) - p_K m_K + p* s*) / (s_K - s*).
-template <typename T, int NV>
+template <typename T, int NV, bool SOFT = true>
 __device__ __forceinline__ void hllc_lean(const Prob& P, const T* uL, const T* uR, int dir, T* F, bool wall = false) {
   constexpr bool two = NV == 4;
+  // fx64 in 2D: the products in integers (SOFT) or by the FP64 pipe, the same bits
+  auto M = [](T a, T b) {
+    if constexpr (two && std::is_same<T, fx64>::value) return SOFT ? product(a, b) : fx64(__dmul_rn(a.v, b.v));
+    else return a * b;
+  };
   constexpr int iE = NV - 1;
   const int in = 1 + dir, it = 2 - dir;
   const T g = pc<T>(P.cgamma), gm1 = pc<T>(P.cgm1), k = pc<T>(P.chk);
@@ -460,19 +465,19 @@ __device__ __forceinline__ void hllc_lean(const Prob& P, const T* uL, const T* u
     iL = rcp(rL);
     iR = rcp(rR);
   }
-  const T mL = uL[in] * iL, mR = uR[in] * iR;
-  const T tL = two ? uL[it] * iL : T(0), tR = two ? uR[it] * iR : T(0);
-  T kL = uL[in] * mL, kR = uR[in] * mR;
+  const T mL = M(uL[in], iL), mR = M(uR[in], iR);
+  const T tL = two ? M(uL[it], iL) : T(0), tR = two ? M(uR[it], iR) : T(0);
+  T kL = M(uL[in], mL), kR = M(uR[in], mR);
   if constexpr (two) { kL = fma(uL[it], tL, kL); kR = fma(uR[it], tR, kR); }
-  const T pL = gm1 * fma(T(-0.5), kL, EL), pR = gm1 * fma(T(-0.5), kR, ER);
-  const T gL = g * iL, gR = g * iR;
-  const T cL = sqrt(gL * pL), cR = sqrt(gR * pR);
-  const T x = (rL + rR) * (cL + cR);                 // four times the mean density times the mean sound speed
-  const T ps = fma((mL - mR) * x, T(0.125), half(pL + pR));
-  const T ss = fma((pL - pR) * rcp(x), T(2), half(mL + mR));
+  const T pL = M(gm1, fma(T(-0.5), kL, EL)), pR = M(gm1, fma(T(-0.5), kR, ER));
+  const T gL = M(g, iL), gR = M(g, iR);
+  const T cL = sqrt(M(gL, pL)), cR = sqrt(M(gR, pR));
+  const T x = M(rL + rR, cL + cR);                 // four times the mean density times the mean sound speed
+  const T ps = fma(M(mL - mR, x), T(0.125), half(pL + pR));
+  const T ss = fma(M(pL - pR, rcp(x)), T(2), half(mL + mR));
   auto speed = [&](T gk, T pk, T ck) {               // c_K coef_K of eq. (COEF)
     const T d = ps - pk;
-    return nonpos(d) ? ck : sqrt(gk * fma(k, d, pk));
+    return nonpos(d) ? ck : sqrt(M(gk, fma(k, d, pk)));
   };
   bool left = nonneg(ss);
   if (!left && !wall && !below(mL, cL)) left = nonneg(mL - speed(gL, pL, cL));
@@ -484,19 +489,19 @@ __device__ __forceinline__ void hllc_lean(const Prob& P, const T* uL, const T* u
     const T q = left ? uL[in] : uR[in];
     F[0] = q;
     F[in] = fma(q, mK, pK);
-    if constexpr (two) F[it] = q * tK;
-    F[iE] = mK * (EK + pK);
+    if constexpr (two) F[it] = M(q, tK);
+    F[iE] = M(mK, EK + pK);
     return;
   }
-  const T a = sK - mK, w = (left ? rL : rR) * a;
+  const T a = sK - mK, w = M(left ? rL : rR, a);
   const T pst = fma(w, ss - mK, pK);
   const T rb = rcp(sK - ss);
-  const T f0 = w * rb * ss;
+  const T f0 = M(M(w, rb), ss);
   F[0] = f0;
   F[in] = fma(f0, ss, pst);
-  if constexpr (two) F[it] = f0 * tK;
-  const T e = fma(pst, ss, fma(EK, a, -(pK * mK)));
-  F[iE] = ss * fma(e, rb, pst);
+  if constexpr (two) F[it] = M(f0, tK);
+  const T e = fma(pst, ss, fma(EK, a, -M(pK, mK)));
+  F[iE] = M(ss, fma(e, rb, pst));
 }
 
 // Scalar laws: local Lax-Friedrichs flux with alpha = max(|f'(uL)|, |f'(uR)|).

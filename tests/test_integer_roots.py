@@ -1,8 +1,9 @@
-"""Host check of the integer reciprocal and square root of the FP64 forms.
+"""Host check of the integer reciprocal, square root and product of the FP64 forms.
 
 The hardware's starting values may be off by its stated error either way; the
 results have to be within 0.52 units in the last place for every start allowed,
-and exact where the true value is representable.
+and exact where the true value is representable.  A product has the bits of the
+FP64 one; below the normal range it is zero.
 """
 import os
 import shutil
@@ -72,4 +73,49 @@ def test_reciprocal_and_root_within_half_a_unit(tmp_path):
     src.write_text(SOURCE)
     subprocess.check_call(["g++", "-O2", "-I", CSRC, "-o", str(tmp_path / "roots"), str(src)])
     out = subprocess.run([str(tmp_path / "roots")], capture_output=True, text=True)
+    assert out.returncode == 0, out.stdout
+
+
+PRODUCT = r"""
+#include "fx64_roots.h"
+#include <cmath>
+#include <cstdio>
+#include <cstring>
+#include <random>
+int main() {
+  std::mt19937_64 g(11);
+  auto draw = [&](long k) {                            // few bits, many bits, powers of two, all exponents, zeros
+    uint64_t m = g() >> 12, e = k % 3 ? 1015 + g() % 16 : g() % 2047;
+    if (k % 5 == 1) m &= ~((1ull << (g() % 52)) - 1);
+    if (k % 5 == 2) m |= (1ull << (g() % 52)) - 1;
+    if (k % 11 == 0) m = 0;
+    if (k % 13 == 0) m &= ~((1ull << 27) - 1);         // products of these meet exact ties
+    if (e == 0) m = 0;
+    return (g() & 1) << 63 | e << 52 | m;
+  };
+  for (long k = 0; k < 2000000; ++k) {
+    const uint64_t x = draw(k), y = draw((long)(g() % 100000));
+    double a, b;
+    memcpy(&a, &x, 8);
+    memcpy(&b, &y, 8);
+    const double c = a * b;
+    uint64_t want;
+    memcpy(&want, &c, 8);
+    const uint64_t got = fxr::product(x >> 32, (uint32_t)x, y >> 32, (uint32_t)y);
+    if (std::fabs(c) <= 2.2250738585072014e-308 && (got << 1) == 0) continue;
+    if (got != want) { printf("%a %a: %llx %llx\n", a, b, (unsigned long long)got, (unsigned long long)want); return 1; }
+  }
+  const uint64_t inf = 0x7FFull << 52, one = 1023ull << 52;
+  const uint64_t n = fxr::product(inf >> 32, 0, one >> 32, 0);
+  return (n >> 52 & 0x7FF) == 0x7FF && (n << 12) != 0 ? 0 : 2;
+}
+"""
+
+
+@pytest.mark.skipif(shutil.which("g++") is None, reason="needs g++")
+def test_product_has_the_fp64_bits(tmp_path):
+    src = tmp_path / "product.cpp"
+    src.write_text(PRODUCT)
+    subprocess.check_call(["g++", "-O2", "-I", CSRC, "-o", str(tmp_path / "product"), str(src)])
+    out = subprocess.run([str(tmp_path / "product")], capture_output=True, text=True)
     assert out.returncode == 0, out.stdout
