@@ -46,9 +46,9 @@ FXR_HD uint32_t seed_fixed(uint32_t bits_1py) { return bits_1py & 0x7FFFFFu; }
 constexpr float RCP_ONE = 1.0f - 5.0f / 16777216.0f;    // D = 5: the approximation's 2^-23 and the mantissa's truncation
 constexpr float ROOT_ONE = 1.0f - 4.0f / 16777216.0f;   // D = 4: 2^-22.9 and half the truncation
 
-// 2^62 / m for the mantissa M = mh:ml (2^52 <= M < 2^53, m = M 2^-52) from y in
-// units of 2^-23: as the mantissa rounded to [2^52, 2^53] of 1/m = it / 2^53.
-FXR_HD uint64_t rcp_mantissa(uint32_t mh, uint32_t ml, uint32_t y) {
+// 2^62 / m (at most a few units too small) for the mantissa M = mh:ml
+// (2^52 <= M < 2^53, m = M 2^-52) from y in units of 2^-23.
+FXR_HD uint64_t rcp62(uint32_t mh, uint32_t ml, uint32_t y) {
   const uint64_t t = wide(ml, y) + ((uint64_t)(uint32_t)(mh * y) << 32);   // m y, units 2^-75, less 1
   const uint64_t r = 0 - t;                                                // e
   uint32_t rh, rl;
@@ -56,8 +56,10 @@ FXR_HD uint64_t rcp_mantissa(uint32_t mh, uint32_t ml, uint32_t y) {
   const uint64_t e = r + (wide(rh, rh) >> 11);                             // e + e^2
   split(e, rh, rl);
   const uint64_t c = wide(y, rh) + (wide(y, rl) >> 32);                    // y (e + e^2), units 2^-66
-  return (((uint64_t)(y << 7) << 32) + (c >> 4) + 256) >> 9;
+  return ((uint64_t)(y << 7) << 32) + (c >> 4);
 }
+// 1/m rounded, in units of 2^-53.
+FXR_HD uint64_t rcp_mantissa(uint32_t mh, uint32_t ml, uint32_t y) { return (rcp62(mh, ml, y) + 256) >> 9; }
 
 // sqrt(m) 2^52, rounded, for m = M 2^-52 in [1, 4) (M = mh:ml below 2^54) from y in units of 2^-23.
 FXR_HD uint64_t sqrt_mantissa(uint32_t mh, uint32_t ml, uint32_t y) {
@@ -73,6 +75,43 @@ FXR_HD uint64_t sqrt_mantissa(uint32_t mh, uint32_t ml, uint32_t y) {
   split(c, ch, cl);
   const uint64_t d = wide(gh, ch) + ((wide(gh, cl) + wide(gl, ch)) >> 32); // m y c, units 2^-65
   return (g + (d >> 3) + 512) >> 10;
+}
+
+// rcp_mantissa's q is at most the correctly rounded one and at least that less 1
+// (every truncation above lowers it): the sign of 2^105 - q M - M/2 tells which.
+FXR_HD uint64_t rcp_nearest(uint32_t mh, uint32_t ml, uint64_t q) {
+  uint32_t qh, ql;
+  split(q, qh, ql);
+  const uint64_t p = wide(ql, ml) + ((uint64_t)(uint32_t)(qh * ml + ql * mh) << 32);
+  const int64_t r2 = (int64_t)((0 - p) << 1);
+  return q + (r2 > (int64_t)(((uint64_t)mh << 32) | ml) ? 1u : 0u);
+}
+// The same for the root: one up if M 2^52 exceeds q (q + 1).
+FXR_HD uint64_t sqrt_nearest(uint32_t mh, uint32_t ml, uint64_t q) {
+  uint32_t qh, ql;
+  split(q, qh, ql);
+  const uint64_t p = wide(ql, ql) + ((uint64_t)(uint32_t)(2u * qh * ql) << 32);
+  const int64_t d = (int64_t)(((uint64_t)(ml << 20) << 32) - p);
+  return q + (d > (int64_t)q ? 1u : 0u);
+}
+
+// A / B for mantissas, rounded to nearest (a quotient of two doubles is never a
+// tie), in units of 2^-52, of 2^-53 (less = 1) if A < B; y as for 1/B.
+FXR_HD uint64_t quotient(uint32_t ah, uint32_t al, uint32_t bh, uint32_t bl, uint32_t y, uint32_t& less) {
+  uint32_t qh, ql, h, l;
+  split(rcp62(bh, bl, y), qh, ql);
+  const uint64_t a = ((uint64_t)ah << 32) | al, b = ((uint64_t)bh << 32) | bl;
+  split(a << 11, h, l);
+  const uint64_t lo = wide(h, ql) + (wide(l, ql) >> 32);                   // A / B, units 2^-61
+  uint32_t xh, xl;
+  split(lo, xh, xl);
+  const uint64_t t = wide(h, qh) + xh + ((wide(l, qh) + xl) >> 32);
+  less = a < b ? 1u : 0u;
+  const uint64_t q = (t + (256u >> less)) >> (9u - less);
+  split(q, qh, ql);
+  const uint64_t p = wide(ql, bl) + ((uint64_t)(uint32_t)(qh * bl + ql * bh) << 32);
+  const int64_t r2 = (int64_t)((((uint64_t)(al << (20u + less)) << 32) - p) << 1);
+  return q + (r2 > (int64_t)b ? 1u : 0u);
 }
 
 // a b for the doubles ah:al and bh:bl, rounded to nearest even as the FP64

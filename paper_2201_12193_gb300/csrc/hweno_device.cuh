@@ -249,14 +249,21 @@ __device__ __forceinline__ double avg_img(const Prob& P, const double* __restric
 // ---------------------------------------------------------------- physics
 // Physical flux of eq. (1D-Euler) / (2D-Euler) or of the scalar laws in
 // direction dir (0 = x, 1 = y); NV = 1 (scalar), 3 (1D Euler), 4 (2D Euler).
-// 1/x.  FP32, double: correctly rounded.  fx64: in integers, within 0.52 units in the
-// last place.
+// 1/x.  FP32, double: correctly rounded (double in integers).  fx64: in integers,
+// within 0.52 units in the last place.
 template <typename T> __device__ __forceinline__ T rcp(T x) { return T(1) / x; }
 template <> __device__ __forceinline__ float rcp<float>(float x) { return __frcp_rn(x); }
-template <> __device__ __forceinline__ double rcp<double>(double x) { return __drcp_rn(x); }
+template <> __device__ __forceinline__ double rcp<double>(double x) { return rcp_ieee(x); }
 template <> __device__ __forceinline__ fx64 rcp<fx64>(fx64 x) { return reciprocal(x); }
 
 __device__ __forceinline__ double rcp64(double x) { return rcp<fx64>(x).v; }
+
+// Root and quotient of the general flux: plain double's in integers where that is the
+// IEEE result (fx64.cuh).
+template <typename T> __device__ __forceinline__ T root(T x) { return sqrt(x); }
+template <> __device__ __forceinline__ double root<double>(double x) { return sqrt_ieee(x); }
+template <typename T> __device__ __forceinline__ T quot(T a, T b) { return a / b; }
+template <> __device__ __forceinline__ double quot<double>(double a, double b) { return div_ieee(a, b); }
 
 // a + b never contracted into an FMA (operands that are products)
 template <typename T> __device__ __forceinline__ T addrn(T a, T b) { return a + b; }
@@ -373,11 +380,11 @@ __device__ __forceinline__ void hllc(const Prob& P, const T* uL, const T* uR, in
   const T pL = gm1 * (EL - T(0.5) * rL * (mL * mL + tL * tL));
   const T pR = gm1 * (ER - T(0.5) * rR * (mR * mR + tR * tR));
   const T gL = g * iL, gR = g * iR;
-  const T cL = sqrt(gL * pL), cR = sqrt(gR * pR);
+  const T cL = root(gL * pL), cR = root(gR * pR);
   const T rs = T(0.5) * (rL + rR), cs = T(0.5) * (cL + cR);
   const T crs = cs * rs;
   const T ps = T(0.5) * (pL + pR + (mL - mR) * crs);
-  const T ss = T(0.5) * (mL + mR + (pL - pR) / crs);
+  const T ss = T(0.5) * (mL + mR + quot(pL - pR, crs));
   // eq. (COEF): c_K coef_K = sqrt(gamma p_K / rho_K) sqrt(1 + k (p* / p_K - 1)) with
   // k = (gamma + 1) / (2 gamma) when p* > p_K, else c_K.  FP64 keeps the two roots
   // (the second only where p* > p_K); FP32 and double-float take one root,
@@ -388,8 +395,8 @@ __device__ __forceinline__ void hllc(const Prob& P, const T* uL, const T* uR, in
   const T k = pc<T>(P.chk);
   T sL, sR;
   if constexpr (one_division<T>::value) {
-    const T coefL = ps <= pL ? T(1) : sqrt(T(1) + k * (ps / pL - T(1)));
-    const T coefR = ps <= pR ? T(1) : sqrt(T(1) + k * (ps / pR - T(1)));
+    const T coefL = ps <= pL ? T(1) : root(T(1) + k * (quot(ps, pL) - T(1)));
+    const T coefR = ps <= pR ? T(1) : root(T(1) + k * (quot(ps, pR) - T(1)));
     sL = mL - cL * coefL;
     sR = mR + cR * coefR;
   } else {

@@ -1,9 +1,10 @@
-"""Host check of the integer reciprocal, square root and product of the FP64 forms.
+"""Host check of the integer reciprocal, square root, quotient and product of the FP64 forms.
 
 The hardware's starting values may be off by its stated error either way; the
 results have to be within 0.52 units in the last place for every start allowed,
 and exact where the true value is representable.  A product has the bits of the
-FP64 one; below the normal range it is zero.
+FP64 one; below the normal range it is zero.  The forms plain double takes have
+IEEE's bits.
 """
 import os
 import shutil
@@ -118,4 +119,60 @@ def test_product_has_the_fp64_bits(tmp_path):
     src.write_text(PRODUCT)
     subprocess.check_call(["g++", "-O2", "-I", CSRC, "-o", str(tmp_path / "product"), str(src)])
     out = subprocess.run([str(tmp_path / "product")], capture_output=True, text=True)
+    assert out.returncode == 0, out.stdout
+
+
+NEAREST = r"""
+#include "fx64_roots.h"
+#include <cmath>
+#include <cstdio>
+#include <cstring>
+#include <random>
+static uint32_t bits(float f) { uint32_t b; memcpy(&b, &f, 4); return b; }
+static float flt(uint32_t b) { float f; memcpy(&f, &b, 4); return f; }
+static uint32_t seed(float y, float one) {          // the sum rounded towards zero
+  const double s = (double)y + one;
+  float f = (float)s;
+  if (f > s) f = nextafterf(f, -1.0f);
+  return fxr::seed_fixed(bits(f));
+}
+int main() {
+  std::mt19937_64 g(3);
+  auto draw = [&](long k) {
+    uint64_t M = (1ull << 52) | (g() >> 12);
+    if (k % 4 == 1) M &= ~((1ull << (g() % 53)) - 1);
+    if (k % 4 == 2) M |= (1ull << (g() % 52)) - 1;
+    return M;
+  };
+  for (long k = 0; k < 600000; ++k) {
+    const uint64_t M = k < 300 ? (1ull << 52) + k / 3 : k < 600 ? (1ull << 53) - 1 - (k - 300) / 3 : draw(k);
+    uint64_t A = k % 5 ? draw(k / 7) : M + k % 3 - 1;                        // equal and neighbouring mantissas too
+    if (A < 1ull << 52 || A >= 1ull << 53) A = M;
+    const double p = k % 3 - 1;
+    const uint32_t h = M >> 32, l = (uint32_t)M, sb = fxr::seed_bits(h, l);
+    const uint32_t y = seed((float)((1.0 / flt(sb)) * (1 + p * std::ldexp(1.0, -23))), fxr::RCP_ONE);
+    const double m = std::ldexp((double)M, -52);
+    if (std::ldexp((double)fxr::rcp_nearest(h, l, fxr::rcp_mantissa(h, l, y)), -53) != 1.0 / m) { printf("1/%a\n", m); return 1; }
+    uint32_t less;
+    const uint64_t q = fxr::quotient(A >> 32, (uint32_t)A, h, l, y, less);
+    if (std::ldexp((double)q, -52 - (int)less) != (double)A / (double)M) { printf("%llx / %llx\n", (unsigned long long)A, (unsigned long long)M); return 1; }
+    for (int odd = 0; odd < 2; ++odd) {
+      const uint64_t N = M << odd;
+      const float z = flt(sb + ((uint32_t)odd << 23));
+      const uint32_t w = seed((float)((1.0 / std::sqrt((double)z)) * (1 + p * std::exp2(-22.9))), fxr::ROOT_ONE);
+      const uint64_t r = fxr::sqrt_nearest(N >> 32, (uint32_t)N, fxr::sqrt_mantissa(N >> 32, (uint32_t)N, w));
+      if (std::ldexp((double)r, -52) != std::sqrt(std::ldexp((double)N, -52))) { printf("sqrt %llx\n", (unsigned long long)N); return 1; }
+    }
+  }
+  return 0;
+}
+"""
+
+
+@pytest.mark.skipif(shutil.which("g++") is None, reason="needs g++")
+def test_corrected_forms_have_the_ieee_bits(tmp_path):
+    src = tmp_path / "nearest.cpp"
+    src.write_text(NEAREST)
+    subprocess.check_call(["g++", "-O2", "-ffp-contract=off", "-I", CSRC, "-o", str(tmp_path / "nearest"), str(src)])
+    out = subprocess.run([str(tmp_path / "nearest")], capture_output=True, text=True)
     assert out.returncode == 0, out.stdout
