@@ -10,7 +10,7 @@
 namespace hw {
 namespace {
 
-constexpr int RT = 256;       // threads per block (64 in the wave speeds of small grids)
+constexpr int RT = 256;       // threads per block (128 in the wave speeds of small grids)
 constexpr int MAXB = 1024;    // blocks of the first pass (partials per quantity)
 
 template <int K, int NT = RT>
@@ -260,11 +260,12 @@ int reduce_partials_len(const Prob&) { return 4 * MAXB + 1; }
 void run_wavespeed(const Prob& P, const double* U, double* partials, double* out, const double* par, double* st,
                    unsigned* status, cudaStream_t s) {
   const long long n = (long long)P.nx * (P.jhi - P.jlo);
-  // few cells: 64-thread blocks, one warp per scheduler of more SMs (the cells' FP64
-  // divisions and roots issue at 2 per clock and SM)
+  // few cells: 128-thread blocks, one warp per scheduler of more SMs (the cells' FP64
+  // divisions and roots issue at 2 per clock and SM); 64 threads doubled the blocks the
+  // last one waits for (2D Burgers 161^2, 12 steps: 2.11 -> 2.09 ms)
   if (n <= 256LL * P.nsm)
-    wavespeed_kernel<64, false><<<(int)std::min<long long>(MAXB, (n + 63) / 64), 64, 0, s>>>(P, U, partials, out, par,
-                                                                                             st, status);
+    wavespeed_kernel<128, false><<<(int)std::min<long long>(MAXB, (n + 127) / 128), 128, 0, s>>>(P, U, partials, out, par,
+                                                                                                st, status);
   else if (P.eq == EQ_EULER)
     wavespeed_kernel<RT, true><<<first_pass_blocks(P), RT, 0, s>>>(P, U, partials, out, par, st, status);
   else
