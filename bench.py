@@ -57,6 +57,11 @@ def _rec_flop_per_cell(nvar=4):
     with open(os.path.join(ROOT, "paper_2201_12193_gb300", "csrc", "hweno_parity.h")) as f:
         sbv = int(re.search(r"D2_FLOP_SBV = (\d+);", f.read()).group(1))
     return nvar * (sbv + 112) + 44
+# FP64-pipe operations per cell of one launch on four-quadrant data, executed and
+# counted by ncu (smsp__inst_executed_pipe_fp64.sum x 32 / cells, 1024^2): the linear
+# part, divisions, roots and most products of the FP64 kernels are integer work, so
+# the pipe's own operations, not the algorithmic flop, stand against its rate.
+FP64_PIPE_OPS_PER_CELL = {"reconstruct": 504.0, "update": 544.4}
 # algorithmic HBM bytes per cell-stage: read U^(k) (12 doubles), read U^n for stages 2-3, write U^(k+1)
 ALGO_BYTES_PER_CELL_STAGE = 12 * 8 * (1 + 2.0 / 3.0 + 1)
 
@@ -349,7 +354,7 @@ MLP_FLOP_PER_CELL = 2 * (108 * 64 + 64 * 64 + 64)    # 11,072 multiply-adds per 
 
 
 KERNEL_SOURCES = ("hweno_2d_kernels.cuh", "hweno_device.cuh", "hweno_parity.h", "hweno_internal.h", "hweno_fused.cuh",
-                  "df64.cuh")
+                  "df64.cuh", "fx64.cuh", "fx64_roots.h", "hweno_fx.cuh")
 # FP32-bulk update kernel, bytes per cell and launch that its inputs and outputs
 # fix: point values 4 x 16 x 4 B, U^(k) 96 B, U^n 96 B in two stages of three
 # (64 B on average), U^(k+1) 96 B and its float copy 48 B
@@ -357,7 +362,8 @@ UPD32_BYTES_PER_CELL = 256 + 96 + 64 + 96 + 48
 
 
 # the fused 1D stage kernel's sources (its ncu figures: profiles/dram_traffic_1d.json)
-KERNEL_SOURCES_1D = ("hweno_fused1d.cuh", "hweno_1d.cu", "hweno_device.cuh", "hweno_parity.h", "df64.cuh")
+KERNEL_SOURCES_1D = ("hweno_fused1d.cuh", "hweno_1d.cu", "hweno_device.cuh", "hweno_parity.h", "df64.cuh", "fx64.cuh",
+                     "fx64_roots.h", "hweno_fx.cuh")
 # fused 1D stage, bytes per cell and launch: U^(k) 48 B, U^n 48 B in two stages
 # of three (32 B on average), U^(k+1) 48 B, the troubled mask 1 B and the
 # previous stage's mask 1 B in two of three
@@ -908,22 +914,33 @@ def run_ours(args, world, rank, local):
     # roofline of the dominant kernel (largest share of device time)
     kind, (kms, kn) = max(prof.items(), key=lambda kv: kv[1][0])
     total_kernel_ms = sum(v[0] for v in prof.values())
-    flop = _rec_flop_per_cell(s64.nvar) * cells * kn if kind == "reconstruct" else None
     roof = None
-    if flop:
+    if args.precision == "fp64" and kind in FP64_PIPE_OPS_PER_CELL:
+        ops = FP64_PIPE_OPS_PER_CELL[kind]
+        achieved = ops * cells * kn / (kms * 1e-3)
+        pk = peaks["fp64_tflops"] * 1e12 / 2                # one FMA is one operation
+        name = "rec2d_split_kernel<fx64>" if kind == "reconstruct" else "update2d_kernel<fx64,4>"
+        roof = {"bound": "alu", "kernel": f"{name} ({kind})", "achieved": achieved / 1e12, "peak": pk / 1e12,
+                "unit": "T FP64-pipe operations/s", "frac": achieved / pk,
+                "peak_source": "FP64 FMA rate measured in this run by hweno_alu_probe (of measured), an FMA one operation; "
+                               f"nominal from unit counts {peaks['fp64_nominal_tflops'] / 2:.3f}",
+                "frac_of_nominal_fp64": achieved / (peaks["fp64_nominal_tflops"] * 0.5e12),
+                "fp64_pipe_ops_per_cell": ops, "traffic": None, "launches": kn, "avg_ms": kms / kn,
+                "share": kms / total_kernel_ms}
+        bpc = traffic_per_cell(("rec2d" if kind == "reconstruct" else "update2d") + "_fp64")
+    elif kind == "reconstruct":
+        flop = _rec_flop_per_cell(s64.nvar) * cells * kn
         achieved = flop / (kms * 1e-3)
-        pk = peaks["fp64_tflops"] * 1e12 if args.precision == "fp64" else peaks["fp32_tflops"] * 1e12
-        roof = {"bound": "alu", "kernel": f"rec2d<{'double' if args.precision == 'fp64' else 'float'},4> ({kind})",
-                "achieved": achieved / 1e12, "peak": pk / 1e12, "unit": "TFLOP/s", "frac": achieved / pk,
-                "peak_source": f"{args.precision.upper()} FMA throughput measured in this run by hweno_alu_probe "
-                               f"(of measured); nominal FP64 from unit counts {peaks['fp64_nominal_tflops']:.3f}",
-                "frac_of_nominal_fp64": achieved / (peaks["fp64_nominal_tflops"] * 1e12),
+        pk = peaks["fp32_tflops"] * 1e12
+        roof = {"bound": "alu", "kernel": f"rec2d<float,4> ({kind})", "achieved": achieved / 1e12, "peak": pk / 1e12,
+                "unit": "TFLOP/s", "frac": achieved / pk,
+                "peak_source": "FP32 FMA throughput measured in this run by hweno_alu_probe (of measured)",
                 "flop_per_cell": _rec_flop_per_cell(s64.nvar), "traffic": None, "launches": kn, "avg_ms": kms / kn,
                 "share": kms / total_kernel_ms}
-        bpc = traffic_per_cell(f"rec2d_{args.precision}") if args.precision == "fp64" else None
-        if bpc:
-            roof["traffic"] = bpc * cells
-            roof["traffic_unit"] = "bytes per launch (ncu dram read+write per cell x cells, profiles/dram_traffic.json)"
+        bpc = None
+    if roof and bpc:
+        roof["traffic"] = bpc * cells
+        roof["traffic_unit"] = "bytes per launch (ncu dram read+write per cell x cells, profiles/dram_traffic.json)"
     kernels = {k: {"ms": v[0], "launches": v[1], "share": v[0] / total_kernel_ms} for k, v in prof.items()}
     hbm = {"algorithmic_GBps": ALGO_BYTES_PER_CELL_STAGE * cells * 3 * args.steps / (ms * 1e-3) / 1e9,
            "peak_GBps": hbm_gbps, "peak_source": hbm_src}

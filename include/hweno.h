@@ -363,12 +363,12 @@ hweno_status hweno_rerecon_count(hweno_t h, long long* cells);
 /* ---------------------------------------------------------------- batches
  * Many independent 2D Euler problems of different sizes in one handle; every
  * problem is the scheme above on its own grid and boundary kinds.  One batched
- * step is one SSP-RK3 step of every problem, run as one persistent cooperative
- * launch per Runge-Kutta stage (all problems' cells and tiles form one work
- * list), captured in a CUDA graph and replayed.  Phases inside a launch are
- * separated by a grid barrier whose waits are bounded; a wait that gives up
- * sets HWENO_ETIMEOUT (reported by the next synchronising call, which rolls the
- * step back).  All grids must be dim 2, eq Euler, and share precision,
+ * step is one SSP-RK3 step of every problem, run as a launch per phase of each
+ * Runge-Kutta stage (all problems' cells and tiles form one work list), captured
+ * in a CUDA graph and replayed.  With extra arrivals (hweno_batch_set_barrier) a
+ * stage is one persistent cooperative launch whose phases are separated by a
+ * grid barrier with bounded waits; a wait that gives up sets HWENO_ETIMEOUT
+ * (reported by the next synchronising call, which rolls the step back).  All grids must be dim 2, eq Euler, and share precision,
  * indicator, gamma_bar and beta_of_q; cells square per problem.
  *
  * hweno_create_batch: n problems (grids[k], bcs[k]).

@@ -293,8 +293,9 @@ __global__ void __launch_bounds__(RB, (std::is_same<T, float>::value ? 8 : fixed
 // between the barriers is shared by the block.  Measured against a thread per cell
 // (ms per launch, FP64): 64^2 0.065 -> 0.021, 256^2 0.123 -> 0.105, 2048^2
 // 5.67 -> 5.52 (18.1 with the linear part in FP64), troubled cells 0.13 -> 0.11;
-// double-float 2048^2 5.44 -> 5.24 (7.6 in pairs).  FP64: 5 resident blocks per SM;
-// 690 FP64 operations per cell (2330 before), that pipe 80 % busy beside 20 k
+// double-float 2048^2 5.44 -> 5.24 (7.6 in pairs); with the reciprocals and the
+// indicators' squares in integers 4.39 and 4.67.  FP64: 5 resident blocks per SM;
+// 504 FP64 operations per cell (2330 before), that pipe 76 % busy beside 19.8 k
 // integer instructions.  Double-float: 4 blocks, 30 k instructions per cell, the
 // ALU 45 % busy; weights in FP64 beside the integers measured alike.
 template <typename T, int MODE, bool FIX = false>
