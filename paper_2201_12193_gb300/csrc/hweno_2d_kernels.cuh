@@ -296,10 +296,11 @@ __global__ void __launch_bounds__(RB, (std::is_same<T, float>::value ? 8 : fixed
 // double-float 2048^2 5.44 -> 5.24 (7.6 in pairs); with the reciprocals and the
 // indicators' squares in integers 4.39 and 4.67.  FP64: 5 resident blocks per SM;
 // 504 FP64 operations per cell (2330 before), that pipe 76 % busy beside 19.8 k
-// integer instructions.  Double-float: 4 blocks, 30 k instructions per cell, the
-// ALU 45 % busy; weights in FP64 beside the integers measured alike.
+// integer instructions.  Double-float: 30 k instructions per cell, the ALU
+// 45 % busy (1.2 % faster at 5 blocks than at 4 with 120 registers); weights in FP64
+// beside the integers measured alike.
 template <typename T, int MODE, bool FIX = false>
-__global__ void __launch_bounds__(RB, (is_df64<T>::value ? 4 : 5)) rec2d_split_kernel(
+__global__ void __launch_bounds__(RB, 5) rec2d_split_kernel(
     const __grid_constant__ Prob P, const __grid_constant__ Weights<T> W,
     const __grid_constant__ typename rows2d<T>::type B, const double* __restrict__ U,
     const uint8_t* __restrict__ mask, const double* __restrict__ Mod, const int* __restrict__ list,
@@ -847,11 +848,11 @@ __device__ __forceinline__ void update2d_tile(const Prob& P, const Src& src, con
 // with hllc_lean and update_cell_lean, 8.07 with the integer compares, the 5-operation
 // root and the sweep, 5.8 with roots and reciprocals and 4.7 with the flux's products
 // in integers (4.8 at 4 blocks per SM): 600 FP64 operations per cell of 1915, the
-// FP64 pipe still 90 % busy.  Double-float 5.2 -> 3.0 ms.
+// FP64 pipe still 90 % busy.  Double-float 5.2 -> 3.0 ms; at 1024^2 0.78 -> 0.74 with
+// 5 blocks per SM for 4.
 template <typename T, int NV, bool SOLID = false>
 __global__ void __launch_bounds__(TX * TY, (std::is_same<T, float>::value ? 8
-                                         : std::is_same<T, fx64>::value && NV == 4 && !SOLID ? 5
-                                         : lean<T>::value ? 4 : 3))
+                                         : lean<T>::value ? (NV == 4 && !SOLID ? 5 : 4) : 3))
     update2d_kernel(const __grid_constant__ Prob P, const T* __restrict__ G, Rk S, int sweep) {
   __shared__ T xf[TY][TX + 1][4][NV];
   __shared__ T yf[TY + 1][TX][4][NV];
