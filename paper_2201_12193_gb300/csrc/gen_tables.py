@@ -510,7 +510,6 @@ def emit_fx(w, dim, P):
     row_of = {sl[c][j]: r for c in classes for j, r in enumerate(basis[c])}
     cname = {(0, 0): "a", (1, 0): "b", (0, 1): "c", (1, 1): "e"}
     args = ", ".join(f"hwfx::Half2 (&{cname[c]})[{len(cols[c])}]" for c in classes)
-    cargs = ", ".join(f"const hwfx::Half2 (&{cname[c]})[{len(cols[c])}]" for c in classes)
     w("\n// Fixed-point form, on the deviations from the target average (d of it is not read): the classes'\n")
     w("// parity combinations" + ("; c is the x <-> y image of b" if dim == 2 else "") + ".\n")
     w(f"__device__ __forceinline__ void fx_split{dim}d(const long long (&d)[{n}], {args}) {{\n")
@@ -528,9 +527,10 @@ def emit_fx(w, dim, P):
     if dim == 1:
         npt = 4
         w("// x[p] = (c2 q2 + c3 q3 + c4 q4)(point p) - (c2 + c3 + c4) u_5 in fixed point; ca = c2 + c3 weights the\n"
-          "// parts q2 and q3 share.\n")
-        w(f"__device__ __forceinline__ void fx_values1d({cargs}, hwfx::Half2 c2, hwfx::Half2 c3, hwfx::Half2 c4, "
-          f"hwfx::Half2 ca, long long (&x)[{npt}]) {{\n")
+          "// parts q2 and q3 share.  The combinations come in the unit of the level that takes them (a2 those q2 takes,\n"
+          "// ...), each weight in the unit that gives all products one.\n")
+        body, rd = [], set()
+        wb = body.append
         seen = {}
         for bi, b in enumerate(bases):
             for ci, cl in enumerate(classes):
@@ -541,22 +541,26 @@ def emit_fx(w, dim, P):
                     key = (cl,) + tuple((j, str(v)) for j, v in terms)
                     if key not in seen:
                         nm = seen[key] = f"q{lvl}_{ci}_{bi}"
-                        w(f"  hwfx::Half2 {nm};\n  {{")
+                        wb(f"  hwfx::Half2 {nm};\n  {{")
+                        rd.add((lvl, cl))
                         for t, (k, v) in enumerate(terms):
                             h, l = _fx_halves(v)
-                            w(f" hwfx::Acc t = hwfx::prod({cname[cl]}[{k}], {h}, {l});" if t == 0 else
-                              f" hwfx::mac(t, {cname[cl]}[{k}], {h}, {l});")
-                        w(f" {nm} = hwfx::halves(hwfx::scaled<{FX_VF}>(t)); }}\n")
+                            s = f"{cname[cl]}{lvl}[{k}]"
+                            wb(f" hwfx::Acc t = hwfx::prod({s}, {h}, {l});" if t == 0 else
+                              f" hwfx::mac(t, {s}, {h}, {l});")
+                        wb(f" {nm} = hwfx::halves(hwfx::scaled<{FX_VF}>(t)); }}\n")
                     names[lvl] = seen[key]
                 parts = [("ca", names[2]), ("c4", names[4])] if names[2] == names[3] else \
                     [("c2", names[2]), ("c3", names[3]), ("c4", names[4])]
-                w(f"  long long E{ci}_{bi};\n  {{")
+                wb(f"  long long E{ci}_{bi};\n  {{")
                 for t, (c, q) in enumerate(parts):
-                    w(f" hwfx::Acc t = hwfx::prod({q}, {c}.h, {c}.l);" if t == 0 else f" hwfx::mac(t, {q}, {c}.h, {c}.l);")
-                w(f" E{ci}_{bi} = hwfx::scaled<hwfx::CF>(t); }}\n")
+                    wb(f" hwfx::Acc t = hwfx::prod({q}, {c}.h, {c}.l);" if t == 0 else f" hwfx::mac(t, {q}, {c}.h, {c}.l);")
+                wb(f" E{ci}_{bi} = hwfx::scaled<hwfx::CF>(t); }}\n")
             k = b[0]
-            w(f"  x[{k}] = E0_{bi} + E1_{bi};\n  x[{3 - k}] = E0_{bi} - E1_{bi};\n")
-        w("}\n\n")
+            wb(f"  x[{k}] = E0_{bi} + E1_{bi};\n  x[{3 - k}] = E0_{bi} - E1_{bi};\n")
+        args = ", ".join(f"const hwfx::Half2 (&{cname[c]}{lvl})[{len(cols[c])}]" for lvl, c in sorted(rd))
+        w(f"__device__ __forceinline__ void fx_values1d({args}, hwfx::Half2 c2, hwfx::Half2 c3, hwfx::Half2 c4, "
+          f"hwfx::Half2 ca, long long (&x)[{npt}]) {{\n" + "".join(body) + "}\n\n")
     else:
         # value coefficients per base point (|xi|, |eta|) = (.2236, .2236), (.2236, .5), (.5, .2236), (.5, .5)
         def row(lvl, c, b, use):

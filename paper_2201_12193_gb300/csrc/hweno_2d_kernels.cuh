@@ -193,7 +193,7 @@ __device__ __forceinline__ void rec2d_cell(const Prob& P, const Weights<T>& W,
       // the point values go out as they are formed (four base points in turn);
       // the partials read them back below
       T* __restrict__ Gv = G + (long long)(v * 16) * P.gplane + o;
-      recon2d_fx<T>(W, B, d, [&](int p, T x) {
+      recon2d_fixed<T>(W, B, d, [&](int p, T x) {
         Gv[p * P.gplane] = x;
         if (!FLAGGED && v == 0) {
           if constexpr (is_df64<T>::value) nrm = tmax(nrm, tabs(x));

@@ -174,7 +174,11 @@ void build_tables(hweno_s* h) {
   // exponent of a row's value times 2^-61).  first[]: a class's rows of levels 2, 3, 4;
   // times: its data sets (the odd class of 2D has two).
   struct FxClass { int (*first)(int); int nc, times; const double *rl, *rm; int2* out; };
-  auto fill_fx = [&](std::initializer_list<FxClass> cls, int* f) {
+  // elin: a level's indicator is below (4 s max|datum|)^2, s the root of its sum of squares (class
+  // data are sums of up to four), and c_4 is at least 1 / (1 + tau / eps) with tau <= beta^2:
+  // 1/4 for max|datum| <= (3 eps)^(1/4) / (4 s).
+  auto fill_fx = [&](std::initializer_list<FxClass> cls, int* f, int& elin) {
+    long double top = 1.0L;
     for (int l = 0; l < 3; ++l) {
       coef(l + 2, a, b);
       long double sq = 0.0L;
@@ -184,6 +188,7 @@ void build_tables(hweno_s* h) {
           for (int k = 0; k < c.nc; ++k) sum += fabsl(a * c.rl[r * c.nc + k] + b * c.rm[r * c.nc + k]);
           sq += c.times * sum * sum;
         }
+      top = std::max(top, sqrtl(sq));
       const int F = sq > 0.0L ? (int)floorl(62.9L - 0.5L * log2l(sq)) : 60;
       f[l] = 61 - F;
       for (const FxClass& c : cls)
@@ -193,6 +198,7 @@ void build_tables(hweno_s* h) {
           c.out[q] = make_int2((int)((x - lo) >> 32), lo);
         }
     }
+    elin = 1022 + (int)floorl(0.25L * log2l(3e-10L) - log2l(4.0L * top));
   };
   if (h->g.dim == 1) {
     fill(2, hwp::D1P_RC2_2, nullptr, hwp::D1_NB2, h->T.b1f.B2, h->T.b1x.B2, nullptr);
@@ -200,7 +206,8 @@ void build_tables(hweno_s* h) {
     fill(4, hwp::D1P_RC4_4, hwp::D1P_RC4_3, hwp::D1_NB4, h->T.b1f.B4, h->T.b1x.B4, nullptr);
     auto& B = h->T.b1d;
     fill_fx({{hwp::D1_RA, hwp::D1_NCA, 1, &hwp::D1P_AL[0][0], &hwp::D1P_AM[0][0], &B.a[0][0]},
-             {hwp::D1_RB, hwp::D1_NCB, 1, &hwp::D1P_BL[0][0], &hwp::D1P_BM[0][0], &B.b[0][0]}}, B.f);
+             {hwp::D1_RB, hwp::D1_NCB, 1, &hwp::D1P_BL[0][0], &hwp::D1P_BM[0][0], &B.b[0][0]}}, B.f, B.elin);
+    B.w = h->T.wd;
   } else {
     fill(2, hwp::D2P_RC2_2, nullptr, hwp::D2_NB2, h->T.b2f.B2, h->T.b2x.B2, h->T.b2l.B2);
     fill(3, hwp::D2P_RC3_3, hwp::D2P_RC3_2, hwp::D2_NB3, h->T.b2f.B3, h->T.b2x.B3, h->T.b2l.B3);
@@ -208,7 +215,8 @@ void build_tables(hweno_s* h) {
     auto& B = h->T.b2d;
     fill_fx({{hwp::D2_RA, hwp::D2_NCA, 1, &hwp::D2P_AL[0][0], &hwp::D2P_AM[0][0], &B.a[0][0]},
              {hwp::D2_RB, hwp::D2_NCB, 2, &hwp::D2P_BL[0][0], &hwp::D2P_BM[0][0], &B.b[0][0]},
-             {hwp::D2_RE, hwp::D2_NCE, 1, &hwp::D2P_EL[0][0], &hwp::D2P_EM[0][0], &B.e[0][0]}}, B.f);
+             {hwp::D2_RE, hwp::D2_NCE, 1, &hwp::D2P_EL[0][0], &hwp::D2P_EM[0][0], &B.e[0][0]}}, B.f, B.elin);
+    B.w = h->T.wd;
   }
 }
 

@@ -106,12 +106,15 @@ struct Weights {
 template <typename T> struct Beta1 { T B2[hwp::D1_NB2]; T B3[hwp::D1_NB3]; T B4[hwp::D1_NB4]; };
 template <typename T> struct Beta2 { T B2[hwp::D2_NB2]; T B3[hwp::D2_NB3]; T B4[hwp::D2_NB4]; };
 // fx64: the rows in fixed point (hweno_fx.cuh), per parity class and over the class's
-// columns; a coefficient is (x = h, y = l): (h 2^32 + l) 2^-F with F the row's own (the
-// sum of its |coefficients| below 2^63 units), f = 60 - F.
+// columns; a coefficient is (x = h, y = l): (h 2^32 + l) 2^-F with one F a level (the root
+// of the sum of squares of its rows' |coefficient| sums between 2^61.9 and 2^62.9 units, which
+// keeps the Squares below 2^122), f = 61 - F.
 template <int RA, int CA, int RB, int CB, int RE, int CE>
 struct FxRows {
   int2 a[RA][CA], b[RB][CB], e[RE][CE];
-  int f[3];           // the unit of a level's rows is 2^f
+  int f[3];           // a row's value times 2^-61 has the unit 2^f
+  int elin;           // data with exponents up to it leave c_4 at least 1/4 (fx_uneven)
+  Weights<fx64> w;    // for recon2d_levels (double-float kernels hold theirs in pairs)
 };
 template <> struct Beta1<fx64> : FxRows<hwp::D1_NRA, hwp::D1_NCA, hwp::D1_NRB, hwp::D1_NCB, 1, 1> {};
 template <> struct Beta2<fx64>
@@ -620,24 +623,45 @@ __device__ __forceinline__ void fx_row(const hwfx::Half2 (&s)[N], const int2 (&c
   hwfx::add_square(q, hwfx::scaled<61>(t));
 }
 
+// A weight's exponent (2047: not finite), and the weight in units of 2^(e - 1022 - CBITS).
+__device__ __forceinline__ int cexp(fx64 c) { return hwfx::bexp(c.v); }
+__device__ __forceinline__ int cexp(df64 c) {
+  const int f = (int)((__float_as_uint(c.hi) >> 23) & 0xFF);
+  return f == 0xFF ? 0x7FF : f + 896;
+}
+__device__ __forceinline__ hwfx::Half2 cfixed(fx64 c, int e) { return hwfx::halves(hwfx::to_fx<hwfx::CBITS>(c.v, e)); }
+__device__ __forceinline__ hwfx::Half2 cfixed(df64 c, int e) {
+  return hwfx::halves(hwfx::to_fx<hwfx::CBITS>(c.hi, e) + hwfx::to_fx<hwfx::CBITS>(c.lo, e));
+}
+
+// Data of different size.  A datum is kept to 2^-57 of the largest that shares its
+// exponent.  That is FP64's accuracy as long as the result is of that datum's size.  But
+// the first moments enter only q_3 (the cell's own) and q_4, and where they are
+// large against the averages the weights discard those: what remains would be left
+// with the low bits of q_2's data (one exponent for all: 5e-9 of the values at a ratio of
+// 1e8).  So each level's data have the unit of the largest datum that the level takes,
+// and the weights the units that give c_l q_l one (that of the largest product).
+// 1D does so throughout; in 2D, where three sets of class data would not fit the
+// registers, the stencils with uneven data leave for recon2d_levels: those whose first
+// moments' exponent em exceeds that of the averages' differences (ea) and of the average
+// (eu: the value's own rounding) by more than `slack`: 1 for fx64 (a truncation below 2^-55 of
+// the scale, FP64's rounding being 2^-54), 8 for double-float (2^-48, the pairs' is
+// 2^-47).  Data below 2^(elin - 1022) leave c_4 at least 1/4 (their indicators are not much
+// above the weights' eps): q_4 is not discarded and its largest datum is the scale, which
+// keeps the small momenta of gas nearly at rest in the one-exponent form.
+template <typename T>
+__device__ __forceinline__ bool fx_uneven(int ea, int em, int eu, int elin) {
+  constexpr int slack = is_df64<T>::value ? 8 : 1;
+  return em > max(ea, eu) + slack && em > elin;
+}
+
 // The weights c_2, c_3, c_4, c_2 + c_3 as fixed-point integers of one exponent;
 // returns it (2047 if one is not finite).
-__device__ __forceinline__ int fx_weights(const fx64 (&c)[4], hwfx::Half2 (&h)[4]) {
-  const int e = max(max(max(hwfx::bexp(c[0].v), hwfx::bexp(c[1].v)), max(hwfx::bexp(c[2].v), hwfx::bexp(c[3].v))),
-                    hwfx::CEMIN);
+template <typename T>
+__device__ __forceinline__ int fx_weights(const T (&c)[4], hwfx::Half2 (&h)[4]) {
+  const int e = max(max(max(cexp(c[0]), cexp(c[1])), max(cexp(c[2]), cexp(c[3]))), hwfx::CEMIN);
 #pragma unroll
-  for (int k = 0; k < 4; ++k) h[k] = hwfx::halves(hwfx::to_fx<hwfx::CBITS>(c[k].v, e));
-  return e;
-}
-__device__ __forceinline__ int fx_weights(const df64 (&c)[4], hwfx::Half2 (&h)[4]) {
-  int f = 1;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) f = max(f, (int)((__float_as_uint(c[k].hi) >> 23) & 0xFF));
-  if (f == 0xFF) f = 0x7FF - 896;
-  const int e = f + 896;
-#pragma unroll
-  for (int k = 0; k < 4; ++k)
-    h[k] = hwfx::halves(hwfx::to_fx<hwfx::CBITS>(c[k].hi, e) + hwfx::to_fx<hwfx::CBITS>(c[k].lo, e));
+  for (int k = 0; k < 4; ++k) h[k] = cfixed(c[k], e);
   return e;
 }
 
@@ -649,24 +673,28 @@ __device__ __forceinline__ void recon1d_fp64(const Weights<fx64>& W, const Beta1
                                              fx64 (&out)[4]) {
   const double dl = d[1].v - d[0].v, dr = d[2].v - d[1].v;
   const double dv[6] = {-dl, 0.0, dr, d[3].v, d[4].v, d[5].v};
-  int e = hwfx::EMIN;
-#pragma unroll
-  for (int k = 0; k < 6; ++k) if (k != 1) e = max(e, hwfx::bexp(dv[k]));
+  // the exponents of the data of q_2, q_3 and q_4
+  const int e2 = max(hwfx::EMIN, max(hwfx::bexp(dl), hwfx::bexp(dr))), e3 = max(e2, hwfx::bexp(dv[4]));
+  const int e4 = max(e3, max(hwfx::bexp(dv[3]), hwfx::bexp(dv[5])));
   long long q[6];
 #pragma unroll
-  for (int k = 0; k < 6; ++k) q[k] = k == 1 ? 0 : hwfx::to_fx<hwfx::BITS>(dv[k], e);
-  hwfx::Half2 sa[2], sb[3];
-  hwp::fx_split1d(q, sa, sb);
+  for (int k = 0; k < 6; ++k) q[k] = k == 1 ? 0 : hwfx::to_fx<hwfx::BITS>(dv[k], k < 3 ? e2 : k == 4 ? e3 : e4);
+  const int s3 = min(e3 - e2, 63), s4 = min(e4 - e2, 63), s34 = min(e4 - e3, 63);
+  const long long qs = q[0] + q[2], qd = q[0] - q[2];
+  hwfx::Half2 a2[2], b2[3];            // each at the exponent of the level that brought it in
+  hwp::fx_split1d(q, a2, b2);
+  hwfx::Half2 a3[2] = {hwfx::halves(qs >> s3), a2[1]}, a4[2] = {hwfx::halves(qs >> s4), a2[1]};
+  hwfx::Half2 b3[3] = {hwfx::halves(qd >> s3), b2[1], b2[2]};
+  hwfx::Half2 b4[3] = {hwfx::halves(qd >> s4), b2[1], hwfx::halves(q[4] >> s34)};
   fx64 beta[4];
-  const int e0 = e - (1022 + hwfx::BITS);
 #pragma unroll
   for (int l = 0; l < 3; ++l) {
     hwfx::Squares bl{0, 0, 0};
 #pragma unroll
-    for (int r = hwp::D1_RA(l); r < hwp::D1_RA(l + 1); ++r) fx_row(sa, B.a[r], bl);
+    for (int r = hwp::D1_RA(l); r < hwp::D1_RA(l + 1); ++r) fx_row(l == 0 ? a2 : l == 1 ? a3 : a4, B.a[r], bl);
 #pragma unroll
-    for (int r = hwp::D1_RB(l); r < hwp::D1_RB(l + 1); ++r) fx_row(sb, B.b[r], bl);
-    beta[l + 1] = from_squares<fx64>(bl, 2 * (e0 + B.f[l]));
+    for (int r = hwp::D1_RB(l); r < hwp::D1_RB(l + 1); ++r) fx_row(l == 0 ? b2 : l == 1 ? b3 : b4, B.b[r], bl);
+    beta[l + 1] = from_squares<fx64>(bl, 2 * ((l == 0 ? e2 : l == 1 ? e3 : e4) - (1022 + hwfx::BITS) + B.f[l]));
   }
   // beta_1: eqs. (beta1-LR), (tau1), (w1_-LR), (w1-LR), (beta1) over a common denominator
   {
@@ -678,12 +706,14 @@ __device__ __forceinline__ void recon1d_fp64(const Weights<fx64>& W, const Beta1
   }
   fx64 c[4];
   weights_c(W, beta, c);
-  hwfx::Half2 h[4];
-  const int ec = fx_weights(c, h);
+  const int x2 = max(cexp(c[0]), cexp(c[3])), x3 = cexp(c[1]), x4 = cexp(c[2]);
+  const int eu = max(max(x2 + e2, x3 + e3), e4 + max(x4, hwfx::CEMIN));   // the largest product's exponent
   long long x[4];
-  hwp::fx_values1d(sa, sb, h[0], h[1], h[2], h[3], x);
-  const double u = e > hwfx::EMAX || ec == 0x7FF ? __longlong_as_double(0x7FF8000000000000LL) : d[1].v;
-  const int eb = ec + e + (hwfx::CF - (1022 + hwfx::CBITS) - (1022 + hwfx::BITS));
+  hwp::fx_values1d(a2, b2, b3, a4, b4, cfixed(c[0], eu - e2), cfixed(c[1], eu - e3), cfixed(c[2], eu - e4),
+                   cfixed(c[3], eu - e2), x);
+  const bool bad = e4 > hwfx::EMAX || max(x2, max(x3, x4)) == 0x7FF;
+  const double u = bad ? __longlong_as_double(0x7FF8000000000000LL) : d[1].v;
+  const int eb = eu + (hwfx::CF - (1022 + hwfx::CBITS) - (1022 + hwfx::BITS));
 #pragma unroll
   for (int p = 0; p < 4; ++p) out[p] = u + hwfx::from_fx(x[p], eb);
 }
@@ -761,35 +791,45 @@ __device__ __forceinline__ T beta1_2d(const Weights<T>& W, T a, T b, T g, T h) {
 // fx64 and double-float: the linear part in block fixed point (hweno_fx.cuh).  The beta rows and
 // the four base points (+-|xi|, +-|eta|) run as loops over coefficient tables:
 // unrolled, a variable's code is 100 KB and the warps wait for instructions.
-template <typename T, typename Put>
-__device__ __forceinline__ void recon2d_fx(const Weights<T>& W, const Beta2<fx64>& B, const double (&d)[23], Put put) {
+// dv: the data as deviations from the average u5 (dv[4] = u5 itself).
+// e: the exponents of the data of q_2, q_3 and q_4.  LEVELS (uneven data): each level's data in
+// its own unit, as in recon1d_fp64; otherwise, and bit for bit where the three are the
+// same, all in that of e[2].
+template <bool LEVELS, typename T, typename Put>
+__device__ __forceinline__ void recon2d_fx(const Weights<T>& W, const Beta2<fx64>& B, const double (&dv)[23],
+                                           const int (&e)[3], Put put) {
   using hwfx::Half2;
-  const double u5 = d[4];
-  double dv[23];
-#pragma unroll
-  for (int k = 0; k < 23; ++k) dv[k] = k < 9 ? d[k] - u5 : d[k];
-  int e = hwfx::EMIN;
-#pragma unroll
-  for (int k = 0; k < 23; ++k) if (k != 4) e = max(e, hwfx::bexp(dv[k]));
+  const double u5 = dv[4];
   Half2 sa[7], sb[6], sc[6], se[3];   // parity classes (even, even), (odd, even), (even, odd), (odd, odd)
   {
     long long q[23];
 #pragma unroll
-    for (int k = 0; k < 23; ++k) q[k] = k == 4 ? 0 : hwfx::to_fx<hwfx::BITS>(dv[k], e);
+    for (int k = 0; k < 23; ++k) {
+      const int l = !LEVELS || !(k < 9 || k == 12 || k == 19) ? 2 : k < 9 ? 0 : 1;   // the level that brings it in
+      q[k] = k == 4 ? 0 : hwfx::to_fx<hwfx::BITS>(dv[k], e[l]);
+    }
     hwp::fx_split2d(q, sa, sb, sc, se);
   }
+  [[maybe_unused]] Half2 a2[3], e2, b2[2], c2[2], b3[6], c3[6];   // LEVELS: what q_2 and q_3 take, in their units
   T beta[4];
   {
-    const int e0 = e - (1022 + hwfx::BITS);
     int ra = 0, rb = 0, re = 0;
 #pragma unroll 1
     for (int l = 0; l < 3; ++l) {
+      if constexpr (LEVELS) {   // from the last level's unit to this one's
+        const int s = l == 0 ? 0 : min(e[l] - e[l - 1], 63);
+        auto shift = [s](Half2& x) { x = hwfx::halves((((long long)x.h << 32) + x.l) >> s); };
+        if (l > 0) {
+          shift(sa[0]); shift(sa[1]); shift(sa[2]); shift(sb[0]); shift(sb[1]); shift(sc[0]); shift(sc[1]); shift(se[0]);
+          if (l == 2) { shift(sb[4]); shift(sc[4]); }
+        }
+      }
       const int na = l == 0 ? hwp::D2_RA(1) : l == 1 ? hwp::D2_RA(2) : hwp::D2_RA(3);
       const int nb = l == 0 ? hwp::D2_RB(1) : l == 1 ? hwp::D2_RB(2) : hwp::D2_RB(3);
       const int ne = l == 0 ? hwp::D2_RE(1) : l == 1 ? hwp::D2_RE(2) : hwp::D2_RE(3);
       hwfx::Squares q{0, 0, 0};
 #pragma unroll 1
-      for (; ra < na; ++ra) fx_row(sa, B.a[ra], q);
+      for (; ra < na; ++ra) fx_row(sa, B.a[ra], q);   // (a lower level's rows are zero where a higher one's data are)
 #pragma unroll 1
       for (; rb < nb; ++rb) {   // the same rows for both odd classes (x <-> y images)
         fx_row(sb, B.b[rb], q);
@@ -797,17 +837,36 @@ __device__ __forceinline__ void recon2d_fx(const Weights<T>& W, const Beta2<fx64
       }
 #pragma unroll 1
       for (; re < ne; ++re) fx_row(se, B.e[re], q);
-      const T bl = from_squares<T>(q, 2 * (e0 + B.f[l]));
+      const T bl = from_squares<T>(q, 2 * (e[LEVELS ? l : 2] - (1022 + hwfx::BITS) + B.f[l]));
       if (l == 0) beta[1] = bl; else if (l == 1) beta[2] = bl; else beta[3] = bl;
+      if constexpr (LEVELS) {
+        if (l == 0) {
+          a2[0] = sa[0]; a2[1] = sa[1]; a2[2] = sa[2]; e2 = se[0];
+          b2[0] = sb[0]; b2[1] = sb[1]; c2[0] = sc[0]; c2[1] = sc[1];
+        } else if (l == 1) {
+          b3[0] = sb[0]; b3[1] = sb[1]; b3[4] = sb[4];
+          c3[0] = sc[0]; c3[1] = sc[1]; c3[4] = sc[4];
+        }
+      }
     }
   }
   beta[0] = beta1_2d<T>(W, from_double<T>(-dv[3]), from_double<T>(dv[5]), from_double<T>(-dv[1]), from_double<T>(dv[7]));
   T c[4];
   weights_c(W, beta, c);
   Half2 hc[4];
-  const int ec = fx_weights(c, hc);
-  const T u = from_double<T>(e > hwfx::EMAX || ec == 0x7FF ? __longlong_as_double(0x7FF8000000000000LL) : u5);
-  const int eb = ec + e + (hwfx::CF - (1022 + hwfx::CBITS) - (1022 + hwfx::BITS));
+  int ec, eu;                          // the largest exponent of a weight, of a product
+  if constexpr (LEVELS) {
+    const int x2 = max(cexp(c[0]), cexp(c[3])), x3 = cexp(c[1]), x4 = cexp(c[2]);
+    ec = max(x2, max(x3, x4));
+    eu = max(max(x2 + e[0], x3 + e[1]), max(x4, hwfx::CEMIN) + e[2]);
+    hc[0] = cfixed(c[0], eu - e[0]); hc[1] = cfixed(c[1], eu - e[1]);
+    hc[2] = cfixed(c[2], eu - e[2]); hc[3] = cfixed(c[3], eu - e[0]);
+  } else {
+    ec = fx_weights(c, hc);
+    eu = ec + e[2];
+  }
+  const T u = from_double<T>(e[2] > hwfx::EMAX || ec == 0x7FF ? __longlong_as_double(0x7FF8000000000000LL) : u5);
+  const int eb = eu + (hwfx::CF - (1022 + hwfx::CBITS) - (1022 + hwfx::BITS));
   using namespace hwp;
 #pragma unroll 1
   for (int b = 0; b < 4; ++b) {
@@ -829,27 +888,28 @@ __device__ __forceinline__ void recon2d_fx(const Weights<T>& W, const Beta2<fx64
       return hwfx::scaled<hwfx::CF>(t);
     };
     {
-      hwfx::Acc t = dot(D2_VA2[b][0], sa[0]);
-      add(t, D2_VA2[b][1], sa[1]); add(t, D2_VA2[b][2], sa[2]);
+      auto x2 = [&](int k) -> const Half2& { if constexpr (LEVELS) return a2[k]; else return sa[k]; };
+      hwfx::Acc t = dot(D2_VA2[b][0], x2(0));
+      add(t, D2_VA2[b][1], x2(1)); add(t, D2_VA2[b][2], x2(2));
       hwfx::Acc r = dot(D2_VA4[b][0], sa[0]);
 #pragma unroll
       for (int k = 1; k < 7; ++k) add(r, D2_VA4[b][k], sa[k]);
       E[0] = comb_a(fin(t), fin(r));
     }
-    auto odd = [&](int p, const Half2 (&x)[6]) {
-      hwfx::Acc t = dot(D2_VB2[p][0], x[0]);
-      add(t, D2_VB2[p][1], x[1]);
-      hwfx::Acc r = dot(D2_VB3[p][0], x[0]);
-      add(r, D2_VB3[p][1], x[1]); add(r, D2_VB3[p][2], x[4]);
+    auto odd = [&](int p, const Half2* x2, const Half2* x3, const Half2 (&x)[6]) {
+      hwfx::Acc t = dot(D2_VB2[p][0], x2[0]);
+      add(t, D2_VB2[p][1], x2[1]);
+      hwfx::Acc r = dot(D2_VB3[p][0], x3[0]);
+      add(r, D2_VB3[p][1], x3[1]); add(r, D2_VB3[p][2], x3[4]);
       hwfx::Acc z = dot(D2_VB4[p][0], x[0]);
 #pragma unroll
       for (int k = 1; k < 6; ++k) add(z, D2_VB4[p][k], x[k]);
       return comb(fin(t), fin(r), fin(z));
     };
-    E[1] = odd(b, sb);
-    E[2] = odd(bt, sc);
+    E[1] = odd(b, LEVELS ? b2 : sb, LEVELS ? b3 : sb, sb);
+    E[2] = odd(bt, LEVELS ? c2 : sc, LEVELS ? c3 : sc, sc);
     {
-      hwfx::Acc t = dot(D2_VE2[b][0], se[0]);
+      hwfx::Acc t = dot(D2_VE2[b][0], LEVELS ? e2 : se[0]);
       hwfx::Acc r = dot(D2_VE4[b][0], se[0]);
       add(r, D2_VE4[b][1], se[1]); add(r, D2_VE4[b][2], se[2]);
       E[3] = comb_a(fin(t), fin(r));
@@ -863,13 +923,57 @@ __device__ __forceinline__ void recon2d_fx(const Weights<T>& W, const Beta2<fx64
   }
 }
 
+// The form for stencils of uneven data, as a call: the common one keeps its registers.
+static __device__ __noinline__ void recon2d_levels(const Beta2<fx64>& B, const double (&dv)[23], int ea, int eo, int em,
+                                                   double (&out)[16]) {
+  const int e[3] = {ea, eo, em};
+  recon2d_fx<true, fx64>(B.w, B, dv, e, [&](int p, fx64 x) { out[p] = x.v; });
+}
+
+// Either.  fx64: for a whole warp, since with one exponent the two agree bit for bit and a
+// warp that held both kinds would run one after the other (double Mach 800 x 200, two steps:
+// 3.03 ms with one exponent for all, 3.10 so, 3.17 by the stencil, 3.20 in plain FP64).
+// Double-float, whose common form has its weights in pairs: by the stencil.
+template <typename T, typename Put>
+__device__ __forceinline__ void recon2d_fixed(const Weights<T>& W, const Beta2<fx64>& B, const double (&d)[23], Put put) {
+  const double u5 = d[4];
+  double dv[23];
+  int ea = hwfx::EMIN, em = 0;
+#pragma unroll
+  for (int k = 0; k < 23; ++k) {
+    dv[k] = k < 9 && k != 4 ? d[k] - u5 : d[k];
+    if (k < 9 && k != 4) ea = max(ea, hwfx::bexp(dv[k]));
+    else if (k > 8) em = max(em, hwfx::bexp(dv[k]));
+  }
+  const bool uneven = fx_uneven<T>(ea, em, hwfx::bexp(u5), B.elin);
+  const int eo = max(ea, max(hwfx::bexp(dv[12]), hwfx::bexp(dv[19])));   // (the cell's own first moments)
+  em = max(ea, em);
+  bool levels = uneven;
+  if constexpr (std::is_same<T, fx64>::value) levels = __any_sync(__activemask(), uneven);
+  double x[23];
+  if (levels) {                        // (kept apart from the call: there the data need no registers)
+#pragma unroll
+    for (int k = 0; k < 23; ++k) x[k] = dv[k];
+  } else {
+    const int e[3] = {em, em, em};
+    recon2d_fx<false, T>(W, B, dv, e, put);
+  }
+  asm volatile("" ::: "memory");
+  if (levels) {
+    double y[16];
+    recon2d_levels(B, x, uneven ? ea : em, uneven ? eo : em, em, y);
+#pragma unroll 1
+    for (int p = 0; p < 16; ++p) put(p, from_double<T>(y[p]));
+  }
+}
+
 template <typename T, typename Put>
 __device__ __forceinline__ void recon2d(const Weights<T>& W, const Beta2<T>& B, const T (&d)[23], Put put) {
   if constexpr (std::is_same<T, fx64>::value) {
     double x[23];
 #pragma unroll
     for (int k = 0; k < 23; ++k) x[k] = d[k].v;
-    recon2d_fx<T>(W, B, x, put);
+    recon2d_fixed<T>(W, B, x, put);
     return;
   } else {
   T s[23];
