@@ -46,10 +46,11 @@ __device__ __forceinline__ long long scaled(const Acc& s) {
 }
 
 constexpr int BITS = 57;        // data: |d| < 2^BITS units
-constexpr int EMIN = 500;       // smallest block exponent (biased): variations below 2^-580 vanish
+constexpr int EMIN = 64;        // smallest block exponent (biased; to_fx asks for 64): the unit is 2^-1015 then,
+                                // about the smallest normal double
 constexpr int EMAX = 1900;      // largest one: above it the FP64 weights overflow (they are not finite)
 constexpr int CBITS = 61;       // weights c_k: |c| < 2^CBITS units
-constexpr int CEMIN = 700;
+constexpr int CEMIN = 64;
 constexpr int CF = 61;          // the weighted sums keep the product times 2^-CF
 
 __device__ __forceinline__ int bexp(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
@@ -101,14 +102,16 @@ __device__ __forceinline__ double sum_of(const Squares& s, int e) {
   return __longlong_as_double(f >= 2046 ? 0x7FF0000000000000LL : (long long)r);
 }
 
-// x 2^eb as a double (integer work; rounded to 53 bits, halves up).  The caller keeps the exponent in range.
+// x 2^eb as a double (integer work; rounded to 53 bits, halves up); results below 2^-1022 become 0, the
+// caller keeps them below the largest.
 __device__ __forceinline__ double from_fx(long long x, int eb) {
   const long long s = x >> 63;
   const unsigned long long a = (unsigned long long)((x ^ s) - s);
   const int n = __clzll((long long)a);
   const unsigned long long m = (((a << (n & 63)) >> 10) + 1) >> 1;   // a carry to 2^53 raises the exponent
-  const unsigned long long r = m + ((unsigned long long)(unsigned)(1085 - n + eb) << 52);
-  return __longlong_as_double(a ? (long long)(r | ((unsigned long long)s << 63)) : 0LL);
+  const int f = 1085 - n + eb;                       // the biased exponent less 1
+  const unsigned long long r = m + ((unsigned long long)(unsigned)f << 52);
+  return __longlong_as_double(a && f >= 0 ? (long long)(r | ((unsigned long long)s << 63)) : 0LL);
 }
 
 // x 2^eb as a double-float pair hi + lo (truncated to 48 bits); magnitudes below 2^-126 become 0.
