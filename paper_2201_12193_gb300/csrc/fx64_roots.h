@@ -12,8 +12,8 @@
 // The residual comes from the low words of a product whose high words cancel.
 // What the series leaves out is below 2^-58 relative, the truncations of the
 // fixed point below 2^-59; the result is rounded to 53 bits once, to within 0.52
-// units in the last place (the FP64 steps had 0.75).  Plain C++: also compiled
-// for the host.
+// units in the last place, and the sign of the remainder corrects it to the nearest
+// (rcp_nearest, sqrt_nearest).  Plain C++: also compiled for the host.
 #pragma once
 
 #include <stdint.h>

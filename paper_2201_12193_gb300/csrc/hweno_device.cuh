@@ -252,8 +252,7 @@ __device__ __forceinline__ double avg_img(const Prob& P, const double* __restric
 // ---------------------------------------------------------------- physics
 // Physical flux of eq. (1D-Euler) / (2D-Euler) or of the scalar laws in
 // direction dir (0 = x, 1 = y); NV = 1 (scalar), 3 (1D Euler), 4 (2D Euler).
-// 1/x.  FP32, double: correctly rounded (double in integers).  fx64: in integers,
-// within 0.52 units in the last place.
+// 1/x, correctly rounded in FP32, double and fx64 (the latter two in integers).
 template <typename T> __device__ __forceinline__ T rcp(T x) { return T(1) / x; }
 template <> __device__ __forceinline__ float rcp<float>(float x) { return __frcp_rn(x); }
 template <> __device__ __forceinline__ double rcp<double>(double x) { return rcp_ieee(x); }
