@@ -1162,7 +1162,7 @@ __device__ __forceinline__ bool nonphysical(double rho, double m, double n, doub
 // Bounds of an Euler average's |velocity| + sound speed per direction from FP32
 // copies: lo <= exact <= hi.  Truncating the conserved values and the FP32
 // arithmetic err by less than 2^-20 relative, the pressure by 2^-20 of E + kinetic
-// energy.  What falls below FP32's normal range (a momentum, its product with the
+// energy (gamma - 1 is rounded from FP64: in FP32 it cancels near 1).  What falls below FP32's normal range (a momentum, its product with the
 // velocity) is below 1e-38 absolute, which density, E and the squared sound speed inside the
 // limits leave far below those margins.  Outside them, and for a non-physical or barely
 // physical average, hi = infinity and lo = 0: the cell takes the exact speed.
@@ -1171,7 +1171,7 @@ __device__ __forceinline__ void speed_bounds(const Prob& P, const double* __rest
   const float r = f32_trunc(U[sidx(P, 0, 0, i, j)]), m = f32_trunc(U[sidx(P, 1, 0, i, j)]);
   const float n = P.nvar == 4 ? f32_trunc(U[sidx(P, 2, 0, i, j)]) : 0.0f, E = f32_trunc(U[sidx(P, P.nvar - 1, 0, i, j)]);
   const float ri = 1.0f / r, u = fabsf(m) * ri, w = fabsf(n) * ri, ke = 0.5f * (fabsf(m) * u + fabsf(n) * w);
-  const float p = E - ke, d = 1e-6f * (E + ke), gg = P.cgamma.f * (P.cgamma.f - 1.0f) * ri, c2 = gg * (p + d);
+  const float p = E - ke, d = 1e-6f * (E + ke), gg = P.cgamma.f * P.cgm1.f * ri, c2 = gg * (p + d);
   const float cl = sqrtf(gg * (p - d)) * 0.999998f, ch = sqrtf(c2) * 1.000002f;
   const bool ok = r > 1e-15f && r < 1e15f && E > 1e-15f && E < 1e15f && p > d && c2 > 1e-30f && c2 < 1e30f;
   lo[0] = ok ? u * 0.999998f + cl : 0.0f;

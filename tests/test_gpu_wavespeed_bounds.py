@@ -39,7 +39,7 @@ def _speeds(r, u, v, p, gamma):
     return (np.abs(u) + c).max(), (np.abs(v) + c).max()
 
 
-CASES = [("thin", 1.4), ("thin", 3.0), ("thin at rest", 1.4), ("close", 1.4)]
+CASES = [("thin", 1.4), ("thin", 3.0), ("thin at rest", 1.4), ("close", 1.0001), ("close", 1.01), ("close", 1.4)]
 
 
 # the kernel's speeds: a few FP64 roundings of 2^-53, amplified by the pressure's cancellation: the
