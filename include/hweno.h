@@ -369,7 +369,10 @@ hweno_status hweno_rerecon_count(hweno_t h, long long* cells);
  * stage is one persistent cooperative launch whose phases are separated by a
  * grid barrier with bounded waits; a wait that gives up sets HWENO_ETIMEOUT
  * (reported by the next synchronising call, which rolls the step back).  All grids must be dim 2, eq Euler, and share precision,
- * indicator, gamma_bar and beta_of_q; cells square per problem.
+ * indicator, gamma_bar and beta_of_q; cells square per problem.  The calls for
+ * single-problem handles that launch work (hweno_step, hweno_stage,
+ * hweno_advance, hweno_max_dt, hweno_wave_speeds, hweno_totals, hweno_rhs)
+ * return HWENO_ESTATE on a batch handle.
  *
  * hweno_create_batch: n problems (grids[k], bcs[k]).
  * hweno_batch_set_moments / get_moments: problem k's moments in the state

@@ -344,7 +344,7 @@ hweno_status read_speeds(hweno_t h) {
   hw::run_wavespeed(h->P, h->U[h->cur], h->red_part, h->red_out, nullptr, nullptr, h->B.status, h->stream);
   CK(h, cudaMemcpyAsync(h->host_buf, h->red_out, 3 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   CK(h, cudaStreamSynchronize(h->stream));
-  return h->host_buf[2] != 0.0 || h->batch ? check_status(h) : HWENO_OK;
+  return h->host_buf[2] != 0.0 ? check_status(h) : HWENO_OK;
 }
 
 // every inflow side has its fixed states
@@ -599,6 +599,7 @@ void finish_step(hweno_t h, int a, double dt) {
 
 hweno_status hweno_step(hweno_t h, double dt) {
   if (!h) return HWENO_EINVAL;
+  if (h->batch) return fail(h, HWENO_ESTATE, "step: single-problem handles only (hweno_step_batch)");
   if (h->next_stage != 0) return fail(h, HWENO_ESTATE, "step: a step begun with hweno_stage is not finished");
   const hweno_status s = step_checks(h, dt, "step");
   if (s != HWENO_OK) return s;
@@ -787,6 +788,7 @@ hweno_status hweno_advance(hweno_t h, double t_end, double cfl, long long max_st
 
 hweno_status hweno_max_dt(hweno_t h, double cfl, double* dt_out) {
   if (!h || !dt_out) return HWENO_EINVAL;
+  if (h->batch) return fail(h, HWENO_ESTATE, "max_dt: single-problem handles only");
   if (!h->have_state) return fail(h, HWENO_ESTATE, "max_dt: no moments set");
   if (!(cfl > 0.0)) return fail(h, HWENO_EINVAL, "max_dt: cfl must be positive");
   const hweno_status s = read_speeds(h);
@@ -813,6 +815,7 @@ hweno_status hweno_troubled_mask(hweno_t h, unsigned char* mask, size_t count) {
 
 hweno_status hweno_totals(hweno_t h, double* sums) {
   if (!h || !sums) return HWENO_EINVAL;
+  if (h->batch) return fail(h, HWENO_ESTATE, "totals: single-problem handles only");
   if (!h->have_state) return fail(h, HWENO_ESTATE, "totals: no moments set");
   hweno_status s = check_status(h);
   if (s != HWENO_OK) return s;
@@ -826,6 +829,7 @@ hweno_status hweno_totals(hweno_t h, double* sums) {
 
 hweno_status hweno_rhs(hweno_t h, const double* U, double* Umod, double* L, unsigned char* mask, double* aleph) {
   if (!h) return HWENO_EINVAL;
+  if (h->batch) return fail(h, HWENO_ESTATE, "rhs: single-problem handles only");
   if (!U || !Umod || !L || !mask) return fail(h, HWENO_EINVAL, "rhs: U, Umod, L and mask are required");
   if (h->g.indicator == 3 && !h->have_mlp) return fail(h, HWENO_ESTATE, "rhs: learned indicator not set (hweno_set_mlp)");
   Prob P = h->P;           // caller arrays are unpadded
