@@ -365,11 +365,13 @@ hweno_status hweno_rerecon_count(hweno_t h, long long* cells);
  * problem is the scheme above on its own grid and boundary kinds.  One batched
  * step is one SSP-RK3 step of every problem, run as a launch per phase of each
  * Runge-Kutta stage (all problems' cells and tiles form one work list), captured
- * in a CUDA graph and replayed.  With extra arrivals (hweno_batch_set_barrier) a
- * stage is one persistent cooperative launch whose phases are separated by a
- * grid barrier with bounded waits; a wait that gives up sets HWENO_ETIMEOUT
- * (reported by the next synchronising call, which rolls the step back).  All grids must be dim 2, eq Euler, and share precision,
- * indicator, gamma_bar and beta_of_q; cells square per problem.  The calls for
+ * in a CUDA graph and replayed.  After hweno_batch_set_barrier a stage is one
+ * persistent cooperative launch whose phases are separated by a grid barrier
+ * with bounded waits (the same results, slower: 4 problems of 13 k cells in
+ * FP64 1.03 against 0.57 ms a step, 64 of 3.8 M cells 44 against 41); a wait
+ * that gives up sets HWENO_ETIMEOUT (reported by the next synchronising call,
+ * which rolls the step back).  All grids must be dim 2, eq Euler, and share
+ * precision, indicator, gamma_bar and beta_of_q; cells square per problem.  The calls for
  * single-problem handles that launch work (hweno_step, hweno_stage,
  * hweno_advance, hweno_max_dt, hweno_wave_speeds, hweno_totals, hweno_rhs)
  * return HWENO_ESTATE on a batch handle.
@@ -391,14 +393,14 @@ hweno_status hweno_step_batch(hweno_t h, const double* dt_device, double cfl);
 hweno_status hweno_batch_dt(hweno_t h, double* dt, int n);
 hweno_status hweno_batch_troubled_mask(hweno_t h, int k, unsigned char* mask, size_t count);
 hweno_status hweno_batch_set_tile(hweno_t h, int variant);
-/* Bound of the grid barrier's waits (no counterpart in the paper): a wait
- * gives up after spin_limit polls (64 ns sleeps each; default 2^26, seconds),
- * sets HWENO_ETIMEOUT for the next synchronising call (which rolls the step
+/* Runs the handle's stages as one persistent launch each from the next
+ * hweno_step_batch on, and bounds its grid barrier's waits (no counterpart in
+ * the paper): a wait gives up after spin_limit polls (64 ns sleeps each; default
+ * 2^26, seconds), sets HWENO_ETIMEOUT for the next synchronising call (which rolls the step
  * back) and lets the block continue, so no wait can hang the GPU.
  * extra_arrivals (0 normally, at most 1024) makes every barrier wait for that
  * many arrivals beyond the launched blocks, so every wait runs out: the way to
- * exercise the timeout path without faulting anything.  Takes effect from the
- * next hweno_step_batch. */
+ * exercise the timeout path without faulting anything. */
 hweno_status hweno_batch_set_barrier(hweno_t h, long long spin_limit, int extra_arrivals);
 /* 1 if the last batched step was replayed from a captured CUDA graph, 0 if its
  * launches were issued directly (capture unavailable), -1 for a non-batch handle. */

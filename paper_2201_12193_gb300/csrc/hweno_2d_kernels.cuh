@@ -1417,12 +1417,11 @@ __global__ void __launch_bounds__(TXV * TYV) batch_stage_kernel(const __grid_con
 // size (ms per step, persistent / per phase: 4 problems of 13 k cells FP32
 // 0.29 / 0.20, FP64 1.03 / 0.57; 64 problems of 3.8 M cells FP32 8.3 / 5.5, FP64
 // 44 / 41; FP32 9.0 with its moments converted per gather).  The persistent form
-// remains where the caller sets the barrier up (hweno_batch_set_barrier with extra
-// arrivals).
+// runs where the caller sets its barrier up (hweno_batch_set_barrier).
 template <typename T, int TXV, int TYV>
 cudaError_t launch_batch(const Weights<T>& W, const typename rows2d<T>::type& Bt, const BatchStage& S, int nsm,
                          cudaStream_t st) {
-  if (S.bar_extra == 0) {
+  if (!S.persistent) {
     if (S.stage == 0) {
       if (!S.dt_in) {
         batch_bounds_kernel<<<S.n_rec, RB, 0, st>>>(S);

@@ -74,6 +74,7 @@ struct hweno_s {
   int stage_a = 0;               // hweno_stage: rotation of the step in progress
   double stage_dt = 0.0;         // hweno_stage: its dt
   unsigned long long spin_limit = hw::BARRIER_SPIN_DEFAULT;   // grid-barrier wait bound
+  bool persistent = false;       // batched stages as one persistent launch (hweno_batch_set_barrier)
   unsigned bar_extra = 0;        // extra arrivals the barrier waits for (timeout-path tests)
 };
 
@@ -1311,6 +1312,7 @@ hweno_status hweno_batch_set_barrier(hweno_t h, long long spin_limit, int extra_
     return fail(h, HWENO_EINVAL, "batch_set_barrier: need spin_limit >= 1 and 0 <= extra_arrivals <= 1024");
   h->spin_limit = (unsigned long long)spin_limit;
   h->bar_extra = (unsigned)extra_arrivals;
+  h->persistent = true;
   drop_graphs(h);
   return HWENO_OK;
 }
@@ -1363,7 +1365,7 @@ cudaError_t batch_enqueue(hweno_t h, int a, const double* dt_in, double cfl, cud
     S.speeds = h->speeds; S.bounds = reinterpret_cast<unsigned*>(h->speeds + 2 * h->nprob);
     S.dt_in = dt_in; S.dt_out = h->dt_out; S.cfl = cfl;
     S.status = h->B.status; S.pstatus = h->pstatus; S.bar = h->bar; S.stage = k;
-    S.spin_limit = h->spin_limit; S.bar_extra = h->bar_extra; S.Un = h->U[a];
+    S.spin_limit = h->spin_limit; S.bar_extra = h->bar_extra; S.persistent = h->persistent; S.Un = h->U[a];
     const int in = k == 0 ? a : (k == 1 ? b : c), out = k == 1 ? c : b;
     S.Uin = h->U[in]; S.Uout = h->U[out]; S.U32in = h->U32[in]; S.U32out = h->U32[out];
     S.cA = k == 0 ? 0.0 : (k == 1 ? 0.75 : 1.0 / 3.0); S.cB = k == 0 ? 1.0 : (k == 1 ? 0.25 : 2.0 / 3.0);

@@ -152,6 +152,7 @@ struct BatchStage {
   unsigned* pstatus;      // per problem: ST_NONFINITE / ST_NONPOSITIVE of its new state
   unsigned* bar;          // grid barrier {arrived, generation}
   unsigned long long spin_limit;   // polls (64 ns sleeps each) before a barrier wait gives up
+  int persistent;         // one cooperative launch a stage, its phases behind grid barriers (else a launch per phase)
   unsigned bar_extra;     // arrivals a barrier waits for beyond the launched blocks (0; > 0 only to
                           //    exercise the timeout path)
 };

@@ -572,8 +572,9 @@ class BatchSolver:
         self._check(lib().hweno_batch_set_tile(self._h, int(variant)))
 
     def set_barrier(self, spin_limit=1 << 26, extra_arrivals=0):
-        """Bound of the grid barrier's waits; extra_arrivals > 0 makes every wait
-        run out (the timeout path: the next synchronising call raises ETIMEOUT)."""
+        """One persistent launch per stage from the next step on, with this bound of its
+        grid barrier's waits; extra_arrivals > 0 makes every wait run out (the timeout
+        path: the next synchronising call raises ETIMEOUT)."""
         self._check(lib().hweno_batch_set_barrier(self._h, int(spin_limit), int(extra_arrivals)))
 
     def uses_graph(self):
