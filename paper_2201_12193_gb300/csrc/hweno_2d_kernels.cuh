@@ -1226,8 +1226,8 @@ __device__ __forceinline__ double batch_dt(const BatchStage& A, const Prob& P, i
 }
 
 // Quarters [q0, q1) of the item's 128 cells (fixed-point precisions: 32 cells at a
-// time, a warp per variable and then per face).
-template <typename T>
+// time, a warp per variable and then per face).  S32: from the float copy of the state.
+template <typename T, bool S32>
 __device__ __forceinline__ void batch_rec_item(const BatchStage& A, const Prob& P, const BProb& Q, int it, int tid,
                                                const Weights<T>& W, const typename rows2d<T>::type& B, int q0 = 0,
                                                int q1 = 4) {
@@ -1245,8 +1245,8 @@ __device__ __forceinline__ void batch_rec_item(const BatchStage& A, const Prob& 
   } else {
     const int cell = (it - Q.rec_first) * RB + tid;
     if (cell < P.nx * P.ny)
-      rec2d_cell<T, 4, REC_PLAIN, false, true>(P, W, B, A.Uin + Q.uoff, nullptr, nullptr, cell % P.nx, cell / P.nx, G,
-                                               aux, A.U32in + Q.uoff);
+      rec2d_cell<T, 4, REC_PLAIN, false, S32>(P, W, B, A.Uin + Q.uoff, nullptr, nullptr, cell % P.nx, cell / P.nx, G,
+                                              aux, S32 ? A.U32in + Q.uoff : nullptr);
   }
 }
 
@@ -1265,10 +1265,10 @@ __device__ __forceinline__ void batch_flag_item(const BatchStage& A, const Prob&
   }
 }
 
-template <typename T>
+template <typename T, bool S32>
 __device__ __forceinline__ void batch_rerec(const BatchStage& A, const Weights<T>& W,
                                             const typename rows2d<T>::type& B) {
-  constexpr bool S32 = std::is_same<T, float>::value, FXD = fixed2d<T>::value;
+  constexpr bool FXD = fixed2d<T>::value;
   const int n = *(volatile int*)A.count;
   // a thread per cell, or (fixed-point precisions) a warp per variable of 32 cells
   const int per = FXD ? 32 : RB, w = threadIdx.x >> 5;
@@ -1291,7 +1291,7 @@ __device__ __forceinline__ void batch_update_item(const BatchStage& A, const Pro
   const int t = it - Q.upd_first;
   Rk S{A.Uin + Q.uoff, A.Un + Q.uoff, A.Uout + Q.uoff, A.mask + Q.coff, A.Mod + Q.moff,
        A.maskN ? A.maskN + Q.coff : nullptr, A.ModN ? A.ModN + Q.moff : nullptr, dt, A.cA, A.cB,
-       nullptr, nullptr, A.pstatus + p, nullptr, std::is_same<T, float>::value ? A.U32out + Q.uoff : nullptr};
+       nullptr, nullptr, A.pstatus + p, nullptr, std::is_same<T, float>::value && A.U32out ? A.U32out + Q.uoff : nullptr};
   update2d_tile<T, 4, TXV, TYV>(P, GlobalSrc<T>{(const T*)A.G + Q.goff}, S, (t % Q.tiles_x) * TXV,
                                 (t / Q.tiles_x) * TYV, tid, xf, yf);
 }
@@ -1330,7 +1330,7 @@ __global__ void batch_dt_kernel(const __grid_constant__ BatchStage A) {
   if (p < A.nprob) A.dt_out[p] = batch_dt(A, A.probs[p].P, p);
 }
 
-template <typename T>
+template <typename T, bool S32>
 __global__ void __launch_bounds__(RB, (is_df64<T>::value ? 4 : std::is_same<T, float>::value ? 8 : 5))
     batch_rec_kernel(const __grid_constant__ BatchStage A, const __grid_constant__ Weights<T> W,
                      const __grid_constant__ typename rows2d<T>::type B) {
@@ -1338,7 +1338,7 @@ __global__ void __launch_bounds__(RB, (is_df64<T>::value ? 4 : std::is_same<T, f
   const int it = fixed2d<T>::value ? blockIdx.x >> 2 : blockIdx.x, q = blockIdx.x & 3;
   const BProb& Q = A.probs[A.rec_owner[it]];
   stage_prob(Q, &sp, threadIdx.x);
-  batch_rec_item<T>(A, sp, Q, it, threadIdx.x, W, B, q, q + 1);
+  batch_rec_item<T, S32>(A, sp, Q, it, threadIdx.x, W, B, q, q + 1);
 }
 
 template <typename T>
@@ -1350,11 +1350,11 @@ __global__ void __launch_bounds__(RB) batch_flag_kernel(const __grid_constant__ 
   batch_flag_item<T>(A, sp, Q, p, it, threadIdx.x);
 }
 
-template <typename T>
+template <typename T, bool S32>
 __global__ void __launch_bounds__(RB) batch_rerec_kernel(const __grid_constant__ BatchStage A,
                                                          const __grid_constant__ Weights<T> W,
                                                          const __grid_constant__ typename rows2d<T>::type B) {
-  batch_rerec<T>(A, W, B);
+  batch_rerec<T, S32>(A, W, B);
 }
 
 template <typename T, int TXV, int TYV>
@@ -1375,6 +1375,7 @@ __global__ void __launch_bounds__(TXV * TYV) batch_stage_kernel(const __grid_con
                                                                 const __grid_constant__ Weights<T> W,
                                                                 const __grid_constant__ typename rows2d<T>::type B) {
   static_assert(TXV * TYV == RB, "tiles and rows use the same block");
+  constexpr bool FP32 = std::is_same<T, float>::value;
   __shared__ T xf[TYV][TXV + 1][4][4];
   __shared__ T yf[TYV + 1][TXV][4][4];
   const int tid = threadIdx.x;
@@ -1390,7 +1391,8 @@ __global__ void __launch_bounds__(TXV * TYV) batch_stage_kernel(const __grid_con
   // Step 1: every cell
   for (int it = blockIdx.x; it < A.n_rec; it += nb) {
     const BProb& Q = A.probs[A.rec_owner[it]];
-    batch_rec_item<T>(A, Q.P, Q, it, tid, W, B);
+    if (FP32 && A.U32in) batch_rec_item<T, FP32>(A, Q.P, Q, it, tid, W, B);
+    else batch_rec_item<T, false>(A, Q.P, Q, it, tid, W, B);
   }
   grid_barrier(A.bar, nb + A.bar_extra, A.status, A.spin_limit);
   // Steps 2.1-2.2
@@ -1400,7 +1402,8 @@ __global__ void __launch_bounds__(TXV * TYV) batch_stage_kernel(const __grid_con
   }
   grid_barrier(A.bar, nb + A.bar_extra, A.status, A.spin_limit);
   // Step 2.3: troubled cells
-  batch_rerec<T>(A, W, B);
+  if (FP32 && A.U32in) batch_rerec<T, FP32>(A, W, B);
+  else batch_rerec<T, false>(A, W, B);
   grid_barrier(A.bar, nb + A.bar_extra, A.status, A.spin_limit);
   // Step 3: fluxes, quadrature, L, Runge-Kutta
   for (int it = blockIdx.x; it < A.n_upd; it += nb) {
@@ -1429,9 +1432,13 @@ cudaError_t launch_batch(const Weights<T>& W, const typename rows2d<T>::type& Bt
       }
       batch_dt_kernel<<<(S.nprob + 127) / 128, 128, 0, st>>>(S);
     }
-    batch_rec_kernel<T><<<fixed2d<T>::value ? 4 * S.n_rec : S.n_rec, RB, 0, st>>>(S, W, Bt);
+    constexpr bool FP32 = std::is_same<T, float>::value;
+    const bool copy = FP32 && S.U32in;
+    if (copy) batch_rec_kernel<T, FP32><<<S.n_rec, RB, 0, st>>>(S, W, Bt);
+    else batch_rec_kernel<T, false><<<fixed2d<T>::value ? 4 * S.n_rec : S.n_rec, RB, 0, st>>>(S, W, Bt);
     batch_flag_kernel<T><<<S.n_rec, RB, 0, st>>>(S);
-    batch_rerec_kernel<T><<<nsm * 8, RB, 0, st>>>(S, W, Bt);
+    if (copy) batch_rerec_kernel<T, FP32><<<nsm * 8, RB, 0, st>>>(S, W, Bt);
+    else batch_rerec_kernel<T, false><<<nsm * 8, RB, 0, st>>>(S, W, Bt);
     batch_update_kernel<T, TXV, TYV><<<S.n_upd, RB, 0, st>>>(S);
     return cudaGetLastError();
   }

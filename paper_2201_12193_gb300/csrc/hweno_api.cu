@@ -24,7 +24,8 @@ struct hweno_s {
   hw::HostTabs T{};
   int fp32 = 0;                  // compute precision (hw::PREC_*)
   double* U[3] = {nullptr, nullptr, nullptr};
-  float* U32[3] = {nullptr, nullptr, nullptr};   // FP32 form (single 2D handles): float copies of U[k]
+  float* U32[3] = {nullptr, nullptr, nullptr};   // FP32 form (2D): float copies of U[k]; a batch does without
+                                                 //    where they do not fit
   CUtensorMap tmG{};             // FP32 2D Euler: tensor map of the point values (TMA-staged update)
   bool tma_ok = false;           // the map is encoded
   bool tma_on = false;           // the update kernel uses it (hweno_set_tma; off by default)
@@ -1206,8 +1207,6 @@ hweno_status hweno_create_batch(const hweno_grid* grids, const hweno_bc* bcs, in
   h->tile_variant = 0;
   layout_batch(h);
   ok = ok && cudaMalloc(&h->owner, (h->n_rec + most) * sizeof(int)) == cudaSuccess;
-  for (int k = 0; k < 3 && h->fp32 == hw::PREC_FP32; ++k)
-    ok = ok && cudaMalloc(&h->U32[k], tu * sizeof(float)) == cudaSuccess;
   ok = ok && cudaMalloc(&h->dt_out, n * sizeof(double)) == cudaSuccess;
   ok = ok && cudaMalloc(&h->bar, 2 * sizeof(unsigned)) == cudaSuccess;
   ok = ok && cudaMalloc(&h->pstatus, n * sizeof(unsigned)) == cudaSuccess;
@@ -1219,6 +1218,14 @@ hweno_status hweno_create_batch(const hweno_grid* grids, const hweno_bc* bcs, in
     delete h;
     fprintf(stderr, "hweno_create_batch: device allocation failed\n");
     return HWENO_ENOMEM;
+  }
+  if (h->fp32 == hw::PREC_FP32) {   // last: without them the kernels convert the state's doubles as they gather
+    bool fits = true;
+    for (int k = 0; k < 3; ++k) fits = fits && cudaMalloc(&h->U32[k], tu * sizeof(float)) == cudaSuccess;
+    if (!fits) {
+      cudaGetLastError();
+      for (int k = 0; k < 3; ++k) { cudaFree(h->U32[k]); h->U32[k] = nullptr; }
+    }
   }
   upload_layout(h);
   cudaMemset(h->B.status, 0, sizeof(unsigned));
