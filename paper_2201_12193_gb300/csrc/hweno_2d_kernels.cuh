@@ -267,7 +267,7 @@ __device__ __forceinline__ void rec2d_cell(const Prob& P, const Weights<T>& W,
 // reconstructed a second time.  A thread per cell: FP32, plain double and the
 // scalar laws.  FP32 with the float copy: 8 blocks (64 registers, 164 B of spills)
 // measured 0.545 ms per 2048^2 launch against 0.685 at 4 blocks (119 registers).
-template <typename T, int NV, int MODE, bool FIX = false, bool S32 = false>
+template <typename T, int NV, int MODE, bool S32 = false>
 __global__ void __launch_bounds__(RB, (std::is_same<T, float>::value ? 8 : fixed2d<T>::value ? 4 : 1)) rec2d_kernel(
     const __grid_constant__ Prob P, const __grid_constant__ Weights<T> W,
     const __grid_constant__ typename rows2d<T>::type B, const double* __restrict__ U,
@@ -282,8 +282,7 @@ __global__ void __launch_bounds__(RB, (std::is_same<T, float>::value ? 8 : fixed
   if (FLAGGED && rerec && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(rerec, (unsigned long long)n);
   for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
     const int cell = FLAGGED ? list[t] : (int)t;
-    if (FIX && is_solid(P, cell % P.nx, cell / P.nx)) continue;   // solid cells are images, never read
-    rec2d_cell<T, NV, MODE, FIX, S32>(P, W, B, U, mask, Mod, cell % P.nx, cell / P.nx, G, aux, U32);
+    rec2d_cell<T, NV, MODE, false, S32>(P, W, B, U, mask, Mod, cell % P.nx, cell / P.nx, G, aux, U32);
     if constexpr (fixed2d<T>::value && !FLAGGED) face_partials<T, NV>(P, G, aux, goff(P, cell % P.nx, cell / P.nx), 0, 4);
   }
 }
@@ -1039,16 +1038,16 @@ __global__ void __launch_bounds__(TX * TY, 4) update2d_tma_kernel(Prob P, const 
 namespace hw {
 namespace {
 
-// Fixed-state ghosts are supported for 2D Euler in FP64 (the library rejects
-// other combinations), so only that instantiation carries the FIX variant.
+// Fixed-state ghosts and the solid block are supported for 2D Euler in FP64 without the
+// learned indicator (the library rejects other combinations), so only fx64's split kernel
+// carries the FIX variant.
 template <typename T, int NV, int MODE>
 void launch_rec2d(int blocks, cudaStream_t st, const Prob& P, const Weights<T>& W, const typename rows2d<T>::type& Bt,
                   const double* U, const uint8_t* mask, const double* Mod, const int* list, const int* count, T* G,
                   T* aux, unsigned long long* rerec, const float* U32 = nullptr) {
   if constexpr (std::is_same<T, float>::value) {
     if (U32) {   // FP32 form with the float copy of the state: no per-moment conversion
-      rec2d_kernel<T, NV, MODE, false, true><<<blocks, RB, 0, st>>>(P, W, Bt, U, mask, Mod, list, count, G, aux,
-                                                                    rerec, U32);
+      rec2d_kernel<T, NV, MODE, true><<<blocks, RB, 0, st>>>(P, W, Bt, U, mask, Mod, list, count, G, aux, rerec, U32);
       return;
     }
   }
