@@ -142,7 +142,7 @@ __device__ __forceinline__ double mod1(double uL, double uR, double vL, double v
   return MOD_WU * (uR - uL) + MOD_WV * (vL + vR);
 }
 
-// Point velocity (rho u) / rho; fx64 by the three-operation reciprocal.
+// Point velocity (rho u) / rho; fx64 by the integer reciprocal.
 template <typename T>
 __device__ __forceinline__ T vel1(T m, T rho) {
   if constexpr (std::is_same<T, fx64>::value) return m * rcp(rho);

@@ -1,4 +1,4 @@
-// Batched persistent stage: FP64 and FP32-bulk instantiations, and the dispatch.
+// Batched stage: FP64 and FP32-bulk instantiations, and the dispatch.
 #include "hweno_2d_kernels.cuh"
 
 namespace hw {

@@ -1,4 +1,4 @@
-// Batched persistent stage: double-float instantiations.
+// Batched stage: double-float instantiations.
 #include "hweno_2d_kernels.cuh"
 
 namespace hw {

@@ -1,5 +1,5 @@
-// Kernels of the two-dimensional stage pipeline and of the batched persistent
-// stage (shared by the per-precision translation units; internal linkage).
+// Kernels of the two-dimensional stage pipeline and of the batched stage (shared
+// by the per-precision translation units; internal linkage).
 #pragma once
 #include <algorithm>
 #include <type_traits>
@@ -937,8 +937,9 @@ __global__ void __launch_bounds__(2 * TX * TY, 2)
   if (nonphysical(avg[0][c], avg[1][c], avg[2][c], avg[3][c])) atomicOr(S.status, ST_NONPOSITIVE);
 }
 
-// Tiles per block: as many as leave six waves of 4 resident blocks per SM, at
-// most 16; small grids keep one, their blocks must reach every SM first.
+// Tiles per block: as many as leave six waves of 4 blocks per SM (the kernels hold
+// 3 in plain double, 4 with the solid block, 5 in fx64 and double-float: five waves or
+// more), at most 16; small grids keep one, their blocks must reach every SM first.
 template <typename T>
 inline int update_sweep(const Prob& P) {
   if (std::is_same<T, float>::value) return 1;
@@ -1153,8 +1154,9 @@ void stage_t(const Prob& P, const HostTabs& HT, const Weights<T>& W, const Beta2
 // Work items of all problems form one list per phase (128-cell rows for the
 // per-cell phases, update tiles for the flux phase).  A stage runs a launch per
 // phase, or one persistent cooperative launch whose resident blocks stride over
-// the lists, phases separated by a grid barrier.  The barrier's wait is bounded: past the limit the block records ST_TIMEOUT and continues (the host
-// reports HWENO_ETIMEOUT), so no wait can hang the GPU.
+// the lists, phases separated by a grid barrier.  The barrier's wait is bounded:
+// past the limit the block records ST_TIMEOUT and continues (the host reports
+// HWENO_ETIMEOUT), so no wait can hang the GPU.
 
 // nblocks: arrivals that release the barrier; limit: polls before the wait gives up.
 __device__ __forceinline__ void grid_barrier(unsigned* bar, unsigned nblocks, unsigned* status,

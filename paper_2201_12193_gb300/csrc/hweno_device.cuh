@@ -1162,10 +1162,11 @@ __device__ __forceinline__ bool nonphysical(double rho, double m, double n, doub
 // Bounds of an Euler average's |velocity| + sound speed per direction from FP32
 // copies: lo <= exact <= hi.  Truncating the conserved values and the FP32
 // arithmetic err by less than 2^-20 relative, the pressure by 2^-20 of E + kinetic
-// energy (gamma - 1 is rounded from FP64: in FP32 it cancels near 1).  What falls below FP32's normal range (a momentum, its product with the
-// velocity) is below 1e-38 absolute, which density, E and the squared sound speed inside the
-// limits leave far below those margins.  Outside them, and for a non-physical or barely
-// physical average, hi = infinity and lo = 0: the cell takes the exact speed.
+// energy (gamma - 1 is rounded from FP64: in FP32 it cancels near 1).  What falls
+// below FP32's normal range (a momentum, its product with the velocity) is below
+// 1e-38 absolute, which density, E and the squared sound speed inside the limits leave
+// far below those margins.  Outside them, and for a non-physical or barely physical
+// average, hi = infinity and lo = 0: the cell takes the exact speed.
 __device__ __forceinline__ void speed_bounds(const Prob& P, const double* __restrict__ U, int i, int j, float (&lo)[2],
                                              float (&hi)[2]) {
   const float r = f32_trunc(U[sidx(P, 0, 0, i, j)]), m = f32_trunc(U[sidx(P, 1, 0, i, j)]);

@@ -7,10 +7,12 @@
 // run in integers: the stencil data of one variable share an exponent and are
 // held as 57-bit integers, a coefficient is a 64-bit integer, and one
 // multiply-add is three 32 x 32 -> 64 products (the low x low one, below the
-// last place kept, is left out): 0.05 clocks per SM against 0.5.  The data are deviations from the target
-// cell's average, so their common exponent is that of the variation: the
-// rounding is 2^-55 to 2^-57 of the largest deviation (FP64's is 2^-53 of the
-// largest datum).  Nonlinear parts stay FP64.
+// last place kept, is left out): 0.05 clocks per SM against 0.5.  The data are
+// deviations from the target cell's average, so their common exponent is that of the
+// variation: the rounding is 2^-55 to 2^-57 of the largest deviation (FP64's is 2^-53
+// of the largest datum).  Data of which a level q_l takes only a part have an exponent
+// per level where their sizes differ (fx_uneven in hweno_device.cuh).  Nonlinear
+// parts stay FP64.
 #pragma once
 
 #include <cuda_runtime.h>

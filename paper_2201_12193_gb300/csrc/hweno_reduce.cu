@@ -69,10 +69,9 @@ __device__ __forceinline__ void advance_dt(const Prob& P, double ax, double ay, 
   st[1] = dt;
 }
 
-// Largest |f'| (scalars) or |velocity| + sound speed (Euler) per direction,
-// from cell averages.  A non-physical average yields +inf (dt = 0).  With the
+// The exact speeds of one cell average: |f'| (scalars) or |velocity| + sound speed
+// (Euler) per direction.  A non-physical average yields +inf (dt = 0).  With the
 // positivity check off the sound speed uses max(p, 0).
-// The exact speeds of one cell average.
 __device__ __forceinline__ void speeds_of(const Prob& P, const double* __restrict__ U, int i, int j, double& sx, double& sy) {
   if (P.eq == EQ_ADV) { sx = fabs(P.adv_a); sy = fabs(P.adv_b); }
   else if (P.eq == EQ_BURGERS) { sx = sy = fabs(U[sidx(P, 0, 0, i, j)]); }
@@ -86,7 +85,7 @@ __device__ __forceinline__ void speeds_of(const Prob& P, const double* __restric
   }
 }
 
-// The last block to arrive (part[4 MAXB] counts them and returns to 0) reduces the
+// The largest speeds over the cells.  The last block to arrive (part[4 MAXB] counts them and returns to 0) reduces the
 // blocks' partials to out[0..1], copies the status word to out[2] (the host then reads
 // speeds and status at once) and, with par set, forms hweno_advance's step
 // length: one launch where the partials, their reduction and the step length took
