@@ -10,8 +10,8 @@ update).  value = cells * 3 stages * steps / device time, FP64 (the scheme as
 specified).  Under "forms": the FP32-bulk and double-float forms (relative L1
 difference to FP64), the 1D Shu-Osher problem run whole (device-driven against
 the host loop; FP32-bulk and double-float beside FP64 with the N = 4000 vs 8000
-resolution gap), the batched form (256 problems of uneven size, one persistent
-launch per stage, CUDA graph), and the learned-indicator form on 4096^2 blast
+resolution gap), the batched form (256 problems of uneven size, a launch per
+phase, CUDA graph), and the learned-indicator form on 4096^2 blast
 data against the plain scheme on the same data (throughputs, network roofline,
 recall / miss / false-alarm rates against KXRCF, L1 drift).  --full-run adds the
 2048^2 problem run whole to t = 0.25 in FP64 and FP32-bulk.
@@ -57,11 +57,12 @@ def _rec_flop_per_cell(nvar=4):
     with open(os.path.join(ROOT, "paper_2201_12193_gb300", "csrc", "hweno_parity.h")) as f:
         sbv = int(re.search(r"D2_FLOP_SBV = (\d+);", f.read()).group(1))
     return nvar * (sbv + 112) + 44
-# FP64-pipe operations per cell of one launch on four-quadrant data, executed and
-# counted by ncu (smsp__inst_executed_pipe_fp64.sum x 32 / cells, 1024^2): the linear
-# part, divisions, roots and most products of the FP64 kernels are integer work, so
-# the pipe's own operations, not the algorithmic flop, stand against its rate.
-FP64_PIPE_OPS_PER_CELL = {"reconstruct": 504.0, "update": 544.4}
+# The FP64 kernels' linear part, divisions, roots and most products are integer work, so
+# the FP64 pipe's own operations, not the algorithmic flop, stand against its rate:
+# counted by ncu (smsp__inst_executed_pipe_fp64.sum x 32 / cells, 1024^2, mean of a
+# step's three launches), in profiles/dram_traffic.json beside the traffic.
+FP64_KERNELS = {"reconstruct": ("rec2d_fp64", "rec2d_split_kernel<fx64>"),
+                "update": ("update2d_fp64", "update2d_kernel<fx64,4>")}
 # algorithmic HBM bytes per cell-stage: read U^(k) (12 doubles), read U^n for stages 2-3, write U^(k+1)
 ALGO_BYTES_PER_CELL_STAGE = 12 * 8 * (1 + 2.0 / 3.0 + 1)
 
@@ -277,10 +278,15 @@ def run_solver(torch, hweno, p, precision, steps, warmup, world, profile=False, 
     return s, ms, prof, clk, out
 
 
+# kernels of one batched step with CFL step lengths: bounds, speeds and step lengths, then
+# reconstruction, indicator, second reconstruction and update in each of three stages
+BATCH_LAUNCHES_PER_STEP = 3 + 3 * 4
+
+
 def run_batched(torch, hweno, args, world, rank):
     """The batched form: 256 independent problems (sizes seeded uniformly in
     {64,128,256,512}^2; four-quadrant on [0,1]^2 and isentropic vortices on periodic
-    [0,10]^2), one persistent launch per RK stage replayed from a CUDA graph, the
+    [0,10]^2), a launch per phase of each RK stage replayed from a CUDA graph, the
     update tile picked by the autotuner; FP32 bulk, and FP64 for the L1 comparison."""
     from paper_2201_12193_gb300 import autotune, workloads as W
     probs = W.batch_problems(256, seed=rank, npts=2)
@@ -340,7 +346,7 @@ def run_batched(torch, hweno, args, world, rank):
         s.close()
         out[f"batched_{prec}"] = {"value": aggregate(cells, 3, steps, world, ms), "ms_per_step": ms / steps,
                                   "problems": len(probs), "cells": cells, "graph": graph,
-                                  "tile": autotune.VARIANTS[variant], "launches_per_step": 3}
+                                  "tile": autotune.VARIANTS[variant], "launches_per_step": BATCH_LAUNCHES_PER_STEP}
     den = sum(float(np.abs(b).sum()) for b in finals["fp64"])
     for prec in ("fp32", "df64"):
         num = sum(float(np.abs(a - b).sum()) for a, b in zip(finals[prec], finals["fp64"]))
@@ -380,10 +386,10 @@ def source_hash(sources=KERNEL_SOURCES):
     return h.hexdigest()
 
 
-def traffic_per_cell(kernel, table="dram_traffic.json", sources=KERNEL_SOURCES):
-    """DRAM bytes per cell of one launch of `kernel` from the committed ncu
-    figures (profiles/<table>), or None when the kernel sources changed since
-    that capture."""
+def traffic_per_cell(kernel, table="dram_traffic.json", sources=KERNEL_SOURCES, figure="bytes_per_cell"):
+    """DRAM bytes per cell (or another figure) of one launch of `kernel` from the
+    committed ncu figures (profiles/<table>), or None when the kernel sources changed
+    since that capture."""
     try:
         with open(os.path.join(ROOT, "profiles", table)) as f:
             d = json.load(f)
@@ -392,7 +398,7 @@ def traffic_per_cell(kernel, table="dram_traffic.json", sources=KERNEL_SOURCES):
     k = d.get("kernels", {}).get(kernel)
     if not k or d.get("source_sha256") != source_hash(sources):
         return None
-    return float(k["bytes_per_cell"])
+    return float(k[figure]) if figure in k else None
 
 
 def _peaks():
@@ -915,19 +921,19 @@ def run_ours(args, world, rank, local):
     kind, (kms, kn) = max(prof.items(), key=lambda kv: kv[1][0])
     total_kernel_ms = sum(v[0] for v in prof.values())
     roof = None
-    if args.precision == "fp64" and kind in FP64_PIPE_OPS_PER_CELL:
-        ops = FP64_PIPE_OPS_PER_CELL[kind]
-        achieved = ops * cells * kn / (kms * 1e-3)
-        pk = peaks["fp64_tflops"] * 1e12 / 2                # one FMA is one operation
-        name = "rec2d_split_kernel<fx64>" if kind == "reconstruct" else "update2d_kernel<fx64,4>"
-        roof = {"bound": "alu", "kernel": f"{name} ({kind})", "achieved": achieved / 1e12, "peak": pk / 1e12,
-                "unit": "T FP64-pipe operations/s", "frac": achieved / pk,
+    if args.precision == "fp64" and kind in FP64_KERNELS:
+        key, name = FP64_KERNELS[kind]
+        ops = traffic_per_cell(key, figure="fp64_pipe_ops_per_cell")   # None: not counted on these sources
+        rate = ops * cells * kn / (kms * 1e-3) / 1e12 if ops else None
+        pk = peaks["fp64_tflops"] / 2                       # one FMA is one operation
+        roof = {"bound": "alu", "kernel": f"{name} ({kind})", "achieved": rate, "peak": pk,
+                "unit": "T FP64-pipe operations/s", "frac": rate / pk if ops else None,
                 "peak_source": "FP64 FMA rate measured in this run by hweno_alu_probe (of measured), an FMA one operation; "
                                f"nominal from unit counts {peaks['fp64_nominal_tflops'] / 2:.3f}",
-                "frac_of_nominal_fp64": achieved / (peaks["fp64_nominal_tflops"] * 0.5e12),
+                "frac_of_nominal_fp64": rate / (peaks["fp64_nominal_tflops"] / 2) if ops else None,
                 "fp64_pipe_ops_per_cell": ops, "traffic": None, "launches": kn, "avg_ms": kms / kn,
                 "share": kms / total_kernel_ms}
-        bpc = traffic_per_cell(("rec2d" if kind == "reconstruct" else "update2d") + "_fp64")
+        bpc = traffic_per_cell(key)
     elif kind == "reconstruct":
         flop = _rec_flop_per_cell(s64.nvar) * cells * kn
         achieved = flop / (kms * 1e-3)
@@ -945,7 +951,7 @@ def run_ours(args, world, rank, local):
     hbm = {"algorithmic_GBps": ALGO_BYTES_PER_CELL_STAGE * cells * 3 * args.steps / (ms * 1e-3) / 1e9,
            "peak_GBps": hbm_gbps, "peak_source": hbm_src}
     hbm["frac"] = hbm["algorithmic_GBps"] / hbm["peak_GBps"]
-    launches = sum(v[1] for v in prof.values()) + 2 * args.steps     # + wave-speed reduction kernels
+    launches = sum(v[1] for v in prof.values()) + args.steps     # + the wave-speed kernel of max_dt
     s64.close()
 
     forms = {}
