@@ -293,10 +293,11 @@ __global__ void __launch_bounds__(RB, (std::is_same<T, float>::value ? 8 : fixed
 // (ms per launch, FP64): 64^2 0.065 -> 0.021, 256^2 0.123 -> 0.105, 2048^2
 // 5.67 -> 5.52 (18.1 with the linear part in FP64), troubled cells 0.13 -> 0.11;
 // double-float 2048^2 5.44 -> 5.24 (7.6 in pairs); with the reciprocals and the
-// indicators' squares in integers 4.39 and 4.67.  FP64: 5 resident blocks per SM;
-// 504 FP64 operations per cell (2330 before), that pipe 76 % busy beside 19.8 k
-// integer instructions.  Double-float: 30 k instructions per cell, the ALU
-// 45 % busy (1.2 % faster at 5 blocks than at 4 with 120 registers); weights in FP64
+// indicators' squares in integers 4.39 and 4.67; with the stencils of uneven data
+// and the reciprocals rounded to nearest 4.51 and 4.72.  FP64: 5 resident blocks per
+// SM; 504 FP64 operations per cell (2330 before), that pipe 74 % busy, 20.4 k
+// instructions.  Double-float: 25.1 k instructions per cell, issue 56 %, the ALU
+// 37 % busy (1.2 % faster at 5 blocks than at 4 with 120 registers); weights in FP64
 // beside the integers measured alike.
 template <typename T, int MODE, bool FIX = false>
 __global__ void __launch_bounds__(RB, 5) rec2d_split_kernel(
@@ -846,8 +847,9 @@ __device__ __forceinline__ void update2d_tile(const Prob& P, const Src& src, con
 // fx64 at 2048^2: 15.2 ms per launch with hllc and the quadrature per point, 9.6
 // with hllc_lean and update_cell_lean, 8.07 with the integer compares, the 5-operation
 // root and the sweep, 5.8 with roots and reciprocals and 4.7 with the flux's products
-// in integers (4.8 at 4 blocks per SM): 600 FP64 operations per cell of 1915, the
-// FP64 pipe still 90 % busy.  Double-float 5.2 -> 3.0 ms; at 1024^2 0.78 -> 0.74 with
+// in integers (4.8 at 4 blocks per SM): 540 FP64 operations per cell of 1915 (mean of
+// the three stages), the FP64 pipe still 80 % busy, 0.92 of the rate that chains of
+// independent FMAs reach.  Double-float 5.2 -> 2.9 ms; at 1024^2 0.78 -> 0.74 with
 // 5 blocks per SM for 4.
 template <typename T, int NV, bool SOLID = false>
 __global__ void __launch_bounds__(TX * TY, (std::is_same<T, float>::value ? 8
