@@ -538,8 +538,8 @@ def run_shu_osher_long(torch, hweno, world, hbm_gbps, hbm_src, nx=1 << 24):
             "bound": "hbm", "achieved": gbs, "peak": hbm_gbps, "unit": "GB/s", "frac": gbs / hbm_gbps,
             "peak_source": hbm_src, "bytes_per_cell": FUSED1D_BYTES_PER_CELL, "avg_ms": f_ms / f_n,
             "traffic": t * nx if t else None,
-            "note": "the FP64 pipe, not HBM, binds: ncu shows it 72 % busy (the Runge-Kutta combination and "
-                    "the flux differences of the average equation stay in FP64)"}
+            "note": "issue (70 to 79 %) and the FP64 pipe (44 to 56 % busy: the Runge-Kutta combination and the flux "
+                    "differences of the average equation), not HBM, bind"}
     return {"shu_osher_1d_long_fp32": out}
 
 

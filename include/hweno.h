@@ -77,6 +77,9 @@ typedef enum {
  *   split with double-float arithmetic (pairs of FP32 numbers, a 48-bit
  *   significand and FP32's exponent range; magnitudes below 2^-74 keep FP32
  *   precision) in place of FP32.
+ *   Precision 0 computes with normal numbers: intermediate results below 2^-1022
+ *   become 0, reciprocals and roots of subnormal or infinite numbers NaN; the
+ *   nonlinear weights overflow (NaN) for variations from about 1e27 on.
  *   indicator: HWENO_IND_KXRCF is the scheme (HWENO6-M5-I); NONE gives HWENO6
  *   (no modification); ALL gives HWENO6-M5-NI (every cell modified) (Sec. 3);
  *   MLP: the learned indicator with KXRCF fallback (see below; 2D Euler).
