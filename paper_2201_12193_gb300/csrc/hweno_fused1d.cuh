@@ -243,14 +243,11 @@ __global__ void __launch_bounds__(NT) fused1d_kernel(const __grid_constant__ Pro
       const int c = t - QF, p = 4 + c;
       if (i0 + c >= P.nx) continue;
       T u[4][NV], Fq[NV];
-      double ub[NV];
 #pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        ub[v] = sm.U[2 * v][p];
+      for (int v = 0; v < NV; ++v)
 #pragma unroll
         for (int k = 0; k < 4; ++k) u[k][v] = sm.G[v * 4 + k][p];
-      }
-      quad1<T, NV>(P, u, ub, Fq);
+      quad1<T, NV>(P, u, Fq);
 #pragma unroll
       for (int v = 0; v < NV; ++v) sm.UT[v][p] = Fq[v];
     }
